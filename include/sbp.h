@@ -210,7 +210,10 @@ int sbp_step_graph(sbp_handle* h, int nsteps, double dt, void* stream);
 
 /* Device bytes a handle for `desc` holds after sbp_grid_create, sbp_set_material and
  * sbp_set_state (fields, coefficients, metric, closure matrices of D_xx^FC, face buffers and
- * interface traces, tensor maps), used to admit solves by HBM footprint.  No device work. */
+ * interface traces, tensor maps), used to admit solves by HBM footprint.  No device work.  FP64
+ * handles keep 18 more planes (order 6; 12 / 6 for order 4 / 2) of interior edge weights where the
+ * device has eight times that much memory free at sbp_grid_create, and give them back when a later
+ * allocation of the handle finds no room; they are not counted. */
 int sbp_grid_footprint(const sbp_grid_desc* desc, long long* bytes_out);
 
 /* Pick the launch tuning for this grid by timing candidates on leapfrog steps from the current

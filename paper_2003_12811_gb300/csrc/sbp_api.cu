@@ -70,6 +70,8 @@ struct HostBlock {
     void* lscr = nullptr;     // leapfrog: the dissipation of the listed nodes between the pre and post kernels
     void* mx = nullptr;       // closure matrices of D_xx^FC along x1 / x2 (k_closure_mats, type T)
     void* my = nullptr;
+    void* e = nullptr;        // FP64 narrow stencil: interior edge weights (6 Q planes, k_edge_weights); given back
+                              // when a later allocation of the handle finds no room (drop_edges)
 };
 
 int order_nb(int o) { return o == 2 ? SBP2_NB : (o == 4 ? SBP4_NB : SBP6_NB); }
@@ -94,6 +96,11 @@ double host_hweight(int o, int N, int i) {
 }
 
 }  // namespace
+
+struct sbp_handle;
+namespace {
+bool drop_edges(sbp_handle* h);
+}
 
 struct sbp_handle {
     int order = 0, precision = 0, nblocks = 0;
@@ -190,7 +197,10 @@ struct sbp_handle {
     }
     void* dalloc(size_t bytes) {
         void* p = nullptr;
-        if (cudaMalloc(&p, bytes) != cudaSuccess) return nullptr;
+        if (cudaMalloc(&p, bytes) != cudaSuccess && (!drop_edges(this) || cudaMalloc(&p, bytes) != cudaSuccess)) {
+            cudaGetLastError();   // reported as SBP_E_OOM by the caller; the next launch check starts clean
+            return nullptr;
+        }
         cudaMemset(p, 0, bytes);
         allocs.push_back(p);
         return p;
@@ -289,6 +299,12 @@ BlockDev make_view(const sbp_handle* h, const HostBlock& hb) {
     b.sg = hb.sg;
     b.mx = hb.mx;
     b.my = hb.my;
+    b.e = hb.e;
+    for (int k = 0; k < order_q(h->order); ++k) {
+        const double ak = h->order == 2 ? sbphost::sbp2_A[k] : (h->order == 4 ? sbphost::sbp4_A[k] : sbphost::sbp6_A[k]);
+        b.ai1[k] = ak * b.ih1;
+        b.ai2[k] = ak * b.ih2;
+    }
     return b;
 }
 
@@ -314,6 +330,25 @@ int sync_views(sbp_handle* h) {
             return h->fail(SBP_E_CUDA, "upload of adjoint block views failed");
     }
     return SBP_OK;
+}
+
+// gives the edge weights of every block back to the device (an allocation of the handle found no room);
+// the interior then forms them in the kernel again.  False if there were none.
+bool drop_edges(sbp_handle* h) {
+    bool any = false;
+    for (auto& hb : h->blocks) any = any || hb.e;
+    if (!any) return false;
+    cudaGetLastError();
+    cudaDeviceSynchronize();
+    for (auto& hb : h->blocks) {
+        h->dfree(hb.e);
+        hb.e = nullptr;
+    }
+    if (h->graph_exec) {
+        cudaGraphExecDestroy(h->graph_exec);
+        h->graph_exec = nullptr;
+    }
+    return !h->d_blocks || sync_views(h) == SBP_OK;
 }
 
 inline unsigned grid_for(long long n, int bs = 256) { return (unsigned)((n + bs - 1) / bs); }
@@ -440,6 +475,57 @@ int launch_wide(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st) {
     return check_cuda(h, "wide operator launch");
 }
 
+// the FP64 interior of every block by k_interior_edges, up to IE_MAX_BLOCKS blocks a launch.  The tile
+// shape is the one whose busiest SM executes the fewest FP64 instructions (the kernel is bound by
+// them): 32 x 16 nodes repeat the fewest fluxes on their halos and win once there are several tiles per
+// SM, 16 x 4 nodes leave no SM idle on a 101^2 grid (138 tiles against 18).   Order 4, 101^2: 13 us
+// against 38 us for 32 x 16 tiles with their own weights.
+template <int O>
+void launch_interior_f64(sbp_handle* h, const BlockDev* tab, const StepArgs& a, int mode, cudaStream_t st) {
+    constexpr int Q = Ord<O>::Q, NODE = 8 * Q * 4 + 12, FLUX = 6 * Q + 4;
+    const int S = std::max(order_nclos(h->order), order_ncol(h->order));
+    constexpr int shapes[4][2] = {{32, 16}, {32, 8}, {32, 4}, {16, 4}};
+    int best = 0;
+    long long least = -1;
+    for (int k = 0; k < 4; ++k) {
+        const int tx = shapes[k][0], ty = shapes[k][1];
+        long long tiles = 0;
+        for (auto& hb : h->blocks)
+            tiles += (long long)((hb.n1 - 2 * S + tx - 1) / tx) * ((hb.n2 - 2 * S + ty - 1) / ty);
+        const long long cost = (tiles + h->num_sms - 1) / h->num_sms *
+                               (tx * ty * NODE + FLUX * ((tx + 2 * Q) * ty + tx * (ty + 2 * Q)));
+        if (least < 0 || cost < least) {
+            least = cost;
+            best = k;
+        }
+    }
+    const int tx = shapes[best][0], ty = shapes[best][1];
+    for (int first = 0; first < h->nblocks; first += IE_MAX_BLOCKS) {
+        InteriorTiles tl{};
+        tl.first = first;
+        int tiles = 0;
+        for (int b = first; b < std::min(h->nblocks, first + IE_MAX_BLOCKS); ++b) {
+            const HostBlock& hb = h->blocks[b];
+            tl.ncx[tl.nb] = (hb.n1 - 2 * S + tx - 1) / tx;
+            tl.start[tl.nb++] = tiles;
+            tiles += tl.ncx[tl.nb - 1] * ((hb.n2 - 2 * S + ty - 1) / ty);
+        }
+        tl.start[tl.nb] = tiles;
+        ProfScope ps(h, 0, st, 1);
+        auto run = [&](auto xc, auto yc) {
+            constexpr int TX = decltype(xc)::value, TY = decltype(yc)::value, NT = TX * TY < 256 ? TX * TY : 256;
+            if (mode == 0) k_interior_edges<double, O, 0, TX, TY><<<tiles, NT, 0, st>>>(tab, tl, a);
+            else if (mode == 2) k_interior_edges<double, O, 2, TX, TY><<<tiles, NT, 0, st>>>(tab, tl, a);
+            else k_interior_edges<double, O, 1, TX, TY><<<tiles, NT, 0, st>>>(tab, tl, a);
+        };
+        using std::integral_constant;
+        if (best == 0) run(integral_constant<int, 32>(), integral_constant<int, 16>());
+        else if (best == 1) run(integral_constant<int, 32>(), integral_constant<int, 8>());
+        else if (best == 2) run(integral_constant<int, 32>(), integral_constant<int, 4>());
+        else run(integral_constant<int, 16>(), integral_constant<int, 4>());
+    }
+}
+
 // one operator application (mode 1) or leapfrog step (mode 0) on the state fields, or, with adj,
 // on the adjoint fields (the same kernels; the sources are skipped)
 template <typename T, int O>
@@ -499,7 +585,9 @@ int launch_operator(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st,
             if (mmul.nb == MARCH_MAX_BLOCKS) flush();
         }
         flush();
-    } else for (auto& hb : h->blocks) {
+    } else if (h->blocks[0].e) {
+        launch_interior_f64<O>(h, tab, a, mode, ist);
+    } else for (auto& hb : h->blocks) {   // no room for the edge weights: the kernel that forms them
         BlockDev b = adj ? make_view_adj(h, hb) : make_view(h, hb);
         const int S = b.strip;
         const int ni1 = hb.n1 - 2 * S, ni2 = hb.n2 - 2 * S;
@@ -756,12 +844,14 @@ void launch_noalloc(sbp_handle* h, const BlockDev* views, int nviews, BlockDev* 
     const int total = h->nface_nodes;
     if (total > 0) k_face_sat<T, O><<<grid_for(total), 256, 0, st>>>(d_views, d_refs, h->nrefs, total, a, h->beta);
     constexpr size_t smem = interior_smem_elems<T, O>() * sizeof(T);
+    const bool edges = std::is_same<T, double>::value && views[0].e;
+    if (edges) launch_interior_f64<O>(h, d_views, a, 1, st);
     for (int b = 0; b < nviews; ++b) {
         const BlockDev& v = views[b];
         const int S = v.strip;
         const int ni1 = v.n1 - 2 * S, ni2 = v.n2 - 2 * S;
         dim3 grid((ni1 + ITX - 1) / ITX, (ni2 + ITY - 1) / ITY);
-        k_interior<T, O, 1><<<grid, dim3(32, 8), smem, st>>>(v, a);
+        if (!edges) k_interior<T, O, 1><<<grid, dim3(32, 8), smem, st>>>(v, a);
         const long long nstrip = (long long)v.n1 * v.n2 - (long long)ni1 * ni2;
         k_boundary<T, O, 1><<<grid_for(nstrip), 256, 0, st>>>(v, a);
     }
@@ -1127,6 +1217,20 @@ int sbp_grid_create(const sbp_grid_desc* desc, sbp_handle** out) {
         cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(0) != cudaSuccess)
         return cleanup(SBP_E_CUDA, "metric setup failed");
     if (flag) return cleanup(SBP_E_JACOBIAN_NONPOSITIVE, "non-positive Jacobian determinant");
+    // FP64: planes for the interior edge weights.  They are no part of what the handle needs
+    // (sbp_grid_footprint), so they are taken only where they leave seven eighths of the free memory to
+    // others, and given back when an allocation of the handle finds no room.
+    if (h->precision == SBP_FP64 && h->stencil == SBP_STENCIL_NARROW) {
+        size_t want = 0, freeb = 0, totalb = 0;
+        for (auto& hb : h->blocks) want += 6 * (size_t)order_q(o) * hb.n2 * hb.pitch * h->esize;
+        bool room = cudaMemGetInfo(&freeb, &totalb) == cudaSuccess && want <= freeb / 8;
+        for (auto& hb : h->blocks)
+            if (room) room = (hb.e = h->dalloc(6 * (size_t)order_q(o) * hb.n2 * hb.pitch * h->esize)) != nullptr;
+        for (auto& hb : h->blocks) room = room && hb.e;    // a failing allocation takes back the ones before it
+        if (!room) drop_edges(h);
+        cudaGetLastError();
+        if (sync_views(h) != SBP_OK) return cleanup(SBP_E_CUDA, h->err);
+    }
     *out = h;
     return SBP_OK;
 }
@@ -1188,6 +1292,11 @@ int sbp_set_material(sbp_handle* h, int block, const double* rho, const double* 
         if (h->order == 2) { k_closure_mats<float, 2><<<grid_for(nx), 256>>>(b, 0, (float*)hb.mx); k_closure_mats<float, 2><<<grid_for(ny), 256>>>(b, 1, (float*)hb.my); }
         else if (h->order == 4) { k_closure_mats<float, 4><<<grid_for(nx), 256>>>(b, 0, (float*)hb.mx); k_closure_mats<float, 4><<<grid_for(ny), 256>>>(b, 1, (float*)hb.my); }
         else { k_closure_mats<float, 6><<<grid_for(nx), 256>>>(b, 0, (float*)hb.mx); k_closure_mats<float, 6><<<grid_for(ny), 256>>>(b, 1, (float*)hb.my); }
+    }
+    if (hb.e) {
+        if (h->order == 2) k_edge_weights<double, 2><<<grid_for((long long)n), 256>>>(b, (double*)hb.e);
+        else if (h->order == 4) k_edge_weights<double, 4><<<grid_for((long long)n), 256>>>(b, (double*)hb.e);
+        else k_edge_weights<double, 6><<<grid_for((long long)n), 256>>>(b, (double*)hb.e);
     }
     cudaError_t e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) return h->fail(SBP_E_CUDA, std::string("material: ") + cudaGetErrorString(e));
@@ -1888,7 +1997,8 @@ int sbp_step_graph(sbp_handle* h, int nsteps, double dt, void* stream) {
     // launches in the graph, per family (counted as if launched one by one)
     {
         const int nb = (int)h->blocks.size();
-        const int nint = h->precision == SBP_FP32 ? (nb + MARCH_MAX_BLOCKS - 1) / MARCH_MAX_BLOCKS : nb;
+        const int nint = h->precision == SBP_FP32 ? (nb + MARCH_MAX_BLOCKS - 1) / MARCH_MAX_BLOCKS
+                                                       : (h->blocks[0].e ? (nb + IE_MAX_BLOCKS - 1) / IE_MAX_BLOCKS : nb);
         h->launches[0] += (long long)nsteps * nint;
         h->launches[1] += (long long)nsteps;
         if (h->n_src_int > 0) h->launches[3] += nsteps;

@@ -82,6 +82,11 @@ template <int O> __host__ __device__ constexpr int edge_lo(int m) {
     return O == 2 ? 0 : (O == 4 ? (m == 1 ? -1 : 0) : (m == 1 ? -2 : (m == 2 ? -1 : 0)));
 }
 
+// Edge weights kept in memory (FP64 handles; k_edge_weights): plane of E_m of coefficient field f
+// (0..2: c_d1d1, c_d1d2, c_d2d2) along direction d (0: x1, 1: x2), already over h_d^2, at the edge's
+// left node.  6 Q planes.
+template <int O> __host__ __device__ constexpr int edge_plane(int d, int f, int m) { return (d * 3 + f) * Ord<O>::Q + m - 1; }
+
 // ------------------------------------------------------------------ 1-D first derivative
 // D[row][col] * h  (row-major SBP operator with mirrored right closure)
 template <int O> __device__ __forceinline__ double dcoef(int N, int row, int col) {
@@ -192,6 +197,20 @@ __device__ __forceinline__ void dxx_interior(int i, FU0 u0, FU1 u1, FB0 b0, FB1 
         r1 += e1p * dp0 + e2p * dp1 + e1m * dm0 + e2m * dm1;
     }
 }
+// the same row with the edge weights read from memory (over h^2): E(f, m, i) is E_m(i) of field f
+template <int O, typename T, class FU0, class FU1, class FE>
+__device__ __forceinline__ void dxx_edges(int i, FU0 u0, FU1 u1, FE E, T& r0, T& r1) {
+    const T uc0 = u0(i), uc1 = u1(i);
+#pragma unroll
+    for (int m = 1; m <= Ord<O>::Q; ++m) {
+        const T p0 = E(0, m, i), p1 = E(1, m, i), p2 = E(2, m, i);
+        const T q0 = E(0, m, i - m), q1 = E(1, m, i - m), q2 = E(2, m, i - m);
+        const T dp0 = u0(i + m) - uc0, dp1 = u1(i + m) - uc1;
+        const T dm0 = u0(i - m) - uc0, dm1 = u1(i - m) - uc1;
+        r0 += p0 * dp0 + p1 * dp1 + q0 * dm0 + q1 * dm1;
+        r1 += p1 * dp0 + p2 * dp1 + q1 * dm0 + q2 * dm1;
+    }
+}
 template <int O, typename T, class FU0, class FU1, class FB0, class FB1, class FB2>
 __device__ __forceinline__ void dxx_vec(int N, int i, FU0 u0, FU1 u1, FB0 b0, FB1 b1, FB2 b2, T& r0, T& r1) {
     using P = Ord<O>;
@@ -273,6 +292,8 @@ struct BlockDev {
     const void* smaps;        // strip-tile band-box tensor maps (CUtensorMap[3]: u[0], u[1], c)
     const void* mx;           // closure rows of D_xx^FC along x1 as matrices, type T (k_closure_mats)
     const void* my;           // the same along x2
+    const void* e;            // FP64: interior edge weights over h_d^2 (edge_plane) or null
+    double ai1[3], ai2[3];    // interior first-derivative coefficients over h1, h2
     FaceDev f[4];
 };
 

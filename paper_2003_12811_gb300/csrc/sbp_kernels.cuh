@@ -193,6 +193,157 @@ __global__ void __launch_bounds__(ITHREADS) k_interior(BlockDev B, StepArgs a) {
     }
 }
 
+// ============================================================================ interior, FP64
+// The FP64 units bound the double-precision interior: an SM retires two FP64 results per clock
+// (152 SMs: 1.26 TFLOP/s against 6.8 TB/s, 0.19 operations per byte), so a warp's FP64 instruction
+// holds its SM for 16 clocks and every one that is left out counts, while 232 B/node of traffic do not.
+//  * The edge weights of the narrow rows depend on the material alone: k_edge_weights forms them once
+//    and the step reads them (18 planes for order 6) instead of spending 100 of its 245 instructions per
+//    node on them again.
+//  * Only the displacement and the mixed fluxes, which neighbours share, sit in shared memory (34 KB for
+//    32 x 16 nodes against the 177 KB that the kernel with its own weights needs, one CTA per SM).
+//  * One launch covers every block (no tail per block), in tiles of a shape that launch_interior_f64
+//    picks so that small grids still spread over all SMs.
+// A step of 4 order-6 blocks of 401^2 (0.6 M interior nodes): 0.19 ms for the one launch, where the kernel
+// with its own weights took 4 launches of 0.132 ms; at the FP64 units' rate the 142 instructions per node
+// take 0.13 ms.
+template <typename T, int O> __global__ void k_edge_weights(BlockDev B, T* __restrict__ E) {
+    constexpr int Q = Ord<O>::Q;
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= (long long)B.n1 * B.n2) return;
+    const int i2 = (int)(t / B.n1), i1 = (int)(t - (long long)i2 * B.n1);
+    const size_t plane = (size_t)B.n2 * B.pitch, gi = (size_t)i2 * B.pitch + i1;
+    const T* __restrict__ C = reinterpret_cast<const T*>(B.c);
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
+        const int i = d == 0 ? i1 : i2, N = d == 0 ? B.n1 : B.n2;
+        const long long st = d == 0 ? 1 : B.pitch;
+        const T ih = d == 0 ? ih1T<T>(B) : ih2T<T>(B);
+#pragma unroll
+        for (int m = 1; m <= Q; ++m) {
+            const bool in = i + edge_lo<O>(m) >= 0 && i + EdgeRange<O>::HI < N;   // the rows that use it are in range
+#pragma unroll
+            for (int f = 0; f < 3; ++f) {
+                const T* b = C + (size_t)(3 * d + f) * plane + gi;
+                const T e = in ? Edge<O>::template e<T>(m, [&](int k) { return b[k * st]; }) : T(0);
+                E[(size_t)edge_plane<O>(d, f, m) * plane + gi] = e * ih * ih;
+            }
+        }
+    }
+}
+
+constexpr int IE_MAX_BLOCKS = 32;
+struct InteriorTiles {
+    int nb, first;                     // blocks of this launch, the first one's index
+    int start[IE_MAX_BLOCKS + 1];      // first tile of each
+    int ncx[IE_MAX_BLOCKS];            // tiles across
+};
+
+template <typename T, int O, int MODE, int TX, int TY>
+__global__ void __launch_bounds__(TX * TY < 256 ? TX * TY : 256)
+k_interior_edges(const BlockDev* __restrict__ blocks, const __grid_constant__ InteriorTiles tl, StepArgs a) {
+    constexpr int Q = Ord<O>::Q, NT = TX * TY < 256 ? TX * TY : 256;
+    constexpr int SX = TX + 2 * Q, SY = TY + 2 * Q;
+    __shared__ T su[2][SY][SX], sg1[2][TY][SX], sg2[2][SY][TX];
+    int b = 0;
+    while (b + 1 < tl.nb && (int)blockIdx.x >= tl.start[b + 1]) ++b;
+    const BlockDev& B = blocks[tl.first + b];
+    const int tile = blockIdx.x - tl.start[b], ncx = tl.ncx[b];
+    const int S = B.strip, n1 = B.n1, n2 = B.n2, P = B.pitch;
+    const int x0 = S + (tile % ncx) * TX, y0 = S + (tile / ncx) * TY;
+    const int lim1 = n1 - S, lim2 = n2 - S;
+    const size_t plane = (size_t)n2 * P;
+    const T* __restrict__ U = reinterpret_cast<const T*>(B.u[a.cur]);
+    const T* __restrict__ M = reinterpret_cast<const T*>(B.c) + 6 * plane;
+    const T* __restrict__ E = reinterpret_cast<const T*>(B.e);
+    // nodes past the last interior row or column by more than Q are nobody's neighbours: zero
+    const int xe = min(x0 - Q + SX, n1), ye = min(y0 - Q + SY, n2);
+    for (int idx = threadIdx.x; idx < SY * SX; idx += NT) {
+        const int r = idx / SX, c = idx - r * SX, gx = x0 - Q + c, gy = y0 - Q + r;
+        const bool in = gx < xe && gy < ye;
+        const size_t gi = (size_t)gy * P + gx;
+        su[0][r][c] = in ? __ldg(U + gi) : T(0);
+        su[1][r][c] = in ? __ldg(U + plane + gi) : T(0);
+    }
+    T a1[Q], a2[Q];
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+        a1[k] = T(B.ai1[k]);
+        a2[k] = T(B.ai2[k]);
+    }
+    __syncthreads();
+    // mixed fluxes g1_j = c_1j2l D_2 u_l on the tile's rows and its columns +- Q, g2_j = c_1l2j D_1 u_l
+    // on its columns and its rows +- Q, one loop over both so that the CTA's warps share them evenly
+    for (int idx = threadIdx.x; idx < TY * SX + SY * TX; idx += NT) {
+        const bool first = idx < TY * SX;
+        const int id = first ? idx : idx - TY * SX, w = first ? SX : TX;
+        const int r = id / w, c = id - r * w;
+        const int gx = first ? x0 - Q + c : x0 + c, gy = first ? y0 + r : y0 - Q + r;
+        if (gx >= xe || gy >= ye) continue;
+        const size_t gi = (size_t)gy * P + gx;
+        const T m6 = __ldg(M + gi), m7 = __ldg(M + plane + gi), m8 = __ldg(M + 2 * plane + gi), m9 = __ldg(M + 3 * plane + gi);
+        const T* p0 = first ? &su[0][r + Q][c] : &su[0][r][c + Q];
+        const T* p1 = p0 + SY * SX;
+        const int st = first ? SX : 1;
+        T d0 = T(0), d1 = T(0);
+#pragma unroll
+        for (int k = 1; k <= Q; ++k) {
+            const T ak = first ? a2[k - 1] : a1[k - 1];
+            d0 += ak * (p0[k * st] - p0[-k * st]);
+            d1 += ak * (p1[k * st] - p1[-k * st]);
+        }
+        if (first) {
+            sg1[0][r][c] = m6 * d0 + m7 * d1;
+            sg1[1][r][c] = m8 * d0 + m9 * d1;
+        } else {
+            sg2[0][r][c] = m6 * d0 + m8 * d1;
+            sg2[1][r][c] = m7 * d0 + m9 * d1;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int n = 0; n < TX * TY / NT; ++n) {
+        const int idx = threadIdx.x + n * NT, r = idx / TX, c = idx - r * TX;
+        const int gx = x0 + c, gy = y0 + r;
+        if (gx >= lim1 || gy >= lim2) continue;
+        const size_t gi = (size_t)gy * P + gx;
+        T r0 = T(0), r1 = T(0);
+        dxx_edges<O, T>(
+            0, [&](int k) { return su[0][r + Q][c + Q + k]; }, [&](int k) { return su[1][r + Q][c + Q + k]; },
+            [&](int f, int m, int k) { return __ldg(E + (size_t)edge_plane<O>(0, f, m) * plane + gi + k); }, r0, r1);
+        dxx_edges<O, T>(
+            0, [&](int k) { return su[0][r + Q + k][c + Q]; }, [&](int k) { return su[1][r + Q + k][c + Q]; },
+            [&](int f, int m, int k) { return __ldg(E + (size_t)edge_plane<O>(1, f, m) * plane + gi + (long long)k * P); },
+            r0, r1);
+#pragma unroll
+        for (int k = 1; k <= Q; ++k) {
+            r0 += a1[k - 1] * (sg1[0][r][c + Q + k] - sg1[0][r][c + Q - k]);
+            r1 += a1[k - 1] * (sg1[1][r][c + Q + k] - sg1[1][r][c + Q - k]);
+            r0 += a2[k - 1] * (sg2[0][r + Q + k][c] - sg2[0][r + Q - k][c]);
+            r1 += a2[k - 1] * (sg2[1][r + Q + k][c] - sg2[1][r + Q - k][c]);
+        }
+        if (a.with_data && B.jf) {
+            const T* __restrict__ JF = reinterpret_cast<const T*>(B.jf);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                if (k >= a.K) break;
+                r0 += T(a.Tk[k]) * JF[(size_t)k * plane + gi];
+                r1 += T(a.Tk[k]) * JF[(size_t)(a.K + k) * plane + gi];
+            }
+        }
+        if (MODE == 0) {
+            leapfrog_store<T>(B, a, gi, plane, su[0][r + Q][c + Q], su[1][r + Q][c + Q],
+                              reinterpret_cast<const T*>(B.w)[gi], r0, r1, false, T(0), T(0), T(0));
+        } else if (MODE == 2) {
+            rk4_store<T>(B, a, gi, plane, reinterpret_cast<const T*>(B.w)[gi], r0, r1);
+        } else {
+            T* __restrict__ R = reinterpret_cast<T*>(B.r);
+            R[gi] = r0;
+            R[gi + plane] = r1;
+        }
+    }
+}
+
 // ============================================================================ faces
 struct FaceRef {
     int block, face, start, nf;
