@@ -159,6 +159,7 @@ struct sbp_handle {
     // strip tiles of every block, costliest first (one k_strip_tile launch per step)
     int4* d_tiles = nullptr;            // (block, tile, first, end source node of the tile) in launch order
     int ntiles = 0;
+    int strip_len = 32;                 // nodes of a strip tile along the face (pick_strip_len)
     std::vector<int4> tiles_host;
     std::vector<std::vector<int>> tile_pos;   // [block][tile of the block] -> position in the launch order
     cudaStream_t aux = nullptr;
@@ -386,18 +387,42 @@ bool make_map(CUtensorMap* m, void* base, int pitch, int n2, int planes, int row
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// strip-tile band box of the block's order (tiles along x1)
-template <int O> void strip_box(int& bw, int& bh) {
-    bw = StripTile<O>::BWB;
+// strip-tile band box of the block's order and tile length (tiles along x1)
+template <int O> void strip_box(int len, int& bw, int& bh) {
+    bw = len == 32 ? StripTile<O, 32>::BWB : (len == 16 ? StripTile<O, 16>::BWB : StripTile<O, 8>::BWB);
     bh = StripTile<O>::BHB;
+}
+
+// Length of the strip tiles of an FP64 grid: the one whose busiest SM executes the fewest FP64
+// instructions, a tile of length L taking about 140 per output node, 26 and 16 per flux on its rows and
+// columns with their halos, and 150 per face node.  (4 order-6 blocks of 401^2: 200 tiles of 32, 76 us;
+// 400 tiles of 16, 55 us.  101^2, order 4: 14 tiles of 32, 30 us; 50 of 8, 26 us.)  FP32 tiles are bound by their
+// latencies instead and stay at 32.
+int pick_strip_len(const sbp_handle* h) {
+    if (h->precision != SBP_FP64) return 32;
+    const int S = std::max(order_nclos(h->order), order_ncol(h->order)), Q = order_q(h->order);
+    const int HT = h->order == 2 ? StripTile<2>::HT : (h->order == 4 ? StripTile<4>::HT : StripTile<6>::HT);
+    int best = 32;
+    long long least = -1;
+    for (int L : {32, 16, 8}) {
+        long long tiles = 0;
+        for (auto& hb : h->blocks) tiles += 2 * ((hb.n1 + L - 1) / L) + 2 * ((hb.n2 - 2 * S + L - 1) / L);
+        const long long cost = (tiles + h->num_sms - 1) / h->num_sms *
+                               (140 * L * S + 26 * S * (L + 2 * HT + 4) + 16 * (S + Q) * L + 150 * L);
+        if (least < 0 || cost < least) {
+            least = cost;
+            best = L;
+        }
+    }
+    return best;
 }
 
 // the strip-tile band-box maps of two displacement buffers and the coefficients, written to dst[0..2]
 bool make_strip_maps(const sbp_handle* h, const HostBlock& hb, void* u0, void* u1, CUtensorMap* dst) {
     int bw, bh;
-    if (h->order == 2) strip_box<2>(bw, bh);
-    else if (h->order == 4) strip_box<4>(bw, bh);
-    else strip_box<6>(bw, bh);
+    if (h->order == 2) strip_box<2>(h->strip_len, bw, bh);
+    else if (h->order == 4) strip_box<4>(h->strip_len, bw, bh);
+    else strip_box<6>(h->strip_len, bw, bh);
     const int es = (int)h->esize;
     return make_map(&dst[0], u0, hb.pitch, hb.n2, 2, bh, bw, es) &&
            make_map(&dst[1], u1, hb.pitch, hb.n2, 2, bh, bw, es) &&
@@ -608,15 +633,25 @@ int launch_operator(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st,
     }
     {
         ProfScope ps(h, 1, sst, 1);
-        using ST = StripTile<O>;
-        constexpr size_t ssm = ST::template bytes<T>();
         const SrcNode* ss = adj ? nullptr : h->d_src_strip;
-        if (mode == 0)
-            k_strip_tile<T, O, 0><<<h->ntiles, ST::THREADS, ssm, sst>>>(tab, h->d_tiles, a, h->beta, h->d_err, ss, h->d_src_params);
-        else if (mode == 2)
-            k_strip_tile<T, O, 2><<<h->ntiles, ST::THREADS, ssm, sst>>>(tab, h->d_tiles, a, h->beta, h->d_err, ss, h->d_src_params);
-        else
-            k_strip_tile<T, O, 1><<<h->ntiles, ST::THREADS, ssm, sst>>>(tab, h->d_tiles, a, h->beta, h->d_err, ss, h->d_src_params);
+        auto run = [&](auto lc) {
+            constexpr int TL = decltype(lc)::value;
+            using ST = StripTile<O, TL>;
+            constexpr size_t ssm = ST::template bytes<T>();
+            if (mode == 0)
+                k_strip_tile<T, O, 0, TL><<<h->ntiles, ST::THREADS, ssm, sst>>>(tab, h->d_tiles, a, h->beta, h->d_err, ss, h->d_src_params);
+            else if (mode == 2)
+                k_strip_tile<T, O, 2, TL><<<h->ntiles, ST::THREADS, ssm, sst>>>(tab, h->d_tiles, a, h->beta, h->d_err, ss, h->d_src_params);
+            else
+                k_strip_tile<T, O, 1, TL><<<h->ntiles, ST::THREADS, ssm, sst>>>(tab, h->d_tiles, a, h->beta, h->d_err, ss, h->d_src_params);
+        };
+        if constexpr (std::is_same<T, double>::value) {
+            if (h->strip_len == 8) run(std::integral_constant<int, 8>());
+            else if (h->strip_len == 16) run(std::integral_constant<int, 16>());
+            else run(std::integral_constant<int, 32>());
+        } else {
+            run(std::integral_constant<int, 32>());
+        }
     }
     if (ovl) {
         cudaEventRecord(h->ev_join, h->aux);
@@ -691,10 +726,18 @@ int run_operator(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st, bo
 
 template <typename T, int O> void set_smem_attr() {
     constexpr size_t smem = interior_smem_elems<T, O>() * sizeof(T);
-    constexpr size_t ssm = StripTile<O>::template bytes<T>();
-    cudaFuncSetAttribute(k_strip_tile<T, O, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm);
-    cudaFuncSetAttribute(k_strip_tile<T, O, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm);
-    cudaFuncSetAttribute(k_strip_tile<T, O, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm);
+    auto strip = [](auto lc) {
+        constexpr int TL = decltype(lc)::value;
+        constexpr int ssm = (int)StripTile<O, TL>::template bytes<T>();
+        cudaFuncSetAttribute(k_strip_tile<T, O, 0, TL>, cudaFuncAttributeMaxDynamicSharedMemorySize, ssm);
+        cudaFuncSetAttribute(k_strip_tile<T, O, 1, TL>, cudaFuncAttributeMaxDynamicSharedMemorySize, ssm);
+        cudaFuncSetAttribute(k_strip_tile<T, O, 2, TL>, cudaFuncAttributeMaxDynamicSharedMemorySize, ssm);
+    };
+    strip(std::integral_constant<int, 32>());
+    if constexpr (std::is_same<T, double>::value) {
+        strip(std::integral_constant<int, 16>());
+        strip(std::integral_constant<int, 8>());
+    }
     cudaFuncSetAttribute(k_interior<T, O, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaFuncSetAttribute(k_interior<T, O, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaFuncSetAttribute(k_interior<T, O, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -730,11 +773,11 @@ void fill_basis(const sbp_handle* h, double t, StepArgs& a) {
 // x2 = 0 and x2 = 1, then the side bands between them), or -1 for a node off the strips
 int strip_tile_of(const sbp_handle* h, const HostBlock& hb, int i1, int i2) {
     const int S = std::max(order_nclos(h->order), order_ncol(h->order));
-    const int nbx = (hb.n1 + 31) / 32, nby = (hb.n2 - 2 * S + 31) / 32;
-    if (i2 < S) return i1 / 32;
-    if (i2 >= hb.n2 - S) return nbx + i1 / 32;
-    if (i1 < S) return 2 * nbx + (i2 - S) / 32;
-    if (i1 >= hb.n1 - S) return 2 * nbx + nby + (i2 - S) / 32;
+    const int L = h->strip_len, nbx = (hb.n1 + L - 1) / L, nby = (hb.n2 - 2 * S + L - 1) / L;
+    if (i2 < S) return i1 / L;
+    if (i2 >= hb.n2 - S) return nbx + i1 / L;
+    if (i1 < S) return 2 * nbx + (i2 - S) / L;
+    if (i1 >= hb.n1 - S) return 2 * nbx + nby + (i2 - S) / L;
     return -1;
 }
 
@@ -1075,6 +1118,11 @@ int sbp_grid_create(const sbp_grid_desc* desc, sbp_handle** out) {
             cudaEventCreateWithFlags(&h->ev_join_hi, cudaEventDisableTiming) != cudaSuccess)
             return cleanup(SBP_E_CUDA, "auxiliary streams");
     }
+    for (int b = 0; b < desc->nblocks; ++b) {
+        h->blocks[b].n1 = desc->blocks[b].n1;
+        h->blocks[b].n2 = desc->blocks[b].n2;
+    }
+    h->strip_len = pick_strip_len(h);
     std::vector<FaceRef> refs;
     int start = 0, nintf = 0;
     for (int b = 0; b < desc->nblocks; ++b) {
@@ -1164,14 +1212,14 @@ int sbp_grid_create(const sbp_grid_desc* desc, sbp_handle** out) {
     h->ntrefs = nintf;
     if (sync_views(h) != SBP_OK) return cleanup(SBP_E_CUDA, h->err);
     {
-        // strip tiles (the tile numbering of k_strip_tile: 2 bands of ceil(n1/32) tiles along x1,
-        // then 2 side bands of ceil((n2 - 2S)/32) tiles), ordered by a cost estimate: side tiles
+        // strip tiles (the tile numbering of k_strip_tile: 2 bands of ceil(n1/L) tiles along x1,
+        // then 2 side bands of ceil((n2 - 2S)/L) tiles), ordered by a cost estimate: side tiles
         // stage narrow rows, interface tiles read the neighbour, corner tiles carry two faces
-        const int S = std::max(order_nclos(o), order_ncol(o));
+        const int S = std::max(order_nclos(o), order_ncol(o)), L = h->strip_len;
         std::vector<std::pair<int, int2>> tl;
         for (int b = 0; b < desc->nblocks; ++b) {
             const HostBlock& hb = h->blocks[b];
-            const int nbx = (hb.n1 + 31) / 32, nby = (hb.n2 - 2 * S + 31) / 32;
+            const int nbx = (hb.n1 + L - 1) / L, nby = (hb.n2 - 2 * S + L - 1) / L;
             for (int t = 0; t < 2 * nbx + 2 * nby; ++t) {
                 int cost;
                 if (t < 2 * nbx) {
@@ -1189,7 +1237,7 @@ int sbp_grid_create(const sbp_grid_desc* desc, sbp_handle** out) {
         h->tile_pos.assign(desc->nblocks, {});
         for (int b = 0; b < desc->nblocks; ++b) {
             const HostBlock& hb = h->blocks[b];
-            h->tile_pos[b].assign(2 * ((hb.n1 + 31) / 32) + 2 * ((hb.n2 - 2 * S + 31) / 32), -1);
+            h->tile_pos[b].assign(2 * ((hb.n1 + L - 1) / L) + 2 * ((hb.n2 - 2 * S + L - 1) / L), -1);
         }
         h->tiles_host.clear();
         for (auto& e : tl) {

@@ -827,7 +827,7 @@ __device__ __forceinline__ double ricker_at(const SrcParam& p, const StepArgs& a
 }
 
 // ============================================================================ boundary strips, tiled
-// The strips are cut into tiles of 32 nodes along the face x (strip width) nodes across it:
+// The strips are cut into tiles of TL (32) nodes along the face x (strip width) nodes across it:
 // bottom and top bands (tiles along x1), left and right bands (tiles along x2, between the
 // bands).  The tile's region of the 2 displacement and 10 coefficient planes is staged in shared
 // memory: for band tiles one elected thread issues two cp.async.bulk.tensor loads (a bounded
@@ -845,18 +845,23 @@ __device__ __forceinline__ double ricker_at(const SrcParam& p, const StepArgs& a
 // face whose first NCOL nodes the tile touches) are formed from the staged data (interfaces read
 // the traces of k_face_trace), so every output node needs only the narrow rows, two <= NCOL-tap
 // sums and shared-memory SAT terms.
-template <int O> struct StripTile {
+//
+// TL, the tile's length along the face: 32 in FP32 (a warp per row).  In FP64 the tile's arithmetic holds
+// its SM (see k_interior_edges), so small grids are cut shorter, 16 or 8 nodes, until the tiles spread
+// over all SMs (the host picks; the halo along the face repeats more of the fluxes the shorter the tile).
+template <int O, int TL = 32> struct StripTile {
     static constexpr int Q = Ord<O>::Q;
     static constexpr int S = Ord<O>::NCLOS > Ord<O>::NCOL ? Ord<O>::NCLOS : Ord<O>::NCOL;
     static constexpr int HN = Q;
     static constexpr int HT = (Q - EdgeRange<O>::LO + 3) / 4 * 4;
-    static constexpr int BWB = 32 + 2 * HT + 4, BHB = S + HN;            // band box (tiles along x1)
-    static constexpr int CWS = S + HN, BWS = CWS | 1, BHS = 32 + 2 * HT; // side region: CWS columns, odd stride
+    static constexpr int BWB = TL + 2 * HT + 4, BHB = S + HN;            // band box (tiles along x1)
+    static constexpr int CWS = S + HN, BWS = CWS | 1, BHS = TL + 2 * HT; // side region: CWS columns, odd stride
     static constexpr int RMAX = BWB * BHB > BWS * BHS ? BWB * BHB : BWS * BHS;
-    static constexpr int FLUXB = 2 * (S * BWB + BHB * 32), FLUXS = 2 * (32 * BWS + BHS * S);
+    static constexpr int FLUXB = 2 * (S * BWB + BHB * TL), FLUXS = 2 * (TL * BWS + BHS * S);
     static constexpr int FLUX = FLUXB > FLUXS ? FLUXB : FLUXS;   // g1 on the tile rows, g2 on its columns
-    static constexpr int SATS = 4 * 32 * 4;             // per face, per face node: Fs0, Fs1, As0, As1
-    static constexpr int THREADS = 32 * S;
+    static constexpr int FN = TL > S ? TL : S;          // face nodes of a tile: along it, or across it at a corner
+    static constexpr int SATS = 4 * FN * 4;             // per face, per face node: Fs0, Fs1, As0, As1
+    static constexpr int THREADS = TL * S < 128 ? 128 : (TL * S + 31) / 32 * 32;
     // element offset of the coefficient box (128-byte aligned TMA destination), of the fluxes, and bytes
     template <typename T> static constexpr int coff() { return (int)((2 * RMAX * sizeof(T) + 127) / 128 * 128 / sizeof(T)); }
     template <typename T> static constexpr int foff() { return coff<T>() + 10 * RMAX; }
@@ -874,27 +879,27 @@ template <int O> struct StripTile {
 // the tile's staging copies ran out (the error word is set).  The staging mbarrier is
 // invalidated before the return, so a persistent caller can reuse the shared memory for its next
 // tile after a CTA barrier.
-template <typename T, int O, int MODE, int NT>
+template <typename T, int O, int MODE, int NT, int TL = 32>
 __device__ __forceinline__ bool strip_tile_body(const BlockDev* __restrict__ blocks, const int4 tt, const StepArgs& a,
                                                 double beta, int* err, const SrcNode* __restrict__ ssrc,
                                                 const SrcParam* __restrict__ spar, unsigned char* strip_smem) {
-    using ST = StripTile<O>;
+    using ST = StripTile<O, TL>;
     constexpr int S = ST::S;
     T* sm = reinterpret_cast<T*>(strip_smem);
     uint64_t* bar = reinterpret_cast<uint64_t*>(strip_smem + ST::template bar_off<T>());
     const BlockDev& B = blocks[tt.x];
     const int n1 = B.n1, n2 = B.n2, P = B.pitch;
-    const int nbx = (n1 + 31) / 32, nby = (n2 - 2 * S + 31) / 32;
+    const int nbx = (n1 + TL - 1) / TL, nby = (n2 - 2 * S + TL - 1) / TL;
     int t = tt.y, x0, y0, w, h, xs, ys, BW, BH, VW;   // VW: staged columns (BW: row stride)
     bool along_x;
     if (t < 2 * nbx) {
         along_x = true;
         const int band = t / nbx;
-        x0 = (t - band * nbx) * 32;
-        w = min(32, n1 - x0);
+        x0 = (t - band * nbx) * TL;
+        w = min(TL, n1 - x0);
         y0 = band ? n2 - S : 0;
         h = S;
-        const int xc = min(x0, max(0, n1 - 32));
+        const int xc = min(x0, max(0, n1 - TL));
         xs = (xc & ~3) - ST::HT;
         ys = band ? n2 - S - ST::HN : 0;
         BW = VW = ST::BWB;
@@ -903,8 +908,8 @@ __device__ __forceinline__ bool strip_tile_body(const BlockDev* __restrict__ blo
         t -= 2 * nbx;
         along_x = false;
         const int side = t / nby;
-        y0 = S + (t - side * nby) * 32;
-        h = min(32, n2 - S - y0);
+        y0 = S + (t - side * nby) * TL;
+        h = min(TL, n2 - S - y0);
         x0 = side ? n1 - S : 0;
         w = S;
         xs = side ? n1 - ST::CWS : 0;
@@ -997,14 +1002,14 @@ __device__ __forceinline__ bool strip_tile_body(const BlockDev* __restrict__ blo
         if (f < 2) return f == 0 ? x0 < Ord<O>::NCOL : x0 + w > n1 - Ord<O>::NCOL;
         return f == 2 ? y0 < Ord<O>::NCOL : y0 + h > n2 - Ord<O>::NCOL;
     };
-    for (int idx = threadIdx.x; idx < 4 * 32; idx += NT) {
-        const int f = idx >> 5, k = idx & 31;
+    for (int idx = threadIdx.x; idx < 4 * ST::FN; idx += NT) {
+        const int f = idx / ST::FN, k = idx % ST::FN;
         if (k >= (f < 2 ? h : w) || !face_meets(f)) continue;
         const int s = (f < 2 ? y0 : x0) + k;
         T f0, f1, a0, a1;
         face_sat_node<T, O>(blocks, B, B.f[f], s, a, beta, [&](int L, int j1, int j2) { return at(L, j1, j2); },
                             [&](int pl, int j1, int j2) { return at(2 + pl, j1, j2); }, f0, f1, a0, a1);
-        T* q = sats + (f * 32 + k) * 4;
+        T* q = sats + (f * ST::FN + k) * 4;
         q[0] = f0;
         q[1] = f1;
         q[2] = a0;
@@ -1014,25 +1019,41 @@ __device__ __forceinline__ bool strip_tile_body(const BlockDev* __restrict__ blo
     // output node of this thread: a warp per row of a band tile (lanes along the row), a warp per
     // column of a side tile (lanes along the column: one closure row per warp, and the odd row
     // stride of the side staging keeps the column accesses free of bank conflicts)
-    const int lane = threadIdx.x & 31;
-    auto out_node = [&](const int wid) {
+    auto out_node = [&](const int lane, const int wid) {
         const int i1 = along_x ? x0 + lane : x0 + wid;
         const int i2 = along_x ? y0 + wid : y0 + lane;
         if (i1 >= x0 + w || i2 >= y0 + h) return;
-        // narrow rows: closure rows through the precomputed matrices, interior rows by edge weights
-        T rx0v = T(0), rx1v = T(0), ry0v = T(0), ry1v = T(0);
+        // narrow rows: closure rows through the precomputed matrices, interior rows by edge weights (in
+        // FP64 read from memory, where they are over h^2 already: into e0, e1)
+        T rx0v = T(0), rx1v = T(0), ry0v = T(0), ry1v = T(0), e0 = T(0), e1 = T(0);
+        const T* __restrict__ E = sizeof(T) == 8 ? reinterpret_cast<const T*>(B.e) : nullptr;
+        const size_t gi = (size_t)i2 * P + i1;
         if (!dxx_closure_mat<O, T>(n1, i1, i2, n2, reinterpret_cast<const T*>(B.mx), [&](int j) { return at(0, j, i2); },
-                                   [&](int j) { return at(1, j, i2); }, rx0v, rx1v))
-            dxx_interior<O, T>(i1, [&](int j) { return at(0, j, i2); }, [&](int j) { return at(1, j, i2); },
+                                   [&](int j) { return at(1, j, i2); }, rx0v, rx1v)) {
+            if (sizeof(T) == 8 && E)
+                dxx_edges<O, T>(i1, [&](int j) { return at(0, j, i2); }, [&](int j) { return at(1, j, i2); },
+                                [&](int f, int m, int k) { return __ldg(E + (size_t)edge_plane<O>(0, f, m) * plane + gi + (k - i1)); },
+                                e0, e1);
+            else dxx_interior<O, T>(i1, [&](int j) { return at(0, j, i2); }, [&](int j) { return at(1, j, i2); },
                                [&](int k) { return at(2, k, i2); }, [&](int k) { return at(3, k, i2); },
                                [&](int k) { return at(4, k, i2); }, rx0v, rx1v);
+        }
         if (!dxx_closure_mat<O, T>(n2, i2, i1, n1, reinterpret_cast<const T*>(B.my), [&](int j) { return at(0, i1, j); },
-                                   [&](int j) { return at(1, i1, j); }, ry0v, ry1v))
-            dxx_interior<O, T>(i2, [&](int j) { return at(0, i1, j); }, [&](int j) { return at(1, i1, j); },
+                                   [&](int j) { return at(1, i1, j); }, ry0v, ry1v)) {
+            if (sizeof(T) == 8 && E)
+                dxx_edges<O, T>(i2, [&](int j) { return at(0, i1, j); }, [&](int j) { return at(1, i1, j); },
+                                [&](int f, int m, int k) { return __ldg(E + (size_t)edge_plane<O>(1, f, m) * plane + gi + (long long)(k - i2) * P); },
+                                e0, e1);
+            else dxx_interior<O, T>(i2, [&](int j) { return at(0, i1, j); }, [&](int j) { return at(1, i1, j); },
                                [&](int k) { return at(5, i1, k); }, [&](int k) { return at(6, i1, k); },
                                [&](int k) { return at(7, i1, k); }, ry0v, ry1v);
+        }
         T r0 = rx0v * ih1 * ih1 + ry0v * ih2 * ih2;
         T r1 = rx1v * ih1 * ih1 + ry1v * ih2 * ih2;
+        if (sizeof(T) == 8) {
+            r0 += e0;
+            r1 += e1;
+        }
         r0 += dsum<O, T>(n1, i1, [&](int aa) { return g1(0, aa, i2); }) * ih1 +
               dsum<O, T>(n2, i2, [&](int bb) { return g2(0, i1, bb); }) * ih2;
         r1 += dsum<O, T>(n1, i1, [&](int aa) { return g1(1, aa, i2); }) * ih1 +
@@ -1044,7 +1065,7 @@ __device__ __forceinline__ bool strip_tile_body(const BlockDev* __restrict__ blo
             const int im = m == 0 ? i1 : i2, Nm = m == 0 ? n1 : n2;
             const int d = F.side ? Nm - 1 - im : im;
             if (d >= Ord<O>::NCOL) continue;
-            const T* q = sats + (f * 32 + (m == 0 ? i2 - y0 : i1 - x0)) * 4;
+            const T* q = sats + (f * ST::FN + (m == 0 ? i2 - y0 : i1 - x0)) * 4;
             const T fac = facT<T>(F, d);
             r0 += fac * q[2];
             r1 += fac * q[3];
@@ -1053,7 +1074,6 @@ __device__ __forceinline__ bool strip_tile_body(const BlockDev* __restrict__ blo
                 r1 += q[1];
             }
         }
-        const size_t gi = (size_t)i2 * P + i1;
         if (a.with_data && B.jf) {
             const T* __restrict__ JF = reinterpret_cast<const T*>(B.jf);
     #pragma unroll
@@ -1092,20 +1112,20 @@ __device__ __forceinline__ bool strip_tile_body(const BlockDev* __restrict__ blo
             R[gi + plane] = r1;
         }
     };
-    // one warp per output row when the CTA has 32 S threads (the strip kernel), else a loop
-    if constexpr (NT == 32 * S) out_node((int)(threadIdx.x >> 5));
+    // one pass when the CTA has a thread per node (the strip kernel), else a loop
+    if constexpr (NT == TL * S) out_node((int)(threadIdx.x % TL), (int)(threadIdx.x / TL));
     else
-        for (int wid = threadIdx.x >> 5; wid < S; wid += NT / 32) out_node(wid);
+        for (int idx = threadIdx.x; idx < TL * S; idx += NT) out_node(idx % TL, idx / TL);
     return true;
 }
 
-template <typename T, int O, int MODE>
-__global__ void __launch_bounds__(StripTile<O>::THREADS, sizeof(T) == 4 ? 4 : 2)
+template <typename T, int O, int MODE, int TL>
+__global__ void __launch_bounds__(StripTile<O, TL>::THREADS, sizeof(T) == 4 ? 4 : (TL == 32 ? 2 : 4))
 k_strip_tile(const BlockDev* __restrict__ blocks, const int4* __restrict__ tiles, StepArgs a, double beta, int* err,
              const SrcNode* __restrict__ ssrc, const SrcParam* __restrict__ spar) {
     extern __shared__ __align__(128) unsigned char strip_smem[];
-    (void)strip_tile_body<T, O, MODE, StripTile<O>::THREADS>(blocks, tiles[blockIdx.x], a, beta, err, ssrc, spar,
-                                                             strip_smem);
+    (void)strip_tile_body<T, O, MODE, StripTile<O, TL>::THREADS, TL>(blocks, tiles[blockIdx.x], a, beta, err, ssrc,
+                                                                     spar, strip_smem);
 }
 
 // ============================================================================ point sources

@@ -1,5 +1,5 @@
-"""The FP64 interior kernel with edge weights kept in memory, against the FP64 oracle: grids at which
-each tile shape is chosen, with full and ragged tiles, more blocks than one launch takes, and a handle
+"""The FP64 interior kernel with edge weights kept in memory and the FP64 boundary strips, against the
+FP64 oracle: grids at which each tile shape and each strip-tile length is chosen, with full and ragged tiles, more blocks than one launch takes, and a handle
 that had to give the edge weights back.  Bar as in test_gpu_parity: 1e-12 relative max-norm of one
 operator application on a random field."""
 import numpy as np
@@ -29,7 +29,8 @@ def _deviation(S, O, u):
 # 32 x 8 / 32 x 16 tiles, long thin blocks
 @pytest.mark.parametrize("order,n", [(2, (5, 5)), (2, (36, 9)), (2, (181, 133)), (4, (18, 18)), (4, (45, 29)),
                                      (4, (131, 127)), (6, (27, 27)), (6, (34, 22 + 5)), (6, (51, 35)),
-                                     (6, (201, 201)), (6, (261, 262)), (6, (700, 28)), (6, (28, 413))])
+                                     (6, (201, 201)), (6, (261, 262)), (6, (700, 28)), (6, (28, 413)),
+                                     (6, (1301, 28)), (6, (28, 1315))])
 def test_apply_matches_oracle(order, n):
     from paper_2003_12811_gb300 import Solver
     P = W.random_problem(kinds=("robin", "displacement", "displacement", "robin"), n=n, order=order)
@@ -37,6 +38,23 @@ def test_apply_matches_oracle(order, n):
     S = Solver(P, "fp64")
     S.set_state(u, u, 0.0)
     assert _deviation(S, Oracle(P), u) <= FP64_TOL
+    S.close()
+
+
+@pytest.mark.parametrize("n", [(61, 57), (413, 29), (1301, 28)])
+def test_point_sources_on_strip_tiles_of_each_length(n):
+    """Sources at a corner, along the bottom band and on the right side: their nodes are found by the
+    strip tile (8, 16, 32 nodes long on these grids) that owns them."""
+    from paper_2003_12811_gb300 import Solver
+    P = W.random_problem(kinds=("robin", "displacement", "displacement", "robin"), n=n, order=6)
+    P.sources = [W.PointSource(0, x, (0.6, -0.8), 1.0, 3.0, 0.1) for x in ((0.0, 0.0), (0.51, 0.07), (1.0, 0.46))]
+    O = Oracle(P)
+    u = W.random_state(P)
+    ref = O.unpack(O.apply(O.pack(u), 0.12))
+    S = Solver(P, "fp64")
+    S.set_state(u, u, 0.0)
+    got = S.apply(True, 0.12)
+    assert max(np.abs(a - b).max() for a, b in zip(got, ref)) <= FP64_TOL * max(np.abs(b).max() for b in ref)
     S.close()
 
 
