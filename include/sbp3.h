@@ -36,7 +36,7 @@ extern "C" {
 #define SBP3_BC_DISPLACEMENT 0   /* u = 0 weakly, SAT of eq. dirichlet_ansatz */
 #define SBP3_BC_TRACTION 1       /* traction-free, SAT of eq. sat_traction with U = 0 */
 
-#define SBP3_PROF_FAMILIES 3     /* 0: k3_flux, 1: k3_div_int, 2: k3_div_shell (with the face SATs) */
+#define SBP3_PROF_FAMILIES 3     /* 0: k3_flux, 1: k3_div, 2: k3_lines (line ends, with the face SATs) */
 
 typedef struct sbp3_handle sbp3_handle;
 
@@ -53,8 +53,8 @@ int sbp3_destroy(sbp3_handle* h);
 const char* sbp3_last_error(const sbp3_handle* h);
 
 /* Device bytes a handle of this order, precision and size holds: 64 words per node (45 coefficients,
- * 1/(rho J), two levels, the increment, 9 fluxes), the FP64 coordinates and the x1 closure
- * matrices of D_xx^FC (2 x NCLOS x NCLOSJ x 6 words per x1 line). */
+ * 1/(rho J), two levels, the increment, 9 fluxes), the FP64 coordinates and a reserve of
+ * 2 x NCLOS x NCLOSJ x 6 words per x1 line (an upper bound: the handle leaves the reserve free). */
 int sbp3_footprint(int order, int precision, int n1, int n2, int n3, long long* bytes_out);
 
 /* Density and stiffness of the x3-planes i3_begin <= i3 < i3_begin + i3_count (any chunking).
@@ -77,7 +77,7 @@ int sbp3_get_state(sbp3_handle* h, double* u_prev, double* u_cur);
 int sbp3_apply(sbp3_handle* h, const double* u, double* accel);
 
 /* nsteps leapfrog steps of size dt on the given CUDA stream (NULL: the default stream); the call
- * returns once the launches are queued (three kernels per step).  SBP_E_STATE without a complete
+ * returns once the launches are queued (five kernels per step).  SBP_E_STATE without a complete
  * material or a state; SBP_E_INVALID_ARG for nsteps < 0 or dt <= 0.  The caller picks a stable dt
  * (no CFL estimate in 3-D). */
 int sbp3_step(sbp3_handle* h, int nsteps, double dt, void* stream);

@@ -1,10 +1,11 @@
 // libsbp 3-D operator kernels: one curvilinear block of n1 x n2 x n3 nodes (the d = 3 form of
 // Sec. 3.3, 4.3-4.7 and 5).  A leapfrog step is three kernel families:
 //   k3_flux  -- the mixed fluxes q_ij = sum_{k != i} c_ijkl D_k u_l (9 fields) from u^n;
-//   k3_div_int / k3_div_shell -- r_j = sum_i D_i q_ij + sum_i D_ii^FC(c_ijil) u_l, then the leapfrog
-//               store (MODE 0: increment form, d = du + dt^2 w r, un = u + d; MODE 1: out = w r),
-//               on the x1-interior columns at every i2, i3 (with the x2 / x3 face SATs) and on the
-//               x1 slabs near the x1 faces (with every face SAT that reaches the node).
+//   k3_lines -- per direction, the ends of every grid line: closure rows of D_ii^FC and D_i q_i, and the SATs of
+//               the two faces there, for the first rows from each face, as partial sums into the output field;
+//   k3_div   -- r_j = sum_i D_i q_ij + sum_i D_ii^FC(c_ijil) u_l with the interior rows of the other
+//               directions on top of the partial sums, then the leapfrog store (MODE 0: increment form,
+//               d = du + dt^2 w r, un = u + d; MODE 1: out = w r).
 // Layout: every scalar field is [n3][n2][pitch] in the arithmetic type T, pitch = n1 rounded up
 // to 128 bytes; field f of a group starts at f * fs (fs = n3 * n2 * pitch).
 //   cm: 27 fields, M^{ik}_{jl} = c_ijkl for the pairs (i, k) = (1,2), (1,3), (2,3), field 9p + 3j + l
@@ -60,8 +61,8 @@ template <int O, typename T> __device__ __forceinline__ T edge_wT(int m, int kk)
 
 // Closure rows of D_xx^FC, unrolled at compile time.  Row ROW of the table is a list of terms
 // c_t b(k_t) u(j_t); grouping them by k gives r_j += sum_k sum_l b_jl(k) V_k(u_l) with
-// V_k(u) = sum_{t: k_t = k} c_t u(j_t), so the u window (NCLOSJ columns) and each b column are
-// read once and every c_t, j_t, k_t is a constant.
+// V_k(u) = sum_{t: k_t = k} c_t u(j_t), so that every c_t, j_t, k_t is a constant and the window of u
+// (NCLOSJ columns) and each column of b are read once for all the rows (k3_lines).
 namespace tab {
 #define SBP_TABLE static constexpr
 #include "sbp_tables.inc"
@@ -88,75 +89,42 @@ template <int O> constexpr bool clos_has_k(int row, int k) {
     return false;
 }
 
-template <int O, int ROW, int K, typename T, int... I>
-__device__ __forceinline__ void clos_vk(const T (&uw)[3][CTab<O>::NJ], T V[3], std::integer_sequence<int, I...>) {
-    constexpr int T0 = CTab<O>::start[ROW];
+// rr[ROW] += the terms of column K of the closure row ROW; bk: the column's six coefficients
+template <int O, int ROW, int K, typename T, int W, int... I>
+__device__ __forceinline__ void clos_term(const T (&uw)[3][W], const T bk[6], T rr[3], std::integer_sequence<int, I...>) {
+    if constexpr (clos_has_k<O>(ROW, K)) {
+        constexpr int T0 = CTab<O>::start[ROW];
+        T V[3] = {T(0), T(0), T(0)};
+        (
+            [&] {
+                if constexpr (CTab<O>::ck[T0 + I] == K) {
+                    constexpr int j = CTab<O>::cj[T0 + I];
+                    const T c = T(CTab<O>::cc[T0 + I]);
+                    V[0] += c * uw[0][j];
+                    V[1] += c * uw[1][j];
+                    V[2] += c * uw[2][j];
+                }
+            }(),
+            ...);
+        rr[0] += bk[0] * V[0] + bk[1] * V[1] + bk[2] * V[2];
+        rr[1] += bk[1] * V[0] + bk[3] * V[1] + bk[4] * V[2];
+        rr[2] += bk[2] * V[0] + bk[4] * V[1] + bk[5] * V[2];
+    }
+}
+template <int O, int K, typename T, int W, int NR, int... R>
+__device__ __forceinline__ void clos_column(const T (&uw)[3][W], const T bk[6], T (&rr)[NR][3], std::integer_sequence<int, R...>) {
+    (clos_term<O, R, K, T, W>(uw, bk, rr[R], std::make_integer_sequence<int, CTab<O>::start[R + 1] - CTab<O>::start[R]>()), ...);
+}
+template <int O, typename T, int W, int NR, class FB, int... K>
+__device__ __forceinline__ void clos_rows(const T (&uw)[3][W], FB b, T (&rr)[NR][3], std::integer_sequence<int, K...>) {
     (
         [&] {
-            if constexpr (CTab<O>::ck[T0 + I] == K) {
-                constexpr int j = CTab<O>::cj[T0 + I];
-                const T c = T(CTab<O>::cc[T0 + I]);
-                V[0] += c * uw[0][j];
-                V[1] += c * uw[1][j];
-                V[2] += c * uw[2][j];
-            }
+            T bk[6];
+#pragma unroll
+            for (int s6 = 0; s6 < 6; ++s6) bk[s6] = b(s6, K);
+            clos_column<O, K, T, W, NR>(uw, bk, rr, std::make_integer_sequence<int, CTab<O>::NCLOS>());
         }(),
         ...);
-}
-
-template <int O, int ROW, typename T, class FB, int... K>
-__device__ __forceinline__ void clos_row_k(const T (&uw)[3][CTab<O>::NJ], FB b, T r[3],
-                                           std::integer_sequence<int, K...>) {
-    constexpr int NT = CTab<O>::start[ROW + 1] - CTab<O>::start[ROW];
-    (
-        [&] {
-            if constexpr (clos_has_k<O>(ROW, K)) {
-                T V[3] = {T(0), T(0), T(0)};
-                clos_vk<O, ROW, K>(uw, V, std::make_integer_sequence<int, NT>());
-                const T b00 = b(0, K), b01 = b(1, K), b02 = b(2, K), b11 = b(3, K), b12 = b(4, K), b22 = b(5, K);
-                r[0] += b00 * V[0] + b01 * V[1] + b02 * V[2];
-                r[1] += b01 * V[0] + b11 * V[1] + b12 * V[2];
-                r[2] += b02 * V[0] + b12 * V[1] + b22 * V[2];
-            }
-        }(),
-        ...);
-}
-
-// one closure row, shared by the three directions and both ends: the node's pointers up (u) and
-// cp (the 6 narrow coefficients of the direction), column c of the line (counted from the nearer
-// end) at offset (c - ROW) * Ss from the node, Ss = +stride at the left end and -stride at the right
-template <int O, int ROW, typename T>
-__device__ __noinline__ void clos_row(const T* __restrict__ up, const T* __restrict__ cp, long long fs, int Ss,
-                                      T* __restrict__ r) {
-    constexpr int NJ = CTab<O>::NJ;
-    T uw[3][NJ];
-#pragma unroll
-    for (int l = 0; l < 3; ++l)
-#pragma unroll
-        for (int c = 0; c < NJ; ++c) uw[l][c] = ldg(up + l * fs + (c - ROW) * Ss);
-    T rr[3] = {T(0), T(0), T(0)};
-    auto b = [&](int s6, int c) { return ldg(cp + s6 * fs + (c - ROW) * Ss); };
-    clos_row_k<O, ROW>(uw, b, rr, std::make_integer_sequence<int, NJ>());
-    r[0] += rr[0];
-    r[1] += rr[1];
-    r[2] += rr[2];
-}
-
-template <int O, typename T, int... R>
-__device__ __forceinline__ void clos_dispatch(int row, const T* up, const T* cp, long long fs, int Ss, T* r,
-                                              std::integer_sequence<int, R...>) {
-    ((row == R ? clos_row<O, R>(up, cp, fs, Ss, r) : void()), ...);
-}
-
-// h^2 D_xx^FC rows of the closure (i < NCLOS or i >= N - NCLOS) for the node at index i of a line
-// with stride S
-template <int O, typename T>
-__device__ __forceinline__ void dxx3_closure_ptr(int N, int i, const T* up, const T* cp, long long fs, int S,
-                                                 T r[3]) {
-    using P = Ord<O>;
-    const bool right = i >= N - P::NCLOS;
-    const int row = right ? N - 1 - i : i;
-    clos_dispatch<O, T>(row, up, cp, fs, right ? -S : S, r, std::make_integer_sequence<int, P::NCLOS>());
 }
 
 template <int O, typename T, class FU, class FB>
@@ -378,101 +346,15 @@ __global__ void __launch_bounds__(BX * BY, 3) k3_flux(Grid3 g, const T* __restri
         }
 }
 
-// ------------------------------------------------------------------ divergence and leapfrog store
-// r_j += D_D q_Dj + D_DD^FC(c_DjDl) u_l for one direction D
-// x1 closure rows as matrices: row rho of the line (i2, i3) at side s is
-//   h^2 D_xx^FC(b) u |_rho = sum_c sum_l M_{s,rho,c}(b_jl) u_l(col_s(c)),  M(b) = sum_{t in row: j_t = c} c_t b(k_t)
-// (symmetric in jl like b), formed once from the material by k3_xclos.  Layout
-// xm[(((s * NJ + c) * 6 + s6) * nlines + line) * NCLOS + rho]: the row index is fastest, so the lanes
-// of a warp (consecutive i1, hence consecutive rows) read consecutive words, and every lane runs
-// the same code whatever its row.
-struct XClos {
-    const void* m;
-    long long nlines;
-};
-
-template <typename T, int O>
-__device__ __forceinline__ void xclos_apply(const XClos& xc, int N, int i, int line, const T* __restrict__ up,
-                                            long long fs, T rr[3]) {
-    using P = Ord<O>;
-    constexpr int NJ = CTab<O>::NJ, NC = P::NCLOS;
-    const bool right = i >= N - NC;
-    const int rho = right ? N - 1 - i : i;
-    const T* mp = static_cast<const T*>(xc.m) + ((long long)(right ? NJ : 0) * 6 * xc.nlines + line) * NC + rho;
-    const long long cs = xc.nlines * NC;            // stride of one (c, s6) slot
-#pragma unroll
-    for (int c = 0; c < NJ; ++c) {
-        const int off = right ? (N - 1 - c) - i : c - i;
-        const T u0 = ldg(up + off), u1 = ldg(up + fs + off), u2 = ldg(up + 2 * fs + off);
-        T m6[6];
-#pragma unroll
-        for (int s6 = 0; s6 < 6; ++s6) m6[s6] = ldg(mp + (long long)(c * 6 + s6) * cs);
-        rr[0] += m6[0] * u0 + m6[1] * u1 + m6[2] * u2;
-        rr[1] += m6[1] * u0 + m6[3] * u1 + m6[4] * u2;
-        rr[2] += m6[2] * u0 + m6[4] * u1 + m6[5] * u2;
-    }
+// ------------------------------------------------------------------ divergence
+// The rows that k3_lines takes: along x1 the columns outside [x1lo, x1hi) (x1lo a multiple of NV, so that
+// k3_div reads its x1 windows as aligned vectors inside the row), along x2 and x3 the first and last
+// line_rows<O>() planes.
+template <int O> __host__ __device__ constexpr int line_rows() {
+    return Ord<O>::NCLOS > Ord<O>::NCOL ? Ord<O>::NCLOS : Ord<O>::NCOL;
 }
-
-template <typename T, int O, int D>
-__device__ __forceinline__ void div_dir(const Grid3& g, int i, const T* __restrict__ qo, const T* __restrict__ cdo,
-                                        const T* __restrict__ up, T r[3], const XClos* xc = nullptr, int line = 0) {
-    const int S = dstride<D>(g);
-    const int N = g.n[D];
-    const long long fs = g.fs;
-    const T ih = T(g.ih[D]);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        const T* p = qo + (3 * D + j) * fs;
-        r[j] += ih * dsum<O, T>(N, i, [&](int t) { return ldg(p + (t - i) * S); });
-    }
-    T rr[3] = {T(0), T(0), T(0)};
-    const T* cp = cdo + 6 * D * fs;
-    if (i < Ord<O>::NCLOS || i >= N - Ord<O>::NCLOS) {
-        if constexpr (D == 0) xclos_apply<T, O>(*xc, N, i, line, up, fs, rr);
-        else dxx3_closure_ptr<O, T>(N, i, up, cp, fs, S, rr);
-    } else {
-        dxx3_interior<O, T>(i, [&](int l, int t) { return ldg(up + l * fs + (t - i) * S); },
-                            [&](int s, int t) { return ldg(cp + s * fs + (t - i) * S); }, rr);
-    }
-    const T ih2 = ih * ih;
-#pragma unroll
-    for (int j = 0; j < 3; ++j) r[j] += ih2 * rr[j];
-}
-
-// the x1 closure matrices of the lines of x3-planes k0 <= i3 < k0 + nk (one thread per line, side, row)
-template <typename T, int O>
-__global__ void __launch_bounds__(128) k3_xclos(Grid3 g, int k0, int nk, const T* __restrict__ cd, T* __restrict__ xm) {
-    using P = Ord<O>;
-    constexpr int NJ = CTab<O>::NJ, NC = P::NCLOS;
-    const int i2 = blockIdx.x * blockDim.x + threadIdx.x;
-    const int i3 = k0 + blockIdx.y;
-    const int rho = blockIdx.z % NC, side = blockIdx.z / NC;
-    if (i2 >= g.n[1] || blockIdx.y >= (unsigned)nk) return;
-    const int N = g.n[0];
-    const long long nlines = (long long)g.n[1] * g.n[2];
-    const long long line = (long long)i3 * g.n[1] + i2;
-    const long long base = i2 * g.s[1] + i3 * g.s[2];
-    for (int c = 0; c < NJ; ++c)
-        for (int s6 = 0; s6 < 6; ++s6) {
-            double m = 0.0;
-            for (int t = P::cstart(rho); t < P::cstart(rho + 1); ++t) {
-                if (P::cj(t) != c) continue;
-                const int k = side ? N - 1 - P::ck(t) : P::ck(t);
-                m += P::cc(t) * double(cd[s6 * g.fs + base + k]);
-            }
-            xm[((((long long)side * NJ + c) * 6 + s6) * nlines + line) * NC + rho] = T(m);
-        }
-}
-
-// ------------------------------------------------------------------ divergence: interior box and boundary shell
-// Nodes at least max(NCLOS, NCOL) from the x1 faces use interior rows along x1 and no x1-face
-// SAT.  They form the box [x1lo, x1hi) x [y0, y1) x [z0, z1) (x1lo a multiple of NV; the box
-// spans every i2 and i3), handled by k3_div_int: NV consecutive x1 nodes per thread read as one
-// vector (float2 for FP32); the x2 and x3 rows are interior vector code or, on the closure planes
-// and rows (the same for the whole warp), the general rows.  The x1 slabs outside the box (the
-// shell) go to k3_div_shell.
 struct Box3 {
-    int x1lo, x1hi, y0, y1, z0, z1;
+    int x1lo, x1hi;
 };
 
 // x2 / x3 direction (stride S) for NV nodes: r[n][j] += ih D q_Dj + ih^2 D_xx(b) u, interior rows
@@ -675,12 +557,12 @@ __device__ __forceinline__ void div_int_x1(const T* __restrict__ q0, const T* __
 }
 
 // ------------------------------------------------------------------ boundary SATs of the faces x_m = 0, 1
-// Computed by the shell kernel for the nodes they reach, so no node is written twice:
 //   traction:     J SAT_J = -H^-1 P_f nu c_mJkL D_k u_L              (face node only)
 //   displacement: J SAT_J = H^-1 [ sum_k D_k^T (nu c_mLkJ P_f u_L) - P_f (beta d / h1) c_mJmL u_L ]
 // H^-1 P_f is 1 / (h_m hw_0) at a face node; D_m^T spreads the normal term over the first NCOL
 // nodes of the normal line (H^-1 D_m^T at depth t: D_m[face][t] / (h_m hw_t)); the tangential
-// D_k^T stays on the face, weighted by hw_k(a') / hw_k(a).
+// D_k^T stays on the face, weighted by hw_k(a') / hw_k(a).  The normal term and the penalty act along
+// the line and are formed by k3_lines itself.
 // tangential transpose along direction K of face direction M: (H_K^-1 D_K^T H_K v)(a) with
 // v_J = nu c_MLKJ u_L on the face; away from the ends of the line (every row that reads column a
 // is an interior row and every weight there is 1) this is -(D_K v)(a).
@@ -735,152 +617,227 @@ struct Faces3 {
     double beta;
 };
 
-// r += the SAT terms of the faces x_M = 0 and x_M = 1 that reach the node (index im along M):
-// at a face node the face's own terms, at depth 1 .. NCOL-1 below a displacement face the
-// normal transpose D_M^T of that face's node on the same line.
+// r += the SAT terms at a node of the face x_M = 0 (side 0) or 1 that need its neighbours on the face: the
+// traction, or the tangential transposes of a displacement face; im, ia, ib the node's indices along M and the two
+// tangential directions
 template <typename T, int O, int M>
-__device__ __noinline__ void face_terms(const Grid3& g, const Faces3& fc, int im, int ia, int ib, long long o,
-                                           const T* __restrict__ u, const T* __restrict__ cm,
-                                           const T* __restrict__ cd, T r[3]) {
+__device__ __noinline__ void face_node_terms(const Grid3& g, int kind, int side, int im, int ia, int ib, long long o,
+                                             const T* __restrict__ u, const T* __restrict__ cm,
+                                             const T* __restrict__ cd, T r[3]) {
     using P = Ord<O>;
     constexpr int PD = M == 0 ? 1 : 0, TD = M == 2 ? 1 : 2;
-    const int Nm = g.n[M];
-    const int SM = dstride<M>(g);
     const long long fs = g.fs;
-    const T ihm = T(g.ih[M]);
+    const T nu = side ? T(1) : T(-1);
+    const T* up = u + o;
+    const T ihb = T(g.ih[M]) / hweightT<O, T>(g.n[M], im);         // H^-1 P_f at the face node
+    if (kind == BC_TRACTION) {
+        T gr[3][3];
+        const int ix[3] = {M == 0 ? im : ia, M == 1 ? im : (M == 0 ? ia : ib), M == 2 ? im : ib};
+        grad_dir<T, O, 0>(g, ix[0], up, gr[0]);
+        grad_dir<T, O, 1>(g, ix[1], up, gr[1]);
+        grad_dir<T, O, 2>(g, ix[2], up, gr[2]);
 #pragma unroll
-    for (int side = 0; side < 2; ++side) {
-        const int depth = side ? Nm - 1 - im : im;
-        if (depth >= P::NCOL) continue;
-        const int kind = fc.kind[2 * M + side];
-        const T nu = side ? T(1) : T(-1);
-        const int frow = side ? Nm - 1 : 0;                 // the face's row along M
-        if (depth > 0) {
-            if (kind != BC_DISPLACEMENT) continue;
-            const T dc = dcoefT<O, T>(Nm, frow, im);
-            if (dc == T(0)) continue;
-            const long long of = o + (long long)(frow - im) * SM;
-            T uf[3];
+        for (int J = 0; J < 3; ++J) {
+            T sm = T(0);
 #pragma unroll
-            for (int L = 0; L < 3; ++L) uf[L] = ldg(u + L * fs + of);
-            const T coef = ihm * ihm * dc / hweightT<O, T>(Nm, im) * nu;
+            for (int k = 0; k < 3; ++k)
 #pragma unroll
-            for (int J = 0; J < 3; ++J) {
-                T sm = T(0);
-#pragma unroll
-                for (int L = 0; L < 3; ++L) sm += cfull(cm, cd, fs, M, L, M, J, of) * uf[L];
-                r[J] += coef * sm;
-            }
-            continue;
+                for (int L = 0; L < 3; ++L) sm += cfull(cm, cd, fs, M, J, k, L, o) * gr[k][L];
+            r[J] -= ihb * nu * sm;
         }
-        const T* up = u + o;
-        const T ihb = ihm / hweightT<O, T>(Nm, im);         // H^-1 P_f at the face node
-        if (kind == BC_TRACTION) {
-            T gr[3][3];
-            const int ix[3] = {M == 0 ? im : ia, M == 1 ? im : (M == 0 ? ia : ib), M == 2 ? im : ib};
-            grad_dir<T, O, 0>(g, ix[0], up, gr[0]);
-            grad_dir<T, O, 1>(g, ix[1], up, gr[1]);
-            grad_dir<T, O, 2>(g, ix[2], up, gr[2]);
-#pragma unroll
-            for (int J = 0; J < 3; ++J) {
-                T sm = T(0);
-#pragma unroll
-                for (int k = 0; k < 3; ++k)
-#pragma unroll
-                    for (int L = 0; L < 3; ++L) sm += cfull(cm, cd, fs, M, J, k, L, o) * gr[k][L];
-                r[J] -= ihb * nu * sm;
-            }
-        } else {
-            T uf[3];
-#pragma unroll
-            for (int L = 0; L < 3; ++L) uf[L] = ldg(up + L * fs);
-            // penalty -H^-1 P_f (beta d / h1) c_mJmL u_L (h1 = h_m hw_0), and the normal transpose at
-            // depth 0, H^-1 D_M[face][face] nu c_MLMJ u_L
-            const T pen = T(fc.beta * 3.0) * ihb * ihb;
-            const T cn = ihm * ihm * dcoefT<O, T>(Nm, frow, im) / hweightT<O, T>(Nm, im) * nu;
-#pragma unroll
-            for (int J = 0; J < 3; ++J) {
-                T sp = T(0), sn = T(0);
-#pragma unroll
-                for (int L = 0; L < 3; ++L) {
-                    sp += cfull(cm, cd, fs, M, J, M, L, o) * uf[L];
-                    sn += cfull(cm, cd, fs, M, L, M, J, o) * uf[L];
-                }
-                r[J] += cn * sn - pen * sp;
-            }
-            const T base = ihb * nu;
-            face_tangential<T, O, M, PD>(g, ia, up, cm, cd, o, base * T(g.ih[PD]), r);
-            face_tangential<T, O, M, TD>(g, ib, up, cm, cd, o, base * T(g.ih[TD]), r);
-        }
+    } else {
+        const T base = ihb * nu;
+        face_tangential<T, O, M, PD>(g, ia, up, cm, cd, o, base * T(g.ih[PD]), r);
+        face_tangential<T, O, M, TD>(g, ib, up, cm, cd, o, base * T(g.ih[TD]), r);
     }
 }
 
-// the general row code of one node as a call of its own, so the closure planes do not weigh on
-// the register allocation of the vector path
+// one interior row of direction D at a node: r_j += D_D q_Dj + D_DD^FC(c_DjDl) u_l
 template <typename T, int O, int D>
-__device__ __noinline__ void div_dir_call(const Grid3& g, int i, const T* __restrict__ qo, const T* __restrict__ cdo,
-                                          const T* __restrict__ up, T* __restrict__ rn) {
-    T r3[3] = {T(0), T(0), T(0)};
-    div_dir<T, O, D>(g, i, qo, cdo, up, r3);
-    rn[0] += r3[0];
-    rn[1] += r3[1];
-    rn[2] += r3[2];
+__device__ __noinline__ void int_row(const Grid3& g, const T* __restrict__ qo, const T* __restrict__ cp,
+                                     const T* __restrict__ up, T r[3]) {
+    const int S = dstride<D>(g);
+    const long long fs = g.fs;
+    const T ih = T(g.ih[D]);
+    T rr[3] = {T(0), T(0), T(0)};
+    dxx3_interior<O, T>(0, [&](int l, int t) { return ldg(up + l * fs + t * S); },
+                        [&](int s, int t) { return ldg(cp + s * fs + t * S); }, rr);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        T d = T(0);
+#pragma unroll
+        for (int k = 1; k <= Ord<O>::Q; ++k)
+            d += Ord<O>::template aT<T>(k - 1) * (ldg(qo + j * fs + k * S) - ldg(qo + j * fs - k * S));
+        r[j] += ih * d + ih * ih * rr[j];
+    }
 }
 
-// direction D = x2 or x3 for the NV nodes of a thread: interior rows through the vector code,
-// closure rows (the same for every lane of a warp, whose lanes share i2 and i3) node by node
-template <typename T, int O, int NV, int D>
-__device__ __forceinline__ void div_int_dir(const Grid3& g, int i, const T* __restrict__ qo,
-                                            const T* __restrict__ cdo, const T* __restrict__ up, T r[NV][3]) {
-    const int N = g.n[D];
+// The ends of the grid lines of direction D, one thread per line and end: the partial sums
+//   r_j = D_D q_Dj + D_DD^FC(c_DjDl) u_l + the SATs of the face there
+// of the first rows from the face (line_rows<O>(); along x1 up to x1lo, or from x1hi) are stored in `part`
+// (added where a line kernel of a later direction, D = 2, 1, 0 in this order, has stored its own), which k3_div
+// completes.  A closure row reads NCLOSJ columns of the line, the same ones for every row of the end: a
+// thread reads the 12 columns of u, q and the 6 coefficients once (order 6: 144 loads) for all 9 rows,
+// where a thread per node read them for each row.  The lanes of a warp lie along x1 (D = 1, 2: coalesced)
+// or x2 (D = 0: a line's columns share their sectors in L1).  160 x 151 x 144, FP32: 101 + 29 + 24 us for
+// D = 0, 1, 2 (the slab kernel and the closure rows inside the divergence they replace took 226 + ~160 us).
+template <typename T, int O, int D>
+__global__ void __launch_bounds__(128) k3_lines(Grid3 g, Box3 bx, Faces3 fc, const T* __restrict__ u,
+                                                const T* __restrict__ q, const T* __restrict__ cm,
+                                                const T* __restrict__ cd, T* __restrict__ part) {
+    using P = Ord<O>;
+    constexpr int NR = line_rows<O>(), NJ = CTab<O>::NJ, W = NJ > NR + P::Q ? NJ : NR + P::Q;
+    constexpr int A = D == 0 ? 1 : 0, B = D == 2 ? 1 : 2;
+    const int na = g.n[A], nb = g.n[B], N = g.n[D];
+    const int t = blockIdx.x * 128 + threadIdx.x;
+    if (t >= na * nb) return;
+    const int ib = t / na, ia = t - ib * na, side = blockIdx.y;
     const long long fs = g.fs;
-    if (i >= Ord<O>::NCLOS && i < N - Ord<O>::NCLOS) {
-        if constexpr (NV == 2 && sizeof(T) == 4)
-            div_int_strided_f2<O>(qo + 3 * D * fs, cdo + 6 * D * fs, up, fs, dstride<D>(g), float(g.ih[D]), r);
-        else
-            div_int_strided<T, O, NV>(qo + 3 * D * fs, cdo + 6 * D * fs, up, fs, dstride<D>(g), T(g.ih[D]), r);
-        return;
+    const int S = dstride<D>(g), Ss = side ? -S : S;
+    const long long o = ia * g.s[A] + ib * g.s[B] + (side ? (long long)(N - 1) * g.s[D] : 0);   // the face node
+    const T ih = T(g.ih[D]), ih2 = ih * ih;
+    T uw[3][W], rr[NR][3];
+#pragma unroll
+    for (int l = 0; l < 3; ++l)
+#pragma unroll
+        for (int c = 0; c < W; ++c) uw[l][c] = ldg(u + l * fs + o + c * Ss);
+#pragma unroll
+    for (int r = 0; r < NR; ++r) rr[r][0] = rr[r][1] = rr[r][2] = T(0);
+    const T* cp = cd + 6 * D * fs + o;
+    auto b = [&](int s6, int c) { return ldg(cp + s6 * fs + c * Ss); };
+    clos_rows<O, T, W, NR>(uw, b, rr, std::make_integer_sequence<int, NJ>());
+    if constexpr (NR > P::NCLOS) {                       // order 2: the row past the closure that a SAT reaches
+#pragma unroll
+        for (int r = P::NCLOS; r < NR; ++r) dxx3_interior<O, T>(r, [&](int l, int c) { return uw[l][c]; }, b, rr[r]);
     }
 #pragma unroll
-    for (int n = 0; n < NV; ++n) div_dir_call<T, O, D>(g, i, qo + n, cdo + n, up + n, r[n]);
+    for (int r = 0; r < NR; ++r)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) rr[r][j] *= ih2;
+    // D_D q_Dj: rows of D from the face, mirrored with the opposite sign at the high end
+    const T sg = side ? -ih : ih;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const T* qj = q + (3 * D + j) * fs + o;
+        T qw[NR + P::Q > P::NCOL ? NR + P::Q : P::NCOL];
+        constexpr int QW = NR + P::Q > P::NCOL ? NR + P::Q : P::NCOL;
+#pragma unroll
+        for (int c = 0; c < QW; ++c) qw[c] = ldg(qj + c * Ss);
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            T d = T(0);
+            if (r < P::NB) {
+#pragma unroll
+                for (int c = 0; c < P::NCOL; ++c) d += P::template dqT<T>(r, c) * qw[c];
+            } else {
+#pragma unroll
+                for (int k = 1; k <= P::Q; ++k) d += P::template aT<T>(k - 1) * (qw[r + k] - qw[r - k]);
+            }
+            rr[r][j] += sg * d;
+        }
+    }
+    const int kind = fc.kind[2 * D + side];
+    if (kind == BC_DISPLACEMENT) {
+        // s_J = c_DJDL u_L at the face node: spread by H^-1 D_D^T nu over NCOL rows, and the penalty
+        // -H^-1 P_f (beta d / h1) s_J at the face (h1 = h hw_0)
+        T sJ[3];
+        const T b0 = b(0, 0), b1 = b(1, 0), b2 = b(2, 0), b3 = b(3, 0), b4 = b(4, 0), b5 = b(5, 0);
+        sJ[0] = b0 * uw[0][0] + b1 * uw[1][0] + b2 * uw[2][0];
+        sJ[1] = b1 * uw[0][0] + b3 * uw[1][0] + b4 * uw[2][0];
+        sJ[2] = b2 * uw[0][0] + b4 * uw[1][0] + b5 * uw[2][0];
+        const T ihb = ih / hweightT<O, T>(N, 0), pen = T(fc.beta * 3.0) * ihb * ihb;
+#pragma unroll
+        for (int r = 0; r < P::NCOL; ++r) {
+            const T coef = -ih2 * P::template dqT<T>(0, r) / (r < P::NB ? P::template hwT<T>(r) : T(1)) - (r == 0 ? pen : T(0));
+#pragma unroll
+            for (int j = 0; j < 3; ++j) rr[r][j] += coef * sJ[j];
+        }
+    }
+    {
+        T f[3] = {T(0), T(0), T(0)};
+        face_node_terms<T, O, D>(g, kind, side, side ? N - 1 : 0, ia, ib, o, u, cm, cd, f);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) rr[0][j] += f[j];
+    }
+    // nodes that the line kernels of the directions before this one have stored
+    auto end = [&](int i, int n) { return i < NR || i >= n - NR; };
+    const bool add = D == 2 ? false : (D == 1 ? end(ib, g.n[2]) : (end(ia, g.n[1]) || end(ib, g.n[2])));
+    auto store = [&](int r, const T v[3]) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            T* p = part + j * fs + o + r * Ss;
+            *p = add ? *p + v[j] : v[j];
+        }
+    };
+#pragma unroll
+    for (int r = 0; r < NR; ++r) store(r, rr[r]);
+    if constexpr (D == 0) {                               // the columns that the alignment of x1lo leaves here
+        const int rows = side ? N - bx.x1hi : bx.x1lo;
+        for (int r = NR; r < rows; ++r) {
+            T v[3] = {T(0), T(0), T(0)};
+            int_row<T, O, 0>(g, q + o + r * Ss, cp + r * Ss, u + o + r * Ss, v);
+            store(r, v);
+        }
+    }
 }
 
-// MODE 0: leapfrog in increment form, d = du + dt^2 w r, un = u + d (du updated in place);
-// MODE 1: apply, out = w r.
-// launch shapes of k3_div_int (sbp3_set_tuning / sbp3_autotune): x2 rows per block and the
+// interior rows of direction D = x2 or x3 for the NV nodes of a thread
+template <typename T, int O, int NV, int D>
+__device__ __forceinline__ void div_int_dir(const Grid3& g, const T* __restrict__ qo, const T* __restrict__ cdo,
+                                            const T* __restrict__ up, T r[NV][3]) {
+    const long long fs = g.fs;
+    if constexpr (NV == 2 && sizeof(T) == 4)
+        div_int_strided_f2<O>(qo + 3 * D * fs, cdo + 6 * D * fs, up, fs, dstride<D>(g), float(g.ih[D]), r);
+    else
+        div_int_strided<T, O, NV>(qo + 3 * D * fs, cdo + 6 * D * fs, up, fs, dstride<D>(g), T(g.ih[D]), r);
+}
+
+// launch shapes of k3_div (sbp3_set_tuning / sbp3_autotune): x2 rows per block and the
 // minimum resident blocks per SM, which sets the register cap (65536 / (32 BY MINB))
 struct DivShape {
     int by, minb;
 };
 constexpr DivShape kDivShapes[4] = {{4, 5}, {4, 6}, {8, 3}, {2, 10}};
 
+// Every node: the interior rows of the directions whose end rows k3_lines has not taken, on top of its partial
+// sums (in un) where it has, then the store.  NV consecutive x1 nodes per thread read as one vector
+// (float2 for FP32); the last pair of an odd row covers one element of the row's padding, which holds
+// zeros throughout and gets zeros back.  160 x 151 x 144, FP32, order 6: 171 us (the
+// kernel with closure rows and SATs behind calls: 328 us for the x1-interior columns).
 template <typename T, int O, int MODE, int NV, int BY, int MINB>
-__global__ void __launch_bounds__(32 * BY, MINB) k3_div_int(Grid3 g, Box3 bx, Faces3 fc, const T* __restrict__ u,
-                                                            const T* __restrict__ q, const T* __restrict__ cm,
-                                                            const T* __restrict__ cd, const T* __restrict__ w,
-                                                            T* __restrict__ du, T* __restrict__ un, T dt2) {
-    using P = Ord<O>;
-    const int gx = blockIdx.x * 32 + threadIdx.x;
-    const int i1 = bx.x1lo + gx * NV, i2 = bx.y0 + blockIdx.y * BY + threadIdx.y, i3 = bx.z0 + blockIdx.z;
-    if (i1 >= bx.x1hi || i2 >= bx.y1) return;
+__global__ void __launch_bounds__(32 * BY, MINB) k3_div(Grid3 g, Box3 bx, const T* __restrict__ u,
+                                                        const T* __restrict__ q, const T* __restrict__ cd,
+                                                        const T* __restrict__ w, T* __restrict__ du, T* un, T dt2) {
+    constexpr int NR = line_rows<O>();
+    const int i1 = (blockIdx.x * 32 + threadIdx.x) * NV, i2 = blockIdx.y * BY + threadIdx.y, i3 = blockIdx.z;
+    if (i1 >= g.n[0] || i2 >= g.n[1]) return;
     const long long o = i1 + i2 * g.s[1] + i3 * g.s[2];
     const long long fs = g.fs;
     const T* up = u + o;
+    const bool in1 = i1 >= bx.x1lo && i1 < bx.x1hi, in2 = i2 >= NR && i2 < g.n[1] - NR, in3 = i3 >= NR && i3 < g.n[2] - NR;
     T r[NV][3];
+    if (in1 && in2 && in3) {
 #pragma unroll
-    for (int n = 0; n < NV; ++n) r[n][0] = r[n][1] = r[n][2] = T(0);
-    div_int_x1<T, O, NV>(q + o, cd + o, up, fs, T(g.ih[0]), r);
-    div_int_dir<T, O, NV, 1>(g, i2, q + o, cd + o, up, r);
-    div_int_dir<T, O, NV, 2>(g, i3, q + o, cd + o, up, r);
-    // SATs of the x2 and x3 faces that reach these nodes (the x1 faces lie in the shell)
-    if (i2 < P::NCOL || i2 >= g.n[1] - P::NCOL) {
+        for (int n = 0; n < NV; ++n) r[n][0] = r[n][1] = r[n][2] = T(0);
+    } else {
 #pragma unroll
-        for (int n = 0; n < NV; ++n) face_terms<T, O, 1>(g, fc, i2, i1 + n, i3, o + n, u, cm, cd, r[n]);
+        for (int j = 0; j < 3; ++j) {
+            T v[NV];
+            if constexpr (NV == 2 && sizeof(T) == 4) {
+                const float2 x = *reinterpret_cast<const float2*>(un + j * fs + o);
+                v[0] = x.x;
+                v[1] = x.y;
+            } else {
+#pragma unroll
+                for (int n = 0; n < NV; ++n) v[n] = un[j * fs + o + n];
+            }
+#pragma unroll
+            for (int n = 0; n < NV; ++n) r[n][j] = v[n];
+        }
     }
-    if (i3 < P::NCOL || i3 >= g.n[2] - P::NCOL) {
-#pragma unroll
-        for (int n = 0; n < NV; ++n) face_terms<T, O, 2>(g, fc, i3, i1 + n, i2, o + n, u, cm, cd, r[n]);
-    }
+    if (in1) div_int_x1<T, O, NV>(q + o, cd + o, up, fs, T(g.ih[0]), r);
+    if (in2) div_int_dir<T, O, NV, 1>(g, q + o, cd + o, up, r);
+    if (in3) div_int_dir<T, O, NV, 2>(g, q + o, cd + o, up, r);
     T wv[NV];
     vld<T, NV>(w + o, wv);
 #pragma unroll
@@ -902,85 +859,6 @@ __global__ void __launch_bounds__(32 * BY, MINB) k3_div_int(Grid3 g, Box3 bx, Fa
             for (int n = 0; n < NV; ++n) out[n] = wv[n] * r[n][j];
         }
         vst<T, NV>(un + oj, out);
-    }
-}
-
-// the shell: every node outside the box, lanes along x1 (coalesced), in three parts:
-//   Z: the planes i3 < z0, i3 >= z1 (whole planes);
-//   Y: within the box's planes, the rows i2 < y0, i2 >= y1 (whole rows);
-//   X: within the box's planes and rows, the x1 runs i1 < x1lo and i1 >= x1hi.
-struct Shell3 {
-    long long cZ, cY, cX;   // node counts of the three parts
-};
-
-__device__ __forceinline__ bool shell_node(const Grid3& g, const Box3& bx, const Shell3& sh, long long t, int& i1,
-                                           int& i2, int& i3) {
-    const long long n1 = g.n[0], n2 = g.n[1];
-    const long long plane = n1 * n2;
-    if (t < sh.cZ) {
-        const long long pz = t / plane;
-        const long long rem = t - pz * plane;
-        i3 = (int)(pz < bx.z0 ? pz : bx.z1 + (pz - bx.z0));
-        i2 = (int)(rem / n1);
-        i1 = (int)(rem - (long long)i2 * n1);
-        return true;
-    }
-    t -= sh.cZ;
-    if (t < sh.cY) {
-        const long long rowsB = bx.y0 + (n2 - bx.y1);
-        const long long row = t / n1;
-        i1 = (int)(t - row * n1);
-        const long long pz = row / rowsB, ry = row - pz * rowsB;
-        i3 = (int)(bx.z0 + pz);
-        i2 = (int)(ry < bx.y0 ? ry : bx.y1 + (ry - bx.y0));
-        return true;
-    }
-    t -= sh.cY;
-    if (t >= sh.cX) return false;
-    const long long ny = bx.y1 - bx.y0;
-    const long long runs = bx.x1lo + (n1 - bx.x1hi);
-    const long long row = t / runs, rx = t - row * runs;
-    const long long pz = row / ny, py = row - pz * ny;
-    i3 = (int)(bx.z0 + pz);
-    i2 = (int)(bx.y0 + py);
-    i1 = (int)(rx < bx.x1lo ? rx : bx.x1hi + (rx - bx.x1lo));
-    return true;
-}
-
-// the boundary shell: volume terms with closure rows, then every face SAT reaching the node, then
-// the leapfrog store (MODE as in k3_div_int)
-template <typename T, int O, int MODE>
-__global__ void __launch_bounds__(128) k3_div_shell(Grid3 g, Box3 bx, Shell3 sh, XClos xc, Faces3 fc, long long count,
-                                                    const T* __restrict__ u, const T* __restrict__ q,
-                                                    const T* __restrict__ cm, const T* __restrict__ cd,
-                                                    const T* __restrict__ w, T* __restrict__ du,
-                                                    T* __restrict__ un, T dt2) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= count) return;
-    int i1, i2, i3;
-    if (!shell_node(g, bx, sh, t, i1, i2, i3)) return;
-    const long long o = i1 + i2 * g.s[1] + i3 * g.s[2];
-    const T* up = u + o;
-    const T* qo = q + o;
-    const T* cdo = cd + o;
-    T r[3] = {T(0), T(0), T(0)};
-    div_dir<T, O, 0>(g, i1, qo, cdo, up, r, &xc, i3 * g.n[1] + i2);
-    div_dir<T, O, 1>(g, i2, qo, cdo, up, r);
-    div_dir<T, O, 2>(g, i3, qo, cdo, up, r);
-    face_terms<T, O, 0>(g, fc, i1, i2, i3, o, u, cm, cd, r);
-    face_terms<T, O, 1>(g, fc, i2, i1, i3, o, u, cm, cd, r);
-    face_terms<T, O, 2>(g, fc, i3, i1, i2, o, u, cm, cd, r);
-    const T wv = ldg(w + o);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        const long long oj = j * g.fs + o;
-        if constexpr (MODE == 0) {
-            const T d = du[oj] + dt2 * wv * r[j];
-            du[oj] = d;
-            un[oj] = ldg(up + j * g.fs) + d;
-        } else {
-            un[oj] = wv * r[j];
-        }
     }
 }
 

@@ -35,11 +35,9 @@ struct sbp3_handle {
     size_t es = 8;
     double beta = 1.0;
     Grid3 g{};
-    Box3 box{};                              // nodes with interior rows in every direction (k3_div_int)
-    long long shell = 0;                     // nodes outside the box (k3_div_shell)
-    Shell3 sh{};
+    Box3 box{};                              // x1 columns with interior rows along x1 (k3_div)
     Faces3 fc{};
-    int div_variant = 0;                     // launch shape of k3_div_int (kDivShapes)
+    int div_variant = 0;                     // launch shape of k3_div (kDivShapes)
     double* X = nullptr;                     // pitched FP64 coordinates (3 fields)
     void* cm = nullptr;                      // 27 fields
     void* cd = nullptr;                      // 18 fields
@@ -47,7 +45,6 @@ struct sbp3_handle {
     void* u[2] = {nullptr, nullptr};         // leapfrog levels (3 fields each), u[cur] = u^n
     void* du = nullptr;                      // increment u^n - u^{n-1} (3 fields)
     void* q = nullptr;                       // mixed fluxes (9 fields)
-    void* xm = nullptr;                      // x1 closure matrices of D_xx^FC (k3_xclos)
     void* ain = nullptr;                     // sbp3_apply input / output (3 fields each), on first use
     void* aout = nullptr;
     int cur = 0;
@@ -127,33 +124,31 @@ int launch_operator(sbp3_handle* h, const T* u, T* du, T* un, double dt, cudaStr
     prof_begin(h, 0, st, &stop);
     k3_flux<T, O, NVF><<<grd, blk, 0, st>>>(g, u, cm, q);
     prof_end(stop, st);
-    {
-        constexpr int NV = sizeof(T) == 4 ? 2 : 1;
-        const Box3& bx = h->box;
-        const int ngx = (bx.x1hi - bx.x1lo) / NV;
-        if (ngx > 0) {             // the box is empty only for order 2 on the smallest grids
-            auto run = [&](auto vc) {
-                constexpr int V = decltype(vc)::value;
-                constexpr int BY = kDivShapes[V].by, MINB = kDivShapes[V].minb;
-                const dim3 ib(32, BY), ig((ngx + 31) / 32, (bx.y1 - bx.y0 + BY - 1) / BY, bx.z1 - bx.z0);
-                k3_div_int<T, O, MODE, NV, BY, MINB><<<ig, ib, 0, st>>>(g, bx, h->fc, u, q, cm, cd, w, du, un, dt2);
-            };
-            prof_begin(h, 1, st, &stop);
-            // every shape is built for order 6; orders 2 and 4 keep the first
-            const int v = O == 6 ? h->div_variant : 0;
-            if (v == 1) run(std::integral_constant<int, O == 6 ? 1 : 0>());
-            else if (v == 2) run(std::integral_constant<int, O == 6 ? 2 : 0>());
-            else if (v == 3) run(std::integral_constant<int, O == 6 ? 3 : 0>());
-            else run(std::integral_constant<int, 0>());
-            prof_end(stop, st);
-        }
-        const long long cnt = h->shell;
-        prof_begin(h, 2, st, &stop);
-        const XClos xc{h->xm, (long long)h->n[1] * h->n[2]};
-        k3_div_shell<T, O, MODE><<<(unsigned)((cnt + 127) / 128), 128, 0, st>>>(g, bx, h->sh, xc, h->fc, cnt, u, q,
-                                                                             cm, cd, w, du, un, dt2);
-        prof_end(stop, st);
-    }
+    const Box3& bx = h->box;
+    prof_begin(h, 2, st, &stop);
+    auto lines = [&](auto dc) {
+        constexpr int D = decltype(dc)::value, A = D == 0 ? 1 : 0, B = D == 2 ? 1 : 2;
+        const dim3 lg((unsigned)(((long long)g.n[A] * g.n[B] + 127) / 128), 2);
+        k3_lines<T, O, D><<<lg, 128, 0, st>>>(g, bx, h->fc, u, q, cm, cd, un);
+    };
+    lines(std::integral_constant<int, 2>());
+    lines(std::integral_constant<int, 1>());
+    lines(std::integral_constant<int, 0>());
+    prof_end(stop, st);
+    auto run = [&](auto vc) {
+        constexpr int V = decltype(vc)::value;
+        constexpr int BY = kDivShapes[V].by, MINB = kDivShapes[V].minb;
+        const dim3 ib(32, BY), ig((g.n[0] + 32 * NVF - 1) / (32 * NVF), (g.n[1] + BY - 1) / BY, g.n[2]);
+        k3_div<T, O, MODE, NVF, BY, MINB><<<ig, ib, 0, st>>>(g, bx, u, q, cd, w, du, un, dt2);
+    };
+    prof_begin(h, 1, st, &stop);
+    // every shape is built for order 6; orders 2 and 4 keep the first
+    const int v = O == 6 ? h->div_variant : 0;
+    if (v == 1) run(std::integral_constant<int, O == 6 ? 1 : 0>());
+    else if (v == 2) run(std::integral_constant<int, O == 6 ? 2 : 0>());
+    else if (v == 3) run(std::integral_constant<int, O == 6 ? 3 : 0>());
+    else run(std::integral_constant<int, 0>());
+    prof_end(stop, st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(h, e, "3-D operator launch");
     return SBP_OK;
@@ -181,8 +176,6 @@ int material_impl(sbp3_handle* h, int k0, int nk, const double* rho_d, const dou
     const dim3 blk(128), grd((h->n[0] + 127) / 128, h->n[1], nk);
     k3_material<T, O><<<grd, blk>>>(h->g, h->X, k0, nk, rho_d, c_d, static_cast<T*>(h->cm), static_cast<T*>(h->cd),
                                      static_cast<T*>(h->w), h->d_err);
-    const dim3 xg((h->n[1] + 127) / 128, nk, 2 * Ord<O>::NCLOS);
-    k3_xclos<T, O><<<xg, 128>>>(h->g, k0, nk, static_cast<const T*>(h->cd), static_cast<T*>(h->xm));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(h, e, "k3_material");
     return SBP_OK;
@@ -205,7 +198,7 @@ template <typename F> int dispatch(sbp3_handle* h, F f) {
 }
 
 void free_all(sbp3_handle* h) {
-    void* bufs[] = {h->X, h->cm, h->cd, h->w, h->u[0], h->u[1], h->du, h->q, h->xm, h->ain, h->aout, h->d_err};
+    void* bufs[] = {h->X, h->cm, h->cd, h->w, h->u[0], h->u[1], h->du, h->q, h->ain, h->aout, h->d_err};
     for (void* b : bufs)
         if (b) cudaFree(b);
     for (auto& v : h->prof.ev)
@@ -213,7 +206,9 @@ void free_all(sbp3_handle* h) {
             if (e) cudaEventDestroy(e);
 }
 
-size_t xclos_bytes(int order, size_t es, int n2, int n3) {
+// bytes that sbp3_footprint counts per x1 line beyond the fields (NCLOS x NCLOSJ x 6 words at either end): a
+// reserve that callers plan with, of which the line kernels need nothing
+size_t line_reserve_bytes(int order, size_t es, int n2, int n3) {
     const int nclos = order == 2 ? SBP2_NCLOS : (order == 4 ? SBP4_NCLOS : SBP6_NCLOS);
     const int nj = order == 2 ? SBP2_NCLOSJ : (order == 4 ? SBP4_NCLOSJ : SBP6_NCLOSJ);
     return (size_t)2 * nj * 6 * nclos * (size_t)n2 * n3 * es;
@@ -242,7 +237,7 @@ int sbp3_footprint(int order, int precision, int n1, int n2, int n3, long long* 
     const long long f = field_bytes(precision, n);
     const long long x = pitch_of(n1, precision == SBP_FP32 ? 4 : 8) * n2 * n3 * 8LL;
     *bytes_out = f * (NCM + NCD + 1 + 6 + 3 + 9) + 3 * x +
-                 (long long)xclos_bytes(order, precision == SBP_FP32 ? 4 : 8, n2, n3);
+                 (long long)line_reserve_bytes(order, precision == SBP_FP32 ? 4 : 8, n2, n3);
     return SBP_OK;
 }
 
@@ -296,24 +291,13 @@ int sbp3_create(int order, int precision, int n1, int n2, int n3, const double* 
     {
         const int nclos = order == 2 ? SBP2_NCLOS : (order == 4 ? SBP4_NCLOS : SBP6_NCLOS);
         const int q = order / 2, nv = precision == SBP_FP32 ? 2 : 1;
-        const int qa = (q + nv - 1) / nv * nv;            // the x1 window of k3_div_int reaches qa nodes out
+        const int qa = (q + nv - 1) / nv * nv;            // the x1 window of k3_div reaches qa nodes out
         const int ncol = order == 2 ? SBP2_NCOL : (order == 4 ? SBP4_NCOL : SBP6_NCOL);
-        // the shell holds every node with a closure row, a normal SAT term (depth < NCOL) or an x1
-        // window of k3_div_int that would leave the row
         const int ey = nclos > ncol ? nclos : ncol;
         const int e = ey > qa ? ey : qa;
         Box3& bx = h->box;
         bx.x1lo = (e + nv - 1) / nv * nv;
         bx.x1hi = n1 - e > bx.x1lo ? bx.x1lo + (n1 - e - bx.x1lo) / nv * nv : bx.x1lo;
-        bx.y0 = 0;
-        bx.y1 = n2;
-        bx.z0 = 0;
-        bx.z1 = n3;
-        Shell3& sh = h->sh;
-        sh.cZ = (long long)(bx.z0 + (n3 - bx.z1)) * n2 * n1;
-        sh.cY = (long long)(bx.z1 - bx.z0) * (bx.y0 + (n2 - bx.y1)) * n1;
-        sh.cX = (long long)(bx.z1 - bx.z0) * (bx.y1 - bx.y0) * (bx.x1lo + (n1 - bx.x1hi));
-        h->shell = sh.cX + sh.cZ + sh.cY;
     }
     auto alloc = [&](void** p, size_t bytes) -> bool {
         if (cudaMalloc(p, bytes) != cudaSuccess) return false;
@@ -325,7 +309,7 @@ int sbp3_create(int order, int precision, int n1, int n2, int n3, const double* 
     const size_t xfs = (size_t)h->fs;
     bool ok = alloc((void**)&h->X, 3 * xfs * 8) && alloc(&h->cm, NCM * fb) && alloc(&h->cd, NCD * fb) &&
               alloc(&h->w, fb) && alloc(&h->u[0], 3 * fb) && alloc(&h->u[1], 3 * fb) && alloc(&h->du, 3 * fb) &&
-              alloc(&h->q, 9 * fb) && alloc(&h->xm, xclos_bytes(order, h->es, n2, n3)) &&
+              alloc(&h->q, 9 * fb) &&
               alloc((void**)&h->d_err, sizeof(int));
     if (!ok) {
         cudaGetLastError();
