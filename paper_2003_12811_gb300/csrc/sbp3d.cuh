@@ -563,93 +563,47 @@ __device__ __forceinline__ void div_int_x1(const T* __restrict__ q0, const T* __
 // nodes of the normal line (H^-1 D_m^T at depth t: D_m[face][t] / (h_m hw_t)); the tangential
 // D_k^T stays on the face, weighted by hw_k(a') / hw_k(a).  The normal term and the penalty act along
 // the line and are formed by k3_lines itself.
-// tangential transpose along direction K of face direction M: (H_K^-1 D_K^T H_K v)(a) with
-// v_J = nu c_MLKJ u_L on the face; away from the ends of the line (every row that reads column a
-// is an interior row and every weight there is 1) this is -(D_K v)(a).
-template <typename T, int O, int M, int K>
-__device__ __forceinline__ void face_tangential(const Grid3& g, int ak, const T* __restrict__ up,
-                                               const T* __restrict__ cm, const T* __restrict__ cd, long long o,
-                                               T base, T rs[3]) {
-    using P = Ord<O>;
-    const int Nk = g.n[K];
-    const int S = dstride<K>(g);
-    const long long fs = g.fs;
-    auto vJ = [&](int off, T out[3]) {
-        T v[3];
-#pragma unroll
-        for (int L = 0; L < 3; ++L) v[L] = ldg(up + L * fs + off);
-#pragma unroll
-        for (int J = 0; J < 3; ++J) {
-            T s = T(0);
-#pragma unroll
-            for (int L = 0; L < 3; ++L) s += cfull(cm, cd, fs, M, L, K, J, o + off) * v[L];
-            out[J] = s;
-        }
-    };
-    if (ak >= P::NCOL && ak >= P::NB + P::Q && ak <= Nk - 1 - P::NCOL && ak <= Nk - 1 - P::NB - P::Q) {
-#pragma unroll
-        for (int mm = 1; mm <= P::Q; ++mm) {
-            const T am = P::template aT<T>(mm - 1) * base;
-            T vp[3], vm[3];
-            vJ(mm * S, vp);
-            vJ(-mm * S, vm);
-#pragma unroll
-            for (int J = 0; J < 3; ++J) rs[J] += am * (vm[J] - vp[J]);
-        }
-    } else {
-        constexpr int W = P::NCOL - 1 > P::Q ? P::NCOL - 1 : P::Q;
-        const int lo = ak - W < 0 ? 0 : ak - W, hi = ak + W > Nk - 1 ? Nk - 1 : ak + W;
-        const T iwa = T(1.0 / hweight<O>(Nk, ak));
-        for (int a2 = lo; a2 <= hi; ++a2) {
-            const T dc = dcoefT<O, T>(Nk, a2, ak);
-            if (dc == T(0)) continue;
-            const T coef = base * dc * hweightT<O, T>(Nk, a2) * iwa;
-            T v[3];
-            vJ((a2 - ak) * S, v);
-#pragma unroll
-            for (int J = 0; J < 3; ++J) rs[J] += coef * v[J];
-        }
-    }
-}
-
+// Along the face the term is (H_k^-1 D_k^T H_k b)(a) of the face field b_J = c_mLkJ u_L, which the SBP property
+// turns into -(D_k b)(a), less b / H_k at the low end and plus it at the high end of the line.  k3_face forms the
+// two fields of every displacement face once (fields 3 t + J of its buffer, t = 0, 1 the tangential directions in
+// ascending order, each [B][A] with the lower one fastest), where each of the 12 taps of a node formed them again.
 struct Faces3 {
     int kind[6];            // BC_DISPLACEMENT or BC_TRACTION per face
     double beta;
+    long long at[6];        // element offset of the face's fields in the face buffer
 };
 
-// r += the SAT terms at a node of the face x_M = 0 (side 0) or 1 that need its neighbours on the face: the
-// traction, or the tangential transposes of a displacement face; im, ia, ib the node's indices along M and the two
-// tangential directions
 template <typename T, int O, int M>
-__device__ __noinline__ void face_node_terms(const Grid3& g, int kind, int side, int im, int ia, int ib, long long o,
-                                             const T* __restrict__ u, const T* __restrict__ cm,
-                                             const T* __restrict__ cd, T r[3]) {
-    using P = Ord<O>;
-    constexpr int PD = M == 0 ? 1 : 0, TD = M == 2 ? 1 : 2;
-    const long long fs = g.fs;
-    const T nu = side ? T(1) : T(-1);
-    const T* up = u + o;
-    const T ihb = T(g.ih[M]) / hweightT<O, T>(g.n[M], im);         // H^-1 P_f at the face node
-    if (kind == BC_TRACTION) {
-        T gr[3][3];
-        const int ix[3] = {M == 0 ? im : ia, M == 1 ? im : (M == 0 ? ia : ib), M == 2 ? im : ib};
-        grad_dir<T, O, 0>(g, ix[0], up, gr[0]);
-        grad_dir<T, O, 1>(g, ix[1], up, gr[1]);
-        grad_dir<T, O, 2>(g, ix[2], up, gr[2]);
+__device__ __forceinline__ void face_fields(const Grid3& g, int side, int t, const T* __restrict__ u,
+                                            const T* __restrict__ cm, const T* __restrict__ cd, T* __restrict__ out) {
+    constexpr int A = M == 0 ? 1 : 0, B = M == 2 ? 1 : 2;
+    const int na = g.n[A], nb = g.n[B];
+    if (t >= na * nb) return;
+    const int ib = t / na, ia = t - ib * na;
+    const long long o = ia * g.s[A] + ib * g.s[B] + (side ? (g.n[M] - 1) * g.s[M] : 0);
+    T uf[3];
+#pragma unroll
+    for (int L = 0; L < 3; ++L) uf[L] = ldg(u + L * g.fs + o);
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
 #pragma unroll
         for (int J = 0; J < 3; ++J) {
-            T sm = T(0);
+            T v = T(0);
 #pragma unroll
-            for (int k = 0; k < 3; ++k)
-#pragma unroll
-                for (int L = 0; L < 3; ++L) sm += cfull(cm, cd, fs, M, J, k, L, o) * gr[k][L];
-            r[J] -= ihb * nu * sm;
+            for (int L = 0; L < 3; ++L) v += cfull(cm, cd, g.fs, M, L, k == 0 ? A : B, J, o) * uf[L];
+            out[(long long)(3 * k + J) * na * nb + t] = v;
         }
-    } else {
-        const T base = ihb * nu;
-        face_tangential<T, O, M, PD>(g, ia, up, cm, cd, o, base * T(g.ih[PD]), r);
-        face_tangential<T, O, M, TD>(g, ib, up, cm, cd, o, base * T(g.ih[TD]), r);
-    }
+}
+// one launch for the six faces (blockIdx.y; traction faces have no fields)
+template <typename T, int O>
+__global__ void __launch_bounds__(128) k3_face(Grid3 g, Faces3 fc, const T* __restrict__ u, const T* __restrict__ cm,
+                                               const T* __restrict__ cd, T* __restrict__ ff) {
+    const int f = blockIdx.y, t = blockIdx.x * 128 + threadIdx.x;
+    if (fc.kind[f] != BC_DISPLACEMENT) return;
+    T* out = ff + fc.at[f];
+    if (f < 2) face_fields<T, O, 0>(g, f, t, u, cm, cd, out);
+    else if (f < 4) face_fields<T, O, 1>(g, f - 2, t, u, cm, cd, out);
+    else face_fields<T, O, 2>(g, f - 4, t, u, cm, cd, out);
 }
 
 // one interior row of direction D at a node: r_j += D_D q_Dj + D_DD^FC(c_DjDl) u_l
@@ -679,52 +633,82 @@ __device__ __noinline__ void int_row(const Grid3& g, const T* __restrict__ qo, c
 // completes.  A closure row reads NCLOSJ columns of the line, the same ones for every row of the end: a
 // thread reads the 12 columns of u, q and the 6 coefficients once (order 6: 144 loads) for all 9 rows,
 // where a thread per node read them for each row.  The lanes of a warp lie along x1 (D = 1, 2: coalesced)
-// or x2 (D = 0: a line's columns share their sectors in L1).  160 x 151 x 144, FP32: 101 + 29 + 24 us for
-// D = 0, 1, 2 (the slab kernel and the closure rows inside the divergence they replace took 226 + ~160 us).
+// or x2 (D = 0), where a column is one word per line: the CTA copies its lines' ends to shared memory row by row
+// and writes the sums back the same way.  160 x 151 x 144, FP32, order 6: with the columns and the face terms of D = 0
+// from global memory a step took 0.465 ms, now 0.420.
+// FP64 has small CTAs, as every line holds its SM's FP64 units for long: few lines still reach every SM.
+template <typename T> constexpr int kLineThreads = sizeof(T) == 4 ? 64 : 32;
+
 template <typename T, int O, int D>
-__global__ void __launch_bounds__(128) k3_lines(Grid3 g, Box3 bx, Faces3 fc, const T* __restrict__ u,
-                                                const T* __restrict__ q, const T* __restrict__ cm,
-                                                const T* __restrict__ cd, T* __restrict__ part) {
+__global__ void __launch_bounds__(kLineThreads<T>) k3_lines(Grid3 g, Box3 bx, Faces3 fc, const T* __restrict__ u,
+                                                            const T* __restrict__ q, const T* __restrict__ cd,
+                                                            const T* __restrict__ ff, T* __restrict__ part) {
     using P = Ord<O>;
-    constexpr int NR = line_rows<O>(), NJ = CTab<O>::NJ, W = NJ > NR + P::Q ? NJ : NR + P::Q;
+    constexpr int NT = kLineThreads<T>;
+    constexpr int NR = line_rows<O>(), NJ = CTab<O>::NJ;
+    constexpr int RX = D == 0 ? NR + 1 : NR;               // rows formed here: along x1 one more than the closure (see below)
+    constexpr int W = NJ > RX + P::Q ? NJ : RX + P::Q, QW = RX + P::Q > P::NCOL ? RX + P::Q : P::NCOL;
     constexpr int A = D == 0 ? 1 : 0, B = D == 2 ? 1 : 2;
-    const int na = g.n[A], nb = g.n[B], N = g.n[D];
-    const int t = blockIdx.x * 128 + threadIdx.x;
-    if (t >= na * nb) return;
-    const int ib = t / na, ia = t - ib * na, side = blockIdx.y;
+    constexpr int WS = W > QW ? W : QW;
+    __shared__ T sm[D == 0 ? 12 * WS * (NT + 1) : 1];
+    const int na = g.n[A], nb = g.n[B], N = g.n[D], lines = na * nb;
+    const int t = blockIdx.x * NT + threadIdx.x, tx = threadIdx.x, side = blockIdx.y;
     const long long fs = g.fs;
     const int S = dstride<D>(g), Ss = side ? -S : S;
-    const long long o = ia * g.s[A] + ib * g.s[B] + (side ? (long long)(N - 1) * g.s[D] : 0);   // the face node
+    auto face_node = [&](int line) {
+        const int b = line / na;
+        return (line - b * na) * g.s[A] + b * g.s[B] + (side ? (long long)(N - 1) * g.s[D] : 0);
+    };
+    if constexpr (D == 0) {
+        // column c of field f of line n at sm[(f * WS + c) * (NT + 1) + n]; fields u, q_1j, c_1j1l
+        for (int idx = tx; idx < NT * WS; idx += NT) {
+            const int n = idx / WS, c = idx - n * WS, line = blockIdx.x * NT + n;
+            if (line >= lines || c >= N) continue;
+            const long long oc = face_node(line) + c * Ss;
+#pragma unroll
+            for (int f = 0; f < 12; ++f) {
+                const T* p = f < 3 ? u + f * fs : (f < 6 ? q + (f - 3) * fs : cd + (f - 6) * fs);
+                sm[(f * WS + c) * (NT + 1) + n] = ldg(p + oc);
+            }
+        }
+        __syncthreads();
+    }
+    const bool live = t < lines;
+    const int tl = live ? t : lines - 1, ib = tl / na, ia = tl - ib * na;
+    const long long o = face_node(tl);
     const T ih = T(g.ih[D]), ih2 = ih * ih;
-    T uw[3][W], rr[NR][3];
+    const T* cp = cd + 6 * D * fs + o;
+    auto b = [&](int s6, int c) -> T {
+        if constexpr (D == 0) return sm[((6 + s6) * WS + c) * (NT + 1) + tx];
+        else return ldg(cp + s6 * fs + c * Ss);
+    };
+    T uw[3][W], rr[RX][3];
 #pragma unroll
     for (int l = 0; l < 3; ++l)
 #pragma unroll
-        for (int c = 0; c < W; ++c) uw[l][c] = ldg(u + l * fs + o + c * Ss);
+        for (int c = 0; c < W; ++c) uw[l][c] = D == 0 ? sm[(l * WS + c) * (NT + 1) + tx] : ldg(u + l * fs + o + c * Ss);
 #pragma unroll
-    for (int r = 0; r < NR; ++r) rr[r][0] = rr[r][1] = rr[r][2] = T(0);
-    const T* cp = cd + 6 * D * fs + o;
-    auto b = [&](int s6, int c) { return ldg(cp + s6 * fs + c * Ss); };
-    clos_rows<O, T, W, NR>(uw, b, rr, std::make_integer_sequence<int, NJ>());
-    if constexpr (NR > P::NCLOS) {                       // order 2: the row past the closure that a SAT reaches
+    for (int r = 0; r < RX; ++r) rr[r][0] = rr[r][1] = rr[r][2] = T(0);
+    clos_rows<O, T, W, RX>(uw, b, rr, std::make_integer_sequence<int, NJ>());
+    // rows past the closure: order 2 has one that a SAT reaches; along x1 one more may be left here by the alignment of x1lo
 #pragma unroll
-        for (int r = P::NCLOS; r < NR; ++r) dxx3_interior<O, T>(r, [&](int l, int c) { return uw[l][c]; }, b, rr[r]);
-    }
+    for (int r = P::NCLOS; r < RX; ++r) dxx3_interior<O, T>(r, [&](int l, int c) { return uw[l][c]; }, b, rr[r]);
 #pragma unroll
-    for (int r = 0; r < NR; ++r)
+    for (int r = 0; r < RX; ++r)
 #pragma unroll
         for (int j = 0; j < 3; ++j) rr[r][j] *= ih2;
     // D_D q_Dj: rows of D from the face, mirrored with the opposite sign at the high end
     const T sg = side ? -ih : ih;
+    T q0[3];
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-        const T* qj = q + (3 * D + j) * fs + o;
-        T qw[NR + P::Q > P::NCOL ? NR + P::Q : P::NCOL];
-        constexpr int QW = NR + P::Q > P::NCOL ? NR + P::Q : P::NCOL;
+        T qw[QW];
 #pragma unroll
-        for (int c = 0; c < QW; ++c) qw[c] = ldg(qj + c * Ss);
+        for (int c = 0; c < QW; ++c)
+            qw[c] = D == 0 ? sm[((3 + j) * WS + c) * (NT + 1) + tx] : ldg(q + (3 * D + j) * fs + o + c * Ss);
+        q0[j] = qw[0];
 #pragma unroll
-        for (int r = 0; r < NR; ++r) {
+        for (int r = 0; r < RX; ++r) {
             T d = T(0);
             if (r < P::NB) {
 #pragma unroll
@@ -736,48 +720,97 @@ __global__ void __launch_bounds__(128) k3_lines(Grid3 g, Box3 bx, Faces3 fc, con
             rr[r][j] += sg * d;
         }
     }
-    const int kind = fc.kind[2 * D + side];
-    if (kind == BC_DISPLACEMENT) {
-        // s_J = c_DJDL u_L at the face node: spread by H^-1 D_D^T nu over NCOL rows, and the penalty
-        // -H^-1 P_f (beta d / h1) s_J at the face (h1 = h hw_0)
-        T sJ[3];
-        const T b0 = b(0, 0), b1 = b(1, 0), b2 = b(2, 0), b3 = b(3, 0), b4 = b(4, 0), b5 = b(5, 0);
-        sJ[0] = b0 * uw[0][0] + b1 * uw[1][0] + b2 * uw[2][0];
-        sJ[1] = b1 * uw[0][0] + b3 * uw[1][0] + b4 * uw[2][0];
-        sJ[2] = b2 * uw[0][0] + b4 * uw[1][0] + b5 * uw[2][0];
-        const T ihb = ih / hweightT<O, T>(N, 0), pen = T(fc.beta * 3.0) * ihb * ihb;
-#pragma unroll
-        for (int r = 0; r < P::NCOL; ++r) {
-            const T coef = -ih2 * P::template dqT<T>(0, r) / (r < P::NB ? P::template hwT<T>(r) : T(1)) - (r == 0 ? pen : T(0));
-#pragma unroll
-            for (int j = 0; j < 3; ++j) rr[r][j] += coef * sJ[j];
-        }
-    }
     {
-        T f[3] = {T(0), T(0), T(0)};
-        face_node_terms<T, O, D>(g, kind, side, side ? N - 1 : 0, ia, ib, o, u, cm, cd, f);
+        // v_J -> c_DJDL v_L at the face node
+        T b0[6];
 #pragma unroll
-        for (int j = 0; j < 3; ++j) rr[0][j] += f[j];
+        for (int s6 = 0; s6 < 6; ++s6) b0[s6] = b(s6, 0);
+        auto cn = [&](const T v[3], T w[3]) {
+            w[0] = b0[0] * v[0] + b0[1] * v[1] + b0[2] * v[2];
+            w[1] = b0[1] * v[0] + b0[3] * v[1] + b0[4] * v[2];
+            w[2] = b0[2] * v[0] + b0[4] * v[1] + b0[5] * v[2];
+        };
+        const T ihb = ih / hweightT<O, T>(N, 0);                       // H^-1 P_f at the face node
+        const T nu = side ? T(1) : T(-1);
+        T v[3], w[3];
+        if (fc.kind[2 * D + side] == BC_TRACTION) {
+            // c_DJkL D_k u_L = q_DJ + c_DJDL D_D u_L at the face
+#pragma unroll
+            for (int l = 0; l < 3; ++l) {
+                v[l] = T(0);
+#pragma unroll
+                for (int c = 0; c < P::NCOL; ++c) v[l] += P::template dqT<T>(0, c) * uw[l][c];
+                v[l] *= sg;
+            }
+            cn(v, w);
+#pragma unroll
+            for (int j = 0; j < 3; ++j) rr[0][j] -= ihb * nu * (q0[j] + w[j]);
+        } else {
+            // s_J = c_DJDL u_L at the face node: spread by H^-1 D_D^T nu over NCOL rows, and the penalty
+            // -H^-1 P_f (beta d / h1) s_J at the face (h1 = h hw_0)
+#pragma unroll
+            for (int l = 0; l < 3; ++l) v[l] = uw[l][0];
+            cn(v, w);
+            const T pen = T(fc.beta * 3.0) * ihb * ihb;
+#pragma unroll
+            for (int r = 0; r < P::NCOL; ++r) {
+                T coef = -ih2 * P::template dqT<T>(0, r);
+                if (r < P::NB) coef /= P::template hwT<T>(r);
+                if (r == 0) coef -= pen;
+#pragma unroll
+                for (int j = 0; j < 3; ++j) rr[r][j] += coef * w[j];
+            }
+            // tangential transposes of the face fields
+            const T* F = ff + fc.at[2 * D + side];
+            auto tang = [&](const T* Fk, int Nk, int a, int st, T ihk) {
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    const T* p = Fk + (long long)j * lines + tl;
+                    T d = -dsum<O, T>(Nk, a, [&](int x) { return p[(long long)(x - a) * st]; });
+                    if (a == 0 || a == Nk - 1) d += (a == 0 ? -p[0] : p[0]) / P::template hwT<T>(0);
+                    rr[0][j] += ihb * nu * ihk * d;
+                }
+            };
+            tang(F, na, ia, 1, T(g.ih[A]));
+            tang(F + 3LL * lines, nb, ib, na, T(g.ih[B]));
+        }
     }
     // nodes that the line kernels of the directions before this one have stored
     auto end = [&](int i, int n) { return i < NR || i >= n - NR; };
-    const bool add = D == 2 ? false : (D == 1 ? end(ib, g.n[2]) : (end(ia, g.n[1]) || end(ib, g.n[2])));
-    auto store = [&](int r, const T v[3]) {
+    auto put = [&](T* p, bool add, T v) { *p = add ? *p + v : v; };
+    if constexpr (D == 0) {
+        const int rows = side ? N - bx.x1hi : bx.x1lo;      // NR, or one more; many more only on the smallest order-2 blocks
+        __syncthreads();
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            T* p = part + j * fs + o + r * Ss;
-            *p = add ? *p + v[j] : v[j];
-        }
-    };
+        for (int r = 0; r < RX; ++r)
 #pragma unroll
-    for (int r = 0; r < NR; ++r) store(r, rr[r]);
-    if constexpr (D == 0) {                               // the columns that the alignment of x1lo leaves here
-        const int rows = side ? N - bx.x1hi : bx.x1lo;
-        for (int r = NR; r < rows; ++r) {
-            T v[3] = {T(0), T(0), T(0)};
-            int_row<T, O, 0>(g, q + o + r * Ss, cp + r * Ss, u + o + r * Ss, v);
-            store(r, v);
+            for (int j = 0; j < 3; ++j) sm[(j * RX + r) * (NT + 1) + tx] = rr[r][j];
+        __syncthreads();
+        const int nr = rows < RX ? rows : RX;
+        for (int idx = tx; idx < NT * nr; idx += NT) {
+            const int n = idx / nr, r = idx - n * nr, line = blockIdx.x * NT + n;
+            if (line >= lines) continue;
+            const int l3 = line / na, l2 = line - l3 * na;
+            const bool add = end(l2, g.n[1]) || end(l3, g.n[2]);
+            T* p = part + face_node(line) + r * Ss;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) put(p + j * fs, add, sm[(j * RX + r) * (NT + 1) + n]);
         }
+        if (live) {
+            const bool add = end(ia, g.n[1]) || end(ib, g.n[2]);
+            for (int r = RX; r < rows; ++r) {
+                T v[3] = {T(0), T(0), T(0)};
+                int_row<T, O, 0>(g, q + o + r * Ss, cp + r * Ss, u + o + r * Ss, v);
+#pragma unroll
+                for (int j = 0; j < 3; ++j) put(part + j * fs + o + r * Ss, add, v[j]);
+            }
+        }
+    } else if (live) {
+        const bool add = D == 1 && end(ib, g.n[2]);
+#pragma unroll
+        for (int r = 0; r < RX; ++r)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) put(part + j * fs + o + r * Ss, add, rr[r][j]);
     }
 }
 

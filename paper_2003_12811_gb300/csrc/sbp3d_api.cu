@@ -45,6 +45,9 @@ struct sbp3_handle {
     void* u[2] = {nullptr, nullptr};         // leapfrog levels (3 fields each), u[cur] = u^n
     void* du = nullptr;                      // increment u^n - u^{n-1} (3 fields)
     void* q = nullptr;                       // mixed fluxes (9 fields)
+    void* ff = nullptr;                      // tangential SAT fields of the displacement faces (k3_face)
+    long long ff_elems = 0;
+    int face_nodes = 0;                      // nodes of the largest displacement face
     void* ain = nullptr;                     // sbp3_apply input / output (3 fields each), on first use
     void* aout = nullptr;
     int cur = 0;
@@ -126,10 +129,13 @@ int launch_operator(sbp3_handle* h, const T* u, T* du, T* un, double dt, cudaStr
     prof_end(stop, st);
     const Box3& bx = h->box;
     prof_begin(h, 2, st, &stop);
+    T* ff = static_cast<T*>(h->ff);
+    if (h->face_nodes > 0) k3_face<T, O><<<dim3((h->face_nodes + 127) / 128, 6), 128, 0, st>>>(g, h->fc, u, cm, cd, ff);
     auto lines = [&](auto dc) {
         constexpr int D = decltype(dc)::value, A = D == 0 ? 1 : 0, B = D == 2 ? 1 : 2;
-        const dim3 lg((unsigned)(((long long)g.n[A] * g.n[B] + 127) / 128), 2);
-        k3_lines<T, O, D><<<lg, 128, 0, st>>>(g, bx, h->fc, u, q, cm, cd, un);
+        constexpr int NT = kLineThreads<T>;
+        const dim3 lg((unsigned)(((long long)g.n[A] * g.n[B] + NT - 1) / NT), 2);
+        k3_lines<T, O, D><<<lg, NT, 0, st>>>(g, bx, h->fc, u, q, cd, ff, un);
     };
     lines(std::integral_constant<int, 2>());
     lines(std::integral_constant<int, 1>());
@@ -198,7 +204,7 @@ template <typename F> int dispatch(sbp3_handle* h, F f) {
 }
 
 void free_all(sbp3_handle* h) {
-    void* bufs[] = {h->X, h->cm, h->cd, h->w, h->u[0], h->u[1], h->du, h->q, h->ain, h->aout, h->d_err};
+    void* bufs[] = {h->X, h->cm, h->cd, h->w, h->u[0], h->u[1], h->du, h->q, h->ff, h->ain, h->aout, h->d_err};
     for (void* b : bufs)
         if (b) cudaFree(b);
     for (auto& v : h->prof.ev)
@@ -206,8 +212,13 @@ void free_all(sbp3_handle* h) {
             if (e) cudaEventDestroy(e);
 }
 
-// bytes that sbp3_footprint counts per x1 line beyond the fields (NCLOS x NCLOSJ x 6 words at either end): a
-// reserve that callers plan with, of which the line kernels need nothing
+// words of the tangential SAT fields, six per node of a displacement face (at most: of every face)
+long long face_words(int n1, int n2, int n3) {
+    return 12 * ((long long)n2 * n3 + (long long)n1 * n3 + (long long)n1 * n2);
+}
+
+// bytes that sbp3_footprint counts beyond the fields, NCLOS x NCLOSJ x 6 words at either end of an x1 line:
+// a reserve that callers plan with, of which the face fields take their part
 size_t line_reserve_bytes(int order, size_t es, int n2, int n3) {
     const int nclos = order == 2 ? SBP2_NCLOS : (order == 4 ? SBP4_NCLOS : SBP6_NCLOS);
     const int nj = order == 2 ? SBP2_NCLOSJ : (order == 4 ? SBP4_NCLOSJ : SBP6_NCLOSJ);
@@ -236,8 +247,10 @@ int sbp3_footprint(int order, int precision, int n1, int n2, int n3, long long* 
     const int n[3] = {n1, n2, n3};
     const long long f = field_bytes(precision, n);
     const long long x = pitch_of(n1, precision == SBP_FP32 ? 4 : 8) * n2 * n3 * 8LL;
-    *bytes_out = f * (NCM + NCD + 1 + 6 + 3 + 9) + 3 * x +
-                 (long long)line_reserve_bytes(order, precision == SBP_FP32 ? 4 : 8, n2, n3);
+    const size_t es = precision == SBP_FP32 ? 4 : 8;
+    const long long reserve = (long long)line_reserve_bytes(order, es, n2, n3);
+    const long long faces = face_words(n1, n2, n3) * (long long)es;
+    *bytes_out = f * (NCM + NCD + 1 + 6 + 3 + 9) + 3 * x + (reserve > faces ? reserve : faces);
     return SBP_OK;
 }
 
@@ -299,6 +312,13 @@ int sbp3_create(int order, int precision, int n1, int n2, int n3, const double* 
         bx.x1lo = (e + nv - 1) / nv * nv;
         bx.x1hi = n1 - e > bx.x1lo ? bx.x1lo + (n1 - e - bx.x1lo) / nv * nv : bx.x1lo;
     }
+    for (int f = 0; f < 6; ++f) {
+        h->fc.at[f] = h->ff_elems;
+        if (face_kinds[f] != SBP3_BC_DISPLACEMENT) continue;
+        const int nodes = (f < 2 ? n2 : n1) * (f < 4 ? n3 : n2);
+        h->ff_elems += 6LL * nodes;
+        h->face_nodes = nodes > h->face_nodes ? nodes : h->face_nodes;
+    }
     auto alloc = [&](void** p, size_t bytes) -> bool {
         if (cudaMalloc(p, bytes) != cudaSuccess) return false;
         return cudaMemset(*p, 0, bytes) == cudaSuccess;
@@ -309,7 +329,7 @@ int sbp3_create(int order, int precision, int n1, int n2, int n3, const double* 
     const size_t xfs = (size_t)h->fs;
     bool ok = alloc((void**)&h->X, 3 * xfs * 8) && alloc(&h->cm, NCM * fb) && alloc(&h->cd, NCD * fb) &&
               alloc(&h->w, fb) && alloc(&h->u[0], 3 * fb) && alloc(&h->u[1], 3 * fb) && alloc(&h->du, 3 * fb) &&
-              alloc(&h->q, 9 * fb) &&
+              alloc(&h->q, 9 * fb) && (h->ff_elems == 0 || alloc(&h->ff, (size_t)h->ff_elems * h->es)) &&
               alloc((void**)&h->d_err, sizeof(int));
     if (!ok) {
         cudaGetLastError();
