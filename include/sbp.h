@@ -191,11 +191,11 @@ int sbp_step(sbp_handle* h, int nsteps, double dt, void* stream);
  * to leapfrog.  The RK4 state of a block is (u, v) (host, 2 planes of n1*n2 values each); t the
  * time.  sbp_set_state_rk4 allocates the block's RK4 buffers (10 planes) on first use.
  * sbp_step_rk4 advances nsteps steps of size dt asynchronously on `stream`: four operator passes
- * per step, each fused with its stage combination (stage input U_{s+1} = u + c h V_s, stage
- * velocity V_{s+1} = v + c h a_s and the running sums of b_s V_s and b_s a_s are formed in the
- * same kernels that apply the operator; c = 1/2, 1/2, 1, b = 1/6, 1/3, 1/3, 1/6).  After the
+ * per step, each fused with its stage combination (the next stage input U_{s+1}, formed from u, v and
+ * the accelerations of the stages before, and the stage's own acceleration are written by the same
+ * kernels that apply the operator; after the fourth stage u and v).  After the
  * steps, SBP_FIELD_CUR holds u and SBP_FIELD_VELOCITY holds v; the leapfrog level
- * SBP_FIELD_PREV and the operator output SBP_FIELD_APPLY (used as scratch for the point sources)
+ * SBP_FIELD_PREV and the operator output SBP_FIELD_APPLY (used as scratch for the layer dissipation)
  * are then meaningless.  Errors: SBP_E_STATE without materials or RK4 state. */
 int sbp_set_state_rk4(sbp_handle* h, int block, const double* u, const double* v, double t);
 int sbp_step_rk4(sbp_handle* h, int nsteps, double dt, void* stream);

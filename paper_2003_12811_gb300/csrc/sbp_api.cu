@@ -62,7 +62,7 @@ struct HostBlock {
     void* psi[2] = {nullptr, nullptr};   // adjoint fields (sbp_misfit_gradient), allocated on first use
     MarchMaps pmaps;          // marching-kernel maps over the adjoint fields
     CUtensorMap* d_smaps = nullptr;   // strip-tile band-box maps on the device: [0..2] state u0, u1, c; [3..5] adjoint
-    void* rk = nullptr;       // RK4 state (u, v, V, S_u, S_v; sbp_set_state_rk4), allocated on first use
+    void* rk = nullptr;       // RK4 state (u, v, a_1, a_2, a_3; sbp_set_state_rk4), allocated on first use
     void* gw = nullptr;       // wide stencil: the fluxes G_1j, G_2j (4 planes, type T)
     void* sg = nullptr;       // layer dissipation coefficient s (1 plane, type T)
     int2* d_lnodes = nullptr; // nodes the layer dissipation reaches, (i1, i2)
@@ -469,14 +469,9 @@ void launch_traces(sbp_handle* h, const StepArgs& a, cudaStream_t tst, bool adj)
 
 // the wide-stencil operator (sbp_wide.cuh): traces, the SAT terms of every face node, the flux and
 // divergence passes of every block, then the point sources (every source node: the wide path has
-// no strip kernel); RK4 stages take the sources into the operator sum first
+// no strip kernel)
 template <typename T, int O>
 int launch_wide(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st) {
-    if (!h->src_nodes.empty() && mode == 2) {
-        ProfScope ps(h, 3, st, 1);
-        const int ns = (int)h->src_nodes.size();
-        k_sources<T, 2><<<grid_for(ns), 256, 0, st>>>(h->d_blocks, h->d_src_nodes, ns, h->d_src_params, a);
-    }
     if (h->ntrefs > 0) launch_traces<T, O>(h, a, st, false);
     if (h->nface_nodes > 0) {
         ProfScope ps(h, 1, st, 1);
@@ -491,10 +486,11 @@ int launch_wide(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st) {
         else if (mode == 2) k_wide_div<T, O, 2><<<grid_for(n), 256, 0, st>>>(b, a, (const T*)hb.gw);
         else k_wide_div<T, O, 1><<<grid_for(n), 256, 0, st>>>(b, a, (const T*)hb.gw);
     }
-    if (!h->src_nodes.empty() && mode != 2) {
+    if (!h->src_nodes.empty()) {
         ProfScope ps(h, 3, st, 1);
         const int ns = (int)h->src_nodes.size();
-        if (mode == 0) k_sources<T, 0><<<grid_for(ns), 256, 0, st>>>(h->d_blocks, h->d_src_nodes, ns, h->d_src_params, a);
+        if (mode == 2) k_sources<T, 2><<<grid_for(ns), 256, 0, st>>>(h->d_blocks, h->d_src_nodes, ns, h->d_src_params, a);
+        else if (mode == 0) k_sources<T, 0><<<grid_for(ns), 256, 0, st>>>(h->d_blocks, h->d_src_nodes, ns, h->d_src_params, a);
         else k_sources<T, 1><<<grid_for(ns), 256, 0, st>>>(h->d_blocks, h->d_src_nodes, ns, h->d_src_params, a);
     }
     return check_cuda(h, "wide operator launch");
@@ -559,10 +555,6 @@ int launch_operator(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st,
     constexpr size_t smem = interior_smem_elems<T, O>() * sizeof(T);
     // interior kernels on st; strip kernels on the auxiliary stream when overlapping (profiling
     // runs serialise so that every family's events time that family alone)
-    if (mode == 2 && !adj && h->n_src_int > 0) {   // RK4 stage: interior sources first (into r)
-        ProfScope ps(h, 3, st, 1);
-        k_sources<T, 2><<<grid_for(h->n_src_int), 256, 0, st>>>(h->d_blocks, h->d_src_int, h->n_src_int, h->d_src_params, a);
-    }
     const bool ovl = h->overlap && h->aux && !h->prof;
     // the interface traces run on the auxiliary stream beside the interior kernel (in its tail
     // or its free slots); the strips that read them follow on that stream or wait for it
@@ -587,7 +579,10 @@ int launch_operator(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st,
             constexpr size_t msm = MarchCfg<O>::BYTES;
             if (mode == 0 && !adj) k_interior_march_multi<O, 3><<<tiles, MTHREADS, msm, ist>>>(mmul, a, h->d_err);
             else if (mode == 0) k_interior_march_multi<O, 0><<<tiles, MTHREADS, msm, ist>>>(mmul, a, h->d_err);
-            else if (mode == 2) k_interior_march_multi<O, 2><<<tiles, MTHREADS, msm, ist>>>(mmul, a, h->d_err);
+            else if (mode == 2 && a.stage == 1) k_interior_march_multi<O, 4><<<tiles, MTHREADS, msm, ist>>>(mmul, a, h->d_err);
+            else if (mode == 2 && a.stage == 2) k_interior_march_multi<O, 5><<<tiles, MTHREADS, msm, ist>>>(mmul, a, h->d_err);
+            else if (mode == 2 && a.stage == 3) k_interior_march_multi<O, 6><<<tiles, MTHREADS, msm, ist>>>(mmul, a, h->d_err);
+            else if (mode == 2) k_interior_march_multi<O, 7><<<tiles, MTHREADS, msm, ist>>>(mmul, a, h->d_err);
             else k_interior_march_multi<O, 1><<<tiles, MTHREADS, msm, ist>>>(mmul, a, h->d_err);
             mmul = MarchMulti{};
             tiles = 0;
@@ -659,10 +654,11 @@ int launch_operator(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st,
         cudaStreamWaitEvent(st, h->ev_join, 0);
         cudaStreamWaitEvent(st, h->ev_join_hi, 0);
     }
-    if (!adj && h->n_src_int > 0 && mode != 2) {   // source nodes off the strips (the strip kernel adds the others)
+    if (!adj && h->n_src_int > 0) {   // source nodes off the strips (the strip kernel adds the others)
         ProfScope ps(h, 3, st, 1);
         const int ns = h->n_src_int;
-        if (mode == 0) k_sources<T, 0><<<grid_for(ns), 256, 0, st>>>(h->d_blocks, h->d_src_int, ns, h->d_src_params, a);
+        if (mode == 2) k_sources<T, 2><<<grid_for(ns), 256, 0, st>>>(h->d_blocks, h->d_src_int, ns, h->d_src_params, a);
+        else if (mode == 0) k_sources<T, 0><<<grid_for(ns), 256, 0, st>>>(h->d_blocks, h->d_src_int, ns, h->d_src_params, a);
         else k_sources<T, 1><<<grid_for(ns), 256, 0, st>>>(h->d_blocks, h->d_src_int, ns, h->d_src_params, a);
     }
     return check_cuda(h, "operator launch");
@@ -694,7 +690,7 @@ void layer_launch(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st, b
         const BlockDev b = make_view(h, hb);
         const unsigned g = grid_for(hb.nln);
         if (mode == 2) {
-            if (!post) k_layer_rk<T, O><<<g, 256, 0, st>>>(b, hb.d_lnodes, hb.nln, a.stage);
+            if (!post) k_layer_rk<T, O><<<g, 256, 0, st>>>(b, hb.d_lnodes, hb.nln, a.stage, a.rkh);
         } else if (!post) {
             k_layer_pre<T, O><<<g, 256, 0, st>>>(b, hb.d_lnodes, hb.nln, a.cur, 1.0 / a.dt, (T*)hb.lscr);
         } else {
@@ -742,13 +738,13 @@ template <typename T, int O> void set_smem_attr() {
     cudaFuncSetAttribute(k_interior<T, O, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaFuncSetAttribute(k_interior<T, O, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (std::is_same<T, float>::value) {
-        cudaFuncSetAttribute(k_interior_march<O, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
-        cudaFuncSetAttribute(k_interior_march<O, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
-        cudaFuncSetAttribute(k_interior_march<O, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
         cudaFuncSetAttribute(k_interior_march_multi<O, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
         cudaFuncSetAttribute(k_interior_march_multi<O, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
         cudaFuncSetAttribute(k_interior_march_multi<O, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
-        cudaFuncSetAttribute(k_interior_march_multi<O, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
+        cudaFuncSetAttribute(k_interior_march_multi<O, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
+        cudaFuncSetAttribute(k_interior_march_multi<O, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
+        cudaFuncSetAttribute(k_interior_march_multi<O, 6>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
+        cudaFuncSetAttribute(k_interior_march_multi<O, 7>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
     }
 }
 
@@ -1707,9 +1703,9 @@ int sbp_step_rk4(sbp_handle* h, int nsteps, double dt, void* stream) {
     for (auto& hb : h->blocks)
         if (!hb.rk) return h->fail(SBP_E_STATE, "set the RK4 state (sbp_set_state_rk4) of every block first");
     cudaStream_t st = (cudaStream_t)stream;
-    // the operator-output planes carry the interior point sources of each stage (zero elsewhere)
+    // with layers the operator-output planes carry their dissipation of each stage (zero elsewhere)
     for (auto& hb : h->blocks)
-        if (cudaMemsetAsync(hb.r, 0, 2 * (size_t)hb.n2 * hb.pitch * h->esize, st) != cudaSuccess)
+        if (h->layers && cudaMemsetAsync(hb.r, 0, 2 * (size_t)hb.n2 * hb.pitch * h->esize, st) != cudaSuccess)
             return h->fail(SBP_E_CUDA, "RK4 scratch clear failed");
     const double cs[4] = {0.0, 0.5, 0.5, 1.0};
     for (int n = 0; n < nsteps; ++n) {
@@ -1720,6 +1716,7 @@ int sbp_step_rk4(sbp_handle* h, int nsteps, double dt, void* stream) {
             a.stage = s;
             a.rkh = dt;
             a.rkhf = (float)dt;
+            a.rk_r = h->layers;
             a.t = h->t + cs[s - 1] * dt;
             fill_basis(h, a.t, a);
             const int rc = run_operator(h, a, 2, st);

@@ -287,7 +287,7 @@ struct BlockDev {
     const double* X;          // coordinates (2 planes)
     double* G;                // metric dX_I/dx_i (4 planes, [2 i + I])
     double* J;                // Jacobian
-    void* rk;                 // RK4 state (10 planes): u, v, stage velocity V, sums S_u, S_v (2 planes each)
+    void* rk;                 // RK4 state (10 planes): u, v, accelerations a_1, a_2, a_3 of the stages (2 planes each)
     const void* sg;           // layer dissipation coefficient s (1 plane, type T) or null
     const void* smaps;        // strip-tile band-box tensor maps (CUtensorMap[3]: u[0], u[1], c)
     const void* mx;           // closure rows of D_xx^FC along x1 as matrices, type T (k_closure_mats)
@@ -311,58 +311,57 @@ struct StepArgs {
     int stage;                // RK4 mode: stage s = 1..4 of the step
     double rkh;               // RK4 mode: step size h
     float rkhf;               // the same in FP32
+    int rk_r;                 // RK4 mode: the operator-output planes hold the stage's layer dissipation
 };
 
 // RK4 stage epilogue (mode 2) of one node.  The classical RK4 of Sec. 7.1 on y = (u, v),
-// y' = (v, a(u, t)), a = (rho J)^-1 [DD(c) u + J SAT + J f], organised by stage inputs
-// Y_s = (U_s, V_s): U_1 = u, V_1 = v, U_{s+1} = u + c_{s+1} h V_s, V_{s+1} = v + c_{s+1} h a_s with
-// a_s = a(U_s, t + c_s h), c = (0, 1/2, 1/2, 1), and u_new = u + h sum_s b_s V_s,
-// v_new = v + h sum_s b_s a_s, b = (1, 2, 2, 1)/6.  The kernel of stage s has read U_s (state
-// buffer u[cur]) and formed r = DD(c) U_s + J SAT + J f at node gi; this writes U_{s+1} (or u_new)
-// into u[1 - cur] and keeps V, S_u = sum b V, S_v = sum b a and, after stage 4, (u, v) in B.rk.
-// B.r holds zeros except at point-source nodes off the strips (their J f, added before the stage).
+// y' = (v, a(u, t)), a = (rho J)^-1 [DD(c) u + J SAT + J f].  Because u' = v, the stages need only the
+// accelerations a_s = a(U_s, t + c_s h) of those before them:
+//   U_1 = u, U_2 = u + h/2 v, U_3 = u + h/2 (v + h/2 a_1), U_4 = u + h (v + h/2 a_2),
+//   u_new = u + h (v + h/6 (a_1 + a_2 + a_3)), v_new = v + h/6 (a_1 + 2 a_2 + 2 a_3 + a_4).
+// The kernel of stage s has read U_s (state buffer u[cur]) and formed r = DD(c) U_s + J SAT + J f at node
+// gi; this writes U_{s+1} (or u_new) into u[1 - cur] and a_s (after stage 4: u and v) into B.rk: 94 words
+// per node and step with the operator's own (U, c, 1/(rho J)), where keeping the stage velocity and the two
+// running sums took 124.  The sources off the strips are added to a_s (or v) after the stage (k_sources).
+// With layers (a.rk_r), B.r holds their dissipation at the nodes they reach and zeros elsewhere.
+template <typename T> __device__ __forceinline__ T rkhT(const StepArgs& a) {
+    if constexpr (sizeof(T) == 4) return a.rkhf; else return a.rkh;
+}
+template <typename T>
+__device__ __forceinline__ void rk4_layer_terms(const BlockDev& B, size_t gi, size_t plane, T& r0, T& r1) {
+    T* __restrict__ Rs = reinterpret_cast<T*>(B.r);
+    const T rs0 = Rs[gi], rs1 = Rs[plane + gi];
+    if (rs0 != T(0) || rs1 != T(0)) {       // taken into the operator sum, then cleared for the next stage
+        r0 += rs0;
+        r1 += rs1;
+        Rs[gi] = T(0);
+        Rs[plane + gi] = T(0);
+    }
+}
 template <typename T>
 __device__ __forceinline__ void rk4_store(const BlockDev& B, const StepArgs& a, size_t gi, size_t plane, T w, T r0,
                                           T r1) {
     T* __restrict__ R = reinterpret_cast<T*>(B.rk);
     T* __restrict__ Un = reinterpret_cast<T*>(B.u[1 - a.cur]);
     const int s = a.stage;
-    T h;
-    if constexpr (sizeof(T) == 4) h = a.rkhf; else h = a.rkh;
-    // point sources off the strips were added into B.r (zero elsewhere) before this kernel ran:
-    // take them into the operator sum, then clear them for the next stage
-    T* __restrict__ Rs = reinterpret_cast<T*>(B.r);
-    const T rs0 = Rs[gi], rs1 = Rs[plane + gi];
-    if (rs0 != T(0) || rs1 != T(0)) {
-        r0 += rs0;
-        r1 += rs1;
-        Rs[gi] = T(0);
-        Rs[plane + gi] = T(0);
-    }
-    const T a0 = w * r0, a1 = w * r1;
-    const T u0 = R[gi], u1 = R[plane + gi], v0 = R[2 * plane + gi], v1 = R[3 * plane + gi];
-    const T V0 = s == 1 ? v0 : R[4 * plane + gi], V1 = s == 1 ? v1 : R[5 * plane + gi];
-    const T su0 = s == 1 ? T(0) : R[6 * plane + gi], su1 = s == 1 ? T(0) : R[7 * plane + gi];
-    const T sv0 = s == 1 ? T(0) : R[8 * plane + gi], sv1 = s == 1 ? T(0) : R[9 * plane + gi];
-    const T b = (s == 1 || s == 4) ? T(1) / T(6) : T(1) / T(3);
-    if (s < 4) {
-        const T ch = s == 3 ? h : T(0.5) * h;
-        Un[gi] = u0 + ch * V0;
-        Un[plane + gi] = u1 + ch * V1;
-        R[4 * plane + gi] = v0 + ch * a0;
-        R[5 * plane + gi] = v1 + ch * a1;
-        R[6 * plane + gi] = su0 + b * V0;
-        R[7 * plane + gi] = su1 + b * V1;
-        R[8 * plane + gi] = sv0 + b * a0;
-        R[9 * plane + gi] = sv1 + b * a1;
-    } else {
-        const T un0 = u0 + h * (su0 + b * V0), un1 = u1 + h * (su1 + b * V1);
-        Un[gi] = un0;
-        Un[plane + gi] = un1;
-        R[gi] = un0;
-        R[plane + gi] = un1;
-        R[2 * plane + gi] = v0 + h * (sv0 + b * a0);
-        R[3 * plane + gi] = v1 + h * (sv1 + b * a1);
+    const T h = rkhT<T>(a), hh = T(0.5) * h;
+    if (a.rk_r) rk4_layer_terms<T>(B, gi, plane, r0, r1);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const T as = w * (j == 0 ? r0 : r1);
+        T* __restrict__ q = R + j * plane + gi;
+        const T u = q[0], v = q[2 * plane];
+        if (s == 4) {
+            const T a1 = q[4 * plane], a2 = q[6 * plane], a3 = q[8 * plane];
+            const T un = u + h * (v + (h / T(6)) * (a1 + a2 + a3));
+            Un[j * plane + gi] = un;
+            q[0] = un;
+            q[2 * plane] = v + (h / T(6)) * (a1 + T(2) * (a2 + a3) + as);
+        } else {
+            const T V = s == 1 ? v : v + hh * q[(s == 2 ? 4 : 6) * plane];
+            Un[j * plane + gi] = u + (s == 3 ? h : hh) * V;
+            q[(2 + 2 * s) * plane] = as;
+        }
     }
 }
 
@@ -391,13 +390,17 @@ __device__ __forceinline__ bool robin_damping_at(const BlockDev& B, int i1, int 
     return any;
 }
 
-// the stage velocity of an RK4 stage at node gi (v for the first stage, V afterwards)
+// the stage velocity V_s of an RK4 stage at node gi: v, v + h/2 a_1, v + h/2 a_2, v + h a_3
 template <typename T>
-__device__ __forceinline__ void rk4_stage_velocity(const BlockDev& B, const StepArgs& a, size_t gi, size_t plane, T& v0, T& v1) {
+__device__ __forceinline__ void rk4_stage_velocity(const BlockDev& B, int stage, T h, size_t gi, size_t plane, T& v0, T& v1) {
     const T* R = reinterpret_cast<const T*>(B.rk);
-    const size_t o = a.stage == 1 ? 2 * plane : 4 * plane;
-    v0 = R[o + gi];
-    v1 = R[o + plane + gi];
+    v0 = R[2 * plane + gi];
+    v1 = R[3 * plane + gi];
+    if (stage == 1) return;
+    const T ch = stage == 4 ? h : T(0.5) * h;
+    const T* As = R + (size_t)2 * stage * plane;
+    v0 += ch * As[gi];
+    v1 += ch * As[plane + gi];
 }
 
 // the per-block and per-face step constants in the arithmetic type T (FP32 kernels read the FP32

@@ -18,7 +18,10 @@
 //  * 1/(rho J) and u^{n-1} of the output row are loaded from global memory two rows ahead;
 //  * MODE 0: leapfrog update from the two levels; 3: leapfrog update in increment form (the
 //    FP32 state: d^{n+1} = d^n + dt^2 w r, u^{n+1} = u^n + d^{n+1}, see leapfrog_store);
-//    1: operator output r; 2: RK4 stage (rk4_store);
+//    1: operator output r; 4 .. 7: RK4 stage 1 .. 4 (the combination of rk4_store, its 3, 7, 7 or 11 words of
+//    the output row read at the start of the row, before the CTA barrier, so that they arrive behind its arithmetic;
+//    2 x 2001 x 1001, order 6: 87, 100, 100, 108 us a stage, where the combination by stage velocities and sums, read
+//    after the row's arithmetic, took 153);
 //  * the two components of the displacement and of every flux are carried as float2 and
 //    combined with packed FP32x2 instructions (one issue slot for both).
 #pragma once
@@ -111,6 +114,8 @@ __device__ __forceinline__ bool march_tile(const MarchMaps& maps, const BV& B, c
                                            int tile, int* err, unsigned char* march_smem) {
     using MC = MarchCfg<O>;
     constexpr int Q = MC::Q, W = MBOXW, L = 2 * Q + 1;
+    constexpr int RK = MODE >= 4 ? MODE - 3 : 0;             // RK4 stage
+    constexpr int NRK = RK == 0 ? 0 : (RK == 1 ? 1 : (RK == 4 ? 5 : 3));   // its float2 operands: v | u v a_{s-1} | u v a_1 a_2 a_3
     float* ring = reinterpret_cast<float*>(march_smem);
     float* g1s = ring + MNCH * MC::CHUNK;
     float2* hqs = reinterpret_cast<float2*>(g1s + MC::G1);
@@ -303,6 +308,16 @@ __device__ __forceinline__ bool march_tile(const MarchMaps& maps, const BV& B, c
     }
 #pragma unroll 4
     for (int r = ys; r < ye; ++r) {
+        float2 rk[NRK > 0 ? NRK : 1];
+        if constexpr (RK > 0) {
+            const float* __restrict__ K = reinterpret_cast<const float*>(B.rk) + (size_t)r * P + gx;
+            constexpr int first[4] = {2, 0, 0, 0};
+#pragma unroll
+            for (int k = 0; k < NRK; ++k) {
+                const size_t pl = RK == 3 && k == 2 ? 6 : first[RK - 1] + 2 * k;
+                rk[k] = col_ok ? make_float2(K[pl * plane], K[(pl + 1) * plane]) : make_float2(0.f, 0.f);
+            }
+        }
         look(r);
         const float2 ry = yflux();
         // --- g1 at (x, r) into the shared row
@@ -414,8 +429,30 @@ __device__ __forceinline__ bool march_tile(const MarchMaps& maps, const BV& B, c
             Un[gi + plane] = nu.y;
             DU[gi] = d.x;
             DU[gi + plane] = d.y;
-        } else if constexpr (MODE == 2) {
-            rk4_store<float>(B, a, gi, plane, w_c, r0, r1);
+        } else if constexpr (RK > 0) {
+            if (a.rk_r) rk4_layer_terms<float>(B, gi, plane, r0, r1);
+            float* __restrict__ Un = reinterpret_cast<float*>(B.u[1 - a.cur]);
+            float* __restrict__ K = reinterpret_cast<float*>(B.rk);
+            const float h = a.rkhf, hh = 0.5f * h;
+            const float2 as = fmul2(bc2(w_c), make_float2(r0, r1));
+            float2 un;
+            if constexpr (RK == 1) un = ffma2(bc2(hh), rk[0], uc);
+            else if constexpr (RK < 4) un = ffma2(bc2(RK == 3 ? h : hh), ffma2(bc2(hh), rk[2], rk[1]), rk[0]);
+            else {
+                const float2 s23 = fadd2(rk[3], rk[4]);
+                un = ffma2(bc2(h), ffma2(bc2(h / 6.f), fadd2(rk[2], s23), rk[1]), rk[0]);
+                const float2 vn = ffma2(bc2(h / 6.f), fadd2(ffma2(bc2(2.f), s23, rk[2]), as), rk[1]);
+                K[gi] = un.x;
+                K[plane + gi] = un.y;
+                K[2 * plane + gi] = vn.x;
+                K[3 * plane + gi] = vn.y;
+            }
+            Un[gi] = un.x;
+            Un[gi + plane] = un.y;
+            if constexpr (RK < 4) {
+                K[(2 + 2 * RK) * plane + gi] = as.x;
+                K[(3 + 2 * RK) * plane + gi] = as.y;
+            }
         } else {
             float* __restrict__ R = reinterpret_cast<float*>(B.r);
             R[gi] = r0;
@@ -430,13 +467,6 @@ __device__ __forceinline__ bool march_tile(const MarchMaps& maps, const BV& B, c
     if (tx == 0)
         for (int k = 0; k < MNCH; ++k) mbar_inval(&bars[k]);
     return true;
-}
-
-template <int O, int MODE>
-__global__ void __launch_bounds__(MTHREADS, 4)
-k_interior_march(const __grid_constant__ MarchMaps maps, BlockDev B, StepArgs a, int rows_per_cta, int* err) {
-    extern __shared__ __align__(128) unsigned char march_smem[];
-    (void)march_tile<O, MODE>(maps, B, a, rows_per_cta, blockIdx.x, err, march_smem);
 }
 
 // The interior tiles of several blocks in one launch: CTA k takes tile k - start[b] of the block b

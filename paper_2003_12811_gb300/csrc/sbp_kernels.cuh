@@ -1101,7 +1101,7 @@ __device__ __forceinline__ bool strip_tile_body(const BlockDev* __restrict__ blo
         } else if (MODE == 2) {
             if (damped) {
                 T v0, v1;
-                rk4_stage_velocity<T>(B, a, gi, plane, v0, v1);
+                rk4_stage_velocity<T>(B, a.stage, rkhT<T>(a), gi, plane, v0, v1);
                 r0 -= dd00 * v0 + dd01 * v1;
                 r1 -= dd01 * v0 + dd11 * v1;
             }
@@ -1151,11 +1151,12 @@ __global__ void k_sources(const BlockDev* __restrict__ blocks, const SrcNode* __
             atomicAdd(DU + plane + nd.gi, T(fac * nd.wt1));
         }
     } else if (MODE == 2) {
-        // RK4 stage: J f at the node into the (otherwise zero) operator-output planes, which the
-        // stage's kernels add to the operator sum before forming the acceleration (rk4_store)
-        T* R = reinterpret_cast<T*>(B.r);
-        atomicAdd(R + nd.gi, T(Wt * nd.wt0));
-        atomicAdd(R + plane + nd.gi, T(Wt * nd.wt1));
+        // RK4, after the stage's kernels: the source's share of a_s, or of v_new = v + ... + h/6 a_4
+        // (no stage input before the next stage depends on a_s: rk4_store)
+        T* R = reinterpret_cast<T*>(B.rk) + (size_t)(a.stage < 4 ? 2 + 2 * a.stage : 2) * plane;
+        const double fac = (double)reinterpret_cast<const T*>(B.w)[nd.gi] * Wt * (a.stage < 4 ? 1.0 : a.rkh / 6.0);
+        atomicAdd(R + nd.gi, T(fac * nd.wt0));
+        atomicAdd(R + plane + nd.gi, T(fac * nd.wt1));
     } else {
         T* R = reinterpret_cast<T*>(B.r);
         atomicAdd(R + nd.gi, T(Wt * nd.wt0));
@@ -1290,15 +1291,17 @@ __global__ void k_layer_post(BlockDev B, const int2* __restrict__ nodes, int n, 
 // RK4 stage, before the stage kernels: -H^-1 K V_s into the point-source planes of the operator
 // output (rk4_store takes them into the operator sum)
 template <typename T, int O>
-__global__ void k_layer_rk(BlockDev B, const int2* __restrict__ nodes, int n, int stage) {
+__global__ void k_layer_rk(BlockDev B, const int2* __restrict__ nodes, int n, int stage, double h) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     const int2 nd = nodes[k];
     const size_t plane = (size_t)B.n2 * B.pitch, gi = (size_t)nd.y * B.pitch + nd.x;
-    const T* __restrict__ V = reinterpret_cast<const T*>(B.rk) + (stage == 1 ? 2 : 4) * plane;
     T k0, k1;
-    layer_kv<T, O>(B, nd.x, nd.y, [&](int j1, int j2, int c) { return V[(size_t)c * plane + (size_t)j2 * B.pitch + j1]; },
-                   k0, k1);
+    layer_kv<T, O>(B, nd.x, nd.y, [&](int j1, int j2, int c) {
+        T v0, v1;
+        rk4_stage_velocity<T>(B, stage, T(h), (size_t)j2 * B.pitch + j1, plane, v0, v1);
+        return c == 0 ? v0 : v1;
+    }, k0, k1);
     T* __restrict__ R = reinterpret_cast<T*>(B.r);
     R[gi] -= k0;
     R[plane + gi] -= k1;

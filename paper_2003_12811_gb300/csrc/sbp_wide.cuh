@@ -92,7 +92,7 @@ __global__ void k_wide_div(BlockDev B, StepArgs a, const T* __restrict__ G) {
     } else if (MODE == 2) {
         if (damped) {
             T v0, v1;
-            rk4_stage_velocity<T>(B, a, gi, plane, v0, v1);
+            rk4_stage_velocity<T>(B, a.stage, rkhT<T>(a), gi, plane, v0, v1);
             r0 -= dd00 * v0 + dd01 * v1;
             r1 -= dd01 * v0 + dd11 * v1;
         }
