@@ -467,24 +467,72 @@ void launch_traces(sbp_handle* h, const StepArgs& a, cudaStream_t tst, bool adj)
     flush();
 }
 
+// rows per CTA of a marching kernel on a block with ncx tiles across: one wave of about 4 CTAs per SM, at least
+// 16 rows (a tile streams 2q rows or more beyond its own), or the height that was tuned
+int march_rows(const sbp_handle* h, int ncx, int n2i) {
+    if (h->rows_per_cta > 0) return std::min(h->rows_per_cta, n2i);
+    const int ncy = std::max(1, (4 * h->num_sms + ncx / 2) / ncx);
+    return std::max((n2i + ncy - 1) / ncy, std::min(16, n2i));
+}
+
 // the wide-stencil operator (sbp_wide.cuh): traces, the SAT terms of every face node, the flux and
-// divergence passes of every block, then the point sources (every source node: the wide path has
+// divergence passes of every block (in FP32 of its frame near the faces, beside one marching kernel over
+// the interior, which they share nothing with), then the point sources (every source node: the wide path has
 // no strip kernel)
 template <typename T, int O>
 int launch_wide(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st) {
-    if (h->ntrefs > 0) launch_traces<T, O>(h, a, st, false);
+    constexpr bool march = std::is_same<T, float>::value;
+    const int S = std::max(order_nclos(h->order), order_ncol(h->order));
+    // the frame's chain of small kernels on the high-priority stream, queued before the interior
+    const bool par = march && h->hi && !h->prof;
+    cudaStream_t fst = par ? h->hi : st;
+    if (par) {
+        cudaEventRecord(h->ev_fork, st);
+        cudaStreamWaitEvent(h->hi, h->ev_fork, 0);
+    }
+    if (h->ntrefs > 0) launch_traces<T, O>(h, a, fst, false);
     if (h->nface_nodes > 0) {
-        ProfScope ps(h, 1, st, 1);
-        k_face_sat<T, O><<<grid_for(h->nface_nodes), 256, 0, st>>>(h->d_blocks, h->d_refs, h->nrefs, h->nface_nodes, a, h->beta);
+        ProfScope ps(h, 1, fst, 1);
+        k_face_sat<T, O><<<grid_for(h->nface_nodes, 64), 64, 0, fst>>>(h->d_blocks, h->d_refs, h->nrefs, h->nface_nodes, a, h->beta);
+    }
+    if constexpr (march) {
+        MarchMulti mm{};
+        int tiles = 0;
+        auto flush = [&]() {
+            if (mm.nb == 0) return;
+            mm.start[mm.nb] = tiles;
+            ProfScope ps(h, 0, st, 1);
+            constexpr size_t msm = MarchCfg<O>::BYTES;
+            if (mode == 0) k_wide_march<O, 3><<<tiles, MTHREADS, msm, st>>>(mm, a, h->d_err);
+            else if (mode == 2) k_wide_march<O, 2><<<tiles, MTHREADS, msm, st>>>(mm, a, h->d_err);
+            else k_wide_march<O, 1><<<tiles, MTHREADS, msm, st>>>(mm, a, h->d_err);
+            mm = MarchMulti{};
+            tiles = 0;
+        };
+        for (auto& hb : h->blocks) {
+            const int ncx = wide_ncx(hb.n1, S), n2i = hb.n2 - 2 * S, rows = march_rows(h, ncx, n2i), k = mm.nb++;
+            mm.maps[k] = hb.mmaps;
+            mm.b[k] = make_view(h, hb);
+            mm.start[k] = tiles;
+            mm.rows[k] = rows;
+            tiles += ncx * ((n2i + rows - 1) / rows);
+            if (mm.nb == MARCH_MAX_BLOCKS) flush();
+        }
+        flush();
     }
     for (auto& hb : h->blocks) {
         const BlockDev b = make_view(h, hb);
-        const long long n = (long long)hb.n1 * hb.n2;
-        ProfScope ps(h, 0, st, 2);
-        k_wide_flux<T, O><<<grid_for(n), 256, 0, st>>>(b, a, (T*)hb.gw);
-        if (mode == 0) k_wide_div<T, O, 0><<<grid_for(n), 256, 0, st>>>(b, a, (const T*)hb.gw);
-        else if (mode == 2) k_wide_div<T, O, 2><<<grid_for(n), 256, 0, st>>>(b, a, (const T*)hb.gw);
-        else k_wide_div<T, O, 1><<<grid_for(n), 256, 0, st>>>(b, a, (const T*)hb.gw);
+        const int ff = march ? S + Ord<O>::Q : 0, fd = march ? S : 0;
+        const long long nf = frame_nodes(hb.n1, hb.n2, ff), nd = frame_nodes(hb.n1, hb.n2, fd);
+        ProfScope ps(h, march ? 1 : 0, fst, 2);
+        k_wide_flux<T, O><<<grid_for(nf), 256, 0, fst>>>(b, a, (T*)hb.gw, ff);
+        if (mode == 0) k_wide_div<T, O, 0><<<grid_for(nd), 256, 0, fst>>>(b, a, (const T*)hb.gw, fd);
+        else if (mode == 2) k_wide_div<T, O, 2><<<grid_for(nd), 256, 0, fst>>>(b, a, (const T*)hb.gw, fd);
+        else k_wide_div<T, O, 1><<<grid_for(nd), 256, 0, fst>>>(b, a, (const T*)hb.gw, fd);
+    }
+    if (par) {
+        cudaEventRecord(h->ev_join_hi, h->hi);
+        cudaStreamWaitEvent(st, h->ev_join_hi, 0);
     }
     if (!h->src_nodes.empty()) {
         ProfScope ps(h, 3, st, 1);
@@ -591,11 +639,7 @@ int launch_operator(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st,
             const int S2 = std::max(order_nclos(h->order), order_ncol(h->order));
             const int ncx = march_ncx(hb.n1, S2);
             const int n2i = hb.n2 - 2 * S2;
-            int ncy = std::max(1, (4 * h->num_sms + ncx / 2) / ncx);
-            int rows = (n2i + ncy - 1) / ncy;
-            if (rows < 16) rows = std::min(16, n2i);
-            if (h->rows_per_cta > 0) rows = std::min(h->rows_per_cta, n2i);
-            ncy = (n2i + rows - 1) / rows;
+            const int rows = march_rows(h, ncx, n2i), ncy = (n2i + rows - 1) / rows;
             const int k = mmul.nb++;
             mmul.maps[k] = adj ? hb.pmaps : hb.mmaps;
             mmul.b[k] = adj ? make_view_adj(h, hb) : make_view(h, hb);
@@ -738,6 +782,9 @@ template <typename T, int O> void set_smem_attr() {
     cudaFuncSetAttribute(k_interior<T, O, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaFuncSetAttribute(k_interior<T, O, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (std::is_same<T, float>::value) {
+        cudaFuncSetAttribute(k_wide_march<O, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
+        cudaFuncSetAttribute(k_wide_march<O, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
+        cudaFuncSetAttribute(k_wide_march<O, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
         cudaFuncSetAttribute(k_interior_march_multi<O, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
         cudaFuncSetAttribute(k_interior_march_multi<O, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
         cudaFuncSetAttribute(k_interior_march_multi<O, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
