@@ -8,7 +8,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsbp.so")
 SOURCES = ["sbp_api.cu", "sbp3d_api.cu"]
 DEPS = ["sbp_api.cu", "sbp_kernels.cuh", "sbp_adjoint.cuh", "sbp_device.cuh", "sbp_interior_march.cuh",
-        "sbp_batch.cuh", "sbp_wide.cuh", "sbp_tables.inc", "sbp3d_api.cu", "sbp3d.cuh"]
+        "sbp_batch.cuh", "sbp_wide.cuh", "sbp_step.cuh", "sbp_tables.inc", "sbp3d_api.cu", "sbp3d.cuh"]
 HEADERS = ["sbp.h", "sbp3.h"]
 NVCC_FLAGS = ["-std=c++17", "-O3", "-gencode", "arch=compute_103a,code=sm_103a", "-lineinfo",
               "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",

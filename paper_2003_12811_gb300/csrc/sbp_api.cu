@@ -19,6 +19,7 @@
 #include "sbp_adjoint.cuh"
 #include "sbp_batch.cuh"
 #include "sbp_wide.cuh"
+#include "sbp_step.cuh"
 
 namespace sbphost {
 #define SBP_TABLE static const
@@ -61,7 +62,8 @@ struct HostBlock {
     MarchMaps mmaps;          // FP32 column-marching interior kernel tensor maps
     void* psi[2] = {nullptr, nullptr};   // adjoint fields (sbp_misfit_gradient), allocated on first use
     MarchMaps pmaps;          // marching-kernel maps over the adjoint fields
-    CUtensorMap* d_smaps = nullptr;   // strip-tile band-box maps on the device: [0..2] state u0, u1, c; [3..5] adjoint
+    CUtensorMap* d_smaps = nullptr;   // strip-tile band-box maps on the device: [0..2] state u0, u1, c; [3..5] adjoint;
+                                      // [6..11] the same for short tiles
     void* rk = nullptr;       // RK4 state (u, v, a_1, a_2, a_3; sbp_set_state_rk4), allocated on first use
     void* gw = nullptr;       // wide stencil: the fluxes G_1j, G_2j (4 planes, type T)
     void* sg = nullptr;       // layer dissipation coefficient s (1 plane, type T)
@@ -162,6 +164,14 @@ struct sbp_handle {
     int strip_len = 32;                 // nodes of a strip tile along the face (pick_strip_len)
     std::vector<int4> tiles_host;
     std::vector<std::vector<int>> tile_pos;   // [block][tile of the block] -> position in the launch order
+    // FP32 grids whose strips make few tiles: a second set, SHORT_TILE nodes long, for the one-launch step (the
+    // batch kernel and the others keep to 32)
+    struct StripSet {
+        int4* d_tiles = nullptr;
+        SrcNode* d_src = nullptr;
+        std::vector<int4> tiles;
+        std::vector<std::vector<int>> pos;
+    } shorts;
     cudaStream_t aux = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     // adjoint: block views whose state buffers are the adjoint fields; receivers
@@ -393,6 +403,9 @@ template <int O> void strip_box(int len, int& bw, int& bh) {
     bh = StripTile<O>::BHB;
 }
 
+// length of the short strip tiles of FP32 grids (sbp_handle::shorts)
+constexpr int SHORT_TILE = 8;
+
 // Length of the strip tiles of an FP64 grid: the one whose busiest SM executes the fewest FP64
 // instructions, a tile of length L taking about 140 per output node, 26 and 16 per flux on its rows and
 // columns with their halos, and 150 per face node.  (4 order-6 blocks of 401^2: 200 tiles of 32, 76 us;
@@ -417,12 +430,44 @@ int pick_strip_len(const sbp_handle* h) {
     return best;
 }
 
+// strip tiles of length L (the tile numbering of k_strip_tile: 2 bands of ceil(n1/L) tiles along x1, then 2
+// side bands of ceil((n2 - 2S)/L) tiles), ordered by a cost estimate: side tiles stage narrow rows,
+// interface tiles read the neighbour, corner tiles carry two faces
+void list_strip_tiles(const sbp_handle* h, int L, std::vector<int4>& tiles, std::vector<std::vector<int>>& pos) {
+    const int S = std::max(order_nclos(h->order), order_ncol(h->order));
+    std::vector<std::pair<int, int2>> tl;
+    pos.assign(h->nblocks, {});
+    for (int b = 0; b < h->nblocks; ++b) {
+        const HostBlock& hb = h->blocks[b];
+        const int nbx = (hb.n1 + L - 1) / L, nby = (hb.n2 - 2 * S + L - 1) / L;
+        pos[b].assign(2 * nbx + 2 * nby, -1);
+        for (int t = 0; t < 2 * nbx + 2 * nby; ++t) {
+            int cost;
+            if (t < 2 * nbx) {
+                const int f = 2 + t / nbx, k = t % nbx;
+                cost = (hb.f[f].kind == SBP_BC_INTERFACE ? 3 : 1) + ((k == 0 || k == nbx - 1) ? 2 : 0);
+            } else {
+                const int f = (t - 2 * nbx) / nby;
+                cost = 2 + (hb.f[f].kind == SBP_BC_INTERFACE ? 3 : 0);
+            }
+            tl.push_back({cost, make_int2(b, t)});
+        }
+    }
+    std::stable_sort(tl.begin(), tl.end(),
+                     [](const std::pair<int, int2>& x, const std::pair<int, int2>& y) { return x.first > y.first; });
+    tiles.clear();
+    for (auto& e : tl) {
+        pos[e.second.x][e.second.y] = (int)tiles.size();
+        tiles.push_back(make_int4(e.second.x, e.second.y, 0, 0));
+    }
+}
+
 // the strip-tile band-box maps of two displacement buffers and the coefficients, written to dst[0..2]
-bool make_strip_maps(const sbp_handle* h, const HostBlock& hb, void* u0, void* u1, CUtensorMap* dst) {
+bool make_strip_maps(const sbp_handle* h, const HostBlock& hb, void* u0, void* u1, CUtensorMap* dst, int len) {
     int bw, bh;
-    if (h->order == 2) strip_box<2>(h->strip_len, bw, bh);
-    else if (h->order == 4) strip_box<4>(h->strip_len, bw, bh);
-    else strip_box<6>(h->strip_len, bw, bh);
+    if (h->order == 2) strip_box<2>(len, bw, bh);
+    else if (h->order == 4) strip_box<4>(len, bw, bh);
+    else strip_box<6>(len, bw, bh);
     const int es = (int)h->esize;
     return make_map(&dst[0], u0, hb.pitch, hb.n2, 2, bh, bw, es) &&
            make_map(&dst[1], u1, hb.pitch, hb.n2, 2, bh, bw, es) &&
@@ -549,56 +594,174 @@ int launch_wide(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st) {
 // them): 32 x 16 nodes repeat the fewest fluxes on their halos and win once there are several tiles per
 // SM, 16 x 4 nodes leave no SM idle on a 101^2 grid (138 tiles against 18).   Order 4, 101^2: 13 us
 // against 38 us for 32 x 16 tiles with their own weights.
-template <int O>
-void launch_interior_f64(sbp_handle* h, const BlockDev* tab, const StepArgs& a, int mode, cudaStream_t st) {
-    constexpr int Q = Ord<O>::Q, NODE = 8 * Q * 4 + 12, FLUX = 6 * Q + 4;
-    const int S = std::max(order_nclos(h->order), order_ncol(h->order));
-    constexpr int shapes[4][2] = {{32, 16}, {32, 8}, {32, 4}, {16, 4}};
+constexpr int kEdgeShapes[4][2] = {{32, 16}, {32, 8}, {32, 4}, {16, 4}};
+int pick_edge_shape(const sbp_handle* h) {
+    const int Q = order_q(h->order), S = std::max(order_nclos(h->order), order_ncol(h->order));
+    const int node = 8 * Q * 4 + 12, flux = 6 * Q + 4;
     int best = 0;
     long long least = -1;
     for (int k = 0; k < 4; ++k) {
-        const int tx = shapes[k][0], ty = shapes[k][1];
+        const int tx = kEdgeShapes[k][0], ty = kEdgeShapes[k][1];
         long long tiles = 0;
         for (auto& hb : h->blocks)
             tiles += (long long)((hb.n1 - 2 * S + tx - 1) / tx) * ((hb.n2 - 2 * S + ty - 1) / ty);
         const long long cost = (tiles + h->num_sms - 1) / h->num_sms *
-                               (tx * ty * NODE + FLUX * ((tx + 2 * Q) * ty + tx * (ty + 2 * Q)));
+                               (tx * ty * node + flux * ((tx + 2 * Q) * ty + tx * (ty + 2 * Q)));
         if (least < 0 || cost < least) {
             least = cost;
             best = k;
         }
     }
-    const int tx = shapes[best][0], ty = shapes[best][1];
+    return best;
+}
+// the interior tiles of blocks [first, first + IE_MAX_BLOCKS) in shape k; returns their number
+int edge_tiles(const sbp_handle* h, int first, int k, InteriorTiles& tl) {
+    const int S = std::max(order_nclos(h->order), order_ncol(h->order)), tx = kEdgeShapes[k][0], ty = kEdgeShapes[k][1];
+    tl = InteriorTiles{};
+    tl.first = first;
+    int tiles = 0;
+    for (int b = first; b < std::min(h->nblocks, first + IE_MAX_BLOCKS); ++b) {
+        const HostBlock& hb = h->blocks[b];
+        tl.ncx[tl.nb] = (hb.n1 - 2 * S + tx - 1) / tx;
+        tl.start[tl.nb++] = tiles;
+        tiles += tl.ncx[tl.nb - 1] * ((hb.n2 - 2 * S + ty - 1) / ty);
+    }
+    tl.start[tl.nb] = tiles;
+    return tiles;
+}
+template <int O>
+void launch_interior_f64(sbp_handle* h, const BlockDev* tab, const StepArgs& a, int mode, cudaStream_t st) {
+    const int best = pick_edge_shape(h);
     for (int first = 0; first < h->nblocks; first += IE_MAX_BLOCKS) {
-        InteriorTiles tl{};
-        tl.first = first;
-        int tiles = 0;
-        for (int b = first; b < std::min(h->nblocks, first + IE_MAX_BLOCKS); ++b) {
-            const HostBlock& hb = h->blocks[b];
-            tl.ncx[tl.nb] = (hb.n1 - 2 * S + tx - 1) / tx;
-            tl.start[tl.nb++] = tiles;
-            tiles += tl.ncx[tl.nb - 1] * ((hb.n2 - 2 * S + ty - 1) / ty);
-        }
-        tl.start[tl.nb] = tiles;
+        InteriorTiles tl;
+        const int tiles = edge_tiles(h, first, best, tl);
         ProfScope ps(h, 0, st, 1);
-        auto run = [&](auto xc, auto yc) {
-            constexpr int TX = decltype(xc)::value, TY = decltype(yc)::value, NT = TX * TY < 256 ? TX * TY : 256;
+        auto run = [&](auto kc) {
+            constexpr int TX = kEdgeShapes[decltype(kc)::value][0], TY = kEdgeShapes[decltype(kc)::value][1], NT = TX * TY < 256 ? TX * TY : 256;
             if (mode == 0) k_interior_edges<double, O, 0, TX, TY><<<tiles, NT, 0, st>>>(tab, tl, a);
             else if (mode == 2) k_interior_edges<double, O, 2, TX, TY><<<tiles, NT, 0, st>>>(tab, tl, a);
             else k_interior_edges<double, O, 1, TX, TY><<<tiles, NT, 0, st>>>(tab, tl, a);
         };
-        using std::integral_constant;
-        if (best == 0) run(integral_constant<int, 32>(), integral_constant<int, 16>());
-        else if (best == 1) run(integral_constant<int, 32>(), integral_constant<int, 8>());
-        else if (best == 2) run(integral_constant<int, 32>(), integral_constant<int, 4>());
-        else run(integral_constant<int, 16>(), integral_constant<int, 4>());
+        if (best == 0) run(std::integral_constant<int, 0>());
+        else if (best == 1) run(std::integral_constant<int, 1>());
+        else if (best == 2) run(std::integral_constant<int, 2>());
+        else run(std::integral_constant<int, 3>());
     }
+}
+
+// Rows of the interior items (128 columns of a marching kernel, bands of equal height per grid) that share `slots`
+// CTAs with `strips` strip tiles.  An item costs its rows and about ITEM_ROWS more (the rows it marches before
+// its first output, its start), a strip tile about STRIP_ROWS; the height minimises the larger of the mean load
+// and the rounds of the longest item.  grids: (tiles across, interior rows).
+int item_rows(int slots, const std::vector<int2>& grids, long long strips) {
+    constexpr double ITEM_ROWS = 14, STRIP_ROWS = 10;
+    double least = 1e300;
+    int best = 64;
+    for (int rows = 8; rows <= 256; rows += rows < 32 ? 1 : 4) {
+        long long items = 0;
+        double work = strips * STRIP_ROWS, longest = 0;
+        for (const int2& s : grids) {
+            const int bands = (s.y + rows - 1) / rows, high = (s.y + bands - 1) / bands;
+            items += (long long)s.x * bands;
+            work += (double)s.x * (s.y + bands * ITEM_ROWS);
+            longest = std::max(longest, high + ITEM_ROWS);
+        }
+        // (strip tiles shorter than an item leave their slots to items of the next round)
+        const double cost = std::max(work / slots, (double)((items + strips + slots - 1) / slots) * longest);
+        if (cost < least) {
+            least = cost;
+            best = rows;
+        }
+    }
+    return best;
+}
+
+// Whether a step runs as one launch (sbp_step.cuh): the blocks fit the launch's tables and the kernels are not being
+// timed one by one.  FP32: leapfrog steps of the state or the adjoint fields, up to as many strip tiles as SMs
+// (1200^2; larger grids fill the chip with either kernel, see the figures there) and without interfaces, whose
+// traces now form beside the interior (2 x 402 x 201: 38 us a step, 41 with the traces first).  FP64: leapfrog steps and RK4 stages
+// with strip tiles of 8 nodes, or 16 without interfaces (4 blocks of 401^2: 264 us in one launch, 258 in two), not on
+// the largest grids, where FP64 arithmetic alone counts.  A user's choice of streams (sbp_set_tuning) keeps the strips
+// in a launch of their own.
+bool one_launch(const sbp_handle* h, int mode) {
+    if (h->prof || h->overlap || h->nblocks > MARCH_MAX_BLOCKS || h->stencil != SBP_STENCIL_NARROW) return false;
+    if (h->precision == SBP_FP32) return mode == 0 && h->ntrefs == 0 && (h->shorts.d_tiles || h->ntiles <= h->num_sms);
+    return mode != 1 && h->blocks[0].e && (h->strip_len == 8 || (h->strip_len == 16 && h->ntrefs == 0));
+}
+// the interior shape that goes with the strip tiles of an FP64 step in one launch
+int step_edge_shape(const sbp_handle* h) { return h->strip_len == 16 ? 0 : std::max(1, pick_edge_shape(h)); }
+
+template <typename T, int O>
+int launch_step(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st, bool adj) {
+    if (h->ntrefs > 0) launch_traces<T, O>(h, a, st, adj);
+    StepStrips ss{};
+    const bool sh = h->shorts.d_tiles != nullptr;
+    ss.blocks = adj ? h->d_blocks_adj : h->d_blocks;
+    ss.tiles = sh ? h->shorts.d_tiles : h->d_tiles;
+    ss.n = sh ? (int)h->shorts.tiles.size() : h->ntiles;
+    ss.ssrc = adj ? nullptr : (sh ? h->shorts.d_src : h->d_src_strip);
+    ss.spar = h->d_src_params;
+    ss.beta = h->beta;
+    const bool inside = !adj && h->n_src_int > 0 && h->n_src_int <= STEP_MAX_SOURCES;
+    ss.isrc = inside ? h->d_src_int : nullptr;
+    ss.nisrc = inside ? h->n_src_int : 0;
+    {
+        ProfScope ps(h, 0, st, 1);
+        if constexpr (std::is_same<T, float>::value) {
+            MarchMulti mm{};
+            int tiles = 0;
+            const int S = std::max(order_nclos(h->order), order_ncol(h->order));
+            std::vector<int2> grids;
+            for (auto& hb : h->blocks) grids.push_back(make_int2(march_ncx(hb.n1, S), hb.n2 - 2 * S));
+            const int even = h->rows_per_cta > 0 ? h->rows_per_cta : item_rows(4 * h->num_sms, grids, ss.n);
+            for (auto& hb : h->blocks) {
+                const int ncx = march_ncx(hb.n1, S), n2i = hb.n2 - 2 * S, bands = (n2i + even - 1) / even;
+                const int rows = h->rows_per_cta > 0 ? std::min(n2i, even) : (n2i + bands - 1) / bands;
+                const int k = mm.nb++;
+                mm.maps[k] = adj ? hb.pmaps : hb.mmaps;
+                mm.b[k] = adj ? make_view_adj(h, hb) : make_view(h, hb);
+                mm.start[k] = tiles;
+                mm.rows[k] = rows;
+                tiles += ncx * ((n2i + rows - 1) / rows);
+            }
+            mm.start[mm.nb] = tiles;
+            constexpr size_t sm = step_smem_f32<O>();
+            const int grid = ss.n + tiles;
+            if (adj && sh) k_step_f32<O, 0, SHORT_TILE><<<grid, MTHREADS, sm, st>>>(mm, ss, a, h->d_err);
+            else if (adj) k_step_f32<O, 0, 32><<<grid, MTHREADS, sm, st>>>(mm, ss, a, h->d_err);
+            else if (sh) k_step_f32<O, 3, SHORT_TILE><<<grid, MTHREADS, sm, st>>>(mm, ss, a, h->d_err);
+            else k_step_f32<O, 3, 32><<<grid, MTHREADS, sm, st>>>(mm, ss, a, h->d_err);
+        } else {
+            const int best = step_edge_shape(h);
+            InteriorTiles tl;
+            const int grid = ss.n + edge_tiles(h, 0, best, tl);
+            auto run = [&](auto kc) {
+                constexpr int TX = kEdgeShapes[decltype(kc)::value][0], TY = kEdgeShapes[decltype(kc)::value][1];
+                constexpr size_t sm = step_smem_f64<O, TX, TY>();
+                constexpr int NT = step_threads_f64<TX, TY>();
+                if (mode == 0) k_step_f64<O, 0, TX, TY><<<grid, NT, sm, st>>>(tl, ss, a, h->d_err);
+                else k_step_f64<O, 2, TX, TY><<<grid, NT, sm, st>>>(tl, ss, a, h->d_err);
+            };
+            if (best == 0) run(std::integral_constant<int, 0>());
+            else if (best == 1) run(std::integral_constant<int, 1>());
+            else if (best == 2) run(std::integral_constant<int, 2>());
+            else run(std::integral_constant<int, 3>());
+        }
+    }
+    if (!adj && h->n_src_int > 0 && !inside) {
+        ProfScope ps(h, 3, st, 1);
+        const int ns = h->n_src_int;
+        if (mode == 2) k_sources<T, 2><<<grid_for(ns), 256, 0, st>>>(h->d_blocks, h->d_src_int, ns, h->d_src_params, a);
+        else k_sources<T, 0><<<grid_for(ns), 256, 0, st>>>(h->d_blocks, h->d_src_int, ns, h->d_src_params, a);
+    }
+    return check_cuda(h, "step launch");
 }
 
 // one operator application (mode 1) or leapfrog step (mode 0) on the state fields, or, with adj,
 // on the adjoint fields (the same kernels; the sources are skipped)
 template <typename T, int O>
 int launch_operator(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st, bool adj) {
+    if (one_launch(h, mode)) return launch_step<T, O>(h, a, mode, st, adj);
     const BlockDev* tab = adj ? h->d_blocks_adj : h->d_blocks;
     constexpr size_t smem = interior_smem_elems<T, O>() * sizeof(T);
     // interior kernels on st; strip kernels on the auxiliary stream when overlapping (profiling
@@ -774,6 +937,24 @@ template <typename T, int O> void set_smem_attr() {
         cudaFuncSetAttribute(k_strip_tile<T, O, 2, TL>, cudaFuncAttributeMaxDynamicSharedMemorySize, ssm);
     };
     strip(std::integral_constant<int, 32>());
+    if constexpr (std::is_same<T, float>::value) {
+        constexpr int sm = (int)step_smem_f32<O>();
+        cudaFuncSetAttribute(k_step_f32<O, 0, SHORT_TILE>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        cudaFuncSetAttribute(k_step_f32<O, 3, SHORT_TILE>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        cudaFuncSetAttribute(k_step_f32<O, 0, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        cudaFuncSetAttribute(k_step_f32<O, 3, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    } else {
+        auto step = [](auto kc) {
+            constexpr int TX = kEdgeShapes[decltype(kc)::value][0], TY = kEdgeShapes[decltype(kc)::value][1];
+            constexpr int sm = (int)step_smem_f64<O, TX, TY>();
+            cudaFuncSetAttribute(k_step_f64<O, 0, TX, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+            cudaFuncSetAttribute(k_step_f64<O, 2, TX, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+        };
+        step(std::integral_constant<int, 0>());
+        step(std::integral_constant<int, 1>());
+        step(std::integral_constant<int, 2>());
+        step(std::integral_constant<int, 3>());
+    }
     if constexpr (std::is_same<T, double>::value) {
         strip(std::integral_constant<int, 16>());
         strip(std::integral_constant<int, 8>());
@@ -814,9 +995,9 @@ void fill_basis(const sbp_handle* h, double t, StepArgs& a) {
 
 // strip tile of node (i1, i2) of a block in the numbering of k_strip_tile (bands of width S along
 // x2 = 0 and x2 = 1, then the side bands between them), or -1 for a node off the strips
-int strip_tile_of(const sbp_handle* h, const HostBlock& hb, int i1, int i2) {
+int strip_tile_of(const sbp_handle* h, const HostBlock& hb, int i1, int i2, int L) {
     const int S = std::max(order_nclos(h->order), order_ncol(h->order));
-    const int L = h->strip_len, nbx = (hb.n1 + L - 1) / L, nby = (hb.n2 - 2 * S + L - 1) / L;
+    const int nbx = (hb.n1 + L - 1) / L, nby = (hb.n2 - 2 * S + L - 1) / L;
     if (i2 < S) return i1 / L;
     if (i2 >= hb.n2 - S) return nbx + i1 / L;
     if (i1 < S) return 2 * nbx + (i2 - S) / L;
@@ -839,31 +1020,43 @@ int upload_sources(sbp_handle* h) {
         cudaMemcpy(h->d_src_params, h->src_params.data(), sizeof(SrcParam) * h->src_params.size(), cudaMemcpyHostToDevice) != cudaSuccess)
         return h->fail(SBP_E_CUDA, "source table upload failed");
     // split: nodes on the boundary strips go with their strip tile, the rest to k_sources
-    std::vector<std::pair<int, SrcNode>> strip;
     std::vector<SrcNode> inner;
-    for (const SrcNode& nd : h->src_nodes) {
-        const HostBlock& hb = h->blocks[nd.block];
-        const int i2 = (int)(nd.gi / hb.pitch), i1 = (int)(nd.gi - (long long)i2 * hb.pitch);
-        const int t = strip_tile_of(h, hb, i1, i2);
-        if (t < 0) inner.push_back(nd);
-        else strip.push_back({h->tile_pos[nd.block][t], nd});
-    }
-    std::stable_sort(strip.begin(), strip.end(),
-                     [](const std::pair<int, SrcNode>& x, const std::pair<int, SrcNode>& y) { return x.first < y.first; });
-    for (int4& tl : h->tiles_host) tl.z = tl.w = 0;
-    std::vector<SrcNode> sv;
-    for (size_t k = 0; k < strip.size(); ++k) {
-        int4& tl = h->tiles_host[strip[k].first];
-        if (tl.z == tl.w) tl.z = tl.w = (int)k;
-        tl.w = (int)k + 1;
-        sv.push_back(strip[k].second);
-    }
-    if (!sv.empty()) {
-        h->d_src_strip = (SrcNode*)h->dalloc(sizeof(SrcNode) * sv.size());
-        if (!h->d_src_strip) return h->fail(SBP_E_OOM, "source tables");
-        if (cudaMemcpy(h->d_src_strip, sv.data(), sizeof(SrcNode) * sv.size(), cudaMemcpyHostToDevice) != cudaSuccess)
-            return h->fail(SBP_E_CUDA, "source table upload failed");
-    }
+    auto split = [&](int L, std::vector<int4>& tiles, const std::vector<std::vector<int>>& pos, int4* d_tiles, SrcNode** d_src) {
+        std::vector<std::pair<int, SrcNode>> strip;
+        inner.clear();
+        for (const SrcNode& nd : h->src_nodes) {
+            const HostBlock& hb = h->blocks[nd.block];
+            const int i2 = (int)(nd.gi / hb.pitch), i1 = (int)(nd.gi - (long long)i2 * hb.pitch);
+            const int t = strip_tile_of(h, hb, i1, i2, L);
+            if (t < 0) inner.push_back(nd);
+            else strip.push_back({pos[nd.block][t], nd});
+        }
+        std::stable_sort(strip.begin(), strip.end(),
+                         [](const std::pair<int, SrcNode>& x, const std::pair<int, SrcNode>& y) { return x.first < y.first; });
+        for (int4& tl : tiles) tl.z = tl.w = 0;
+        std::vector<SrcNode> sv;
+        for (size_t k = 0; k < strip.size(); ++k) {
+            int4& tl = tiles[strip[k].first];
+            if (tl.z == tl.w) tl.z = tl.w = (int)k;
+            tl.w = (int)k + 1;
+            sv.push_back(strip[k].second);
+        }
+        if (!sv.empty()) {
+            *d_src = (SrcNode*)h->dalloc(sizeof(SrcNode) * sv.size());
+            if (!*d_src) return h->fail(SBP_E_OOM, "source tables");
+            if (cudaMemcpy(*d_src, sv.data(), sizeof(SrcNode) * sv.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+                return h->fail(SBP_E_CUDA, "source table upload failed");
+        }
+        if (cudaMemcpy(d_tiles, tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+            return h->fail(SBP_E_CUDA, "tile table upload failed");
+        return (int)SBP_OK;
+    };
+    h->dfree(h->shorts.d_src);
+    h->shorts.d_src = nullptr;
+    int rc = split(h->strip_len, h->tiles_host, h->tile_pos, h->d_tiles, &h->d_src_strip);
+    if (rc == SBP_OK && h->shorts.d_tiles)
+        rc = split(SHORT_TILE, h->shorts.tiles, h->shorts.pos, h->shorts.d_tiles, &h->shorts.d_src);
+    if (rc != SBP_OK) return rc;
     if (!inner.empty()) {
         h->d_src_int = (SrcNode*)h->dalloc(sizeof(SrcNode) * inner.size());
         if (!h->d_src_int) return h->fail(SBP_E_OOM, "source tables");
@@ -871,8 +1064,6 @@ int upload_sources(sbp_handle* h) {
             return h->fail(SBP_E_CUDA, "source table upload failed");
         h->n_src_int = (int)inner.size();
     }
-    if (cudaMemcpy(h->d_tiles, h->tiles_host.data(), sizeof(int4) * h->tiles_host.size(), cudaMemcpyHostToDevice) != cudaSuccess)
-        return h->fail(SBP_E_CUDA, "tile table upload failed");
     if (h->graph_exec) {   // captured launches hold the old tables and launch counts
         cudaGraphExecDestroy(h->graph_exec);
         h->graph_exec = nullptr;
@@ -967,9 +1158,11 @@ int ensure_adjoint_buffers(sbp_handle* h) {
                 return h->fail(SBP_E_CUDA, "tensor map encoding failed (adjoint fields)");
             hb.pmaps.c = hb.mmaps.c;
         }
-        CUtensorMap sm[3];
-        if (!make_strip_maps(h, hb, hb.psi[0], hb.psi[1], sm) ||
-            cudaMemcpy(hb.d_smaps + 3, sm, sizeof(sm), cudaMemcpyHostToDevice) != cudaSuccess)
+        CUtensorMap sm[3], sh[3];
+        if (!make_strip_maps(h, hb, hb.psi[0], hb.psi[1], sm, h->strip_len) ||
+            !make_strip_maps(h, hb, hb.psi[0], hb.psi[1], sh, SHORT_TILE) ||
+            cudaMemcpy(hb.d_smaps + 3, sm, sizeof(sm), cudaMemcpyHostToDevice) != cudaSuccess ||
+            cudaMemcpy(hb.d_smaps + 9, sh, sizeof(sh), cudaMemcpyHostToDevice) != cudaSuccess)
             return h->fail(SBP_E_CUDA, "tensor map encoding failed (adjoint strip maps)");
         fresh = true;
     }
@@ -1227,11 +1420,13 @@ int sbp_grid_create(const sbp_grid_desc* desc, sbp_handle** out) {
                 return cleanup(SBP_E_CUDA, "tensor map encoding failed");
         }
         {
-            hb.d_smaps = (CUtensorMap*)h->dalloc(6 * sizeof(CUtensorMap));
-            CUtensorMap sm[3];
+            hb.d_smaps = (CUtensorMap*)h->dalloc(12 * sizeof(CUtensorMap));
+            CUtensorMap sm[3], sh[3];
             if (!hb.d_smaps) return cleanup(SBP_E_OOM, "strip tensor maps");
-            if (!make_strip_maps(h, hb, hb.u[0], hb.u[1], sm) ||
-                cudaMemcpy(hb.d_smaps, sm, sizeof(sm), cudaMemcpyHostToDevice) != cudaSuccess)
+            if (!make_strip_maps(h, hb, hb.u[0], hb.u[1], sm, h->strip_len) ||
+                !make_strip_maps(h, hb, hb.u[0], hb.u[1], sh, SHORT_TILE) ||
+                cudaMemcpy(hb.d_smaps, sm, sizeof(sm), cudaMemcpyHostToDevice) != cudaSuccess ||
+                cudaMemcpy(hb.d_smaps + 6, sh, sizeof(sh), cudaMemcpyHostToDevice) != cudaSuccess)
                 return cleanup(SBP_E_CUDA, "tensor map encoding failed (strip tiles)");
         }
         // coordinates -> pitched device planes
@@ -1255,43 +1450,20 @@ int sbp_grid_create(const sbp_grid_desc* desc, sbp_handle** out) {
     h->ntrefs = nintf;
     if (sync_views(h) != SBP_OK) return cleanup(SBP_E_CUDA, h->err);
     {
-        // strip tiles (the tile numbering of k_strip_tile: 2 bands of ceil(n1/L) tiles along x1,
-        // then 2 side bands of ceil((n2 - 2S)/L) tiles), ordered by a cost estimate: side tiles
-        // stage narrow rows, interface tiles read the neighbour, corner tiles carry two faces
-        const int S = std::max(order_nclos(o), order_ncol(o)), L = h->strip_len;
-        std::vector<std::pair<int, int2>> tl;
-        for (int b = 0; b < desc->nblocks; ++b) {
-            const HostBlock& hb = h->blocks[b];
-            const int nbx = (hb.n1 + L - 1) / L, nby = (hb.n2 - 2 * S + L - 1) / L;
-            for (int t = 0; t < 2 * nbx + 2 * nby; ++t) {
-                int cost;
-                if (t < 2 * nbx) {
-                    const int f = 2 + t / nbx, k = t % nbx;
-                    cost = (hb.f[f].kind == SBP_BC_INTERFACE ? 3 : 1) + ((k == 0 || k == nbx - 1) ? 2 : 0);
-                } else {
-                    const int f = (t - 2 * nbx) / nby;
-                    cost = 2 + (hb.f[f].kind == SBP_BC_INTERFACE ? 3 : 0);
-                }
-                tl.push_back({cost, make_int2(b, t)});
-            }
-        }
-        std::stable_sort(tl.begin(), tl.end(),
-                         [](const std::pair<int, int2>& x, const std::pair<int, int2>& y) { return x.first > y.first; });
-        h->tile_pos.assign(desc->nblocks, {});
-        for (int b = 0; b < desc->nblocks; ++b) {
-            const HostBlock& hb = h->blocks[b];
-            h->tile_pos[b].assign(2 * ((hb.n1 + L - 1) / L) + 2 * ((hb.n2 - 2 * S + L - 1) / L), -1);
-        }
-        h->tiles_host.clear();
-        for (auto& e : tl) {
-            h->tile_pos[e.second.x][e.second.y] = (int)h->tiles_host.size();
-            h->tiles_host.push_back(make_int4(e.second.x, e.second.y, 0, 0));
-        }
+        list_strip_tiles(h, h->strip_len, h->tiles_host, h->tile_pos);
         h->ntiles = (int)h->tiles_host.size();
         h->d_tiles = (int4*)h->dalloc(sizeof(int4) * h->tiles_host.size());
         if (!h->d_tiles) return cleanup(SBP_E_OOM, "tile table");
         if (cudaMemcpy(h->d_tiles, h->tiles_host.data(), sizeof(int4) * h->tiles_host.size(), cudaMemcpyHostToDevice) != cudaSuccess)
             return cleanup(SBP_E_CUDA, "tile table upload failed");
+        auto& sh = h->shorts;
+        list_strip_tiles(h, SHORT_TILE, sh.tiles, sh.pos);
+        if (h->precision == SBP_FP32 && (int)sh.tiles.size() <= 2 * h->num_sms) {
+            sh.d_tiles = (int4*)h->dalloc(sizeof(int4) * sh.tiles.size());
+            if (!sh.d_tiles) return cleanup(SBP_E_OOM, "tile table");
+            if (cudaMemcpy(sh.d_tiles, sh.tiles.data(), sizeof(int4) * sh.tiles.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+                return cleanup(SBP_E_CUDA, "tile table upload failed");
+        }
     }
     // metric
     cudaMemset(h->d_flag, 0, sizeof(int));
@@ -2089,11 +2261,12 @@ int sbp_step_graph(sbp_handle* h, int nsteps, double dt, void* stream) {
     // launches in the graph, per family (counted as if launched one by one)
     {
         const int nb = (int)h->blocks.size();
-        const int nint = h->precision == SBP_FP32 ? (nb + MARCH_MAX_BLOCKS - 1) / MARCH_MAX_BLOCKS
-                                                       : (h->blocks[0].e ? (nb + IE_MAX_BLOCKS - 1) / IE_MAX_BLOCKS : nb);
+        const bool one = one_launch(h, 0);
+        const int nint = one ? 1 : (h->precision == SBP_FP32 ? (nb + MARCH_MAX_BLOCKS - 1) / MARCH_MAX_BLOCKS
+                                    : (h->blocks[0].e ? (nb + IE_MAX_BLOCKS - 1) / IE_MAX_BLOCKS : nb));
         h->launches[0] += (long long)nsteps * nint;
-        h->launches[1] += (long long)nsteps;
-        if (h->n_src_int > 0) h->launches[3] += nsteps;
+        if (!one) h->launches[1] += (long long)nsteps;
+        if (h->n_src_int > (one ? STEP_MAX_SOURCES : 0)) h->launches[3] += nsteps;
     }
     h->t = tt;
     return SBP_OK;
@@ -2118,7 +2291,7 @@ int sbp_grid_footprint(const sbp_grid_desc* desc, long long* bytes_out) {
         // closure matrices of D_xx^FC along x1 and x2, strip-tile tensor maps
         if (desc->order == 2 || desc->order == 4 || desc->order == 6)
             total += al((long long)closure_elems(desc->order, bd.n2) * es) + al((long long)closure_elems(desc->order, bd.n1) * es);
-        total += al(6 * (long long)sizeof(CUtensorMap));
+        total += al(12 * (long long)sizeof(CUtensorMap));
         if (desc->stencil == SBP_STENCIL_WIDE) total += al(4 * plane * es);   // flux planes
         for (int f = 0; f < 4; ++f) {
             const long long nf = f < 2 ? bd.n2 : bd.n1;

@@ -239,16 +239,19 @@ struct InteriorTiles {
     int ncx[IE_MAX_BLOCKS];            // tiles across
 };
 
-template <typename T, int O, int MODE, int TX, int TY>
-__global__ void __launch_bounds__(TX * TY < 256 ? TX * TY : 256)
-k_interior_edges(const BlockDev* __restrict__ blocks, const __grid_constant__ InteriorTiles tl, StepArgs a) {
-    constexpr int Q = Ord<O>::Q, NT = TX * TY < 256 ? TX * TY : 256;
+// shared-memory elements of a tile: the displacement with its halo, g1 and g2
+template <int O, int TX, int TY> constexpr int edge_tile_elems() {
+    constexpr int SX = TX + 2 * Ord<O>::Q, SY = TY + 2 * Ord<O>::Q;
+    return 2 * (SY * SX + TY * SX + SY * TX);
+}
+// tile `tile` (of ncx across) of block B by the NT threads of the CTA
+template <typename T, int O, int MODE, int TX, int TY, int NT>
+__device__ __forceinline__ void interior_edges_tile(const BlockDev& B, int tile, int ncx, const StepArgs& a, T* sm) {
+    constexpr int Q = Ord<O>::Q;
     constexpr int SX = TX + 2 * Q, SY = TY + 2 * Q;
-    __shared__ T su[2][SY][SX], sg1[2][TY][SX], sg2[2][SY][TX];
-    int b = 0;
-    while (b + 1 < tl.nb && (int)blockIdx.x >= tl.start[b + 1]) ++b;
-    const BlockDev& B = blocks[tl.first + b];
-    const int tile = blockIdx.x - tl.start[b], ncx = tl.ncx[b];
+    T(*su)[SY][SX] = reinterpret_cast<T(*)[SY][SX]>(sm);
+    T(*sg1)[TY][SX] = reinterpret_cast<T(*)[TY][SX]>(sm + 2 * SY * SX);
+    T(*sg2)[SY][TX] = reinterpret_cast<T(*)[SY][TX]>(sm + 2 * (SY * SX + TY * SX));
     const int S = B.strip, n1 = B.n1, n2 = B.n2, P = B.pitch;
     const int x0 = S + (tile % ncx) * TX, y0 = S + (tile / ncx) * TY;
     const int lim1 = n1 - S, lim2 = n2 - S;
@@ -302,10 +305,10 @@ k_interior_edges(const BlockDev* __restrict__ blocks, const __grid_constant__ In
     }
     __syncthreads();
 #pragma unroll
-    for (int n = 0; n < TX * TY / NT; ++n) {
+    for (int n = 0; n < (TX * TY + NT - 1) / NT; ++n) {
         const int idx = threadIdx.x + n * NT, r = idx / TX, c = idx - r * TX;
         const int gx = x0 + c, gy = y0 + r;
-        if (gx >= lim1 || gy >= lim2) continue;
+        if (r >= TY || gx >= lim1 || gy >= lim2) continue;
         const size_t gi = (size_t)gy * P + gx;
         T r0 = T(0), r1 = T(0);
         dxx_edges<O, T>(
@@ -342,6 +345,16 @@ k_interior_edges(const BlockDev* __restrict__ blocks, const __grid_constant__ In
             R[gi + plane] = r1;
         }
     }
+}
+
+template <typename T, int O, int MODE, int TX, int TY>
+__global__ void __launch_bounds__(TX * TY < 256 ? TX * TY : 256)
+k_interior_edges(const BlockDev* __restrict__ blocks, const __grid_constant__ InteriorTiles tl, StepArgs a) {
+    constexpr int NT = TX * TY < 256 ? TX * TY : 256;
+    __shared__ T sm[edge_tile_elems<O, TX, TY>()];
+    int b = 0;
+    while (b + 1 < tl.nb && (int)blockIdx.x >= tl.start[b + 1]) ++b;
+    interior_edges_tile<T, O, MODE, TX, TY, NT>(blocks[tl.first + b], blockIdx.x - tl.start[b], tl.ncx[b], a, sm);
 }
 
 // ============================================================================ faces
@@ -931,7 +944,8 @@ __device__ __forceinline__ bool strip_tile_body(const BlockDev* __restrict__ blo
             // the region may have been read and written by this CTA's threads for an earlier tile
             // (persistent callers): order those accesses before the bulk copies overwrite it
             fence_proxy_async();
-            const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(B.smaps);
+            // (FP32 handles have a second set of maps for short tiles)
+            const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(B.smaps) + (sizeof(T) == 4 && TL != 32 ? 6 : 0);
             mbar_expect_tx(bar, (uint32_t)(12 * PS * sizeof(T)));
             tma_load_3d(sm, &maps[a.cur], xs, ys, 0, bar);
             tma_load_3d(sm + ST::template coff<T>(), &maps[2], xs, ys, 0, bar);
@@ -1130,17 +1144,13 @@ k_strip_tile(const BlockDev* __restrict__ blocks, const int4* __restrict__ tiles
 
 // ============================================================================ point sources
 
+// the share of source node nd in the step's output, after the node's own update
 template <typename T, int MODE>
-__global__ void k_sources(const BlockDev* __restrict__ blocks, const SrcNode* __restrict__ nodes, int nnodes,
-                          const SrcParam* __restrict__ par, StepArgs a) {
-    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-    if (tid >= nnodes || !a.with_data) return;
-    const SrcNode nd = nodes[tid];
+__device__ __forceinline__ void source_add(const BlockDev& B, const SrcNode& nd, const SrcParam* __restrict__ par, const StepArgs& a) {
     const double Wt = ricker_at(par[nd.src], a);
-    const BlockDev& B = blocks[nd.block];
     const size_t plane = (size_t)B.n2 * B.pitch;
     if (MODE == 0) {
-        // the source's share of dt^2 w r, into u^{n+1} and, in increment form, into d^{n+1}
+        // its share of dt^2 w r, into u^{n+1} and, in increment form, into d^{n+1}
         T* Un = reinterpret_cast<T*>(B.u[1 - a.cur]);
         T* DU = reinterpret_cast<T*>(B.du);
         const double fac = a.dt2 * (double)reinterpret_cast<const T*>(B.w)[nd.gi] * Wt;
@@ -1162,6 +1172,15 @@ __global__ void k_sources(const BlockDev* __restrict__ blocks, const SrcNode* __
         atomicAdd(R + nd.gi, T(Wt * nd.wt0));
         atomicAdd(R + plane + nd.gi, T(Wt * nd.wt1));
     }
+}
+
+template <typename T, int MODE>
+__global__ void k_sources(const BlockDev* __restrict__ blocks, const SrcNode* __restrict__ nodes, int nnodes,
+                          const SrcParam* __restrict__ par, StepArgs a) {
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+    if (tid >= nnodes || !a.with_data) return;
+    const SrcNode nd = nodes[tid];
+    source_add<T, MODE>(blocks[nd.block], nd, par, a);
 }
 
 // ============================================================================ wait probe
