@@ -572,6 +572,202 @@ __device__ void face_sat_node(const BlockDev* __restrict__ blocks, const BlockDe
     Fs1 = inv_h0 * f1;
 }
 
+// The same terms in SAT_PARTS independent parts, for as many threads; adds the part's share to Fs, As.  Part 0 has As
+// and what needs the face node alone; the others the normal and the tangential share of a Robin face's traction, or
+// the taps of the tangential transpose.  (One function for both, the parts chosen at compile time or run in turn,
+// made face_sat_node spill in the strip kernels: 2001^2 FP32 100.5 -> 104.7 us a step.)
+constexpr int SAT_PARTS = 4;
+// face_traction's part of the normal derivative (NORMAL) or of the tangential one, added to t0, t1
+template <typename T, int O, bool NORMAL, class UA, class CA>
+__device__ __forceinline__ void face_traction_part(const BlockDev& B, const FaceDev& F, int s, UA u, CA c, T& t0, T& t1) {
+    const int m = F.m, Nm = m == 0 ? B.n1 : B.n2, Nt = m == 0 ? B.n2 : B.n1;
+    const T ih = ((m == 0) == NORMAL ? ih1T<T>(B) : ih2T<T>(B));
+    T d[2];
+#pragma unroll
+    for (int L = 0; L < 2; ++L)
+        d[L] = NORMAL ? dsum<O, T>(Nm, F.side ? Nm - 1 : 0, [&](int j) {
+                            int j1, j2;
+                            face_at(B, F, s, F.side ? Nm - 1 - j : j, j1, j2);
+                            return u(L, j1, j2);
+                        }) * ih
+                      : dsum<O, T>(Nt, s, [&](int j) {
+                            int j1, j2;
+                            face_at(B, F, j, 0, j1, j2);
+                            return u(L, j1, j2);
+                        }) * ih;
+    int i1, i2;
+    face_at(B, F, s, 0, i1, i2);
+    const T nu = T(F.nu);
+    auto pl = [&](int J, int L) { return NORMAL ? plane_nn(m, J, L) : plane_nt(m, J, L); };
+    t0 += nu * (c(pl(0, 0), i1, i2) * d[0] + c(pl(0, 1), i1, i2) * d[1]);
+    t1 += nu * (c(pl(1, 0), i1, i2) * d[0] + c(pl(1, 1), i1, i2) * d[1]);
+}
+template <typename T, int O, class UA, class CA>
+__device__ __forceinline__ void face_sat_part(int part, const BlockDev* __restrict__ blocks, const BlockDev& B, const FaceDev& F,
+                                              int s, const StepArgs& a, double beta, UA u, CA c, T& Fs0, T& Fs1, T& As0,
+                                              T& As1) {
+    const int m = F.m, nf = F.nf;
+    const T nu = T(F.nu);
+    const T inv_h0 = T(F.inv_h0);
+    int i1, i2;
+    face_at(B, F, s, 0, i1, i2);
+    const bool has_data = a.with_data && F.g;
+    const T* __restrict__ g = reinterpret_cast<const T*>(F.g);
+    if (F.kind == FACE_ROBIN) {
+        T f0 = T(0), f1 = T(0);
+        if (part == 1) face_traction_part<T, O, true>(B, F, s, u, c, f0, f1);
+        else if (part == 2) face_traction_part<T, O, false>(B, F, s, u, c, f0, f1);
+        else if (part == 0) {
+            if (F.ju) {
+                const T u0 = u(0, i1, i2), u1 = u(1, i1, i2);
+                const T* ju = reinterpret_cast<const T*>(F.ju);
+                const T a11 = ju[s], a12 = ju[nf + s], a22 = ju[2 * nf + s];
+                f0 = a11 * u0 + a12 * u1;
+                f1 = a12 * u0 + a22 * u1;
+            }
+            if (has_data) {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    if (k >= a.K) break;
+                    f0 -= T(a.Tk[k]) * g[(size_t)k * nf + s];
+                    f1 -= T(a.Tk[k]) * g[(size_t)(a.K + k) * nf + s];
+                }
+            }
+        }
+        Fs0 -= inv_h0 * f0;
+        Fs1 -= inv_h0 * f1;
+        return;
+    }
+    const bool intf = F.kind == FACE_INTF;
+    // the neighbour across an interface: its block, face, current level and coefficients
+    const BlockDev* V = intf ? &blocks[F.nbr_block] : nullptr;
+    const FaceDev* FV = intf ? &V->f[F.nbr_face] : nullptr;
+    const T* __restrict__ Uv = intf ? reinterpret_cast<const T*>(V->u[a.cur]) : nullptr;
+    const T* __restrict__ Cv = intf ? reinterpret_cast<const T*>(V->c) : nullptr;
+    const size_t pv = intf ? (size_t)V->n2 * V->pitch : 0;
+    auto uv = [&](int L, int j1, int j2) { return Uv[(size_t)L * pv + (size_t)j2 * V->pitch + j1]; };
+    auto cv = [&](int pl, int j1, int j2) { return Cv[(size_t)pl * pv + (size_t)j2 * V->pitch + j1]; };
+    // traces of both sides (k_face_trace, same level): replace the neighbour's reads and both tractions
+    const T* __restrict__ trU = intf ? reinterpret_cast<const T*>(F.tr) : nullptr;
+    const T* __restrict__ trV = intf ? reinterpret_cast<const T*>(FV->tr) : nullptr;
+    const bool traced = trU != nullptr && trV != nullptr;
+    // jump w_L at face node sp (displacement: u - g(t); interface: u - v)
+    auto jump = [&](int sp, T& w0, T& w1) {
+        int j1, j2;
+        face_at(B, F, sp, 0, j1, j2);
+        w0 = u(0, j1, j2);
+        w1 = u(1, j1, j2);
+        if (intf) {
+            const int svp = F.reversed ? nf - 1 - sp : sp;
+            if (traced) {
+                w0 -= trV[svp];
+                w1 -= trV[nf + svp];
+            } else {
+                int v1, v2;
+                face_at(*V, *FV, svp, 0, v1, v2);
+                w0 -= uv(0, v1, v2);
+                w1 -= uv(1, v1, v2);
+            }
+        } else if (has_data) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                if (k >= a.K) break;
+                w0 -= T(a.Tk[k]) * g[(size_t)k * nf + sp];
+                w1 -= T(a.Tk[k]) * g[(size_t)(a.K + k) * nf + sp];
+            }
+        }
+    };
+    const T half = intf ? T(0.5) : T(1);
+    if (part == 0) {
+        const double dd = 2.0;   // spatial dimension d
+        T w0, w1;
+        jump(s, w0, w1);
+        const T c00 = c(plane_nn(m, 0, 0), i1, i2), c01 = c(plane_nn(m, 0, 1), i1, i2), c11 = c(plane_nn(m, 1, 1), i1, i2);
+        T z00, z01, z11;
+        if (!intf) {
+            const T k = T(beta * dd * F.inv_h0);
+            z00 = k * c00; z01 = k * c01; z11 = k * c11;
+        } else if (traced) {
+            const int sv = F.reversed ? nf - 1 - s : s;
+            z00 = trU[4 * nf + s] + trV[4 * nf + sv];
+            z01 = trU[5 * nf + s] + trV[5 * nf + sv];
+            z11 = trU[6 * nf + s] + trV[6 * nf + sv];
+        } else {
+            const int sv = F.reversed ? nf - 1 - s : s;
+            int v1, v2;
+            face_at(*V, *FV, sv, 0, v1, v2);
+            const int mv = FV->m;
+            const T ku = T(beta * dd / 4.0 * F.inv_h0), kv = T(beta * dd / 4.0 * FV->inv_h0);
+            const T zu00 = ku * c00, zu01 = ku * c01, zu11 = ku * c11;
+            const T zv00 = kv * cv(plane_nn(mv, 0, 0), v1, v2), zv01 = kv * cv(plane_nn(mv, 0, 1), v1, v2),
+                    zv11 = kv * cv(plane_nn(mv, 1, 1), v1, v2);
+            z00 = zu00 + zv00;
+            z01 = zu01 + zv01;
+            z11 = zu11 + zv11;
+        }
+        // normal-spread amplitude a_J = half nu c_mJmL w_L
+        As0 += half * nu * (c00 * w0 + c01 * w1);
+        As1 += half * nu * (c01 * w0 + c11 * w1);
+        T f0 = -(z00 * w0 + z01 * w1), f1 = -(z01 * w0 + z11 * w1);
+        if (intf) {
+            T tu0, tu1, tv0, tv1;
+            const int sv = F.reversed ? nf - 1 - s : s;
+            if (traced) {
+                tu0 = trU[2 * nf + s];
+                tu1 = trU[3 * nf + s];
+                tv0 = trV[2 * nf + sv];
+                tv1 = trV[3 * nf + sv];
+            } else {
+                face_traction<T, O>(B, F, s, u, c, tu0, tu1);
+                face_traction<T, O>(*V, *FV, sv, uv, cv, tv0, tv1);
+            }
+            f0 -= T(0.5) * (tu0 + tv0);
+            f1 -= T(0.5) * (tu1 + tv1);
+        }
+        Fs0 += inv_h0 * f0;
+        Fs1 += inv_h0 * f1;
+        return;
+    }
+    // tangential transpose term (1/H_t(s)) sum_s' D_t[s'][s] H_t(s') b_J(s'),  b_J = nu c_mLtJ w_L;
+    // rows of D with a non-zero in column s: the interior band s-Q..s+Q plus, near an end, every
+    // boundary row (boundary rows span columns 0..NCOL-1, which can reach past s+Q)
+    const int Nt = nf;
+    T tt0 = T(0), tt1 = T(0);
+    auto tterm = [&](int sp, T wgt) {
+        T v0, v1;
+        jump(sp, v0, v1);
+        int j1, j2;
+        face_at(B, F, sp, 0, j1, j2);
+        tt0 += wgt * nu * (c(plane_nt(m, 0, 0), j1, j2) * v0 + c(plane_nt(m, 1, 0), j1, j2) * v1);
+        tt1 += wgt * nu * (c(plane_nt(m, 0, 1), j1, j2) * v0 + c(plane_nt(m, 1, 1), j1, j2) * v1);
+    };
+    constexpr int TP = SAT_PARTS - 1;
+    T tfac = m == 0 ? ih2T<T>(B) : ih1T<T>(B);
+    if (s >= Ord<O>::NCOL && s < Nt - Ord<O>::NCOL) {
+        // column s meets only interior rows s-Q..s+Q of D (weight 1): s-k with a_k and s+k with -a_k, k = part
+        static_assert(Ord<O>::Q <= TP, "a part per tap distance");
+        if (part <= Ord<O>::Q) {
+            const T ak = Ord<O>::template aT<T>(part - 1);
+            tterm(s - part, ak);
+            tterm(s + part, -ak);
+        }
+    } else {
+        int lo = s - Ord<O>::Q, hi = s + Ord<O>::Q;
+        if (s < Ord<O>::NCOL) { lo = 0; hi = max(hi, Ord<O>::NB - 1); }
+        if (s >= Nt - Ord<O>::NCOL) { hi = Nt - 1; lo = min(lo, Nt - Ord<O>::NB); }
+        if (lo < 0) lo = 0;
+        if (hi > Nt - 1) hi = Nt - 1;
+        for (int sp = lo + part - 1; sp <= hi; sp += TP) {
+            const T dc = dcoefT<O, T>(Nt, sp, s);
+            if (dc == T(0)) continue;
+            tterm(sp, dc * hweightT<O, T>(Nt, sp));
+        }
+        tfac /= hweightT<O, T>(Nt, s);
+    }
+    Fs0 += inv_h0 * half * tfac * tt0;
+    Fs1 += inv_h0 * half * tfac * tt1;
+}
+
 // SAT terms of every face node from global memory into F.sat (face term 2 x nf, spread amplitude
 // 2 x nf); used with k_boundary (the strip tile kernel computes them itself)
 template <typename T, int O>
@@ -862,7 +1058,7 @@ __device__ __forceinline__ double ricker_at(const SrcParam& p, const StepArgs& a
 // TL, the tile's length along the face: 32 in FP32 (a warp per row).  In FP64 the tile's arithmetic holds
 // its SM (see k_interior_edges), so small grids are cut shorter, 16 or 8 nodes, until the tiles spread
 // over all SMs (the host picks; the halo along the face repeats more of the fluxes the shorter the tile).
-template <int O, int TL = 32> struct StripTile {
+template <int O, int TL = 32, bool SPLIT = false> struct StripTile {
     static constexpr int Q = Ord<O>::Q;
     static constexpr int S = Ord<O>::NCLOS > Ord<O>::NCOL ? Ord<O>::NCLOS : Ord<O>::NCOL;
     static constexpr int HN = Q;
@@ -873,7 +1069,8 @@ template <int O, int TL = 32> struct StripTile {
     static constexpr int FLUXB = 2 * (S * BWB + BHB * TL), FLUXS = 2 * (TL * BWS + BHS * S);
     static constexpr int FLUX = FLUXB > FLUXS ? FLUXB : FLUXS;   // g1 on the tile rows, g2 on its columns
     static constexpr int FN = TL > S ? TL : S;          // face nodes of a tile: along it, or across it at a corner
-    static constexpr int SATS = 4 * FN * 4;             // per face, per face node: Fs0, Fs1, As0, As1
+    static constexpr int SN = 2 + 2 * (SPLIT ? SAT_PARTS : 1);   // per face node: As0, As1, and Fs0, Fs1 of each part
+    static constexpr int SATS = 4 * FN * SN;
     static constexpr int THREADS = TL * S < 128 ? 128 : (TL * S + 31) / 32 * 32;
     // element offset of the coefficient box (128-byte aligned TMA destination), of the fluxes, and bytes
     template <typename T> static constexpr int coff() { return (int)((2 * RMAX * sizeof(T) + 127) / 128 * 128 / sizeof(T)); }
@@ -892,11 +1089,15 @@ template <int O, int TL = 32> struct StripTile {
 // the tile's staging copies ran out (the error word is set).  The staging mbarrier is
 // invalidated before the return, so a persistent caller can reuse the shared memory for its next
 // tile after a CTA barrier.
-template <typename T, int O, int MODE, int NT, int TL = 32>
+// SPLIT: a warp per part of the SAT terms.  One thread for all of a face node's terms is the tile's longest chain of
+// dependent operations: the one-launch steps, which wait for it, gain (FP32 order 6: 101^2 20.6 -> 16.5 us, 601^2
+// 24.8 -> 22.7; FP64 order 4: 101^2 31 -> 27), where many tiles fill the chip the repeated indexing costs (2 x
+// 802 x 401: 43.4 -> 45.3 us).
+template <typename T, int O, int MODE, int NT, int TL = 32, bool SPLIT = false>
 __device__ __forceinline__ bool strip_tile_body(const BlockDev* __restrict__ blocks, const int4 tt, const StepArgs& a,
                                                 double beta, int* err, const SrcNode* __restrict__ ssrc,
                                                 const SrcParam* __restrict__ spar, unsigned char* strip_smem) {
-    using ST = StripTile<O, TL>;
+    using ST = StripTile<O, TL, SPLIT>;
     constexpr int S = ST::S;
     T* sm = reinterpret_cast<T*>(strip_smem);
     uint64_t* bar = reinterpret_cast<uint64_t*>(strip_smem + ST::template bar_off<T>());
@@ -989,6 +1190,37 @@ __device__ __forceinline__ bool strip_tile_body(const BlockDev* __restrict__ blo
     auto g1 = [&](int J, int j1, int j2) -> T& { return g1s[(J * h + (j2 - y0)) * BW + (j1 - xs)]; };
     auto g2 = [&](int J, int j1, int j2) -> T& { return g2s[(J * BH + (j2 - ys)) * w + (j1 - x0)]; };
     const T ih1 = ih1T<T>(B), ih2 = ih2T<T>(B);
+    // SAT terms of the face nodes whose first NCOL nodes meet the tile: face f's tangential range
+    // is the tile's y range (f = 0, 1) or x range (f = 2, 3)
+    T* sats = sm + ST::template foff<T>() + ST::FLUX;
+    auto face_meets = [&](int f) {
+        if (f < 2) return f == 0 ? x0 < Ord<O>::NCOL : x0 + w > n1 - Ord<O>::NCOL;
+        return f == 2 ? y0 < Ord<O>::NCOL : y0 + h > n2 - Ord<O>::NCOL;
+    };
+    // (split: two groups of warps where the CTA has eight, each with every other face)
+    if constexpr (SPLIT) {
+        const int wid = threadIdx.x >> 5, part = wid % SAT_PARTS, group = wid / SAT_PARTS;
+        constexpr int GROUPS = NT / 32 / SAT_PARTS;
+        static_assert(GROUPS >= 1, "a warp for every part");
+        int nth = 0;
+        for (int f = 0; f < 4; ++f) {
+            if (!face_meets(f)) continue;
+            if (nth++ % GROUPS != group) continue;
+            for (int k = threadIdx.x & 31; k < (f < 2 ? h : w); k += 32) {
+                T f0 = T(0), f1 = T(0), a0 = T(0), a1 = T(0);
+                face_sat_part<T, O>(part, blocks, B, B.f[f], (f < 2 ? y0 : x0) + k, a, beta,
+                                    [&](int L, int j1, int j2) { return at(L, j1, j2); },
+                                    [&](int pl, int j1, int j2) { return at(2 + pl, j1, j2); }, f0, f1, a0, a1);
+                T* q = sats + (f * ST::FN + k) * ST::SN;
+                if (part == 0) {
+                    q[0] = a0;
+                    q[1] = a1;
+                }
+                q[2 + 2 * part] = f0;
+                q[3 + 2 * part] = f1;
+            }
+        }
+    }
     // g1 on the tile's rows (the staged columns inside the block), g2 on the tile's columns (the
     // staged rows inside the block)
     const int cx0 = max(0, xs), cx1 = min(n1, xs + VW), RWc = cx1 - cx0;
@@ -1009,25 +1241,20 @@ __device__ __forceinline__ bool strip_tile_body(const BlockDev* __restrict__ blo
         g2(0, j1, j2) = at(8, j1, j2) * d0 + at(10, j1, j2) * d1;
         g2(1, j1, j2) = at(9, j1, j2) * d0 + at(11, j1, j2) * d1;
     }
-    // SAT terms of the face nodes whose first NCOL nodes meet the tile: face f's tangential range
-    // is the tile's y range (f = 0, 1) or x range (f = 2, 3)
-    T* sats = sm + ST::template foff<T>() + ST::FLUX;
-    auto face_meets = [&](int f) {
-        if (f < 2) return f == 0 ? x0 < Ord<O>::NCOL : x0 + w > n1 - Ord<O>::NCOL;
-        return f == 2 ? y0 < Ord<O>::NCOL : y0 + h > n2 - Ord<O>::NCOL;
-    };
-    for (int idx = threadIdx.x; idx < 4 * ST::FN; idx += NT) {
-        const int f = idx / ST::FN, k = idx % ST::FN;
-        if (k >= (f < 2 ? h : w) || !face_meets(f)) continue;
-        const int s = (f < 2 ? y0 : x0) + k;
-        T f0, f1, a0, a1;
-        face_sat_node<T, O>(blocks, B, B.f[f], s, a, beta, [&](int L, int j1, int j2) { return at(L, j1, j2); },
-                            [&](int pl, int j1, int j2) { return at(2 + pl, j1, j2); }, f0, f1, a0, a1);
-        T* q = sats + (f * ST::FN + k) * 4;
-        q[0] = f0;
-        q[1] = f1;
-        q[2] = a0;
-        q[3] = a1;
+    if constexpr (!SPLIT) {
+        for (int idx = threadIdx.x; idx < 4 * ST::FN; idx += NT) {
+            const int f = idx / ST::FN, k = idx % ST::FN;
+            if (k >= (f < 2 ? h : w) || !face_meets(f)) continue;
+            T f0, f1, a0, a1;
+            face_sat_node<T, O>(blocks, B, B.f[f], (f < 2 ? y0 : x0) + k, a, beta,
+                                [&](int L, int j1, int j2) { return at(L, j1, j2); },
+                                [&](int pl, int j1, int j2) { return at(2 + pl, j1, j2); }, f0, f1, a0, a1);
+            T* q = sats + (f * ST::FN + k) * ST::SN;
+            q[0] = a0;
+            q[1] = a1;
+            q[2] = f0;
+            q[3] = f1;
+        }
     }
     __syncthreads();
     // output node of this thread: a warp per row of a band tile (lanes along the row), a warp per
@@ -1079,13 +1306,16 @@ __device__ __forceinline__ bool strip_tile_body(const BlockDev* __restrict__ blo
             const int im = m == 0 ? i1 : i2, Nm = m == 0 ? n1 : n2;
             const int d = F.side ? Nm - 1 - im : im;
             if (d >= Ord<O>::NCOL) continue;
-            const T* q = sats + (f * ST::FN + (m == 0 ? i2 - y0 : i1 - x0)) * 4;
+            const T* q = sats + (f * ST::FN + (m == 0 ? i2 - y0 : i1 - x0)) * ST::SN;
             const T fac = facT<T>(F, d);
-            r0 += fac * q[2];
-            r1 += fac * q[3];
+            r0 += fac * q[0];
+            r1 += fac * q[1];
             if (d == 0) {
-                r0 += q[0];
-                r1 += q[1];
+#pragma unroll
+                for (int p = 0; p < (SPLIT ? SAT_PARTS : 1); ++p) {
+                    r0 += q[2 + 2 * p];
+                    r1 += q[3 + 2 * p];
+                }
             }
         }
         if (a.with_data && B.jf) {

@@ -4,10 +4,10 @@
 // middling grid leaves most of the chip idle in either kernel and waits for each one's latency and launch in
 // turn.  An interior tile then adds the off-strip source nodes that lie in it (as k_sources does after the step kernels; the same
 // arithmetic), which saves that launch as well.
-// A step of one block, FP32, order 6, with a source inside, against separate launches: 201^2 36.6 -> 18.6 us, 601^2
-// 37.7 -> 24.7, 1001^2 46.1 -> 30.9, but 1401^2 67.8 -> 72.7 (the strips by 128 threads then cost more than the
-// launches do); FP64, order 6: 201^2 45 -> 35 us,
-// 601^2 158 -> 137; order 4: 101^2 41 -> 31.
+// A step of one block, FP32, order 6, with a source inside, against separate launches: 201^2 36.6 -> 16.5 us, 601^2
+// 37.7 -> 22.7, 1001^2 46.1 -> 29.9, but 1401^2 67.8 -> 72.7 (the strips by 128 threads then cost more than the
+// launches do); FP64, order 6: 201^2 45 -> 33 us,
+// 601^2 158 -> 136; order 4: 101^2 41 -> 27.
 #pragma once
 #include "sbp_interior_march.cuh"
 #include "sbp_kernels.cuh"
@@ -42,7 +42,8 @@ __device__ __forceinline__ void tile_sources(const StepStrips& s, int b, int lo1
 }
 
 template <int O> constexpr size_t step_smem_f32() {
-    return MarchCfg<O>::BYTES > StripTile<O>::template bytes<float>() ? MarchCfg<O>::BYTES : StripTile<O>::template bytes<float>();
+    return MarchCfg<O>::BYTES > StripTile<O, 32, (O > 2)>::template bytes<float>() ? MarchCfg<O>::BYTES
+                                                                                  : StripTile<O, 32, (O > 2)>::template bytes<float>();
 }
 
 // FP32 leapfrog step; MODE 3: increment form, 0: the adjoint fields' two levels
@@ -52,7 +53,7 @@ k_step_f32(const __grid_constant__ MarchMulti mm, const __grid_constant__ StepSt
     extern __shared__ __align__(128) unsigned char step_smem[];
     const int k = (int)blockIdx.x - ss.n;
     if (k < 0) {
-        (void)strip_tile_body<float, O, 0, MTHREADS, TL>(ss.blocks, ss.tiles[blockIdx.x], a, ss.beta, err, ss.ssrc, ss.spar, step_smem);
+        (void)strip_tile_body<float, O, 0, MTHREADS, TL, (O > 2)>(ss.blocks, ss.tiles[blockIdx.x], a, ss.beta, err, ss.ssrc, ss.spar, step_smem);
         return;
     }
     int b = 0;
@@ -69,7 +70,7 @@ k_step_f32(const __grid_constant__ MarchMulti mm, const __grid_constant__ StepSt
 template <int TX, int TY> constexpr int step_len_f64() { return TX * TY == 512 ? 16 : 8; }
 template <int TX, int TY> constexpr int step_threads_f64() { return TX * TY == 512 ? 256 : 128; }
 template <int O, int TX, int TY> constexpr size_t step_smem_f64() {
-    constexpr size_t strip = StripTile<O, step_len_f64<TX, TY>()>::template bytes<double>();
+    constexpr size_t strip = StripTile<O, step_len_f64<TX, TY>(), (O > 2)>::template bytes<double>();
     return edge_tile_elems<O, TX, TY>() * sizeof(double) > strip ? edge_tile_elems<O, TX, TY>() * sizeof(double) : strip;
 }
 template <int O, int MODE, int TX, int TY>
@@ -79,7 +80,7 @@ k_step_f64(const __grid_constant__ InteriorTiles tl, const __grid_constant__ Ste
     extern __shared__ __align__(128) unsigned char step_smem[];
     const int k = (int)blockIdx.x - ss.n;
     if (k < 0) {
-        (void)strip_tile_body<double, O, MODE, NT, step_len_f64<TX, TY>()>(ss.blocks, ss.tiles[blockIdx.x], a, ss.beta, err,
+        (void)strip_tile_body<double, O, MODE, NT, step_len_f64<TX, TY>(), (O > 2)>(ss.blocks, ss.tiles[blockIdx.x], a, ss.beta, err,
                                                                            ss.ssrc, ss.spar, step_smem);
         return;
     }
