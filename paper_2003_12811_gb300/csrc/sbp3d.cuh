@@ -194,6 +194,17 @@ template <typename T, int NV> __device__ __forceinline__ void vld(const T* p, T 
         for (int n = 0; n < NV; ++n) v[n] = __ldg(p + n);
     }
 }
+// Field access of the flux kernel: the field's base is the same for the whole grid and the node's
+// offset, in bytes of type I, is 32 bits wide where the fields stay below 4 GB.  A neighbour then costs one 32-bit
+// addition, shared by all the fields that are read there, where a pointer per field costs a 64-bit one for
+// each of them.  160 x 151 x 144, FP32: k3_flux 140 -> 131 us (k3_div, whose offsets then take the registers that
+// its rows need, 171 -> 189: it keeps pointers).
+template <typename T, typename I> __device__ __forceinline__ const T* at(const T* base, I off) {
+    return reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) + off);
+}
+template <typename T, int NV, typename I> __device__ __forceinline__ void vldo(const T* base, I off, T v[NV]) {
+    vld<T, NV>(at(base, off), v);
+}
 template <typename T, int NV> __device__ __forceinline__ void vst(T* p, const T v[NV]) {
     if constexpr (NV == 2 && sizeof(T) == 4) {
         *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
@@ -218,14 +229,15 @@ __device__ __noinline__ void grad_call(const Grid3& g, int i, const T* __restric
 // reads its x1 stencil as aligned vector windows; its x2 / x3 rows are vector loads at +-k
 // strides (interior) or the general rows node by node (closure rows, the same for a whole warp).
 // A pair near the x1 faces takes the general rows for everything.
-template <typename T, int O, int NV>
-__device__ __forceinline__ void flux_pair(const Grid3& g, int i1, int i2, int i3, const T* __restrict__ up,
+template <typename T, int O, int NV, typename I>
+__device__ __forceinline__ void flux_pair(const Grid3& g, int i1, int i2, int i3, const T* __restrict__ u, I ob,
                                           T gr[NV][3][3]) {
     using P = Ord<O>;
     constexpr int Q = P::Q;
     constexpr int QA = (Q + NV - 1) / NV * NV;
     constexpr int WN = NV + 2 * QA;
     const long long fs = g.fs;
+    const T* up = at(u, ob);
     const bool x1int = i1 >= P::NB && i1 + NV - 1 <= g.n[0] - 1 - P::NB && i1 >= QA;
     if (x1int) {
         const T ih = T(g.ih[0]);
@@ -233,7 +245,7 @@ __device__ __forceinline__ void flux_pair(const Grid3& g, int i1, int i2, int i3
         for (int l = 0; l < 3; ++l) {
             T w[WN];
 #pragma unroll
-            for (int v = 0; v < WN / NV; ++v) vld<T, NV>(up + l * fs - QA + v * NV, w + v * NV);
+            for (int v = 0; v < WN / NV; ++v) vldo<T, NV>(u + l * fs, ob + I((v * NV - QA) * (int)sizeof(T)), w + v * NV);
 #pragma unroll
             for (int n = 0; n < NV; ++n) {
                 T acc = T(0);
@@ -250,25 +262,30 @@ __device__ __forceinline__ void flux_pair(const Grid3& g, int i1, int i2, int i3
         constexpr int D = decltype(dc)::value;
         const int N = g.n[D];
         if (i >= P::NB && i <= N - 1 - P::NB) {
-            const int S = dstride<D>(g);
+            const I S = I(dstride<D>(g)) * I(sizeof(T));
             const T ih = T(g.ih[D]);
+            T acc[3][NV];
 #pragma unroll
-            for (int l = 0; l < 3; ++l) {
-                T acc[NV];
+            for (int l = 0; l < 3; ++l)
 #pragma unroll
-                for (int n = 0; n < NV; ++n) acc[n] = T(0);
+                for (int n = 0; n < NV; ++n) acc[l][n] = T(0);
 #pragma unroll
-                for (int k = 1; k <= Q; ++k) {
+            for (int k = 1; k <= Q; ++k) {
+                const I op = ob + I(k) * S, om = ob - I(k) * S;
+                const T ak = P::template aT<T>(k - 1);
+#pragma unroll
+                for (int l = 0; l < 3; ++l) {
                     T a[NV], b[NV];
-                    vld<T, NV>(up + l * fs + k * S, a);
-                    vld<T, NV>(up + l * fs - k * S, b);
-                    const T ak = P::template aT<T>(k - 1);
+                    vldo<T, NV>(u + l * fs, op, a);
+                    vldo<T, NV>(u + l * fs, om, b);
 #pragma unroll
-                    for (int n = 0; n < NV; ++n) acc[n] += ak * (a[n] - b[n]);
+                    for (int n = 0; n < NV; ++n) acc[l][n] += ak * (a[n] - b[n]);
                 }
-#pragma unroll
-                for (int n = 0; n < NV; ++n) gr[n][D][l] = ih * acc[n];
             }
+#pragma unroll
+            for (int l = 0; l < 3; ++l)
+#pragma unroll
+                for (int n = 0; n < NV; ++n) gr[n][D][l] = ih * acc[l][n];
         } else {
 #pragma unroll
             for (int n = 0; n < NV; ++n) grad_call<T, O, D>(g, i, up + n, gr[n][D]);
@@ -278,7 +295,7 @@ __device__ __forceinline__ void flux_pair(const Grid3& g, int i1, int i2, int i3
     strided(std::integral_constant<int, 2>(), i3);
 }
 
-template <typename T, int O, int NV>
+template <typename T, int O, int NV, typename I>
 __global__ void __launch_bounds__(BX * BY, 3) k3_flux(Grid3 g, const T* __restrict__ u, const T* __restrict__ cm,
                                                    T* __restrict__ q) {
     const int i1 = (blockIdx.x * BX + threadIdx.x) * NV, i2 = blockIdx.y * BY + threadIdx.y, i3 = blockIdx.z;
@@ -286,11 +303,12 @@ __global__ void __launch_bounds__(BX * BY, 3) k3_flux(Grid3 g, const T* __restri
     const long long o = i1 + i2 * g.s[1] + i3 * g.s[2];
     const long long fs = g.fs;
     const T* up = u + o;
+    const I ob = I(o) * I(sizeof(T));
     // the last pair of an odd row has one node: it runs alone through the general rows
     const bool full = i1 + NV - 1 < g.n[0];
     T gr[NV][3][3];                               // gr[n][k][l] = D_k u_l at node n
     if (full) {
-        flux_pair<T, O, NV>(g, i1, i2, i3, up, gr);
+        flux_pair<T, O, NV, I>(g, i1, i2, i3, u, ob, gr);
     } else {
 #pragma unroll
         for (int n = 0; n < NV; ++n) {
@@ -306,7 +324,6 @@ __global__ void __launch_bounds__(BX * BY, 3) k3_flux(Grid3 g, const T* __restri
         for (int i = 0; i < 3; ++i)
 #pragma unroll
             for (int j = 0; j < 3; ++j) qq[n][i][j] = T(0);
-    const T* cmo = cm + o;
 #pragma unroll
     for (int p = 0; p < 3; ++p) {
         const int i = p == 2 ? 1 : 0, k = p == 0 ? 1 : 2;
@@ -316,9 +333,9 @@ __global__ void __launch_bounds__(BX * BY, 3) k3_flux(Grid3 g, const T* __restri
             for (int l = 0; l < 3; ++l) {
                 T M[NV];
                 if (full) {
-                    vld<T, NV>(cmo + (9 * p + 3 * j + l) * fs, M);
+                    vldo<T, NV>(cm + (9 * p + 3 * j + l) * fs, ob, M);
                 } else {
-                    M[0] = ldg(cmo + (9 * p + 3 * j + l) * fs);
+                    M[0] = ldg(at(cm + (9 * p + 3 * j + l) * fs, ob));
 #pragma unroll
                     for (int n = 1; n < NV; ++n) M[n] = T(0);
                 }
@@ -329,19 +346,18 @@ __global__ void __launch_bounds__(BX * BY, 3) k3_flux(Grid3 g, const T* __restri
                 }
             }
     }
-    T* qo = q + o;
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            const long long f = (3 * i + j) * fs;
+            T* qo = const_cast<T*>(at(static_cast<const T*>(q + (3 * i + j) * fs), ob));
             if (full) {
                 T v[NV];
 #pragma unroll
                 for (int n = 0; n < NV; ++n) v[n] = qq[n][i][j];
-                vst<T, NV>(qo + f, v);
+                vst<T, NV>(qo, v);
             } else {
-                qo[f] = qq[0][i][j];
+                *qo = qq[0][i][j];
             }
         }
 }

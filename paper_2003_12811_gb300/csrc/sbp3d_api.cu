@@ -125,7 +125,8 @@ int launch_operator(sbp3_handle* h, const T* u, T* du, T* un, double dt, cudaStr
     const T dt2 = T(dt * dt);
     cudaEvent_t stop;
     prof_begin(h, 0, st, &stop);
-    k3_flux<T, O, NVF><<<grd, blk, 0, st>>>(g, u, cm, q);
+    if ((unsigned long long)h->fs * sizeof(T) <= 0xffffffffull) k3_flux<T, O, NVF, unsigned><<<grd, blk, 0, st>>>(g, u, cm, q);
+    else k3_flux<T, O, NVF, long long><<<grd, blk, 0, st>>>(g, u, cm, q);
     prof_end(stop, st);
     const Box3& bx = h->box;
     prof_begin(h, 2, st, &stop);
