@@ -349,7 +349,8 @@ int sbp_batch_poll(sbp_batch* b, int* remaining, void* stream);
  * on `stream`); otherwise `stream` is synchronised and the state read. */
 int sbp_batch_remove(sbp_batch* b, int slot, void* stream);
 
-/* Rows of an interior work item (the tile shape; 0 = default 64).  Only while the batch is empty. */
+/* Rows of an interior work item (the tile shape; 0 = default: bands of equal height that divide the work
+ * of the admitted shots evenly over the CTAs).  Only while the batch is empty. */
 int sbp_batch_set_rows(sbp_batch* b, int rows);
 
 /* Pick the tile shape (rows of an interior work item: 32, 64, 128 or 256) by timing batch steps of

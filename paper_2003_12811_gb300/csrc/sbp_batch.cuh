@@ -3,7 +3,8 @@
 //
 // One launch advances every active shot of the batch by one leapfrog step.  Its CTAs (a fixed
 // number per SM) pull work items from one device-wide queue -- an interior tile of a shot (128
-// columns x `rows` rows of the column-marching stencil) or a boundary-strip tile of a shot
+// columns x as many rows of the column-marching stencil as divide the batch evenly, item_rows) or a
+// boundary-strip tile of a shot
 // (closures, SAT terms, strip point sources) -- until the queue is empty; the items of a step are
 // independent (they read level n and write level n+1 of disjoint nodes).  The last CTA to finish
 // (detected with a fence and a counter, no waiting) adds the point-source nodes off the strips,
@@ -25,7 +26,6 @@ struct alignas(64) BatchShot {
     const SrcNode* isrc;            // point-source nodes off the strips or null
     const SrcParam* spar;
     int nisrc;
-    int rows;                       // rows of an interior item
     double dt, dt2, beta;
     float dt2f;
 };
@@ -38,7 +38,7 @@ struct BatchState {
 };
 
 struct BatchHead {
-    const int4* items;              // (shot, kind 0 interior / 1 strip, item index, 0)
+    const int4* items;              // (shot, kind 0 interior / 1 strip, item index, rows of an interior item)
     int nitems;
     int nshots;
     const BatchShot* shots;
@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(MTHREADS, 4) k_batch_step(BatchHead* __restric
         if (!run) continue;
         const BatchShot& sh = H->shots[w.x];
         bool ok;
-        if (w.y == 0) ok = march_tile<O, 3>(sh.maps, s_v, s_a, sh.rows, w.z, err, batch_smem);
+        if (w.y == 0) ok = march_tile<O, 3>(sh.maps, s_v, s_a, w.w, w.z, err, batch_smem);
         else ok = strip_tile_body<float, O, 0, MTHREADS>(&sh.view, sh.tiles[w.z], s_a, sh.beta, err, sh.ssrc, sh.spar,
                                                         batch_smem);
         __syncthreads();                                    // the next item reuses the shared memory
