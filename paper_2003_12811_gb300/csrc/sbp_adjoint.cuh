@@ -13,9 +13,44 @@
 // D_ii^FC(b) (closure triples and interior edge weights, Sec. 4.4), the mixed terms D_i c D_k
 // (Sec. 4.6), and the SAT terms of Sec. 5.1, 5.2 and 6, which involve c only at face nodes.
 #pragma once
+#include <utility>
+
 #include "sbp_kernels.cuh"
 
 namespace sbp {
+
+// the gradient tables as compile-time constants (k_grad_lines)
+namespace ctab {
+#define SBP_TABLE static constexpr
+#include "sbp_tables.inc"
+#undef SBP_TABLE
+}  // namespace ctab
+template <int O> struct GTab;
+#define SBP_GTAB(O)                                                                                    \
+    template <> struct GTab<O> {                                                                       \
+        static constexpr const int* start = ctab::sbp##O##_GN_START;                                   \
+        static constexpr const int* row = ctab::sbp##O##_GN_ROW;                                       \
+        static constexpr const int* j = ctab::sbp##O##_GN_J;                                           \
+        static constexpr const double* c = ctab::sbp##O##_GN_C;                                        \
+    };
+SBP_GTAB(2)
+SBP_GTAB(4)
+SBP_GTAB(6)
+#undef SBP_GTAB
+// rows and columns of a line that the gradient at its first GS nodes reads
+template <int O> constexpr int grad_line_width() {
+    int w = 0;
+    for (int t = 0; t < GTab<O>::start[Ord<O>::GS]; ++t) {
+        if (GTab<O>::row[t] + 1 > w) w = GTab<O>::row[t] + 1;
+        if (GTab<O>::j[t] + 1 > w) w = GTab<O>::j[t] + 1;
+    }
+    return w;
+}
+template <int O> constexpr bool grad_has(int k, int row) {
+    for (int t = GTab<O>::start[k]; t < GTab<O>::start[k + 1]; ++t)
+        if (GTab<O>::row[t] == row) return true;
+    return false;
+}
 
 struct GradDev {
     const void* seg;          // recomputed forward levels: level l (2 planes) at seg + l * lvl_elems
@@ -23,7 +58,7 @@ struct GradDev {
     long long lvl_elems;
     void* gc;                 // 10 accumulator planes (dPhi/dc, plane layout of BlockDev::c)
     void* grho;               // 1 accumulator plane (dPhi/drho)
-    void* gsat[4];            // per face: 7 x nf SAT contributions (planes 3m, 3m+1, 3m+2, 6..9)
+    void* gsat[4];            // per face and level chunk: 7 x nf SAT contributions (planes 3m, 3m+1, 3m+2, 6..9)
     void* part;               // strip nodes: per level chunk, 11 partial sums (10 c planes, rho)
 };
 
@@ -121,68 +156,41 @@ template <int O> struct GradCfg {
     static constexpr int EHI = O == 2 ? SBP2_EHI : (O == 4 ? SBP4_EHI : SBP6_EHI);
 };
 
-// Gradient of the narrow rows of one grid line with respect to b at line index x, contracted with
-// phi (per row) and u: s_JL = sum_rows phi_J(row) d(row of h^2 D_xx(b) u_L)/d b_x, with s01
-// collecting (J, L) = (0, 1) and (1, 0).  Nodes at least GS from both ends: the edge-pair form
-//   -sum_m sum_k e_{m,k} (phi(j+m) - phi(j)) (u(j+m) - u(j)),  j = x - k;
-// nodes near an end: the tabulated (row, u-column, coefficient) lists (mirrored at the high end).
-template <int O, typename T, class FP, class FU>
-__device__ __forceinline__ void narrow_grad_line(int N, int x, FP phi, FU u, T& s00, T& s01, T& s11) {
-    using P = Ord<O>;
-    s00 = s01 = s11 = T(0);
-    if (x >= P::GS && x < N - P::GS) {
-#pragma unroll
-        for (int m = 1; m <= P::Q; ++m) {
-#pragma unroll
-            for (int k = GradCfg<O>::ELO; k <= GradCfg<O>::EHI; ++k) {
-                const double e = edge_coef<O>(m, k);
-                if (e == 0.0) continue;
-                const T ee = T(e);
-                const int j = x - k;
-                const T dp0 = phi(0, j + m) - phi(0, j), dp1 = phi(1, j + m) - phi(1, j);
-                const T du0 = u(0, j + m) - u(0, j), du1 = u(1, j + m) - u(1, j);
-                s00 -= ee * dp0 * du0;
-                s01 -= ee * (dp0 * du1 + dp1 * du0);
-                s11 -= ee * dp1 * du1;
-            }
-        }
-        return;
-    }
-    const bool right = x >= N - P::GS;
-    const int kk = right ? N - 1 - x : x;
-    for (int t = P::gn_start(kk); t < P::gn_start(kk + 1); ++t) {
-        int r = P::gn_row(t), j = P::gn_j(t);
-        if (right) { r = N - 1 - r; j = N - 1 - j; }
-        const T c = P::template gn_c<T>(t);
-        const T p0 = phi(0, r), p1 = phi(1, r), u0 = u(0, j), u1 = u(1, j);
-        s00 += c * p0 * u0;
-        s01 += c * (p0 * u1 + p1 * u0);
-        s11 += c * p1 * u1;
+// Gradient of the narrow rows of a line end with respect to b at its first GS nodes:
+//   S[k] = sum over rows r of phi(r) dr/db_k u, the entries (r, j, c) of node k in the table grouped by row,
+//   s00 += p_0 V_0, s01 += p_0 V_1 + p_1 V_0, s11 += p_1 V_1 with V_J = sum_{j in row} c u_J(j).
+template <int O, int K, int ROW, typename T, int W, int... I>
+__device__ __forceinline__ void grad_term(const T (&p)[2][W], const T (&u)[2][W], T s[3], std::integer_sequence<int, I...>) {
+    if constexpr (grad_has<O>(K, ROW)) {
+        constexpr int T0 = GTab<O>::start[K];
+        T v0 = T(0), v1 = T(0);
+        (
+            [&] {
+                if constexpr (GTab<O>::row[T0 + I] == ROW) {
+                    constexpr int j = GTab<O>::j[T0 + I];
+                    const T c = T(GTab<O>::c[T0 + I]);
+                    v0 += c * u[0][j];
+                    v1 += c * u[1][j];
+                }
+            }(),
+            ...);
+        s[0] += p[0][ROW] * v0;
+        s[1] += p[0][ROW] * v1 + p[1][ROW] * v0;
+        s[2] += p[1][ROW] * v1;
     }
 }
-
-// (D^T phi)(x) * h on a line of N nodes: -D in the interior, tabulated columns near the ends
-// (the high end mirrors the low end with the sign of D flipped)
-template <int O, typename T, class FP>
-__device__ __forceinline__ T dt_line(int N, int x, FP phi) {
-    using P = Ord<O>;
-    T s = T(0);
-    if (x >= P::GS && x < N - P::GS) {
-#pragma unroll
-        for (int k = 1; k <= P::Q; ++k) s += P::template aT<T>(k - 1) * (phi(x - k) - phi(x + k));
-        return s;
-    }
-    const bool right = x >= N - P::GS;
-    const int kk = right ? N - 1 - x : x;
-    for (int t = P::dt_start(kk); t < P::dt_start(kk + 1); ++t) {
-        const int r = P::dt_row(t);
-        s += P::template dt_c<T>(t) * phi(right ? N - 1 - r : r);
-    }
-    return right ? -s : s;
+template <int O, int K, typename T, int W, int... R>
+__device__ __forceinline__ void grad_node(const T (&p)[2][W], const T (&u)[2][W], T s[3], std::integer_sequence<int, R...>) {
+    (grad_term<O, K, R, T, W>(p, u, s, std::make_integer_sequence<int, GTab<O>::start[K + 1] - GTab<O>::start[K]>()), ...);
+}
+template <int O, typename T, int W, int GS, int... K>
+__device__ __forceinline__ void grad_line(const T (&p)[2][W], const T (&u)[2][W], T (&s)[GS][3], std::integer_sequence<int, K...>) {
+    (grad_node<O, K, T, W>(p, u, s[K], std::make_integer_sequence<int, W>()), ...);
 }
 
 // ------------------------------------------------------------------ SAT part of the gradient
-// One thread per face node: the derivatives of (H psi)^T SAT(c, u) with respect to the c planes
+// One thread per face node and level chunk (blockIdx.y; a thread for all levels is a chain of hundreds of
+// loads on a chip that a few thousand face nodes cannot fill): the derivatives of (H psi)^T SAT(c, u) with respect to the c planes
 // at that node (the SATs involve c only at face nodes).  For face F with normal direction m,
 // tangential direction t, outward sign nu, w = u - v (interface) or u (displacement), and
 // H_t = h_t hw_t(s) (H = H_m H_t on the face, H_m[0] cancels against the SAT's 1/H_m[0]):
@@ -194,7 +202,7 @@ __device__ __forceinline__ T dt_line(int N, int x, FP phi) {
 //                    the interface average (weight -H_t (psi_J + psi^v_J) / 2)
 template <typename T, int O>
 __global__ void k_grad_face(const BlockDev* __restrict__ adj, const GradDev* __restrict__ gd,
-                            const FaceRef* __restrict__ refs, int nrefs, int total, int nl, double beta) {
+                            const FaceRef* __restrict__ refs, int nrefs, int total, int nl, int nchunk, double beta) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= total) return;
     const FaceRef fr = refs[find_face(refs, nrefs, t)];
@@ -202,8 +210,9 @@ __global__ void k_grad_face(const BlockDev* __restrict__ adj, const GradDev* __r
     const BlockDev& B = adj[fr.block];
     const FaceDev& F = B.f[fr.face];
     const GradDev& G = gd[fr.block];
-    T* out = reinterpret_cast<T*>(G.gsat[fr.face]);
-    const int nf = F.nf;
+    const int nf = F.nf, c = blockIdx.y;
+    const int l0 = (int)((long long)nl * c / nchunk), l1 = (int)((long long)nl * (c + 1) / nchunk);
+    T* out = reinterpret_cast<T*>(G.gsat[fr.face]) + (size_t)c * 7 * nf;
     T g[7];
 #pragma unroll
     for (int k = 0; k < 7; ++k) g[k] = T(0);
@@ -244,7 +253,7 @@ __global__ void k_grad_face(const BlockDev* __restrict__ adj, const GradDev* __r
         Uv = reinterpret_cast<const T*>(GV.seg) + GV.lvl_elems;
         lv = GV.lvl_elems;
     }
-    for (int l = 0; l < nl; ++l) {
+    for (int l = l0; l < l1; ++l) {
     const T* __restrict__ Ps = reinterpret_cast<const T*>(G.pseg) + (size_t)l * G.lvl_elems;
     const T* __restrict__ U = reinterpret_cast<const T*>(G.seg) + (size_t)(l + 1) * G.lvl_elems;
     const T ps0 = Ps[gi], ps1 = Ps[gi + plane];
@@ -387,26 +396,44 @@ __device__ __forceinline__ void grad_level(const BlockDev& B, const T* __restric
 #pragma unroll
             for (int b = 0; b < 2; ++b) acc[6 + 2 * a + b] += d1p[a] * d2u[b] + d2p[b] * d1u[a];
     } else {
-        const T hh = T(B.h1 * B.h2);
-        auto phi = [&](int L, int j1, int j2) {
-            return hh * hweightT<O, T>(n1, j1) * hweightT<O, T>(n2, j2) * ps(L, j1, j2);
+        // a direction in which the node is within GS of an end has its narrow rows from k_grad_lines; D^T phi
+        // with phi = H psi is (e_N e_N^T - e_0 e_0^T) psi - H D psi by the SBP property
+        const T hh = T(B.h1 * B.h2), hw1 = hweightT<O, T>(n1, i1), hw2 = hweightT<O, T>(n2, i2);
+        auto pairs = [&](int e1, int e2, T sc, T* out) {
+            T s00 = T(0), s01 = T(0), s11 = T(0);
+#pragma unroll
+            for (int m = 1; m <= PO::Q; ++m) {
+#pragma unroll
+                for (int k = GradCfg<O>::ELO; k <= GradCfg<O>::EHI; ++k) {
+                    const double e = edge_coef<O>(m, k);
+                    if (e == 0.0) continue;
+                    const T ee = T(e);
+                    const int a1 = i1 - k * e1, a2 = i2 - k * e2, b1 = a1 + m * e1, b2 = a2 + m * e2;
+                    const T dp0 = ps(0, b1, b2) - ps(0, a1, a2), dp1 = ps(1, b1, b2) - ps(1, a1, a2);
+                    const T du0 = uu(0, b1, b2) - uu(0, a1, a2), du1 = uu(1, b1, b2) - uu(1, a1, a2);
+                    s00 += ee * dp0 * du0;
+                    s01 += ee * (dp0 * du1 + dp1 * du0);
+                    s11 += ee * dp1 * du1;
+                }
+            }
+            out[0] -= sc * s00;
+            out[1] -= sc * s01;
+            out[2] -= sc * s11;
         };
-        T s00, s01, s11;
-        narrow_grad_line<O, T>(n1, i1, [&](int L, int j) { return phi(L, j, i2); }, [&](int L, int j) { return uu(L, j, i2); },
-                               s00, s01, s11);
-        acc[0] += s00 * ih1 * ih1;
-        acc[1] += s01 * ih1 * ih1;
-        acc[2] += s11 * ih1 * ih1;
-        narrow_grad_line<O, T>(n2, i2, [&](int L, int j) { return phi(L, i1, j); }, [&](int L, int j) { return uu(L, i1, j); },
-                               s00, s01, s11);
-        acc[3] += s00 * ih2 * ih2;
-        acc[4] += s01 * ih2 * ih2;
-        acc[5] += s11 * ih2 * ih2;
+        if (i1 >= PO::GS && i1 < n1 - PO::GS) pairs(1, 0, hh * hw2 * ih1 * ih1, acc);
+        if (i2 >= PO::GS && i2 < n2 - PO::GS) pairs(0, 1, hh * hw1 * ih2 * ih2, acc + 3);
         T d1p[2], d2p[2], d1u[2], d2u[2];
 #pragma unroll
         for (int L = 0; L < 2; ++L) {
-            d1p[L] = dt_line<O, T>(n1, i1, [&](int j) { return phi(L, j, i2); }) * ih1;
-            d2p[L] = dt_line<O, T>(n2, i2, [&](int j) { return phi(L, i1, j); }) * ih2;
+            const T pc = ps(L, i1, i2);
+            T t1 = -hw1 * dsum<O, T>(n1, i1, [&](int j) { return ps(L, j, i2); });
+            T t2 = -hw2 * dsum<O, T>(n2, i2, [&](int j) { return ps(L, i1, j); });
+            if (i1 == 0) t1 -= pc;
+            if (i1 == n1 - 1) t1 += pc;
+            if (i2 == 0) t2 -= pc;
+            if (i2 == n2 - 1) t2 += pc;
+            d1p[L] = hh * hw2 * ih1 * t1;
+            d2p[L] = hh * hw1 * ih2 * t2;
             d1u[L] = dsum<O, T>(n1, i1, [&](int j) { return uu(L, j, i2); }) * ih1;
             d2u[L] = dsum<O, T>(n2, i2, [&](int j) { return uu(L, i1, j); }) * ih2;
         }
@@ -446,7 +473,7 @@ __device__ __forceinline__ void grad_levels(const BlockDev& B, const GradDev& G,
 
 // adds the SAT sums at face nodes, then gc += dt^2 acc[0..9], grho -= H J acc[10]
 template <typename T, int O, bool INTERIOR>
-__device__ __forceinline__ void grad_finish(const BlockDev& B, const GradDev& G, double dt2, int i1, int i2, T* acc) {
+__device__ __forceinline__ void grad_finish(const BlockDev& B, const GradDev& G, double dt2, int i1, int i2, T* acc, int nfc = 0) {
     const int n1 = B.n1, n2 = B.n2;
     const size_t plane = (size_t)n2 * B.pitch, gi = (size_t)i2 * B.pitch + i1;
     if (!INTERIOR) {
@@ -460,11 +487,13 @@ __device__ __forceinline__ void grad_finish(const BlockDev& B, const GradDev& G,
             const int s = m == 0 ? i2 : i1;
             const T* gs = reinterpret_cast<const T*>(G.gsat[f]);
             const int nf = F.nf;
-            acc[3 * m] += gs[s];
-            acc[3 * m + 1] += gs[nf + s];
-            acc[3 * m + 2] += gs[2 * nf + s];
+            for (int c = 0; c < nfc; ++c, gs += 7 * (size_t)nf) {
+                acc[3 * m] += gs[s];
+                acc[3 * m + 1] += gs[nf + s];
+                acc[3 * m + 2] += gs[2 * nf + s];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) acc[6 + k] += gs[(3 + k) * nf + s];
+                for (int k = 0; k < 4; ++k) acc[6 + k] += gs[(3 + k) * nf + s];
+            }
         }
     }
     T* __restrict__ GC = reinterpret_cast<T*>(G.gc);
@@ -506,7 +535,66 @@ __device__ __forceinline__ void grad_strip_node(const BlockDev& B, long long t, 
     }
 }
 
-// strip nodes, phase 1: level chunk blockIdx.y of nchunk; partial sums to G.part
+// the inverse: the strip index of a node
+template <int O> __device__ __forceinline__ long long grad_strip_index(const BlockDev& B, int i1, int i2) {
+    constexpr int S = GradCfg<O>::GS;
+    const long long n1 = B.n1, n2 = B.n2, top = S * n1;
+    if (i2 < S) return i2 * n1 + i1;
+    if (i2 >= n2 - S) return top + (i2 - n2 + S) * n1 + i1;
+    return 2 * top + (i1 < S ? i1 : i1 - n1 + 2 * S) * (n2 - 2 * S) + (i2 - S);
+}
+
+// Narrow rows of the line ends, one thread per line and end (lines of x1 = 0, x1 = 1, x2 = 0, x2 = 1 after one
+// another) and level chunk blockIdx.y: the sums over the chunk's levels for the first GS nodes go to the planes 3 m
+// .. 3 m + 2 of G.part.  A thread reads the line's first columns of psi and u once per level (order 6: 60 loads)
+// and runs the 522 table entries of its 12 nodes as constants; a thread per node looped over the entries of its
+// own node, four loads and two norm weights each.  501^2, 64 levels, FP32:
+// k_grad_strip 1716 us without this kernel, 319 with it.
+template <typename T, int O>
+__global__ void __launch_bounds__(64) k_grad_lines(BlockDev B, GradDev G, int nl, int nchunk, long long nstrip) {
+    constexpr int GS = GradCfg<O>::GS, W = grad_line_width<O>();
+    const int n1 = B.n1, n2 = B.n2, P = B.pitch;
+    int t = blockIdx.x * 64 + threadIdx.x;
+    if (t >= 2 * (n1 + n2)) return;
+    const int m = t < 2 * n2 ? 0 : 1;
+    if (m == 1) t -= 2 * n2;
+    const int nt = m == 0 ? n2 : n1, nn = m == 0 ? n1 : n2, side = t / nt, s = t - side * nt;
+    const size_t plane = (size_t)n2 * P;
+    const long long st = (m == 0 ? 1 : P) * (side ? -1 : 1);
+    const size_t o = m == 0 ? (size_t)s * P + (side ? n1 - 1 : 0) : (size_t)(side ? n2 - 1 : 0) * P + s;
+    const int c = blockIdx.y;
+    const int l0 = (int)((long long)nl * c / nchunk), l1 = (int)((long long)nl * (c + 1) / nchunk);
+    T acc[GS][3];
+#pragma unroll
+    for (int k = 0; k < GS; ++k) acc[k][0] = acc[k][1] = acc[k][2] = T(0);
+    for (int l = l0; l < l1; ++l) {
+        const T* __restrict__ Ps = reinterpret_cast<const T*>(G.pseg) + (size_t)l * G.lvl_elems + o;
+        const T* __restrict__ U = reinterpret_cast<const T*>(G.seg) + (size_t)(l + 1) * G.lvl_elems + o;
+        T p[2][W], u[2][W];
+#pragma unroll
+        for (int L = 0; L < 2; ++L)
+#pragma unroll
+            for (int d = 0; d < W; ++d) {
+                p[L][d] = __ldg(Ps + L * plane + d * st);
+                if (d < Ord<O>::NB) p[L][d] *= Ord<O>::template hwT<T>(d);
+                u[L][d] = __ldg(U + L * plane + d * st);
+            }
+        grad_line<O, T, W, GS>(p, u, acc, std::make_integer_sequence<int, GS>());
+    }
+    const T ih = m == 0 ? ih1T<T>(B) : ih2T<T>(B);
+    const T sc = T(B.h1 * B.h2) * hweightT<O, T>(nt, s) * ih * ih;
+    T* part = reinterpret_cast<T*>(G.part) + ((size_t)c * 11 + 3 * m) * nstrip;
+#pragma unroll
+    for (int k = 0; k < GS; ++k) {
+        const int d = side ? nn - 1 - k : k;
+        const long long idx = m == 0 ? grad_strip_index<O>(B, d, s) : grad_strip_index<O>(B, s, d);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) part[q * nstrip + idx] = sc * acc[k][q];
+    }
+}
+
+// strip nodes, phase 1: level chunk blockIdx.y of nchunk; partial sums to G.part (the planes of a direction
+// in which the node is within GS of an end come from k_grad_lines)
 template <typename T, int O>
 __global__ void __launch_bounds__(256, 2) k_grad_strip(BlockDev B, GradDev G, int nl, int nchunk, long long nstrip) {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -520,13 +608,16 @@ __global__ void __launch_bounds__(256, 2) k_grad_strip(BlockDev B, GradDev G, in
     for (int p = 0; p < 11; ++p) acc[p] = T(0);
     grad_levels<T, O, false>(B, G, l0, l1, i1, i2, acc);
     T* part = reinterpret_cast<T*>(G.part) + (size_t)c * 11 * nstrip;
+    constexpr int GS = GradCfg<O>::GS;
+    const bool in1 = i1 >= GS && i1 < B.n1 - GS, in2 = i2 >= GS && i2 < B.n2 - GS;
 #pragma unroll
-    for (int p = 0; p < 11; ++p) part[(size_t)p * nstrip + t] = acc[p];
+    for (int p = 0; p < 11; ++p)
+        if (p >= 6 || (p < 3 ? in1 : in2)) part[(size_t)p * nstrip + t] = acc[p];
 }
 
 // strip nodes, phase 2: the chunks in order, the SAT sums, and the accumulator update
 template <typename T, int O>
-__global__ void __launch_bounds__(256) k_grad_strip_sum(BlockDev B, GradDev G, int nchunk, long long nstrip, double dt2) {
+__global__ void __launch_bounds__(256) k_grad_strip_sum(BlockDev B, GradDev G, int nchunk, int nfc, long long nstrip, double dt2) {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nstrip) return;
     int i1, i2;
@@ -538,7 +629,7 @@ __global__ void __launch_bounds__(256) k_grad_strip_sum(BlockDev B, GradDev G, i
     for (int c = 0; c < nchunk; ++c)
 #pragma unroll
         for (int p = 0; p < 11; ++p) acc[p] += part[((size_t)c * 11 + p) * nstrip + t];
-    grad_finish<T, O, false>(B, G, dt2, i1, i2, acc);
+    grad_finish<T, O, false>(B, G, dt2, i1, i2, acc, nfc);
 }
 
 // dPhi/dC (pair layout, 10 planes of the upper triangle of M[2I+J][2K+L]) and dPhi/drho as dense

@@ -206,13 +206,13 @@ struct sbp_handle {
         stage_bytes = stage ? bytes + bytes / 4 : 0;
         return stage;
     }
-    void* dalloc(size_t bytes) {
+    void* dalloc(size_t bytes, bool clear = true) {
         void* p = nullptr;
         if (cudaMalloc(&p, bytes) != cudaSuccess && (!drop_edges(this) || cudaMalloc(&p, bytes) != cudaSuccess)) {
             cudaGetLastError();   // reported as SBP_E_OOM by the caller; the next launch check starts clean
             return nullptr;
         }
-        cudaMemset(p, 0, bytes);
+        if (clear) cudaMemset(p, 0, bytes);
         allocs.push_back(p);
         return p;
     }
@@ -1219,10 +1219,10 @@ int grad_strip_chunks(const sbp_handle* h, long long nstrip, int nl) {
 template <typename T, int O>
 void launch_grad(sbp_handle* h, const GradDev* d_grad, const std::vector<GradDev>& grads, int nl, double dt2,
                  cudaStream_t st) {
-    const int total = h->nface_nodes;
+    const int total = h->nface_nodes, nfc = std::min(GRAD_MAX_CHUNKS, nl);
     if (total > 0) {
         ProfScope ps(h, 6, st, 1);
-        k_grad_face<T, O><<<grid_for(total, 128), 128, 0, st>>>(h->d_blocks_adj, d_grad, h->d_refs, h->nrefs, total, nl, h->beta);
+        k_grad_face<T, O><<<dim3(grid_for(total, 64), nfc), 64, 0, st>>>(h->d_blocks_adj, d_grad, h->d_refs, h->nrefs, total, nl, nfc, h->beta);
     }
     constexpr int GS = GradCfg<O>::GS;
     for (size_t b = 0; b < h->blocks.size(); ++b) {
@@ -1234,11 +1234,12 @@ void launch_grad(sbp_handle* h, const GradDev* d_grad, const std::vector<GradDev
             k_grad_interior<T, O><<<gi, dim3(32, 8), 0, st>>>(v, grads[b], nl, dt2);
         }
         {
-            ProfScope ps(h, 5, st, 2);
+            ProfScope ps(h, 5, st, 3);
             const long long nstrip = grad_strip_nodes(hb, GS);
             const int nchunk = grad_strip_chunks(h, nstrip, nl);
+            k_grad_lines<T, O><<<dim3(grid_for(2LL * (hb.n1 + hb.n2), 64), nchunk), 64, 0, st>>>(v, grads[b], nl, nchunk, nstrip);
             k_grad_strip<T, O><<<dim3(grid_for(nstrip), nchunk), 256, 0, st>>>(v, grads[b], nl, nchunk, nstrip);
-            k_grad_strip_sum<T, O><<<grid_for(nstrip), 256, 0, st>>>(v, grads[b], nchunk, nstrip, dt2);
+            k_grad_strip_sum<T, O><<<grid_for(nstrip), 256, 0, st>>>(v, grads[b], nchunk, nfc, nstrip, dt2);
         }
     }
 }
@@ -1256,19 +1257,27 @@ void run_grad(sbp_handle* h, const GradDev* d_grad, const std::vector<GradDev>& 
     }
 }
 
-// temporaries of one sbp_misfit_gradient call, released on every exit path
+// temporaries of one sbp_misfit_gradient or sbp_record call: one allocation, cut up, released on every exit path
+// (allocations and frees of their own cost about 0.1 ms each and a clear of every level; nothing here is read
+// before it is written)
 struct GradScratch {
     sbp_handle* h;
-    std::vector<void*> ptrs;
+    void* base = nullptr;
+    size_t bytes = 0;
+    std::vector<std::pair<void**, size_t>> parts;
     explicit GradScratch(sbp_handle* hh) : h(hh) {}
-    void* get(size_t bytes) {
-        void* p = h->dalloc(bytes);
-        if (p) ptrs.push_back(p);
-        return p;
+    template <typename P> void want(P** p, size_t n) {
+        parts.push_back({reinterpret_cast<void**>(p), bytes});
+        bytes += (n + 255) / 256 * 256;
+    }
+    bool get() {
+        base = h->dalloc(bytes, false);
+        for (auto& q : parts) *q.first = base ? (unsigned char*)base + q.second : nullptr;
+        return base != nullptr;
     }
     ~GradScratch() {
         cudaDeviceSynchronize();
-        for (void* p : ptrs) h->dfree(p);
+        h->dfree(base);
     }
 };
 
@@ -2528,8 +2537,9 @@ int sbp_record(sbp_handle* h, int nsteps, double dt, double* traces) {
     if (h->recs.empty()) return h->fail(SBP_E_STATE, "set the receivers first");
     const size_t per = 2 * h->recs.size();
     GradScratch sc(h);
-    double* d_tr = (double*)sc.get(sizeof(double) * per * std::max(nsteps, 1));
-    if (!d_tr) return h->fail(SBP_E_OOM, "trace buffer");
+    double* d_tr = nullptr;
+    sc.want(&d_tr, sizeof(double) * per * std::max(nsteps, 1));
+    if (!sc.get()) return h->fail(SBP_E_OOM, "trace buffer");
     for (int n = 0; n < nsteps; ++n) {
         int rc = step_once(h, dt, 0);
         if (rc != SBP_OK) return rc;
@@ -2579,36 +2589,42 @@ int sbp_misfit_gradient(sbp_handle* h, int nsteps, double dt, const double* obse
     const int nb = (int)h->blocks.size();
     GradScratch sc(h);
     std::vector<void*> ck(nb), seg(nb), pseg(nb), fin(nb);
+    std::vector<double*> dC(nb), dR(nb);       // outputs: dPhi/dC (in the layout) and dPhi/drho as dense FP64 arrays
     std::vector<size_t> lvl_bytes(nb);
     // a checkpoint holds (u_{n-1}, u_n) and, for FP32, the leapfrog increment
     const int nck = h->precision == SBP_FP32 ? 3 : 2;
     std::vector<GradDev> grads(nb);
     for (int b = 0; b < nb; ++b) {
         HostBlock& hb = h->blocks[b];
-        const size_t plane = (size_t)hb.n2 * hb.pitch;
+        const size_t plane = (size_t)hb.n2 * hb.pitch, n = (size_t)hb.n1 * hb.n2;
         lvl_bytes[b] = 2 * plane * es;
-        ck[b] = sc.get((size_t)nseg * nck * lvl_bytes[b]);
-        seg[b] = sc.get((size_t)(K + 2) * lvl_bytes[b]);
-        pseg[b] = sc.get((size_t)K * lvl_bytes[b]);
-        fin[b] = sc.get(nck * lvl_bytes[b]);
+        sc.want(&ck[b], (size_t)nseg * nck * lvl_bytes[b]);
+        sc.want(&seg[b], (size_t)(K + 2) * lvl_bytes[b]);
+        sc.want(&pseg[b], (size_t)K * lvl_bytes[b]);
+        sc.want(&fin[b], nck * lvl_bytes[b]);
         GradDev& G = grads[b];
-        G.seg = seg[b];
-        G.pseg = pseg[b];
         G.lvl_elems = (long long)(2 * plane);
-        G.gc = sc.get(10 * plane * es);
-        G.grho = sc.get(plane * es);
-        for (int f = 0; f < 4; ++f) G.gsat[f] = sc.get(7 * (size_t)hb.f[f].nf * es);
-        G.part = sc.get((size_t)GRAD_MAX_CHUNKS * 11 * grad_strip_nodes(hb, order_gs(h->order)) * es);
-        if (!ck[b] || !seg[b] || !pseg[b] || !fin[b] || !G.part || !G.gc || !G.grho || !G.gsat[0] || !G.gsat[1] || !G.gsat[2] || !G.gsat[3])
-            return h->fail(SBP_E_OOM, "misfit-gradient workspace (checkpoints every " + std::to_string(K) + " steps)");
+        sc.want(&G.gc, 10 * plane * es);
+        sc.want(&G.grho, plane * es);
+        for (int f = 0; f < 4; ++f) sc.want(&G.gsat[f], GRAD_MAX_CHUNKS * 7 * (size_t)hb.f[f].nf * es);
+        sc.want(&G.part, (size_t)GRAD_MAX_CHUNKS * 11 * grad_strip_nodes(hb, order_gs(h->order)) * es);
+        sc.want(&dC[b], (size_t)ncp * n * sizeof(double));
+        sc.want(&dR[b], n * sizeof(double));
     }
-    GradDev* d_grad = (GradDev*)sc.get(sizeof(GradDev) * nb);
-    double* d_tr = (double*)sc.get(sizeof(double) * per * nsteps);
-    double* d_obs = (double*)sc.get(sizeof(double) * per * nsteps);
-    double* d_res = (double*)sc.get(sizeof(double) * per * nsteps);
-    double* d_part = (double*)sc.get(sizeof(double) * nsteps);
-    double* d_phi = (double*)sc.get(sizeof(double));
-    if (!d_grad || !d_tr || !d_obs || !d_res || !d_part || !d_phi) return h->fail(SBP_E_OOM, "misfit-gradient tables");
+    GradDev* d_grad = nullptr;
+    double *d_tr = nullptr, *d_obs = nullptr, *d_res = nullptr, *d_part = nullptr, *d_phi = nullptr;
+    sc.want(&d_grad, sizeof(GradDev) * nb);
+    sc.want(&d_tr, sizeof(double) * per * nsteps);
+    sc.want(&d_obs, sizeof(double) * per * nsteps);
+    sc.want(&d_res, sizeof(double) * per * nsteps);
+    sc.want(&d_part, sizeof(double) * nsteps);
+    sc.want(&d_phi, sizeof(double));
+    if (!sc.get())
+        return h->fail(SBP_E_OOM, "misfit-gradient workspace (checkpoints every " + std::to_string(K) + " steps)");
+    for (int b = 0; b < nb; ++b) {
+        grads[b].seg = seg[b];
+        grads[b].pseg = pseg[b];
+    }
     if (cudaMemcpy(d_grad, grads.data(), sizeof(GradDev) * nb, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(d_obs, observed, sizeof(double) * per * nsteps, cudaMemcpyHostToDevice) != cudaSuccess)
         return h->fail(SBP_E_CUDA, "misfit-gradient table upload failed");
@@ -2726,22 +2742,18 @@ int sbp_misfit_gradient(sbp_handle* h, int nsteps, double dt, const double* obse
     }
     rc = check_cuda(h, "misfit gradient");
     if (rc != SBP_OK) return rc;
-    // outputs: dPhi/dC (pair layout) and dPhi/drho as dense FP64 arrays
     for (int b = 0; b < nb; ++b) {
         HostBlock& hb = h->blocks[b];
         const size_t n = (size_t)hb.n1 * hb.n2;
-        double* dC = (double*)sc.get((size_t)ncp * n * sizeof(double));
-        double* dR = (double*)sc.get(n * sizeof(double));
-        if (!dC || !dR) return h->fail(SBP_E_OOM, "gradient download staging");
         const BlockDev v = make_view(h, hb);
         ProfScope ps(h, 7, st, 1);
         if (h->precision == SBP_FP64)
-            k_grad_to_C<double><<<grid_for((long long)n), 256, 0, st>>>(v, (const double*)grads[b].gc, (const double*)grads[b].grho, dC, dR, ncp == 6);
+            k_grad_to_C<double><<<grid_for((long long)n), 256, 0, st>>>(v, (const double*)grads[b].gc, (const double*)grads[b].grho, dC[b], dR[b], ncp == 6);
         else
-            k_grad_to_C<float><<<grid_for((long long)n), 256, 0, st>>>(v, (const float*)grads[b].gc, (const float*)grads[b].grho, dC, dR, ncp == 6);
-        if (grad_C && grad_C[b] && cudaMemcpy(grad_C[b], dC, (size_t)ncp * n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess)
+            k_grad_to_C<float><<<grid_for((long long)n), 256, 0, st>>>(v, (const float*)grads[b].gc, (const float*)grads[b].grho, dC[b], dR[b], ncp == 6);
+        if (grad_C && grad_C[b] && cudaMemcpy(grad_C[b], dC[b], (size_t)ncp * n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess)
             return h->fail(SBP_E_CUDA, "gradient download");
-        if (grad_rho && grad_rho[b] && cudaMemcpy(grad_rho[b], dR, n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess)
+        if (grad_rho && grad_rho[b] && cudaMemcpy(grad_rho[b], dR[b], n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess)
             return h->fail(SBP_E_CUDA, "gradient download");
     }
     // leave the state where the forward pass ended
