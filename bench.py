@@ -40,7 +40,7 @@ BYTES_PER_NODE = {"fp32": 76, "fp64": 136}
 # DRAM bytes per node of one FP32 interior launch (dram__bytes_read.sum + dram__bytes_write.sum of
 # k_interior_march_multi<6,3> captured at 2 x 1601x801, scaled by nodes).  Set to None whenever that
 # kernel changes until it is measured again.
-TRAFFIC_BYTES_PER_NODE = {"fp32": 71.75, "fp64": None}
+TRAFFIC_BYTES_PER_NODE = {"fp32": None, "fp64": None}
 FALLBACK_HBM_GBS = 6800.0
 N1, N2 = 4001, 2001
 # crop of the workload the oracle is timed on: a 401-column window around the source spanning
@@ -362,19 +362,18 @@ def adjoint_bench(n=1001, nsteps=2000, prec="fp32"):
                          "frac": achieved / peak, "peak_source": src, "traffic": None}}
 
 
-# algorithmic bytes per node: an RK4 stage reads U_s (2), c (10), 1/(rho J) (1), u, v, V, S_u, S_v
-# (10) and writes U_{s+1}, V, S_u, S_v (8): 31 words; four stages per step
-RK4_WORDS_PER_STAGE = 31
-# the wide operator's two passes move: fluxes u (2) + c (10) -> G (4); divergence G (4), 1/(rho J) (1),
-# u^n (2), u^{n-1} (2) -> u^{n+1} (2): 27 words (FP32 increment form: d^n (2) in place of u^{n-1},
-# d^{n+1} (2) written as well: 29), against the 17 (19) of a fused step
-WIDE_WORDS_IMPLEMENTED = {"fp32": 29, "fp64": 27}
+# algorithmic words per node of the four RK4 stages (rk4_store): U_s (2), c (10), 1/(rho J) (1) each, and of the
+# combination v | u, v, a_1 | u, v, a_2 | u, v, a_1, a_2, a_3 in, U_{s+1} and a_s (u_new twice and v_new last) out
+RK4_WORDS_PER_STAGE = (4 * 13 + 2 + 6 + 6 + 10 + 3 * 4 + 6) / 4
+# the wide operator: FP32 in one march over the interior (the words of the narrow step); FP64 in two passes, fluxes
+# u (2) + c (10) -> G (4), divergence G (4), 1/(rho J) (1), u^n (2), u^{n-1} (2) -> u^{n+1} (2)
+WIDE_WORDS_IMPLEMENTED = {"fp32": 19, "fp64": 27}
 
 
-# FP64 operations of k_interior<double, 6, 0> per interior node (ncu thread-level counts
-# 2 x DFMA + DADD + DMUL over the 299,889 interior nodes of one 801 x 401 block) and the FP64 peak
+# FP64 operations of k_interior_edges<double, 6, 0, 32, 16> per interior node, counted from its source (narrow rows
+# 120, mixed fluxes with their halos 56, their divergence 36, update 9), and the FP64 peak
 # of the part: 152 SMs x 2 FP64 FMA per clock x 2 flops x 2.07 GHz
-FP64_FLOPS_PER_NODE = 431.6
+FP64_FLOPS_PER_NODE = 221.0
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 
 
@@ -409,7 +408,7 @@ def fp64_bench(P, nsteps=20):
     return {"node_updates_per_s": nodes / (ms / 1e3), "ms_per_step": ms, "interior_ms_per_step": k_ms,
             "hbm": {"bytes_per_node": BYTES_PER_NODE["fp64"], "achieved_GBs": BYTES_PER_NODE["fp64"] * inner / (k_ms / 1e3) / 1e9,
                     "frac": BYTES_PER_NODE["fp64"] * inner / (k_ms / 1e3) / 1e9 / peak, "peak_source": src},
-            "alu": {"bound": "alu", "kernel": "k_interior<double,6,0>", "flops_per_node": FP64_FLOPS_PER_NODE,
+            "alu": {"bound": "alu", "kernel": "k_interior_edges<double,6,0>", "flops_per_node": FP64_FLOPS_PER_NODE,
                     "achieved": tflops, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": tflops / FP64_PEAK_TFLOPS,
                     "peak_source": "derived: 152 SMs x 2 FP64 FMA per clock x 2 flops x 2.07 GHz"},
             "steps": nsteps}
@@ -417,9 +416,9 @@ def fp64_bench(P, nsteps=20):
 
 # 3-D operator: words per node each bulk kernel must move (FP32 words; FP64 doubles them)
 #   k3_flux: u (3) and the 27 mixed coefficients in, the 9 fluxes q out            = 39
-#   k3_div:  q (9), the 18 narrow coefficients, w, u (3), du (3) in; du, u^{n+1} out = 40
+#   divergence (k3_div with k3_lines): q (9), the 18 narrow coefficients, w, u (3), du (3) in; du, u^{n+1} out = 40
 #   one fused pass at the minimum: u, du, 45 coefficients, w in; du, u^{n+1} out     = 58
-OP3D_WORDS = {"k3_flux": 39, "k3_div": 40, "fused_min": 58}
+OP3D_WORDS = {"k3_flux": 39, "divergence": 40, "fused_min": 58}
 
 
 def bench3d(n=256, nsteps=40, prec="fp32"):
@@ -877,7 +876,7 @@ def main():
                          "frac": achieved / peak,
                          "traffic": (TRAFFIC_BYTES_PER_NODE[prec] * units_per_launch
                                      if TRAFFIC_BYTES_PER_NODE[prec] else None),
-                         "kernel": "k_interior_march_multi" if prec == "fp32" else "k_interior",
+                         "kernel": "k_interior_march_multi" if prec == "fp32" else "k_interior_edges",
                          "peak_source": peak_src,
                          "bytes_per_node": bpn, "units_per_launch": units_per_launch,
                          "kernel_ms_per_step": interior_ms,

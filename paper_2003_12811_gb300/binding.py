@@ -454,7 +454,7 @@ class Batch:
 
 # ----------------------------------------------------------------------------- 3-D operator (include/sbp3.h)
 BC3 = {"displacement": 0, "traction": 1}
-PROF3_FAMILIES = 3     # SBP3_PROF_FAMILIES: k3_flux, k3_div_int, k3_div_shell (with the face SATs)
+PROF3_FAMILIES = 3     # SBP3_PROF_FAMILIES: k3_flux, k3_div, k3_lines (line ends, with the face SATs)
 
 
 def footprint3_bytes(N, precision="fp32", order=6):
