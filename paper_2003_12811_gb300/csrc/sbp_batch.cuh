@@ -48,8 +48,8 @@ struct BatchHead {
 };
 
 template <int O> constexpr size_t batch_smem_bytes() {
-    return MarchCfg<O>::BYTES > StripTile<O>::template bytes<float>() ? MarchCfg<O>::BYTES
-                                                                        : StripTile<O>::template bytes<float>();
+    return MarchCfg<O>::BYTES > StripTile<O, 32, (O > 2)>::template bytes<float>() ? MarchCfg<O>::BYTES
+                                                                        : StripTile<O, 32, (O > 2)>::template bytes<float>();
 }
 
 template <int O>
@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(MTHREADS, 4) k_batch_step(BatchHead* __restric
         const BatchShot& sh = H->shots[w.x];
         bool ok;
         if (w.y == 0) ok = march_tile<O, 3>(sh.maps, s_v, s_a, w.w, w.z, err, batch_smem);
-        else ok = strip_tile_body<float, O, 0, MTHREADS>(&sh.view, sh.tiles[w.z], s_a, sh.beta, err, sh.ssrc, sh.spar,
+        else ok = strip_tile_body<float, O, 0, MTHREADS, 32, (O > 2)>(&sh.view, sh.tiles[w.z], s_a, sh.beta, err, sh.ssrc, sh.spar,
                                                         batch_smem);
         __syncthreads();                                    // the next item reuses the shared memory
         if (!ok) break;                                     // uniform: set by a CTA-wide vote
