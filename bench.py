@@ -481,7 +481,7 @@ def bench3d(n=256, nsteps=40, prec="fp32"):
             "node_updates_per_s": nodes / (ms / 1e3), "ms_per_step": ms, "kernels": kern,
             "step_vs_fused_minimum": {"bytes_per_node": OP3D_WORDS["fused_min"] * es, "achieved_GBs": fused,
                                       "frac": fused / peak},
-            "peak_GBs": peak, "peak_source": src, "launches_per_step": 6, "steps": nsteps, "state_finite": finite,
+            "peak_GBs": peak, "peak_source": src, "launches_per_step": 4, "steps": nsteps, "state_finite": finite,
             "tuning": {"variant": variant, "apply_ms_per_variant": variant_ms}}
 
 

@@ -54,8 +54,8 @@ const char* sbp3_last_error(const sbp3_handle* h);
 
 /* Device bytes a handle of this order, precision and size holds: 64 words per node (45 coefficients,
  * 1/(rho J), two levels, the increment, 9 fluxes), the FP64 coordinates and a reserve of
- * 2 x NCLOS x NCLOSJ x 6 words per x1 line, of which the face fields of the SATs take their part (an upper
- * bound; more only where 12 words per node of the faces are more). */
+ * 2 x NCLOS x NCLOSJ x 6 words per x1 line, of which the face fields of the SATs and the partial sums of
+ * the line ends take their part (an upper bound; more only where these need more: order 2, blocks long in x1). */
 int sbp3_footprint(int order, int precision, int n1, int n2, int n3, long long* bytes_out);
 
 /* Density and stiffness of the x3-planes i3_begin <= i3 < i3_begin + i3_count (any chunking).
@@ -78,7 +78,7 @@ int sbp3_get_state(sbp3_handle* h, double* u_prev, double* u_cur);
 int sbp3_apply(sbp3_handle* h, const double* u, double* accel);
 
 /* nsteps leapfrog steps of size dt on the given CUDA stream (NULL: the default stream); the call
- * returns once the launches are queued (six kernels per step).  SBP_E_STATE without a complete
+ * returns once the launches are queued (four kernels per step).  SBP_E_STATE without a complete
  * material or a state; SBP_E_INVALID_ARG for nsteps < 0 or dt <= 0.  The caller picks a stable dt
  * (no CFL estimate in 3-D). */
 int sbp3_step(sbp3_handle* h, int nsteps, double dt, void* stream);

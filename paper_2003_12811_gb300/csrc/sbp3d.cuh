@@ -1,8 +1,9 @@
 // libsbp 3-D operator kernels: one curvilinear block of n1 x n2 x n3 nodes (the d = 3 form of
 // Sec. 3.3, 4.3-4.7 and 5).  A leapfrog step is three kernel families:
 //   k3_flux  -- the mixed fluxes q_ij = sum_{k != i} c_ijkl D_k u_l (9 fields) from u^n;
-//   k3_lines -- per direction, the ends of every grid line: closure rows of D_ii^FC and D_i q_i, and the SATs of
-//               the two faces there, for the first rows from each face, as partial sums into the output field;
+//   k3_lines -- the ends of every grid line of the three directions: closure rows of D_ii^FC and D_i q_i, and the
+//               SATs of the two faces there (k3_face forms their fields along the face first), for the first rows
+//               from each face, as partial sums;
 //   k3_div   -- r_j = sum_i D_i q_ij + sum_i D_ii^FC(c_ijil) u_l with the interior rows of the other
 //               directions on top of the partial sums, then the leapfrog store (MODE 0: increment form,
 //               d = du + dt^2 w r, un = u + d; MODE 1: out = w r).
@@ -89,7 +90,7 @@ template <int O> constexpr bool clos_has_k(int row, int k) {
     return false;
 }
 
-// rr[ROW] += the terms of column K of the closure row ROW; bk: the column's six coefficients
+// rr[ROW - R0] += the terms of column K of the closure row ROW; bk: the column's six coefficients
 template <int O, int ROW, int K, typename T, int W, int... I>
 __device__ __forceinline__ void clos_term(const T (&uw)[3][W], const T bk[6], T rr[3], std::integer_sequence<int, I...>) {
     if constexpr (clos_has_k<O>(ROW, K)) {
@@ -111,18 +112,20 @@ __device__ __forceinline__ void clos_term(const T (&uw)[3][W], const T bk[6], T 
         rr[2] += bk[2] * V[0] + bk[4] * V[1] + bk[5] * V[2];
     }
 }
-template <int O, int K, typename T, int W, int NR, int... R>
+template <int O, int K, int R0, typename T, int W, int NR, int... R>
 __device__ __forceinline__ void clos_column(const T (&uw)[3][W], const T bk[6], T (&rr)[NR][3], std::integer_sequence<int, R...>) {
-    (clos_term<O, R, K, T, W>(uw, bk, rr[R], std::make_integer_sequence<int, CTab<O>::start[R + 1] - CTab<O>::start[R]>()), ...);
+    (clos_term<O, R0 + R, K, T, W>(uw, bk, rr[R], std::make_integer_sequence<int, CTab<O>::start[R0 + R + 1] - CTab<O>::start[R0 + R]>()), ...);
 }
-template <int O, typename T, int W, int NR, class FB, int... K>
+// the closure rows R0 .. R0 + NR - 1 (those of them that are closure rows)
+template <int O, int R0, typename T, int W, int NR, class FB, int... K>
 __device__ __forceinline__ void clos_rows(const T (&uw)[3][W], FB b, T (&rr)[NR][3], std::integer_sequence<int, K...>) {
+    constexpr int NC = CTab<O>::NCLOS - R0 < NR ? CTab<O>::NCLOS - R0 : NR;
     (
         [&] {
             T bk[6];
 #pragma unroll
             for (int s6 = 0; s6 < 6; ++s6) bk[s6] = b(s6, K);
-            clos_column<O, K, T, W, NR>(uw, bk, rr, std::make_integer_sequence<int, CTab<O>::NCLOS>());
+            clos_column<O, K, R0, T, W, NR>(uw, bk, rr, std::make_integer_sequence<int, (NC > 0 ? NC : 0)>());
         }(),
         ...);
 }
@@ -371,6 +374,7 @@ template <int O> __host__ __device__ constexpr int line_rows() {
 }
 struct Box3 {
     int x1lo, x1hi;
+    int rows;               // rows of the longer x1 end: max(x1lo, n1 - x1hi)
 };
 
 // x2 / x3 direction (stride S) for NV nodes: r[n][j] += ih D q_Dj + ih^2 D_xx(b) u, interior rows
@@ -469,14 +473,20 @@ __device__ __forceinline__ void div_int_strided_f2(const float* __restrict__ qD,
     float2 dp[3][Q], dm[3][Q];
 #pragma unroll
     for (int l = 0; l < 3; ++l) {
-        const float2 uc = ld2(up + l * fs);
+        const float *ul = up + l * fs, *pp = ul, *pm = ul;
+        const float2 uc = ld2(ul);
 #pragma unroll
         for (int m = 1; m <= Q; ++m) {
-            dp[l][m - 1] = p2fsub(ld2(up + l * fs + m * S), uc);
-            dm[l][m - 1] = p2fsub(ld2(up + l * fs - m * S), uc);
+            pp += S;
+            pm -= S;
+            dp[l][m - 1] = p2fsub(ld2(pp), uc);
+            dm[l][m - 1] = p2fsub(ld2(pm), uc);
         }
     }
     const float2 ih2 = p2s(ih * ih);
+    const float* ck[6];
+#pragma unroll
+    for (int s6 = 0; s6 < 6; ++s6) ck[s6] = cdD + s6 * fs - Q * S;
 #pragma unroll
     for (int k = -Q; k <= Q; ++k) {
         float2 L[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
@@ -491,7 +501,10 @@ __device__ __forceinline__ void div_int_strided_f2(const float* __restrict__ qD,
         }
         float2 bb[6];
 #pragma unroll
-        for (int s6 = 0; s6 < 6; ++s6) bb[s6] = ld2(cdD + s6 * fs + k * S);
+        for (int s6 = 0; s6 < 6; ++s6) {
+            bb[s6] = ld2(ck[s6]);
+            ck[s6] += S;
+        }
         const float2 t0 = p2ffma(bb[2], L[2], p2ffma(bb[1], L[1], p2fmul(bb[0], L[0])));
         const float2 t1 = p2ffma(bb[4], L[2], p2ffma(bb[3], L[1], p2fmul(bb[1], L[0])));
         const float2 t2 = p2ffma(bb[5], L[2], p2ffma(bb[4], L[1], p2fmul(bb[2], L[0])));
@@ -642,75 +655,71 @@ __device__ __noinline__ void int_row(const Grid3& g, const T* __restrict__ qo, c
     }
 }
 
-// The ends of the grid lines of direction D, one thread per line and end: the partial sums
+// The ends of the grid lines of direction D: the partial sums
 //   r_j = D_D q_Dj + D_DD^FC(c_DjDl) u_l + the SATs of the face there
-// of the first rows from the face (line_rows<O>(); along x1 up to x1lo, or from x1hi) are stored in `part`
-// (added where a line kernel of a later direction, D = 2, 1, 0 in this order, has stored its own), which k3_div
-// completes.  A closure row reads NCLOSJ columns of the line, the same ones for every row of the end: a
-// thread reads the 12 columns of u, q and the 6 coefficients once (order 6: 144 loads) for all 9 rows,
+// of the first rows from the face (line_rows<O>(); along x1 up to x1lo, or from x1hi), which k3_div completes.
+// Nodes near several faces get a sum from each direction, so every direction stores where no other does (x3: in
+// the output field; x2, x1: in planes of their own, LineParts) and one launch takes all three.
+// A closure row reads NCLOSJ columns of the line, the same ones for every row of the end: a
+// thread reads the columns of u, q and the 6 coefficients once (order 6: 144 loads) for all its rows,
 // where a thread per node read them for each row.  The lanes of a warp lie along x1 (D = 1, 2: coalesced)
 // or x2 (D = 0), where a column is one word per line: the CTA copies its lines' ends to shared memory row by row
-// and writes the sums back the same way.  160 x 151 x 144, FP32, order 6: with the columns and the face terms of D = 0
-// from global memory a step took 0.465 ms, now 0.420.
-// FP64 has small CTAs, as every line holds its SM's FP64 units for long: few lines still reach every SM.
-template <typename T> constexpr int kLineThreads = sizeof(T) == 4 ? 64 : 32;
+// and writes the sums back the same way.
+// A line end is taken by three warps of a CTA, a third of the rows each (orders 4 and 6): the rows are straight-line code
+// that a thread runs once (order 6: 2070 FP64 instructions; order 4: 780), and small blocks have few lines (40^3: 100 warps
+// of line ends per direction for 152 SMs).  With a thread for all rows of an end, in a launch per direction one after the
+// other, nothing hid the latencies of loads and instruction fetches: FP64 steps were slower than with a thread per node
+// (a step of 40^3, order 6: 321 us with a thread per node, 436 with a thread per end, now 199; order 4: 184, 258, 147; the
+// three launches of 64 x 61 x 57, order 4: 143 us, now 64).  FP32, 160 x 151 x 144, order 6: 91 us, now 76.
+constexpr int kLines = 32;                                    // line ends of a CTA
+template <int O> constexpr int kLineGroups = O == 2 ? 1 : 3;      // groups of rows
+template <int O> constexpr int kLineThreads = kLines * kLineGroups<O>;
+// rows formed here: along x1 one more than the closure for node pairs (the alignment of x1lo)
+template <typename T, int O, int D> constexpr int kLineRows = line_rows<O>() + (D == 0 && sizeof(T) == 4 ? 1 : 0);
+template <typename T, int O, int D> constexpr int line_window() {      // columns that the rows read
+    constexpr int RX = kLineRows<T, O, D> + Ord<O>::Q, NJ = CTab<O>::NJ, NC = Ord<O>::NCOL;
+    return NJ > RX ? (NJ > NC ? NJ : NC) : (RX > NC ? RX : NC);
+}
+template <typename T, int O> constexpr int line_smem() { return 12 * line_window<T, O, 0>() * (kLines + 1); }
 
-template <typename T, int O, int D>
-__global__ void __launch_bounds__(kLineThreads<T>) k3_lines(Grid3 g, Box3 bx, Faces3 fc, const T* __restrict__ u,
-                                                            const T* __restrict__ q, const T* __restrict__ cd,
-                                                            const T* __restrict__ ff, T* __restrict__ part) {
+// partial sums of the line ends of x2 and x1 (see Box3 for x1's rows)
+template <typename T> struct LineParts {
+    T *x2, *x1;
+};
+// element of the sum j at the node e-th row from the nearer face x2 (the rows of the high face after those of the low one)
+template <int O> __device__ __forceinline__ long long part_x2(const Grid3& g, int e, int j, int i1, int i3) {
+    return ((long long)(e * 3 + j) * g.n[2] + i3) * g.s[1] + i1;
+}
+// ... r-th row from the face x1 at `side`; line: i3 n2 + i2
+__device__ __forceinline__ long long part_x1(const Grid3& g, const Box3& bx, int side, int j, long long line, int r) {
+    return ((long long)(side * 3 + j) * g.n[1] * g.n[2] + line) * bx.rows + r;
+}
+
+// rows R0 .. of a line end, as many as rr holds or are left: u, q and the six coefficients through uat(l, c), qat(j, c),
+// b(s6, c)
+template <typename T, int O, int D, int R0, int NG, class FU, class FQ, class FB>
+__device__ __forceinline__ void line_end_rows(const Grid3& g, const Faces3& fc, int side, int tl, int ia, int ib, FU uat, FQ qat,
+                                              FB b, const T* __restrict__ ff, T (&rr)[NG][3]) {
     using P = Ord<O>;
-    constexpr int NT = kLineThreads<T>;
-    constexpr int NR = line_rows<O>(), NJ = CTab<O>::NJ;
-    constexpr int RX = D == 0 ? NR + 1 : NR;               // rows formed here: along x1 one more than the closure (see below)
-    constexpr int W = NJ > RX + P::Q ? NJ : RX + P::Q, QW = RX + P::Q > P::NCOL ? RX + P::Q : P::NCOL;
+    constexpr int LEFT = kLineRows<T, O, D> - R0, NR = NG < LEFT ? NG : LEFT;
+    constexpr int NJ = CTab<O>::NJ, W = line_window<T, O, D>();
     constexpr int A = D == 0 ? 1 : 0, B = D == 2 ? 1 : 2;
-    constexpr int WS = W > QW ? W : QW;
-    __shared__ T sm[D == 0 ? 12 * WS * (NT + 1) : 1];
     const int na = g.n[A], nb = g.n[B], N = g.n[D], lines = na * nb;
-    const int t = blockIdx.x * NT + threadIdx.x, tx = threadIdx.x, side = blockIdx.y;
-    const long long fs = g.fs;
-    const int S = dstride<D>(g), Ss = side ? -S : S;
-    auto face_node = [&](int line) {
-        const int b = line / na;
-        return (line - b * na) * g.s[A] + b * g.s[B] + (side ? (long long)(N - 1) * g.s[D] : 0);
-    };
-    if constexpr (D == 0) {
-        // column c of field f of line n at sm[(f * WS + c) * (NT + 1) + n]; fields u, q_1j, c_1j1l
-        for (int idx = tx; idx < NT * WS; idx += NT) {
-            const int n = idx / WS, c = idx - n * WS, line = blockIdx.x * NT + n;
-            if (line >= lines || c >= N) continue;
-            const long long oc = face_node(line) + c * Ss;
-#pragma unroll
-            for (int f = 0; f < 12; ++f) {
-                const T* p = f < 3 ? u + f * fs : (f < 6 ? q + (f - 3) * fs : cd + (f - 6) * fs);
-                sm[(f * WS + c) * (NT + 1) + n] = ldg(p + oc);
-            }
-        }
-        __syncthreads();
-    }
-    const bool live = t < lines;
-    const int tl = live ? t : lines - 1, ib = tl / na, ia = tl - ib * na;
-    const long long o = face_node(tl);
     const T ih = T(g.ih[D]), ih2 = ih * ih;
-    const T* cp = cd + 6 * D * fs + o;
-    auto b = [&](int s6, int c) -> T {
-        if constexpr (D == 0) return sm[((6 + s6) * WS + c) * (NT + 1) + tx];
-        else return ldg(cp + s6 * fs + c * Ss);
-    };
-    T uw[3][W], rr[RX][3];
+    T uw[3][W];
 #pragma unroll
     for (int l = 0; l < 3; ++l)
 #pragma unroll
-        for (int c = 0; c < W; ++c) uw[l][c] = D == 0 ? sm[(l * WS + c) * (NT + 1) + tx] : ldg(u + l * fs + o + c * Ss);
+        for (int c = 0; c < W; ++c) uw[l][c] = uat(l, c);
 #pragma unroll
-    for (int r = 0; r < RX; ++r) rr[r][0] = rr[r][1] = rr[r][2] = T(0);
-    clos_rows<O, T, W, RX>(uw, b, rr, std::make_integer_sequence<int, NJ>());
+    for (int r = 0; r < NG; ++r) rr[r][0] = rr[r][1] = rr[r][2] = T(0);
+    clos_rows<O, R0, T, W, NG>(uw, b, rr, std::make_integer_sequence<int, NJ>());
     // rows past the closure: order 2 has one that a SAT reaches; along x1 one more may be left here by the alignment of x1lo
 #pragma unroll
-    for (int r = P::NCLOS; r < RX; ++r) dxx3_interior<O, T>(r, [&](int l, int c) { return uw[l][c]; }, b, rr[r]);
+    for (int r = 0; r < NR; ++r)
+        if (R0 + r >= P::NCLOS) dxx3_interior<O, T>(R0 + r, [&](int l, int c) { return uw[l][c]; }, b, rr[r]);
 #pragma unroll
-    for (int r = 0; r < RX; ++r)
+    for (int r = 0; r < NR; ++r)
 #pragma unroll
         for (int j = 0; j < 3; ++j) rr[r][j] *= ih2;
     // D_D q_Dj: rows of D from the face, mirrored with the opposite sign at the high end
@@ -718,13 +727,12 @@ __global__ void __launch_bounds__(kLineThreads<T>) k3_lines(Grid3 g, Box3 bx, Fa
     T q0[3];
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-        T qw[QW];
+        T qw[W];
 #pragma unroll
-        for (int c = 0; c < QW; ++c)
-            qw[c] = D == 0 ? sm[((3 + j) * WS + c) * (NT + 1) + tx] : ldg(q + (3 * D + j) * fs + o + c * Ss);
+        for (int c = 0; c < W; ++c) qw[c] = qat(j, c);
         q0[j] = qw[0];
 #pragma unroll
-        for (int r = 0; r < RX; ++r) {
+        for (int r = R0; r < R0 + NR; ++r) {
             T d = T(0);
             if (r < P::NB) {
 #pragma unroll
@@ -733,10 +741,10 @@ __global__ void __launch_bounds__(kLineThreads<T>) k3_lines(Grid3 g, Box3 bx, Fa
 #pragma unroll
                 for (int k = 1; k <= P::Q; ++k) d += P::template aT<T>(k - 1) * (qw[r + k] - qw[r - k]);
             }
-            rr[r][j] += sg * d;
+            rr[r - R0][j] += sg * d;
         }
     }
-    {
+    if constexpr (R0 < P::NCOL) {
         // v_J -> c_DJDL v_L at the face node
         T b0[6];
 #pragma unroll
@@ -750,17 +758,19 @@ __global__ void __launch_bounds__(kLineThreads<T>) k3_lines(Grid3 g, Box3 bx, Fa
         const T nu = side ? T(1) : T(-1);
         T v[3], w[3];
         if (fc.kind[2 * D + side] == BC_TRACTION) {
-            // c_DJkL D_k u_L = q_DJ + c_DJDL D_D u_L at the face
+            if constexpr (R0 == 0) {
+                // c_DJkL D_k u_L = q_DJ + c_DJDL D_D u_L at the face
 #pragma unroll
-            for (int l = 0; l < 3; ++l) {
-                v[l] = T(0);
+                for (int l = 0; l < 3; ++l) {
+                    v[l] = T(0);
 #pragma unroll
-                for (int c = 0; c < P::NCOL; ++c) v[l] += P::template dqT<T>(0, c) * uw[l][c];
-                v[l] *= sg;
+                    for (int c = 0; c < P::NCOL; ++c) v[l] += P::template dqT<T>(0, c) * uw[l][c];
+                    v[l] *= sg;
+                }
+                cn(v, w);
+#pragma unroll
+                for (int j = 0; j < 3; ++j) rr[0][j] -= ihb * nu * (q0[j] + w[j]);
             }
-            cn(v, w);
-#pragma unroll
-            for (int j = 0; j < 3; ++j) rr[0][j] -= ihb * nu * (q0[j] + w[j]);
         } else {
             // s_J = c_DJDL u_L at the face node: spread by H^-1 D_D^T nu over NCOL rows, and the penalty
             // -H^-1 P_f (beta d / h1) s_J at the face (h1 = h hw_0)
@@ -769,65 +779,132 @@ __global__ void __launch_bounds__(kLineThreads<T>) k3_lines(Grid3 g, Box3 bx, Fa
             cn(v, w);
             const T pen = T(fc.beta * 3.0) * ihb * ihb;
 #pragma unroll
-            for (int r = 0; r < P::NCOL; ++r) {
+            for (int r = R0; r < R0 + NR && r < P::NCOL; ++r) {
                 T coef = -ih2 * P::template dqT<T>(0, r);
                 if (r < P::NB) coef /= P::template hwT<T>(r);
                 if (r == 0) coef -= pen;
 #pragma unroll
-                for (int j = 0; j < 3; ++j) rr[r][j] += coef * w[j];
+                for (int j = 0; j < 3; ++j) rr[r - R0][j] += coef * w[j];
             }
-            // tangential transposes of the face fields
-            const T* F = ff + fc.at[2 * D + side];
-            auto tang = [&](const T* Fk, int Nk, int a, int st, T ihk) {
+            if constexpr (R0 == 0) {
+                // tangential transposes of the face fields
+                const T* F = ff + fc.at[2 * D + side];
+                auto tang = [&](const T* Fk, int Nk, int a, int st, T ihk) {
 #pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    const T* p = Fk + (long long)j * lines + tl;
-                    T d = -dsum<O, T>(Nk, a, [&](int x) { return p[(long long)(x - a) * st]; });
-                    if (a == 0 || a == Nk - 1) d += (a == 0 ? -p[0] : p[0]) / P::template hwT<T>(0);
-                    rr[0][j] += ihb * nu * ihk * d;
-                }
-            };
-            tang(F, na, ia, 1, T(g.ih[A]));
-            tang(F + 3LL * lines, nb, ib, na, T(g.ih[B]));
+                    for (int j = 0; j < 3; ++j) {
+                        const T* p = Fk + (long long)j * lines + tl;
+                        T d = -dsum<O, T>(Nk, a, [&](int x) { return p[(long long)(x - a) * st]; });
+                        if (a == 0 || a == Nk - 1) d += (a == 0 ? -p[0] : p[0]) / P::template hwT<T>(0);
+                        rr[0][j] += ihb * nu * ihk * d;
+                    }
+                };
+                tang(F, na, ia, 1, T(g.ih[A]));
+                tang(F + 3LL * lines, nb, ib, na, T(g.ih[B]));
+            }
         }
     }
-    // nodes that the line kernels of the directions before this one have stored
-    auto end = [&](int i, int n) { return i < NR || i >= n - NR; };
-    auto put = [&](T* p, bool add, T v) { *p = add ? *p + v : v; };
+}
+
+// the line ends `blk` kLines .. of direction D at `side`
+template <typename T, int O, int D>
+__device__ __forceinline__ void line_ends(const Grid3& g, const Box3& bx, const Faces3& fc, int blk, int side,
+                                          const T* __restrict__ u, const T* __restrict__ q, const T* __restrict__ cd,
+                                          const T* __restrict__ ff, T* __restrict__ un, const LineParts<T>& parts, T* sm) {
+    constexpr int NL = kLines, G = kLineGroups<O>, NT = NL * G;
+    constexpr int RX = kLineRows<T, O, D>, WS = line_window<T, O, D>();
+    constexpr int A = D == 0 ? 1 : 0, B = D == 2 ? 1 : 2;
+    const int na = g.n[A], nb = g.n[B], N = g.n[D], lines = na * nb;
+    const int tx = threadIdx.x % NL, group = threadIdx.x / NL, t = blk * NL + tx;
+    const long long fs = g.fs;
+    const int S = dstride<D>(g), Ss = side ? -S : S;
+    auto face_node = [&](int line) {
+        const int b = line / na;
+        return (line - b * na) * g.s[A] + b * g.s[B] + (side ? (long long)(N - 1) * g.s[D] : 0);
+    };
     if constexpr (D == 0) {
-        const int rows = side ? N - bx.x1hi : bx.x1lo;      // NR, or one more; many more only on the smallest order-2 blocks
-        __syncthreads();
+        // column c of field f of line n at sm[(f * WS + c) * (NL + 1) + n]; fields u, q_1j, c_1j1l
+        for (int idx = threadIdx.x; idx < NL * WS; idx += NT) {
+            const int n = idx / WS, c = idx - n * WS, line = blk * NL + n;
+            if (line >= lines || c >= N) continue;
+            const long long oc = face_node(line) + c * Ss;
 #pragma unroll
-        for (int r = 0; r < RX; ++r)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) sm[(j * RX + r) * (NT + 1) + tx] = rr[r][j];
-        __syncthreads();
-        const int nr = rows < RX ? rows : RX;
-        for (int idx = tx; idx < NT * nr; idx += NT) {
-            const int n = idx / nr, r = idx - n * nr, line = blockIdx.x * NT + n;
-            if (line >= lines) continue;
-            const int l3 = line / na, l2 = line - l3 * na;
-            const bool add = end(l2, g.n[1]) || end(l3, g.n[2]);
-            T* p = part + face_node(line) + r * Ss;
-#pragma unroll
-            for (int j = 0; j < 3; ++j) put(p + j * fs, add, sm[(j * RX + r) * (NT + 1) + n]);
+            for (int f = 0; f < 12; ++f) {
+                const T* p = f < 3 ? u + f * fs : (f < 6 ? q + (f - 3) * fs : cd + (f - 6) * fs);
+                sm[(f * WS + c) * (NL + 1) + n] = ldg(p + oc);
+            }
         }
-        if (live) {
-            const bool add = end(ia, g.n[1]) || end(ib, g.n[2]);
-            for (int r = RX; r < rows; ++r) {
+        __syncthreads();
+    }
+    const bool live = t < lines;
+    const int tl = live ? t : lines - 1, ib = tl / na, ia = tl - ib * na;
+    const long long o = face_node(tl);
+    const T* cp = cd + 6 * D * fs + o;
+    auto uat = [&](int l, int c) -> T {
+        if constexpr (D == 0) return sm[(l * WS + c) * (NL + 1) + tx];
+        else return ldg(u + l * fs + o + c * Ss);
+    };
+    auto qat = [&](int j, int c) -> T {
+        if constexpr (D == 0) return sm[((3 + j) * WS + c) * (NL + 1) + tx];
+        else return ldg(q + (3 * D + j) * fs + o + c * Ss);
+    };
+    auto b = [&](int s6, int c) -> T {
+        if constexpr (D == 0) return sm[((6 + s6) * WS + c) * (NL + 1) + tx];
+        else return ldg(cp + s6 * fs + c * Ss);
+    };
+    constexpr int R3 = (RX + G - 1) / G;                     // rows of a group (fewer in the last)
+    T rr[R3][3];
+    if (G == 1 || group == 0) line_end_rows<T, O, D, 0>(g, fc, side, tl, ia, ib, uat, qat, b, ff, rr);
+    else if constexpr (G == 3) {
+        if (group == 1) line_end_rows<T, O, D, R3>(g, fc, side, tl, ia, ib, uat, qat, b, ff, rr);
+        else line_end_rows<T, O, D, 2 * R3>(g, fc, side, tl, ia, ib, uat, qat, b, ff, rr);
+    }
+    const int r0 = group * R3;
+    if constexpr (D == 0) __syncthreads();                   // every thread has read the staged columns
+#pragma unroll
+    for (int r = 0; r < R3; ++r)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            if (G * R3 > RX && r0 + r >= RX) continue;
+            if constexpr (D == 0) sm[(j * RX + r0 + r) * (NL + 1) + tx] = rr[r][j];
+            else if (live) {
+                if constexpr (D == 2) un[j * fs + o + (r0 + r) * Ss] = rr[r][j];
+                else parts.x2[part_x2<O>(g, side * line_rows<O>() + r0 + r, j, ia, ib)] = rr[r][j];
+            }
+        }
+    if constexpr (D == 0) {
+        const int rows1 = side ? N - bx.x1hi : bx.x1lo;     // at most RX; more only on the smallest order-2 blocks
+        __syncthreads();
+        const int nr = rows1 < RX ? rows1 : RX;
+        for (int idx = threadIdx.x; idx < NL * nr; idx += NT) {
+            const int n = idx / nr, r = idx - n * nr, line = blk * NL + n;
+            if (line >= lines) continue;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) parts.x1[part_x1(g, bx, side, j, line, r)] = sm[(j * RX + r) * (NL + 1) + n];
+        }
+        if (live && group == 0) {
+            for (int r = RX; r < rows1; ++r) {
                 T v[3] = {T(0), T(0), T(0)};
                 int_row<T, O, 0>(g, q + o + r * Ss, cp + r * Ss, u + o + r * Ss, v);
 #pragma unroll
-                for (int j = 0; j < 3; ++j) put(part + j * fs + o + r * Ss, add, v[j]);
+                for (int j = 0; j < 3; ++j) parts.x1[part_x1(g, bx, side, j, tl, r)] = v[j];
             }
         }
-    } else if (live) {
-        const bool add = D == 1 && end(ib, g.n[2]);
-#pragma unroll
-        for (int r = 0; r < RX; ++r)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) put(part + j * fs + o + r * Ss, add, rr[r][j]);
     }
+}
+
+// CTAs of the three directions
+struct LineGrid {
+    int c2, c1;             // CTAs of x3's lines, then of x2's; the rest take x1's
+};
+template <typename T, int O>
+__global__ void __launch_bounds__(kLineThreads<O>) k3_lines(Grid3 g, Box3 bx, Faces3 fc, LineGrid lg, const T* __restrict__ u,
+                                                               const T* __restrict__ q, const T* __restrict__ cd,
+                                                               const T* __restrict__ ff, T* __restrict__ un, LineParts<T> parts) {
+    __shared__ T sm[line_smem<T, O>()];
+    const int k = blockIdx.x, side = blockIdx.y;
+    if (k < lg.c2) line_ends<T, O, 2>(g, bx, fc, k, side, u, q, cd, ff, un, parts, sm);
+    else if (k < lg.c2 + lg.c1) line_ends<T, O, 1>(g, bx, fc, k - lg.c2, side, u, q, cd, ff, un, parts, sm);
+    else line_ends<T, O, 0>(g, bx, fc, k - lg.c2 - lg.c1, side, u, q, cd, ff, un, parts, sm);
 }
 
 // interior rows of direction D = x2 or x3 for the NV nodes of a thread
@@ -849,14 +926,15 @@ struct DivShape {
 constexpr DivShape kDivShapes[4] = {{4, 5}, {4, 6}, {8, 3}, {2, 10}};
 
 // Every node: the interior rows of the directions whose end rows k3_lines has not taken, on top of its partial
-// sums (in un) where it has, then the store.  NV consecutive x1 nodes per thread read as one vector
-// (float2 for FP32); the last pair of an odd row covers one element of the row's padding, which holds
-// zeros throughout and gets zeros back.  160 x 151 x 144, FP32, order 6: 171 us (the
+// sums where it has, then the store.  NV consecutive x1 nodes per thread read as one vector
+// (float2 for FP32); the last pair of an odd row covers one element of the row's padding, whose value no
+// node reads.  160 x 151 x 144, FP32, order 6: 191 us (the
 // kernel with closure rows and SATs behind calls: 328 us for the x1-interior columns).
 template <typename T, int O, int MODE, int NV, int BY, int MINB>
 __global__ void __launch_bounds__(32 * BY, MINB) k3_div(Grid3 g, Box3 bx, const T* __restrict__ u,
                                                         const T* __restrict__ q, const T* __restrict__ cd,
-                                                        const T* __restrict__ w, T* __restrict__ du, T* un, T dt2) {
+                                                        const T* __restrict__ w, T* __restrict__ du, T* un, LineParts<T> parts,
+                                                        T dt2) {
     constexpr int NR = line_rows<O>();
     const int i1 = (blockIdx.x * 32 + threadIdx.x) * NV, i2 = blockIdx.y * BY + threadIdx.y, i3 = blockIdx.z;
     if (i1 >= g.n[0] || i2 >= g.n[1]) return;
@@ -865,23 +943,33 @@ __global__ void __launch_bounds__(32 * BY, MINB) k3_div(Grid3 g, Box3 bx, const 
     const T* up = u + o;
     const bool in1 = i1 >= bx.x1lo && i1 < bx.x1hi, in2 = i2 >= NR && i2 < g.n[1] - NR, in3 = i3 >= NR && i3 < g.n[2] - NR;
     T r[NV][3];
-    if (in1 && in2 && in3) {
 #pragma unroll
-        for (int n = 0; n < NV; ++n) r[n][0] = r[n][1] = r[n][2] = T(0);
-    } else {
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
+    for (int n = 0; n < NV; ++n) r[n][0] = r[n][1] = r[n][2] = T(0);
+    if (!(in1 && in2 && in3)) {
+        auto add = [&](const T* p, int j) {
             T v[NV];
             if constexpr (NV == 2 && sizeof(T) == 4) {
-                const float2 x = *reinterpret_cast<const float2*>(un + j * fs + o);
+                const float2 x = *reinterpret_cast<const float2*>(p);
                 v[0] = x.x;
                 v[1] = x.y;
             } else {
 #pragma unroll
-                for (int n = 0; n < NV; ++n) v[n] = un[j * fs + o + n];
+                for (int n = 0; n < NV; ++n) v[n] = p[n];
             }
 #pragma unroll
-            for (int n = 0; n < NV; ++n) r[n][j] = v[n];
+            for (int n = 0; n < NV; ++n) r[n][j] += v[n];
+        };
+        const int e2 = i2 < NR ? i2 : NR + g.n[1] - 1 - i2, side = i1 >= bx.x1hi;
+        const long long line = (long long)i3 * g.n[1] + i2;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            if (!in3) add(un + j * fs + o, j);
+            if (!in2) add(parts.x2 + part_x2<O>(g, e2, j, i1, i3), j);
+            if (!in1) {
+#pragma unroll
+                for (int n = 0; n < NV; ++n)
+                    if (i1 + n < g.n[0]) r[n][j] += parts.x1[part_x1(g, bx, side, j, line, side ? g.n[0] - 1 - i1 - n : i1 + n)];
+            }
         }
     }
     if (in1) div_int_x1<T, O, NV>(q + o, cd + o, up, fs, T(g.ih[0]), r);

@@ -48,6 +48,8 @@ struct sbp3_handle {
     void* ff = nullptr;                      // tangential SAT fields of the displacement faces (k3_face)
     long long ff_elems = 0;
     int face_nodes = 0;                      // nodes of the largest displacement face
+    void* part = nullptr;                    // partial sums of the line ends of x2, then of x1 (k3_lines)
+    long long part_x2 = 0;                   // elements of the former
     void* ain = nullptr;                     // sbp3_apply input / output (3 fields each), on first use
     void* aout = nullptr;
     int cur = 0;
@@ -132,21 +134,16 @@ int launch_operator(sbp3_handle* h, const T* u, T* du, T* un, double dt, cudaStr
     prof_begin(h, 2, st, &stop);
     T* ff = static_cast<T*>(h->ff);
     if (h->face_nodes > 0) k3_face<T, O><<<dim3((h->face_nodes + 127) / 128, 6), 128, 0, st>>>(g, h->fc, u, cm, cd, ff);
-    auto lines = [&](auto dc) {
-        constexpr int D = decltype(dc)::value, A = D == 0 ? 1 : 0, B = D == 2 ? 1 : 2;
-        constexpr int NT = kLineThreads<T>;
-        const dim3 lg((unsigned)(((long long)g.n[A] * g.n[B] + NT - 1) / NT), 2);
-        k3_lines<T, O, D><<<lg, NT, 0, st>>>(g, bx, h->fc, u, q, cd, ff, un);
-    };
-    lines(std::integral_constant<int, 2>());
-    lines(std::integral_constant<int, 1>());
-    lines(std::integral_constant<int, 0>());
+    const LineParts<T> parts{static_cast<T*>(h->part), static_cast<T*>(h->part) + h->part_x2};
+    auto ctas = [&](int na, int nb) { return (int)(((long long)na * nb + kLines - 1) / kLines); };
+    const LineGrid lg{ctas(g.n[0], g.n[1]), ctas(g.n[0], g.n[2])};
+    k3_lines<T, O><<<dim3(lg.c2 + lg.c1 + ctas(g.n[1], g.n[2]), 2), kLineThreads<O>, 0, st>>>(g, bx, h->fc, lg, u, q, cd, ff, un, parts);
     prof_end(stop, st);
     auto run = [&](auto vc) {
         constexpr int V = decltype(vc)::value;
         constexpr int BY = kDivShapes[V].by, MINB = kDivShapes[V].minb;
         const dim3 ib(32, BY), ig((g.n[0] + 32 * NVF - 1) / (32 * NVF), (g.n[1] + BY - 1) / BY, g.n[2]);
-        k3_div<T, O, MODE, NVF, BY, MINB><<<ig, ib, 0, st>>>(g, bx, u, q, cd, w, du, un, dt2);
+        k3_div<T, O, MODE, NVF, BY, MINB><<<ig, ib, 0, st>>>(g, bx, u, q, cd, w, du, un, parts, dt2);
     };
     prof_begin(h, 1, st, &stop);
     // every shape is built for order 6; orders 2 and 4 keep the first
@@ -205,7 +202,7 @@ template <typename F> int dispatch(sbp3_handle* h, F f) {
 }
 
 void free_all(sbp3_handle* h) {
-    void* bufs[] = {h->X, h->cm, h->cd, h->w, h->u[0], h->u[1], h->du, h->q, h->ff, h->ain, h->aout, h->d_err};
+    void* bufs[] = {h->X, h->cm, h->cd, h->w, h->u[0], h->u[1], h->du, h->q, h->ff, h->part, h->ain, h->aout, h->d_err};
     for (void* b : bufs)
         if (b) cudaFree(b);
     for (auto& v : h->prof.ev)
@@ -218,8 +215,27 @@ long long face_words(int n1, int n2, int n3) {
     return 12 * ((long long)n2 * n3 + (long long)n1 * n3 + (long long)n1 * n2);
 }
 
+// words of the partial sums of the line ends of x2 and x1 (k3_lines), `rows` rows at either end of an x1 line
+long long part_x2_words(int order, long long pitch, int n3) {
+    const int nr = order == 2 ? line_rows<2>() : (order == 4 ? line_rows<4>() : line_rows<6>());
+    return 2LL * nr * 3 * n3 * pitch;
+}
+long long part_x1_words(int rows, int n2, int n3) { return 2LL * rows * 3 * n2 * n3; }
+
+// the x1 columns with interior rows for k3_div, whose x1 window reaches qa nodes out, in whole vectors
+Box3 x1_box(int order, int precision, int n1) {
+    const int nr = order == 2 ? line_rows<2>() : (order == 4 ? line_rows<4>() : line_rows<6>());
+    const int q = order / 2, nv = precision == SBP_FP32 ? 2 : 1;
+    const int qa = (q + nv - 1) / nv * nv, e = nr > qa ? nr : qa;
+    Box3 bx;
+    bx.x1lo = (e + nv - 1) / nv * nv;
+    bx.x1hi = n1 - e > bx.x1lo ? bx.x1lo + (n1 - e - bx.x1lo) / nv * nv : bx.x1lo;
+    bx.rows = bx.x1lo > n1 - bx.x1hi ? bx.x1lo : n1 - bx.x1hi;
+    return bx;
+}
+
 // bytes that sbp3_footprint counts beyond the fields, NCLOS x NCLOSJ x 6 words at either end of an x1 line:
-// a reserve that callers plan with, of which the face fields take their part
+// a reserve that callers plan with, of which the face fields and the partial sums of the line ends take their part
 size_t line_reserve_bytes(int order, size_t es, int n2, int n3) {
     const int nclos = order == 2 ? SBP2_NCLOS : (order == 4 ? SBP4_NCLOS : SBP6_NCLOS);
     const int nj = order == 2 ? SBP2_NCLOSJ : (order == 4 ? SBP4_NCLOSJ : SBP6_NCLOSJ);
@@ -250,8 +266,9 @@ int sbp3_footprint(int order, int precision, int n1, int n2, int n3, long long* 
     const long long x = pitch_of(n1, precision == SBP_FP32 ? 4 : 8) * n2 * n3 * 8LL;
     const size_t es = precision == SBP_FP32 ? 4 : 8;
     const long long reserve = (long long)line_reserve_bytes(order, es, n2, n3);
-    const long long faces = face_words(n1, n2, n3) * (long long)es;
-    *bytes_out = f * (NCM + NCD + 1 + 6 + 3 + 9) + 3 * x + (reserve > faces ? reserve : faces);
+    const long long ends = (face_words(n1, n2, n3) + part_x2_words(order, pitch_of(n1, es), n3) +
+                            part_x1_words(x1_box(order, precision, n1).rows, n2, n3)) * (long long)es;
+    *bytes_out = f * (NCM + NCD + 1 + 6 + 3 + 9) + 3 * x + (reserve > ends ? reserve : ends);
     return SBP_OK;
 }
 
@@ -302,17 +319,8 @@ int sbp3_create(int order, int precision, int n1, int n2, int n3, const double* 
     g.s[1] = h->pitch;
     g.s[2] = h->pitch * n2;
     g.fs = h->fs;
-    {
-        const int nclos = order == 2 ? SBP2_NCLOS : (order == 4 ? SBP4_NCLOS : SBP6_NCLOS);
-        const int q = order / 2, nv = precision == SBP_FP32 ? 2 : 1;
-        const int qa = (q + nv - 1) / nv * nv;            // the x1 window of k3_div reaches qa nodes out
-        const int ncol = order == 2 ? SBP2_NCOL : (order == 4 ? SBP4_NCOL : SBP6_NCOL);
-        const int ey = nclos > ncol ? nclos : ncol;
-        const int e = ey > qa ? ey : qa;
-        Box3& bx = h->box;
-        bx.x1lo = (e + nv - 1) / nv * nv;
-        bx.x1hi = n1 - e > bx.x1lo ? bx.x1lo + (n1 - e - bx.x1lo) / nv * nv : bx.x1lo;
-    }
+    h->box = x1_box(order, precision, n1);
+    h->part_x2 = part_x2_words(order, h->pitch, n3);
     for (int f = 0; f < 6; ++f) {
         h->fc.at[f] = h->ff_elems;
         if (face_kinds[f] != SBP3_BC_DISPLACEMENT) continue;
@@ -331,6 +339,7 @@ int sbp3_create(int order, int precision, int n1, int n2, int n3, const double* 
     bool ok = alloc((void**)&h->X, 3 * xfs * 8) && alloc(&h->cm, NCM * fb) && alloc(&h->cd, NCD * fb) &&
               alloc(&h->w, fb) && alloc(&h->u[0], 3 * fb) && alloc(&h->u[1], 3 * fb) && alloc(&h->du, 3 * fb) &&
               alloc(&h->q, 9 * fb) && (h->ff_elems == 0 || alloc(&h->ff, (size_t)h->ff_elems * h->es)) &&
+              alloc(&h->part, (size_t)(h->part_x2 + part_x1_words(h->box.rows, n2, n3)) * h->es) &&
               alloc((void**)&h->d_err, sizeof(int));
     if (!ok) {
         cudaGetLastError();
