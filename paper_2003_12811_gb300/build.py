@@ -6,13 +6,17 @@ import subprocess
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsbp.so")
-SOURCES = ["sbp_api.cu", "sbp3d_api.cu"]
-DEPS = ["sbp_api.cu", "sbp_kernels.cuh", "sbp_adjoint.cuh", "sbp_device.cuh", "sbp_interior_march.cuh",
-        "sbp_batch.cuh", "sbp_wide.cuh", "sbp_step.cuh", "sbp_tables.inc", "sbp3d_api.cu", "sbp3d.cuh"]
+# translation units, compiled side by side: (source, object, macros).  The 2-D kernels of each precision and order
+# are a unit of their own (sbp_ops.cu)
+UNITS = [("sbp_ops.cu", f"sbp_ops_{t}_{o}", [f"-DSBP_T={t}", f"-DSBP_O={o}"] + (["-DSBP_BATCH"] if t == "float" else []))
+         for o in (6, 4, 2) for t in ("float", "double")]
+UNITS += [("sbp3d_api.cu", "sbp3d_api", []), ("sbp_api.cu", "sbp_api", [])]
+DEPS = ["sbp_api.cu", "sbp_ops.cu", "sbp_host.cuh", "sbp_launch.cuh", "sbp_kernels.cuh", "sbp_adjoint.cuh", "sbp_device.cuh",
+        "sbp_interior_march.cuh", "sbp_batch.cuh", "sbp_wide.cuh", "sbp_step.cuh", "sbp_tables.inc", "sbp3d_api.cu",
+        "sbp3d.cuh"]
 HEADERS = ["sbp.h", "sbp3.h"]
 NVCC_FLAGS = ["-std=c++17", "-O3", "-gencode", "arch=compute_103a,code=sm_103a", "-lineinfo",
-              "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
-              "--split-compile", "0"]   # device code compiled in parallel on all host cores
+              "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 
 
 def nvcc_path():
@@ -38,11 +42,11 @@ def build(force=False, verbose=False):
     if nvcc is None:
         raise RuntimeError("nvcc not found: cannot build libsbp")
     tmp = LIB + ".tmp"
-    # one object per translation unit, compiled side by side, then one shared library
-    objs = [os.path.join(HERE, "_" + os.path.splitext(s)[0] + ".tmp.o") for s in SOURCES]
-    procs = [subprocess.Popen([nvcc] + NVCC_FLAGS + ["-c", "-o", o, os.path.join(CSRC, s)],
+    # one object per translation unit, then one shared library
+    objs = [os.path.join(HERE, f"_{name}.tmp.o") for _, name, _ in UNITS]
+    procs = [subprocess.Popen([nvcc] + NVCC_FLAGS + macros + ["-c", "-o", o, os.path.join(CSRC, src)],
                               stdout=subprocess.PIPE, stderr=subprocess.PIPE, text=True)
-             for s, o in zip(SOURCES, objs)]
+             for (src, _, macros), o in zip(UNITS, objs)]
     outs = [p.communicate() for p in procs]
     log = "".join(a + b for a, b in outs)
     try:

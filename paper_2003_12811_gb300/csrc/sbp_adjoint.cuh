@@ -83,7 +83,7 @@ __global__ void k_record(const BlockDev* __restrict__ blocks, const RecDev* __re
 }
 
 // res = traces - observed per step (one CTA per step) and the per-step sum of squares
-__global__ void k_residual(const double* __restrict__ tr, const double* __restrict__ obs, double* __restrict__ res,
+static __global__ void k_residual(const double* __restrict__ tr, const double* __restrict__ obs, double* __restrict__ res,
                            int per_step, double* __restrict__ partial) {
     const size_t base = (size_t)blockIdx.x * per_step;
     double acc = 0.0;
@@ -103,7 +103,7 @@ __global__ void k_residual(const double* __restrict__ tr, const double* __restri
 }
 
 // out = scale * sum(partial[0..n))   (one CTA of 256 threads, fixed summation order)
-__global__ void k_sum_scaled(const double* __restrict__ partial, int n, double scale, double* out) {
+static __global__ void k_sum_scaled(const double* __restrict__ partial, int n, double scale, double* out) {
     double acc = 0.0;
     for (int k = threadIdx.x; k < n; k += blockDim.x) acc += partial[k];
     __shared__ double red[256];

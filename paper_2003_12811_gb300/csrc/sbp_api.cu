@@ -1,333 +1,12 @@
 // libsbp host implementation: handle, validation, device memory, setup and the leapfrog step
 // loop.  The declarations and their documentation are in include/sbp.h.
-#include <cuda_runtime.h>
+#include "sbp_host.cuh"
 
-#include <algorithm>
-#include <cmath>
-#include <cstdio>
-#include <cstring>
-#include <string>
-#include <type_traits>
-#include <vector>
-
-#include <cuda.h>
-#include <cudaTypedefs.h>
-
-#include "../../include/sbp.h"
-#include "sbp_interior_march.cuh"
-#include "sbp_kernels.cuh"
-#include "sbp_adjoint.cuh"
-#include "sbp_batch.cuh"
-#include "sbp_wide.cuh"
-#include "sbp_step.cuh"
-
-namespace sbphost {
-#define SBP_TABLE static const
-#include "sbp_tables.inc"
-#undef SBP_TABLE
-}  // namespace sbphost
-
-using namespace sbp;
+using namespace sbphost;
 
 namespace {
 
 thread_local std::string g_create_error;
-
-struct HostFace {
-    int kind = -1, nbr_block = -1, nbr_face = -1, reversed = 0;
-    int nf = 0;
-    double* jhat = nullptr;
-    void* ju = nullptr;
-    void* g = nullptr;
-    void* sat = nullptr;      // wide stencil: SAT terms of the face nodes (k_face_sat); else unused (sbp_apply_noalloc
-                              // points its views at its own scratch)
-    void* tr = nullptr;       // interface faces: trace of this side (k_face_trace), 7 x nf
-    void* jv = nullptr;       // Robin faces with damping: J^ V (3 x nf, type T)
-};
-
-struct HostBlock {
-    int n1 = 0, n2 = 0, pitch = 0;
-    double h1 = 0, h2 = 0;
-    void* u[2] = {nullptr, nullptr};
-    void* du = nullptr;       // FP32: the leapfrog increment u^n - u^{n-1} (2 planes)
-    void* c = nullptr;
-    void* w = nullptr;
-    void* jf = nullptr;
-    void* r = nullptr;
-    double* X = nullptr;
-    double* G = nullptr;
-    double* J = nullptr;
-    bool material = false;
-    HostFace f[4];
-    MarchMaps mmaps;          // FP32 column-marching interior kernel tensor maps
-    void* psi[2] = {nullptr, nullptr};   // adjoint fields (sbp_misfit_gradient), allocated on first use
-    MarchMaps pmaps;          // marching-kernel maps over the adjoint fields
-    CUtensorMap* d_smaps = nullptr;   // strip-tile band-box maps on the device: [0..2] state u0, u1, c; [3..5] adjoint;
-                                      // [6..11] the same for short tiles
-    void* rk = nullptr;       // RK4 state (u, v, a_1, a_2, a_3; sbp_set_state_rk4), allocated on first use
-    void* gw = nullptr;       // wide stencil: the fluxes G_1j, G_2j (4 planes, type T)
-    void* sg = nullptr;       // layer dissipation coefficient s (1 plane, type T)
-    int2* d_lnodes = nullptr; // nodes the layer dissipation reaches, (i1, i2)
-    int nln = 0;
-    void* lscr = nullptr;     // leapfrog: the dissipation of the listed nodes between the pre and post kernels
-    void* mx = nullptr;       // closure matrices of D_xx^FC along x1 / x2 (k_closure_mats, type T)
-    void* my = nullptr;
-    void* e = nullptr;        // FP64 narrow stencil: interior edge weights (6 Q planes, k_edge_weights); given back
-                              // when a later allocation of the handle finds no room (drop_edges)
-};
-
-int order_nb(int o) { return o == 2 ? SBP2_NB : (o == 4 ? SBP4_NB : SBP6_NB); }
-int order_ncol(int o) { return o == 2 ? SBP2_NCOL : (o == 4 ? SBP4_NCOL : SBP6_NCOL); }
-int order_nclos(int o) { return o == 2 ? SBP2_NCLOS : (o == 4 ? SBP4_NCLOS : SBP6_NCLOS); }
-int order_nclosj(int o) { return o == 2 ? SBP2_NCLOSJ : (o == 4 ? SBP4_NCLOSJ : SBP6_NCLOSJ); }
-// elements of the closure matrices of one direction with `lines` lines (layout of dxx_closure_mat)
-size_t closure_elems(int o, int lines) { return 2 * (size_t)order_nclos(o) * order_nclosj(o) * 3 * lines; }
-int order_q(int o) { return o / 2; }
-int order_min_n(int o) { return o == 2 ? 5 : (o == 4 ? 18 : 27); }
-double order_hw(int o, int i) {
-    return o == 2 ? sbphost::sbp2_HW[i] : (o == 4 ? sbphost::sbp4_HW[i] : sbphost::sbp6_HW[i]);
-}
-double order_dq0(int o, int c) {
-    return o == 2 ? sbphost::sbp2_DQ[0][c] : (o == 4 ? sbphost::sbp4_DQ[0][c] : sbphost::sbp6_DQ[0][c]);
-}
-double host_hweight(int o, int N, int i) {
-    const int nb = order_nb(o);
-    if (i < nb) return order_hw(o, i);
-    if (i >= N - nb) return order_hw(o, N - 1 - i);
-    return 1.0;
-}
-
-}  // namespace
-
-struct sbp_handle;
-namespace {
-bool drop_edges(sbp_handle* h);
-}
-
-struct sbp_handle {
-    int order = 0, precision = 0, nblocks = 0;
-    int stencil = SBP_STENCIL_NARROW;
-    bool layers = false;          // some block has layer dissipation (sbp_set_layer_dissipation)
-    bool damping = false;         // some face has Robin damping or some block layers
-    double beta = 1.0;
-    size_t esize = 8;
-    std::vector<HostBlock> blocks;
-    BlockDev* d_blocks = nullptr;
-    FaceRef* d_refs = nullptr;
-    int nrefs = 0, nface_nodes = 0;
-    int ntrefs = 0;               // interface faces (their traces: k_face_trace)
-    int cur = 0;
-    double t = 0.0;
-    int nbasis = 0;
-    int basis_kind[8] = {0};
-    double basis_omega[8] = {0};
-    std::vector<SrcNode> src_nodes;
-    std::vector<SrcParam> src_params;
-    SrcNode* d_src_nodes = nullptr;     // every source node (sbp_apply_noalloc)
-    SrcNode* d_src_int = nullptr;       // source nodes off the boundary strips (k_sources)
-    int n_src_int = 0;
-    SrcNode* d_src_strip = nullptr;     // source nodes on the strips, grouped by strip tile (k_strip_tile)
-    SrcParam* d_src_params = nullptr;
-    bool src_dirty = false;
-    double* d_scalar = nullptr;
-    int* d_flag = nullptr;
-    int* d_err = nullptr;       // kernel error flags (bounded waits that ran out)
-    int num_sms = 0;
-    int device = 0;             // CUDA device current at sbp_grid_create (holds every buffer)
-    std::string err;
-    std::vector<void*> allocs;
-    // kernel timing (benchmarks): the families of sbp_profile in include/sbp.h
-    bool prof = false;
-    double prof_ms[SBP_PROF_FAMILIES] = {0};
-    long long launches[SBP_PROF_FAMILIES] = {0};
-    std::vector<cudaEvent_t> ev_pool;
-    struct Pending { int fam; cudaEvent_t a, b; };
-    std::vector<Pending> pending;
-    // CUDA-graph step loop (sbp_step_graph): graph of `graph_steps` steps of size `graph_dt`
-    cudaGraphExec_t graph_exec = nullptr;
-    int graph_steps = 0;
-    double graph_dt = 0.0;
-    double* d_time = nullptr;     // device copies of the step times of a graph launch
-    int d_time_cap = 0;
-    // marching-kernel rows per CTA chosen by sbp_autotune (0 = default heuristic)
-    int rows_per_cta = 0;
-    // optionally (sbp_autotune, sbp_set_tuning) the boundary strips run on a second stream
-    // concurrently with the interior kernel (they write disjoint nodes); both are forked from and
-    // joined back into the launch stream every step, the interior on a high-priority stream so
-    // that its CTAs are placed first
-    bool overlap = false;
-    cudaStream_t hi = nullptr;
-    cudaEvent_t ev_join_hi = nullptr;
-    // strip tiles of every block, costliest first (one k_strip_tile launch per step)
-    int4* d_tiles = nullptr;            // (block, tile, first, end source node of the tile) in launch order
-    int ntiles = 0;
-    int strip_len = 32;                 // nodes of a strip tile along the face (pick_strip_len)
-    std::vector<int4> tiles_host;
-    std::vector<std::vector<int>> tile_pos;   // [block][tile of the block] -> position in the launch order
-    // FP32 grids whose strips make few tiles: a second set, SHORT_TILE nodes long, for the one-launch step (the
-    // batch kernel and the others keep to 32)
-    struct StripSet {
-        int4* d_tiles = nullptr;
-        SrcNode* d_src = nullptr;
-        std::vector<int4> tiles;
-        std::vector<std::vector<int>> pos;
-    } shorts;
-    cudaStream_t aux = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    // adjoint: block views whose state buffers are the adjoint fields; receivers
-    BlockDev* d_blocks_adj = nullptr;
-    std::vector<RecDev> recs;
-    RecDev* d_recs = nullptr;
-
-    cudaEvent_t get_event() {
-        if (!ev_pool.empty()) {
-            cudaEvent_t e = ev_pool.back();
-            ev_pool.pop_back();
-            return e;
-        }
-        cudaEvent_t e;
-        cudaEventCreate(&e);
-        return e;
-    }
-
-    int fail(int code, const std::string& msg) {
-        err = msg;
-        return code;
-    }
-    // one grow-only device staging buffer for host uploads and downloads: setup and transfer calls
-    // use it instead of allocating and freeing temporaries (a free synchronises the whole device,
-    // which would stall work other streams run meanwhile, e.g. a batch of served shots)
-    void* stage = nullptr;
-    size_t stage_bytes = 0;
-    void* staging(size_t bytes) {
-        if (bytes <= stage_bytes) return stage;
-        if (stage) dfree(stage);
-        stage = dalloc(bytes + bytes / 4);
-        stage_bytes = stage ? bytes + bytes / 4 : 0;
-        return stage;
-    }
-    void* dalloc(size_t bytes, bool clear = true) {
-        void* p = nullptr;
-        if (cudaMalloc(&p, bytes) != cudaSuccess && (!drop_edges(this) || cudaMalloc(&p, bytes) != cudaSuccess)) {
-            cudaGetLastError();   // reported as SBP_E_OOM by the caller; the next launch check starts clean
-            return nullptr;
-        }
-        if (clear) cudaMemset(p, 0, bytes);
-        allocs.push_back(p);
-        return p;
-    }
-    void dfree(void* p) {
-        if (!p) return;
-        allocs.erase(std::remove(allocs.begin(), allocs.end(), p), allocs.end());
-        cudaFree(p);
-    }
-};
-
-namespace {
-
-// records CUDA events around one kernel family when profiling is on; counts launches always
-struct ProfScope {
-    sbp_handle* h;
-    int fam;
-    cudaStream_t st;
-    cudaEvent_t a = nullptr, b = nullptr;
-    ProfScope(sbp_handle* h_, int fam_, cudaStream_t st_, int nlaunch) : h(h_), fam(fam_), st(st_) {
-        h->launches[fam] += nlaunch;
-        if (h->prof) {
-            a = h->get_event();
-            b = h->get_event();
-            cudaEventRecord(a, st);
-        }
-    }
-    ~ProfScope() {
-        if (h->prof) {
-            cudaEventRecord(b, st);
-            h->pending.push_back({fam, a, b});
-        }
-    }
-};
-
-int check_cuda(sbp_handle* h, const char* where) {
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return h->fail(SBP_E_CUDA, std::string(where) + ": " + cudaGetErrorString(e));
-    return SBP_OK;
-}
-
-BlockDev make_view(const sbp_handle* h, const HostBlock& hb) {
-    BlockDev b{};
-    b.n1 = hb.n1;
-    b.n2 = hb.n2;
-    b.pitch = hb.pitch;
-    b.strip = std::max(order_nclos(h->order), order_ncol(h->order));
-    b.h1 = hb.h1;
-    b.h2 = hb.h2;
-    b.ih1 = 1.0 / hb.h1;
-    b.ih2 = 1.0 / hb.h2;
-    b.ih1f = (float)b.ih1;
-    b.ih2f = (float)b.ih2;
-    b.u[0] = hb.u[0];
-    b.u[1] = hb.u[1];
-    b.du = hb.du;
-    b.c = hb.c;
-    b.w = hb.w;
-    b.jf = hb.jf;
-    b.r = hb.r;
-    b.X = hb.X;
-    b.G = hb.G;
-    b.J = hb.J;
-    for (int f = 0; f < 4; ++f) {
-        const HostFace& F = hb.f[f];
-        FaceDev& D = b.f[f];
-        D.kind = F.kind;
-        D.m = f / 2;
-        D.side = f % 2;
-        D.nf = F.nf;
-        D.nbr_block = F.nbr_block;
-        D.nbr_face = F.nbr_face;
-        D.reversed = F.reversed;
-        D.nu = (f % 2 == 0) ? -1.0 : 1.0;
-        const int Nm = (f / 2 == 0) ? hb.n1 : hb.n2;
-        const double hm = (f / 2 == 0) ? hb.h1 : hb.h2;
-        D.hm0 = hm * host_hweight(h->order, Nm, 0);
-        D.inv_h0 = 1.0 / D.hm0;
-        // D_m[face row][i_m] / (h_m^2 hw(i_m)) at depth d: the boundary row of D (mirrored with the
-        // opposite sign at the high end) over the norm weight
-        for (int d = 0; d < 12; ++d) {
-            const double dq0 = d < order_ncol(h->order) ? order_dq0(h->order, d) : 0.0;
-            D.fac[d] = ((f % 2) ? -dq0 : dq0) / (hm * hm * host_hweight(h->order, Nm, (f % 2) ? Nm - 1 - d : d));
-            D.facf[d] = (float)D.fac[d];
-        }
-        D.jhat = F.jhat;
-        D.ju = F.ju;
-        D.g = F.g;
-        D.sat = F.sat;
-        D.tr = F.tr;
-        D.jv = F.jv;
-        if (F.jv) b.damped = 1;
-    }
-    b.smaps = hb.d_smaps;
-    b.rk = hb.rk;
-    b.sg = hb.sg;
-    b.mx = hb.mx;
-    b.my = hb.my;
-    b.e = hb.e;
-    for (int k = 0; k < order_q(h->order); ++k) {
-        const double ak = h->order == 2 ? sbphost::sbp2_A[k] : (h->order == 4 ? sbphost::sbp4_A[k] : sbphost::sbp6_A[k]);
-        b.ai1[k] = ak * b.ih1;
-        b.ai2[k] = ak * b.ih2;
-    }
-    return b;
-}
-
-// the same view with the adjoint fields as its state buffers
-BlockDev make_view_adj(const sbp_handle* h, const HostBlock& hb) {
-    BlockDev b = make_view(h, hb);
-    b.u[0] = hb.psi[0];
-    b.u[1] = hb.psi[1];
-    b.du = nullptr;             // the adjoint fields step from their two levels
-    b.smaps = hb.d_smaps ? hb.d_smaps + 3 : nullptr;
-    return b;
-}
 
 int sync_views(sbp_handle* h) {
     std::vector<BlockDev> v;
@@ -343,9 +22,11 @@ int sync_views(sbp_handle* h) {
     return SBP_OK;
 }
 
+}  // namespace
+
 // gives the edge weights of every block back to the device (an allocation of the handle found no room);
 // the interior then forms them in the kernel again.  False if there were none.
-bool drop_edges(sbp_handle* h) {
+bool sbphost::drop_edges(sbp_handle* h) {
     bool any = false;
     for (auto& hb : h->blocks) any = any || hb.e;
     if (!any) return false;
@@ -362,7 +43,7 @@ bool drop_edges(sbp_handle* h) {
     return !h->d_blocks || sync_views(h) == SBP_OK;
 }
 
-inline unsigned grid_for(long long n, int bs = 256) { return (unsigned)((n + bs - 1) / bs); }
+namespace {
 
 // the FP32 leapfrog increment of a block re-formed from its two levels (after the levels were
 // written by something other than a leapfrog step)
@@ -402,9 +83,6 @@ template <int O> void strip_box(int len, int& bw, int& bh) {
     bw = len == 32 ? StripTile<O, 32>::BWB : (len == 16 ? StripTile<O, 16>::BWB : StripTile<O, 8>::BWB);
     bh = StripTile<O>::BHB;
 }
-
-// length of the short strip tiles of FP32 grids (sbp_handle::shorts)
-constexpr int SHORT_TILE = 8;
 
 // Length of the strip tiles of an FP64 grid: the one whose busiest SM executes the fewest FP64
 // instructions, a tile of length L taking about 140 per output node, 26 and 16 per flux on its rows and
@@ -474,403 +152,6 @@ bool make_strip_maps(const sbp_handle* h, const HostBlock& hb, void* u0, void* u
            make_map(&dst[2], hb.c, hb.pitch, hb.n2, 10, bh, bw, es);
 }
 
-// interface traces of the level being read (k_face_trace), TRACE_MAX faces per launch, on stream tst
-template <typename T, int O>
-void launch_traces(sbp_handle* h, const StepArgs& a, cudaStream_t tst, bool adj) {
-    TraceArgs ta{};
-    auto flush = [&]() {
-        if (ta.nfaces == 0) return;
-        ProfScope ps(h, 2, tst, 1);
-        k_face_trace<T, O><<<grid_for(ta.total, 128), 128, 0, tst>>>(ta);
-        ta = TraceArgs{};
-    };
-    for (size_t b = 0; b < h->blocks.size(); ++b) {
-        const HostBlock& hb = h->blocks[b];
-        for (int f = 0; f < 4; ++f) {
-            const HostFace& HF = hb.f[f];
-            if (HF.kind != FACE_INTF) continue;
-            TraceFace& F = ta.f[ta.nfaces++];
-            F.u = adj ? hb.psi[a.cur] : hb.u[a.cur];
-            F.c = hb.c;
-            F.tr = HF.tr;
-            F.plane = (long long)hb.n2 * hb.pitch;
-            F.nf = HF.nf;
-            F.start = ta.total;
-            F.m = f / 2;
-            F.side = f % 2;
-            F.pitch = hb.pitch;
-            F.nm = F.m == 0 ? hb.n1 : hb.n2;
-            F.nu = (f % 2 == 0) ? -1.0 : 1.0;
-            const double hm = F.m == 0 ? hb.h1 : hb.h2, ht = F.m == 0 ? hb.h2 : hb.h1;
-            F.ihm = 1.0 / hm;
-            F.iht = 1.0 / ht;
-            F.k = h->beta * 2.0 / 4.0 * (1.0 / (hm * host_hweight(h->order, F.nm, 0)));
-            ta.total += HF.nf;
-            if (ta.nfaces == TRACE_MAX) flush();
-        }
-    }
-    flush();
-}
-
-// rows per CTA of a marching kernel on a block with ncx tiles across: one wave of about 4 CTAs per SM, at least
-// 16 rows (a tile streams 2q rows or more beyond its own), or the height that was tuned
-int march_rows(const sbp_handle* h, int ncx, int n2i) {
-    if (h->rows_per_cta > 0) return std::min(h->rows_per_cta, n2i);
-    const int ncy = std::max(1, (4 * h->num_sms + ncx / 2) / ncx);
-    return std::max((n2i + ncy - 1) / ncy, std::min(16, n2i));
-}
-
-// the wide-stencil operator (sbp_wide.cuh): traces, the SAT terms of every face node, the flux and
-// divergence passes of every block (in FP32 of its frame near the faces, beside one marching kernel over
-// the interior, which they share nothing with), then the point sources (every source node: the wide path has
-// no strip kernel)
-template <typename T, int O>
-int launch_wide(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st) {
-    constexpr bool march = std::is_same<T, float>::value;
-    const int S = std::max(order_nclos(h->order), order_ncol(h->order));
-    // the frame's chain of small kernels on the high-priority stream, queued before the interior
-    const bool par = march && h->hi && !h->prof;
-    cudaStream_t fst = par ? h->hi : st;
-    if (par) {
-        cudaEventRecord(h->ev_fork, st);
-        cudaStreamWaitEvent(h->hi, h->ev_fork, 0);
-    }
-    if (h->ntrefs > 0) launch_traces<T, O>(h, a, fst, false);
-    if (h->nface_nodes > 0) {
-        ProfScope ps(h, 1, fst, 1);
-        k_face_sat<T, O><<<grid_for(h->nface_nodes, 64), 64, 0, fst>>>(h->d_blocks, h->d_refs, h->nrefs, h->nface_nodes, a, h->beta);
-    }
-    if constexpr (march) {
-        MarchMulti mm{};
-        int tiles = 0;
-        auto flush = [&]() {
-            if (mm.nb == 0) return;
-            mm.start[mm.nb] = tiles;
-            ProfScope ps(h, 0, st, 1);
-            constexpr size_t msm = MarchCfg<O>::BYTES;
-            if (mode == 0) k_wide_march<O, 3><<<tiles, MTHREADS, msm, st>>>(mm, a, h->d_err);
-            else if (mode == 2) k_wide_march<O, 2><<<tiles, MTHREADS, msm, st>>>(mm, a, h->d_err);
-            else k_wide_march<O, 1><<<tiles, MTHREADS, msm, st>>>(mm, a, h->d_err);
-            mm = MarchMulti{};
-            tiles = 0;
-        };
-        for (auto& hb : h->blocks) {
-            const int ncx = wide_ncx(hb.n1, S), n2i = hb.n2 - 2 * S, rows = march_rows(h, ncx, n2i), k = mm.nb++;
-            mm.maps[k] = hb.mmaps;
-            mm.b[k] = make_view(h, hb);
-            mm.start[k] = tiles;
-            mm.rows[k] = rows;
-            tiles += ncx * ((n2i + rows - 1) / rows);
-            if (mm.nb == MARCH_MAX_BLOCKS) flush();
-        }
-        flush();
-    }
-    for (auto& hb : h->blocks) {
-        const BlockDev b = make_view(h, hb);
-        const int ff = march ? S + Ord<O>::Q : 0, fd = march ? S : 0;
-        const long long nf = frame_nodes(hb.n1, hb.n2, ff), nd = frame_nodes(hb.n1, hb.n2, fd);
-        ProfScope ps(h, march ? 1 : 0, fst, 2);
-        k_wide_flux<T, O><<<grid_for(nf), 256, 0, fst>>>(b, a, (T*)hb.gw, ff);
-        if (mode == 0) k_wide_div<T, O, 0><<<grid_for(nd), 256, 0, fst>>>(b, a, (const T*)hb.gw, fd);
-        else if (mode == 2) k_wide_div<T, O, 2><<<grid_for(nd), 256, 0, fst>>>(b, a, (const T*)hb.gw, fd);
-        else k_wide_div<T, O, 1><<<grid_for(nd), 256, 0, fst>>>(b, a, (const T*)hb.gw, fd);
-    }
-    if (par) {
-        cudaEventRecord(h->ev_join_hi, h->hi);
-        cudaStreamWaitEvent(st, h->ev_join_hi, 0);
-    }
-    if (!h->src_nodes.empty()) {
-        ProfScope ps(h, 3, st, 1);
-        const int ns = (int)h->src_nodes.size();
-        if (mode == 2) k_sources<T, 2><<<grid_for(ns), 256, 0, st>>>(h->d_blocks, h->d_src_nodes, ns, h->d_src_params, a);
-        else if (mode == 0) k_sources<T, 0><<<grid_for(ns), 256, 0, st>>>(h->d_blocks, h->d_src_nodes, ns, h->d_src_params, a);
-        else k_sources<T, 1><<<grid_for(ns), 256, 0, st>>>(h->d_blocks, h->d_src_nodes, ns, h->d_src_params, a);
-    }
-    return check_cuda(h, "wide operator launch");
-}
-
-// the FP64 interior of every block by k_interior_edges, up to IE_MAX_BLOCKS blocks a launch.  The tile
-// shape is the one whose busiest SM executes the fewest FP64 instructions (the kernel is bound by
-// them): 32 x 16 nodes repeat the fewest fluxes on their halos and win once there are several tiles per
-// SM, 16 x 4 nodes leave no SM idle on a 101^2 grid (138 tiles against 18).   Order 4, 101^2: 13 us
-// against 38 us for 32 x 16 tiles with their own weights.
-constexpr int kEdgeShapes[4][2] = {{32, 16}, {32, 8}, {32, 4}, {16, 4}};
-int pick_edge_shape(const sbp_handle* h) {
-    const int Q = order_q(h->order), S = std::max(order_nclos(h->order), order_ncol(h->order));
-    const int node = 8 * Q * 4 + 12, flux = 6 * Q + 4;
-    int best = 0;
-    long long least = -1;
-    for (int k = 0; k < 4; ++k) {
-        const int tx = kEdgeShapes[k][0], ty = kEdgeShapes[k][1];
-        long long tiles = 0;
-        for (auto& hb : h->blocks)
-            tiles += (long long)((hb.n1 - 2 * S + tx - 1) / tx) * ((hb.n2 - 2 * S + ty - 1) / ty);
-        const long long cost = (tiles + h->num_sms - 1) / h->num_sms *
-                               (tx * ty * node + flux * ((tx + 2 * Q) * ty + tx * (ty + 2 * Q)));
-        if (least < 0 || cost < least) {
-            least = cost;
-            best = k;
-        }
-    }
-    return best;
-}
-// the interior tiles of blocks [first, first + IE_MAX_BLOCKS) in shape k; returns their number
-int edge_tiles(const sbp_handle* h, int first, int k, InteriorTiles& tl) {
-    const int S = std::max(order_nclos(h->order), order_ncol(h->order)), tx = kEdgeShapes[k][0], ty = kEdgeShapes[k][1];
-    tl = InteriorTiles{};
-    tl.first = first;
-    int tiles = 0;
-    for (int b = first; b < std::min(h->nblocks, first + IE_MAX_BLOCKS); ++b) {
-        const HostBlock& hb = h->blocks[b];
-        tl.ncx[tl.nb] = (hb.n1 - 2 * S + tx - 1) / tx;
-        tl.start[tl.nb++] = tiles;
-        tiles += tl.ncx[tl.nb - 1] * ((hb.n2 - 2 * S + ty - 1) / ty);
-    }
-    tl.start[tl.nb] = tiles;
-    return tiles;
-}
-template <int O>
-void launch_interior_f64(sbp_handle* h, const BlockDev* tab, const StepArgs& a, int mode, cudaStream_t st) {
-    const int best = pick_edge_shape(h);
-    for (int first = 0; first < h->nblocks; first += IE_MAX_BLOCKS) {
-        InteriorTiles tl;
-        const int tiles = edge_tiles(h, first, best, tl);
-        ProfScope ps(h, 0, st, 1);
-        auto run = [&](auto kc) {
-            constexpr int TX = kEdgeShapes[decltype(kc)::value][0], TY = kEdgeShapes[decltype(kc)::value][1], NT = TX * TY < 256 ? TX * TY : 256;
-            if (mode == 0) k_interior_edges<double, O, 0, TX, TY><<<tiles, NT, 0, st>>>(tab, tl, a);
-            else if (mode == 2) k_interior_edges<double, O, 2, TX, TY><<<tiles, NT, 0, st>>>(tab, tl, a);
-            else k_interior_edges<double, O, 1, TX, TY><<<tiles, NT, 0, st>>>(tab, tl, a);
-        };
-        if (best == 0) run(std::integral_constant<int, 0>());
-        else if (best == 1) run(std::integral_constant<int, 1>());
-        else if (best == 2) run(std::integral_constant<int, 2>());
-        else run(std::integral_constant<int, 3>());
-    }
-}
-
-// Rows of the interior items (128 columns of a marching kernel, bands of equal height per grid) that share `slots`
-// CTAs with `strips` strip tiles.  An item costs its rows and about ITEM_ROWS more (the rows it marches before
-// its first output, its start), a strip tile about STRIP_ROWS; the height minimises the larger of the mean load
-// and the rounds of the longest item.  grids: (tiles across, interior rows).
-int item_rows(int slots, const std::vector<int2>& grids, long long strips, bool queued) {
-    constexpr double ITEM_ROWS = 14, STRIP_ROWS = 10;
-    double least = 1e300;
-    int best = 64;
-    for (int rows = 8; rows <= 256; rows += rows < 32 ? 1 : 4) {
-        long long items = 0;
-        double work = strips * STRIP_ROWS, longest = 0;
-        for (const int2& s : grids) {
-            const int bands = (s.y + rows - 1) / rows, high = (s.y + bands - 1) / bands;
-            items += (long long)s.x * bands;
-            work += (double)s.x * (s.y + bands * ITEM_ROWS);
-            longest = std::max(longest, high + ITEM_ROWS);
-        }
-        // (strip tiles first, one per slot, or queued behind the items)
-        const double cost = std::max(work / slots, (double)((items + (queued ? 0 : strips) + slots - 1) / slots) * longest);
-        if (cost < least) {
-            least = cost;
-            best = rows;
-        }
-    }
-    return best;
-}
-
-// Whether a step runs as one launch (sbp_step.cuh): the blocks fit the launch's tables and the kernels are not being
-// timed one by one.  FP32: leapfrog steps of the state or the adjoint fields, up to as many strip tiles as SMs
-// (1200^2; larger grids fill the chip with either kernel, see the figures there) and without interfaces, whose
-// traces now form beside the interior (2 x 402 x 201: 38 us a step, 41 with the traces first).  FP64: leapfrog steps and RK4 stages
-// with strip tiles of 8 nodes, or 16 without interfaces (4 blocks of 401^2: 264 us in one launch, 258 in two), not on
-// the largest grids, where FP64 arithmetic alone counts.  A user's choice of streams (sbp_set_tuning) keeps the strips
-// in a launch of their own.
-bool one_launch(const sbp_handle* h, int mode) {
-    if (h->prof || h->overlap || h->nblocks > MARCH_MAX_BLOCKS || h->stencil != SBP_STENCIL_NARROW) return false;
-    if (h->precision == SBP_FP32) return mode == 0 && h->ntrefs == 0 && (h->shorts.d_tiles || h->ntiles <= h->num_sms);
-    return mode != 1 && h->blocks[0].e && (h->strip_len == 8 || (h->strip_len == 16 && h->ntrefs == 0));
-}
-// the interior shape that goes with the strip tiles of an FP64 step in one launch
-int step_edge_shape(const sbp_handle* h) { return h->strip_len == 16 ? 0 : std::max(1, pick_edge_shape(h)); }
-
-template <typename T, int O>
-int launch_step(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st, bool adj) {
-    if (h->ntrefs > 0) launch_traces<T, O>(h, a, st, adj);
-    StepStrips ss{};
-    const bool sh = h->shorts.d_tiles != nullptr;
-    ss.blocks = adj ? h->d_blocks_adj : h->d_blocks;
-    ss.tiles = sh ? h->shorts.d_tiles : h->d_tiles;
-    ss.n = sh ? (int)h->shorts.tiles.size() : h->ntiles;
-    ss.ssrc = adj ? nullptr : (sh ? h->shorts.d_src : h->d_src_strip);
-    ss.spar = h->d_src_params;
-    ss.beta = h->beta;
-    const bool inside = !adj && h->n_src_int > 0 && h->n_src_int <= STEP_MAX_SOURCES;
-    ss.isrc = inside ? h->d_src_int : nullptr;
-    ss.nisrc = inside ? h->n_src_int : 0;
-    {
-        ProfScope ps(h, 0, st, 1);
-        if constexpr (std::is_same<T, float>::value) {
-            MarchMulti mm{};
-            int tiles = 0;
-            const int S = std::max(order_nclos(h->order), order_ncol(h->order));
-            std::vector<int2> grids;
-            for (auto& hb : h->blocks) grids.push_back(make_int2(march_ncx(hb.n1, S), hb.n2 - 2 * S));
-            const int even = h->rows_per_cta > 0 ? h->rows_per_cta : item_rows(4 * h->num_sms, grids, ss.n, false);
-            for (auto& hb : h->blocks) {
-                const int ncx = march_ncx(hb.n1, S), n2i = hb.n2 - 2 * S, bands = (n2i + even - 1) / even;
-                const int rows = h->rows_per_cta > 0 ? std::min(n2i, even) : (n2i + bands - 1) / bands;
-                const int k = mm.nb++;
-                mm.maps[k] = adj ? hb.pmaps : hb.mmaps;
-                mm.b[k] = adj ? make_view_adj(h, hb) : make_view(h, hb);
-                mm.start[k] = tiles;
-                mm.rows[k] = rows;
-                tiles += ncx * ((n2i + rows - 1) / rows);
-            }
-            mm.start[mm.nb] = tiles;
-            constexpr size_t sm = step_smem_f32<O>();
-            const int grid = ss.n + tiles;
-            if (adj && sh) k_step_f32<O, 0, SHORT_TILE><<<grid, MTHREADS, sm, st>>>(mm, ss, a, h->d_err);
-            else if (adj) k_step_f32<O, 0, 32><<<grid, MTHREADS, sm, st>>>(mm, ss, a, h->d_err);
-            else if (sh) k_step_f32<O, 3, SHORT_TILE><<<grid, MTHREADS, sm, st>>>(mm, ss, a, h->d_err);
-            else k_step_f32<O, 3, 32><<<grid, MTHREADS, sm, st>>>(mm, ss, a, h->d_err);
-        } else {
-            const int best = step_edge_shape(h);
-            InteriorTiles tl;
-            const int grid = ss.n + edge_tiles(h, 0, best, tl);
-            auto run = [&](auto kc) {
-                constexpr int TX = kEdgeShapes[decltype(kc)::value][0], TY = kEdgeShapes[decltype(kc)::value][1];
-                constexpr size_t sm = step_smem_f64<O, TX, TY>();
-                constexpr int NT = step_threads_f64<TX, TY>();
-                if (mode == 0) k_step_f64<O, 0, TX, TY><<<grid, NT, sm, st>>>(tl, ss, a, h->d_err);
-                else k_step_f64<O, 2, TX, TY><<<grid, NT, sm, st>>>(tl, ss, a, h->d_err);
-            };
-            if (best == 0) run(std::integral_constant<int, 0>());
-            else if (best == 1) run(std::integral_constant<int, 1>());
-            else if (best == 2) run(std::integral_constant<int, 2>());
-            else run(std::integral_constant<int, 3>());
-        }
-    }
-    if (!adj && h->n_src_int > 0 && !inside) {
-        ProfScope ps(h, 3, st, 1);
-        const int ns = h->n_src_int;
-        if (mode == 2) k_sources<T, 2><<<grid_for(ns), 256, 0, st>>>(h->d_blocks, h->d_src_int, ns, h->d_src_params, a);
-        else k_sources<T, 0><<<grid_for(ns), 256, 0, st>>>(h->d_blocks, h->d_src_int, ns, h->d_src_params, a);
-    }
-    return check_cuda(h, "step launch");
-}
-
-// one operator application (mode 1) or leapfrog step (mode 0) on the state fields, or, with adj,
-// on the adjoint fields (the same kernels; the sources are skipped)
-template <typename T, int O>
-int launch_operator(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st, bool adj) {
-    if (one_launch(h, mode)) return launch_step<T, O>(h, a, mode, st, adj);
-    const BlockDev* tab = adj ? h->d_blocks_adj : h->d_blocks;
-    constexpr size_t smem = interior_smem_elems<T, O>() * sizeof(T);
-    // interior kernels on st; strip kernels on the auxiliary stream when overlapping (profiling
-    // runs serialise so that every family's events time that family alone)
-    const bool ovl = h->overlap && h->aux && !h->prof;
-    // the interface traces run on the auxiliary stream beside the interior kernel (in its tail
-    // or its free slots); the strips that read them follow on that stream or wait for it
-    const bool tr_async = h->aux && !h->prof && h->ntrefs > 0;
-    cudaStream_t sst = ovl ? h->aux : st;
-    cudaStream_t ist = ovl ? h->hi : st;
-    cudaStream_t tst = (ovl || tr_async) ? h->aux : st;
-    if (ovl || tr_async) {
-        cudaEventRecord(h->ev_fork, st);
-        cudaStreamWaitEvent(h->aux, h->ev_fork, 0);
-        if (ovl) cudaStreamWaitEvent(h->hi, h->ev_fork, 0);
-    }
-    if constexpr (std::is_same<T, float>::value) {
-        // column-marching kernel: the interior tiles of up to MARCH_MAX_BLOCKS blocks per launch,
-        // rows per tile chosen for one wave of ~4 CTAs per SM per block
-        MarchMulti mmul{};
-        int tiles = 0;
-        auto flush = [&]() {
-            if (mmul.nb == 0) return;
-            mmul.start[mmul.nb] = tiles;
-            ProfScope ps(h, 0, ist, 1);
-            constexpr size_t msm = MarchCfg<O>::BYTES;
-            if (mode == 0 && !adj) k_interior_march_multi<O, 3><<<tiles, MTHREADS, msm, ist>>>(mmul, a, h->d_err);
-            else if (mode == 0) k_interior_march_multi<O, 0><<<tiles, MTHREADS, msm, ist>>>(mmul, a, h->d_err);
-            else if (mode == 2 && a.stage == 1) k_interior_march_multi<O, 4><<<tiles, MTHREADS, msm, ist>>>(mmul, a, h->d_err);
-            else if (mode == 2 && a.stage == 2) k_interior_march_multi<O, 5><<<tiles, MTHREADS, msm, ist>>>(mmul, a, h->d_err);
-            else if (mode == 2 && a.stage == 3) k_interior_march_multi<O, 6><<<tiles, MTHREADS, msm, ist>>>(mmul, a, h->d_err);
-            else if (mode == 2) k_interior_march_multi<O, 7><<<tiles, MTHREADS, msm, ist>>>(mmul, a, h->d_err);
-            else k_interior_march_multi<O, 1><<<tiles, MTHREADS, msm, ist>>>(mmul, a, h->d_err);
-            mmul = MarchMulti{};
-            tiles = 0;
-        };
-        for (auto& hb : h->blocks) {
-            const int S2 = std::max(order_nclos(h->order), order_ncol(h->order));
-            const int ncx = march_ncx(hb.n1, S2);
-            const int n2i = hb.n2 - 2 * S2;
-            const int rows = march_rows(h, ncx, n2i), ncy = (n2i + rows - 1) / rows;
-            const int k = mmul.nb++;
-            mmul.maps[k] = adj ? hb.pmaps : hb.mmaps;
-            mmul.b[k] = adj ? make_view_adj(h, hb) : make_view(h, hb);
-            mmul.start[k] = tiles;
-            mmul.rows[k] = rows;
-            tiles += ncx * ncy;
-            if (mmul.nb == MARCH_MAX_BLOCKS) flush();
-        }
-        flush();
-    } else if (h->blocks[0].e) {
-        launch_interior_f64<O>(h, tab, a, mode, ist);
-    } else for (auto& hb : h->blocks) {   // no room for the edge weights: the kernel that forms them
-        BlockDev b = adj ? make_view_adj(h, hb) : make_view(h, hb);
-        const int S = b.strip;
-        const int ni1 = hb.n1 - 2 * S, ni2 = hb.n2 - 2 * S;
-        dim3 grid((ni1 + ITX - 1) / ITX, (ni2 + ITY - 1) / ITY);
-        {
-            ProfScope ps(h, 0, ist, 1);
-            {
-                if (mode == 0) k_interior<T, O, 0><<<grid, dim3(32, 8), smem, ist>>>(b, a);
-                else if (mode == 2) k_interior<T, O, 2><<<grid, dim3(32, 8), smem, ist>>>(b, a);
-                else k_interior<T, O, 1><<<grid, dim3(32, 8), smem, ist>>>(b, a);
-            }
-        }
-    }
-    if (h->ntrefs > 0) launch_traces<T, O>(h, a, tst, adj);
-    if (tr_async && !ovl) {    // the strips wait for the traces formed beside the interior
-        cudaEventRecord(h->ev_join, h->aux);
-        cudaStreamWaitEvent(st, h->ev_join, 0);
-    }
-    {
-        ProfScope ps(h, 1, sst, 1);
-        const SrcNode* ss = adj ? nullptr : h->d_src_strip;
-        auto run = [&](auto lc) {
-            constexpr int TL = decltype(lc)::value;
-            using ST = StripTile<O, TL>;
-            constexpr size_t ssm = ST::template bytes<T>();
-            if (mode == 0)
-                k_strip_tile<T, O, 0, TL><<<h->ntiles, ST::THREADS, ssm, sst>>>(tab, h->d_tiles, a, h->beta, h->d_err, ss, h->d_src_params);
-            else if (mode == 2)
-                k_strip_tile<T, O, 2, TL><<<h->ntiles, ST::THREADS, ssm, sst>>>(tab, h->d_tiles, a, h->beta, h->d_err, ss, h->d_src_params);
-            else
-                k_strip_tile<T, O, 1, TL><<<h->ntiles, ST::THREADS, ssm, sst>>>(tab, h->d_tiles, a, h->beta, h->d_err, ss, h->d_src_params);
-        };
-        if constexpr (std::is_same<T, double>::value) {
-            if (h->strip_len == 8) run(std::integral_constant<int, 8>());
-            else if (h->strip_len == 16) run(std::integral_constant<int, 16>());
-            else run(std::integral_constant<int, 32>());
-        } else {
-            run(std::integral_constant<int, 32>());
-        }
-    }
-    if (ovl) {
-        cudaEventRecord(h->ev_join, h->aux);
-        cudaEventRecord(h->ev_join_hi, h->hi);
-        cudaStreamWaitEvent(st, h->ev_join, 0);
-        cudaStreamWaitEvent(st, h->ev_join_hi, 0);
-    }
-    if (!adj && h->n_src_int > 0) {   // source nodes off the strips (the strip kernel adds the others)
-        ProfScope ps(h, 3, st, 1);
-        const int ns = h->n_src_int;
-        if (mode == 2) k_sources<T, 2><<<grid_for(ns), 256, 0, st>>>(h->d_blocks, h->d_src_int, ns, h->d_src_params, a);
-        else if (mode == 0) k_sources<T, 0><<<grid_for(ns), 256, 0, st>>>(h->d_blocks, h->d_src_int, ns, h->d_src_params, a);
-        else k_sources<T, 1><<<grid_for(ns), 256, 0, st>>>(h->d_blocks, h->d_src_int, ns, h->d_src_params, a);
-    }
-    return check_cuda(h, "operator launch");
-}
-
 template <typename T>
 int dispatch_operator(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st, bool adj) {
     if (h->stencil == SBP_STENCIL_WIDE) {
@@ -884,25 +165,6 @@ int dispatch_operator(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t s
         case 2: return launch_operator<T, 2>(h, a, mode, st, adj);
         case 4: return launch_operator<T, 4>(h, a, mode, st, adj);
         default: return launch_operator<T, 6>(h, a, mode, st, adj);
-    }
-}
-
-// layer dissipation around the step kernels (leapfrog: the backward-velocity term is formed before
-// the step overwrites u^{n-1} and added after it; RK4: added into the stage's operator sum before)
-template <typename T, int O>
-void layer_launch(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st, bool post) {
-    if (mode == 0 && !(a.dt > 0)) return;   // tuning steps advance nothing (dt = 0)
-    for (auto& hb : h->blocks) {
-        if (hb.nln == 0) continue;
-        const BlockDev b = make_view(h, hb);
-        const unsigned g = grid_for(hb.nln);
-        if (mode == 2) {
-            if (!post) k_layer_rk<T, O><<<g, 256, 0, st>>>(b, hb.d_lnodes, hb.nln, a.stage, a.rkh);
-        } else if (!post) {
-            k_layer_pre<T, O><<<g, 256, 0, st>>>(b, hb.d_lnodes, hb.nln, a.cur, 1.0 / a.dt, (T*)hb.lscr);
-        } else {
-            k_layer_post<T><<<g, 256, 0, st>>>(b, hb.d_lnodes, hb.nln, a.cur, a.dt, (const T*)hb.lscr);
-        }
     }
 }
 
@@ -925,55 +187,6 @@ int run_operator(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st, bo
                                             : dispatch_operator<float>(h, a, mode, st, adj);
     if (rc == SBP_OK && layers && mode == 0) run_layers(h, a, mode, st, true);
     return rc;
-}
-
-template <typename T, int O> void set_smem_attr() {
-    constexpr size_t smem = interior_smem_elems<T, O>() * sizeof(T);
-    auto strip = [](auto lc) {
-        constexpr int TL = decltype(lc)::value;
-        constexpr int ssm = (int)StripTile<O, TL>::template bytes<T>();
-        cudaFuncSetAttribute(k_strip_tile<T, O, 0, TL>, cudaFuncAttributeMaxDynamicSharedMemorySize, ssm);
-        cudaFuncSetAttribute(k_strip_tile<T, O, 1, TL>, cudaFuncAttributeMaxDynamicSharedMemorySize, ssm);
-        cudaFuncSetAttribute(k_strip_tile<T, O, 2, TL>, cudaFuncAttributeMaxDynamicSharedMemorySize, ssm);
-    };
-    strip(std::integral_constant<int, 32>());
-    if constexpr (std::is_same<T, float>::value) {
-        constexpr int sm = (int)step_smem_f32<O>();
-        cudaFuncSetAttribute(k_step_f32<O, 0, SHORT_TILE>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-        cudaFuncSetAttribute(k_step_f32<O, 3, SHORT_TILE>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-        cudaFuncSetAttribute(k_step_f32<O, 0, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-        cudaFuncSetAttribute(k_step_f32<O, 3, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    } else {
-        auto step = [](auto kc) {
-            constexpr int TX = kEdgeShapes[decltype(kc)::value][0], TY = kEdgeShapes[decltype(kc)::value][1];
-            constexpr int sm = (int)step_smem_f64<O, TX, TY>();
-            cudaFuncSetAttribute(k_step_f64<O, 0, TX, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_step_f64<O, 2, TX, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-        };
-        step(std::integral_constant<int, 0>());
-        step(std::integral_constant<int, 1>());
-        step(std::integral_constant<int, 2>());
-        step(std::integral_constant<int, 3>());
-    }
-    if constexpr (std::is_same<T, double>::value) {
-        strip(std::integral_constant<int, 16>());
-        strip(std::integral_constant<int, 8>());
-    }
-    cudaFuncSetAttribute(k_interior<T, O, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(k_interior<T, O, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(k_interior<T, O, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (std::is_same<T, float>::value) {
-        cudaFuncSetAttribute(k_wide_march<O, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
-        cudaFuncSetAttribute(k_wide_march<O, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
-        cudaFuncSetAttribute(k_wide_march<O, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
-        cudaFuncSetAttribute(k_interior_march_multi<O, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
-        cudaFuncSetAttribute(k_interior_march_multi<O, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
-        cudaFuncSetAttribute(k_interior_march_multi<O, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
-        cudaFuncSetAttribute(k_interior_march_multi<O, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
-        cudaFuncSetAttribute(k_interior_march_multi<O, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
-        cudaFuncSetAttribute(k_interior_march_multi<O, 6>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
-        cudaFuncSetAttribute(k_interior_march_multi<O, 7>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MarchCfg<O>::BYTES);
-    }
 }
 
 // kernel error word: ERR_* bits (sbp_device.cuh) set by kernels whose bounded wait ran out
@@ -1115,29 +328,6 @@ inline size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 constexpr int NOALLOC_MAX_BLOCKS = 32;
 
-template <typename T, int O>
-void launch_noalloc(sbp_handle* h, const BlockDev* views, int nviews, BlockDev* d_views, FaceRef* d_refs,
-                    const StepArgs& a, cudaStream_t st) {
-    const int total = h->nface_nodes;
-    if (total > 0) k_face_sat<T, O><<<grid_for(total), 256, 0, st>>>(d_views, d_refs, h->nrefs, total, a, h->beta);
-    constexpr size_t smem = interior_smem_elems<T, O>() * sizeof(T);
-    const bool edges = std::is_same<T, double>::value && views[0].e;
-    if (edges) launch_interior_f64<O>(h, d_views, a, 1, st);
-    for (int b = 0; b < nviews; ++b) {
-        const BlockDev& v = views[b];
-        const int S = v.strip;
-        const int ni1 = v.n1 - 2 * S, ni2 = v.n2 - 2 * S;
-        dim3 grid((ni1 + ITX - 1) / ITX, (ni2 + ITY - 1) / ITY);
-        if (!edges) k_interior<T, O, 1><<<grid, dim3(32, 8), smem, st>>>(v, a);
-        const long long nstrip = (long long)v.n1 * v.n2 - (long long)ni1 * ni2;
-        k_boundary<T, O, 1><<<grid_for(nstrip), 256, 0, st>>>(v, a);
-    }
-    if (!h->src_nodes.empty()) {
-        const int ns = (int)h->src_nodes.size();
-        k_sources<T, 1><<<grid_for(ns), 256, 0, st>>>(d_views, h->d_src_nodes, ns, h->d_src_params, a);
-    }
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------------------------------------
@@ -1197,51 +387,6 @@ int record_receivers(sbp_handle* h, double* d_row, cudaStream_t st) {
     if (h->precision == SBP_FP64) k_record<double><<<grid_for(nr, 128), 128, 0, st>>>(h->d_blocks, h->d_recs, nr, h->cur, d_row);
     else k_record<float><<<grid_for(nr, 128), 128, 0, st>>>(h->d_blocks, h->d_recs, nr, h->cur, d_row);
     return SBP_OK;
-}
-
-// strip nodes of the gradient (bands of width gs along every face)
-long long grad_strip_nodes(const HostBlock& hb, int gs) {
-    return (long long)hb.n1 * hb.n2 - (long long)(hb.n1 - 2 * gs) * (hb.n2 - 2 * gs);
-}
-int order_gs(int o) { return o == 2 ? SBP2_GS : (o == 4 ? SBP4_GS : SBP6_GS); }
-// level chunks of the strip gradient: about 4 waves of 256-thread CTAs over the SMs, at most
-// one chunk per level and at most GRAD_MAX_CHUNKS
-constexpr int GRAD_MAX_CHUNKS = 16;
-int grad_strip_chunks(const sbp_handle* h, long long nstrip, int nl) {
-    const long long want = 4LL * h->num_sms * 2048;
-    long long c = (want + nstrip - 1) / std::max(1LL, nstrip);
-    c = std::min<long long>(c, GRAD_MAX_CHUNKS);
-    c = std::min<long long>(c, nl);
-    return (int)std::max(1LL, c);
-}
-
-// gradient contributions of the nl levels of one segment
-template <typename T, int O>
-void launch_grad(sbp_handle* h, const GradDev* d_grad, const std::vector<GradDev>& grads, int nl, double dt2,
-                 cudaStream_t st) {
-    const int total = h->nface_nodes, nfc = std::min(GRAD_MAX_CHUNKS, nl);
-    if (total > 0) {
-        ProfScope ps(h, 6, st, 1);
-        k_grad_face<T, O><<<dim3(grid_for(total, 64), nfc), 64, 0, st>>>(h->d_blocks_adj, d_grad, h->d_refs, h->nrefs, total, nl, nfc, h->beta);
-    }
-    constexpr int GS = GradCfg<O>::GS;
-    for (size_t b = 0; b < h->blocks.size(); ++b) {
-        const HostBlock& hb = h->blocks[b];
-        const BlockDev v = make_view_adj(h, hb);
-        {
-            ProfScope ps(h, 4, st, 1);
-            dim3 gi((hb.n1 - 2 * GS + 31) / 32, (hb.n2 - 2 * GS + 7) / 8);
-            k_grad_interior<T, O><<<gi, dim3(32, 8), 0, st>>>(v, grads[b], nl, dt2);
-        }
-        {
-            ProfScope ps(h, 5, st, 3);
-            const long long nstrip = grad_strip_nodes(hb, GS);
-            const int nchunk = grad_strip_chunks(h, nstrip, nl);
-            k_grad_lines<T, O><<<dim3(grid_for(2LL * (hb.n1 + hb.n2), 64), nchunk), 64, 0, st>>>(v, grads[b], nl, nchunk, nstrip);
-            k_grad_strip<T, O><<<dim3(grid_for(nstrip), nchunk), 256, 0, st>>>(v, grads[b], nl, nchunk, nstrip);
-            k_grad_strip_sum<T, O><<<grid_for(nstrip), 256, 0, st>>>(v, grads[b], nchunk, nfc, nstrip, dt2);
-        }
-    }
 }
 
 void run_grad(sbp_handle* h, const GradDev* d_grad, const std::vector<GradDev>& grads, int nl, double dt2,
@@ -2799,15 +1944,10 @@ struct sbp_batch {
 
 namespace {
 
-template <int O> void batch_smem_attr() {
-    cudaFuncSetAttribute(k_batch_step<O>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)batch_smem_bytes<O>());
-}
-template <int O> size_t batch_smem() { return batch_smem_bytes<O>(); }
-
 void batch_launch(sbp_batch* b, cudaStream_t st) {
-    if (b->order == 2) k_batch_step<2><<<b->ctas, MTHREADS, batch_smem<2>(), st>>>(b->d_head, b->d_err);
-    else if (b->order == 4) k_batch_step<4><<<b->ctas, MTHREADS, batch_smem<4>(), st>>>(b->d_head, b->d_err);
-    else k_batch_step<6><<<b->ctas, MTHREADS, batch_smem<6>(), st>>>(b->d_head, b->d_err);
+    if (b->order == 2) batch_step_launch<2>(b->ctas, b->d_head, b->d_err, st);
+    else if (b->order == 4) batch_step_launch<4>(b->ctas, b->d_head, b->d_err, st);
+    else batch_step_launch<6>(b->ctas, b->d_head, b->d_err, st);
 }
 
 // rebuild and upload the work list: interior tiles of every active shot first (the long items),
@@ -2893,13 +2033,7 @@ int sbp_batch_create(int order, int max_shots, sbp_batch** out) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&b->num_sms, cudaDevAttrMultiProcessorCount, dev);
     if (b->num_sms <= 0) b->num_sms = 1;
-    if (order == 2) batch_smem_attr<2>();
-    else if (order == 4) batch_smem_attr<4>();
-    else batch_smem_attr<6>();
-    int per_sm = 0;
-    if (order == 2) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_step<2>, MTHREADS, batch_smem<2>());
-    else if (order == 4) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_step<4>, MTHREADS, batch_smem<4>());
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_step<6>, MTHREADS, batch_smem<6>());
+    const int per_sm = order == 2 ? batch_ctas_per_sm<2>() : (order == 4 ? batch_ctas_per_sm<4>() : batch_ctas_per_sm<6>());
     b->ctas = std::max(1, per_sm) * b->num_sms;      // persistent: every CTA resident at once
     if (cudaMalloc(&b->d_head, sizeof(BatchHead)) != cudaSuccess || cudaMalloc(&b->d_shots, sizeof(BatchShot) * max_shots) != cudaSuccess ||
         cudaMalloc(&b->d_state, sizeof(BatchState) * max_shots) != cudaSuccess || cudaMalloc(&b->d_err, 64) != cudaSuccess) {

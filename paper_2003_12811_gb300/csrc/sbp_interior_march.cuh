@@ -347,6 +347,20 @@ __device__ __forceinline__ bool march_tile(const MarchMaps& maps, const BV& B, c
             const float2 g = ffma2(make_float2(m6, m8), bc2(d.x), fmul2(make_float2(m7, m9), bc2(d.y)));
             reinterpret_cast<float2*>(g1s)[par * W + hc] = g;
         }
+        // the part of the RK4 combination that needs no operator value, so that its operands leave their registers to the
+        // narrow rows
+        float2 rku = make_float2(0.f, 0.f), rkv = rku, rka = rku;       // next input; stage 4: v, a_1 + 2 (a_2 + a_3)
+        if constexpr (RK > 0) {
+            const float h = a.rkhf, hh = 0.5f * h;
+            if constexpr (RK == 1) rku = ffma2(bc2(hh), rk[0], qu[Q]);
+            else if constexpr (RK < 4) rku = ffma2(bc2(RK == 3 ? h : hh), ffma2(bc2(hh), rk[2], rk[1]), rk[0]);
+            else {
+                const float2 s23 = fadd2(rk[3], rk[4]);
+                rku = ffma2(bc2(h), ffma2(bc2(h / 6.f), fadd2(rk[2], s23), rk[1]), rk[0]);
+                rka = ffma2(bc2(2.f), s23, rk[2]);
+                rkv = rk[1];
+            }
+        }
         if (__syncthreads_or(!ok)) {
             // a bounded wait ran out: record it, drain this CTA's issued copies (bounded), stop
             if (tx == 0) {
@@ -436,15 +450,10 @@ __device__ __forceinline__ bool march_tile(const MarchMaps& maps, const BV& B, c
             if (a.rk_r) rk4_layer_terms<float>(B, gi, plane, r0, r1);
             float* __restrict__ Un = reinterpret_cast<float*>(B.u[1 - a.cur]);
             float* __restrict__ K = reinterpret_cast<float*>(B.rk);
-            const float h = a.rkhf, hh = 0.5f * h;
             const float2 as = fmul2(bc2(w_c), make_float2(r0, r1));
-            float2 un;
-            if constexpr (RK == 1) un = ffma2(bc2(hh), rk[0], uc);
-            else if constexpr (RK < 4) un = ffma2(bc2(RK == 3 ? h : hh), ffma2(bc2(hh), rk[2], rk[1]), rk[0]);
-            else {
-                const float2 s23 = fadd2(rk[3], rk[4]);
-                un = ffma2(bc2(h), ffma2(bc2(h / 6.f), fadd2(rk[2], s23), rk[1]), rk[0]);
-                const float2 vn = ffma2(bc2(h / 6.f), fadd2(ffma2(bc2(2.f), s23, rk[2]), as), rk[1]);
+            const float2 un = rku;
+            if constexpr (RK == 4) {
+                const float2 vn = ffma2(bc2(a.rkhf / 6.f), fadd2(rka, as), rkv);
                 K[gi] = un.x;
                 K[plane + gi] = un.y;
                 K[2 * plane + gi] = vn.x;
