@@ -440,6 +440,20 @@ inline int grad_strip_chunks(const sbp_handle* h, long long nstrip, int nl) {
     return (int)std::max(1LL, c);
 }
 
+// Whether an FP32 wide-stencil operator marches over the interior (k_wide_march beside the frame's kernels) or takes
+// two passes over every node.  The march reads each node once, but costs a launch and a fork and join of streams, which the
+// host pays where the kernels are short.  The line lies where the two are equal, in nodes of all blocks (a block's own two
+// launches move it up): order 6 about 300 k on one block, 450 k on four (us a step, two passes / march: 601 x 477 38.2 /
+// 42.4, 801 x 627 43.1 / 41.4; 4 x 301^2 87 / 98, 4 x 401^2 103 / 99; 2 x 201 x 177 59 / 62, 2 x 601 x 477 68 / 65); orders 2
+// and 4, whose marches save less, 350 k and 950 k (order 4: 601 x 477 33.7 / 33.9, 801 x 627 38.6 / 34.3; order 2: 2 x
+// 401 x 327 43.4 / 50.8, 2 x 801 x 627 65 / 52; 4 x 401^2 77 / 84, 4 x 601^2 124 / 118).
+inline bool wide_by_march(const sbp_handle* h) {
+    long long nodes = 0;
+    for (auto& hb : h->blocks) nodes += (long long)hb.n1 * hb.n2;
+    const long long nb = h->nblocks;
+    return nodes >= (h->order == 6 ? 250000 + 50000 * nb : 150000 + 200000 * nb);
+}
+
 // ------------------------------------------------------------------ per precision and order (sbp_launch.cuh)
 template <typename T, int O> int launch_operator(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st, bool adj);
 template <typename T, int O> int launch_wide(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st);

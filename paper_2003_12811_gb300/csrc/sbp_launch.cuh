@@ -43,12 +43,13 @@ void launch_traces(sbp_handle* h, const StepArgs& a, cudaStream_t tst, bool adj)
 }
 
 // the wide-stencil operator (sbp_wide.cuh): traces, the SAT terms of every face node, the flux and
-// divergence passes of every block (in FP32 of its frame near the faces, beside one marching kernel over
+// divergence passes of every block (by wide_by_march only of its frame near the faces, beside one marching kernel over
 // the interior, which they share nothing with), then the point sources (every source node: the wide path has
 // no strip kernel)
 template <typename T, int O>
 int launch_wide(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st) {
-    constexpr bool march = std::is_same<T, float>::value;
+    constexpr bool f32 = std::is_same<T, float>::value;
+    const bool march = f32 && wide_by_march(h);
     const int S = std::max(order_nclos(h->order), order_ncol(h->order));
     // the frame's chain of small kernels on the high-priority stream, queued before the interior
     const bool par = march && h->hi && !h->prof;
@@ -62,7 +63,7 @@ int launch_wide(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st) {
         ProfScope ps(h, 1, fst, 1);
         k_face_sat<T, O><<<grid_for(h->nface_nodes, 64), 64, 0, fst>>>(h->d_blocks, h->d_refs, h->nrefs, h->nface_nodes, a, h->beta);
     }
-    if constexpr (march) {
+    if constexpr (f32) {
         MarchMulti mm{};
         int tiles = 0;
         auto flush = [&]() {
@@ -77,6 +78,7 @@ int launch_wide(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st) {
             tiles = 0;
         };
         for (auto& hb : h->blocks) {
+            if (!march) break;
             const int ncx = wide_ncx(hb.n1, S), n2i = hb.n2 - 2 * S, rows = march_rows(h, ncx, n2i), k = mm.nb++;
             mm.maps[k] = hb.mmaps;
             mm.b[k] = make_view(h, hb);
@@ -87,15 +89,24 @@ int launch_wide(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st) {
         }
         flush();
     }
-    for (auto& hb : h->blocks) {
-        const BlockDev b = make_view(h, hb);
-        const int ff = march ? S + Ord<O>::Q : 0, fd = march ? S : 0;
-        const long long nf = frame_nodes(hb.n1, hb.n2, ff), nd = frame_nodes(hb.n1, hb.n2, fd);
-        ProfScope ps(h, march ? 1 : 0, fst, 2);
-        k_wide_flux<T, O><<<grid_for(nf), 256, 0, fst>>>(b, a, (T*)hb.gw, ff);
-        if (mode == 0) k_wide_div<T, O, 0><<<grid_for(nd), 256, 0, fst>>>(b, a, (const T*)hb.gw, fd);
-        else if (mode == 2) k_wide_div<T, O, 2><<<grid_for(nd), 256, 0, fst>>>(b, a, (const T*)hb.gw, fd);
-        else k_wide_div<T, O, 1><<<grid_for(nd), 256, 0, fst>>>(b, a, (const T*)hb.gw, fd);
+    auto passes = [&](auto fc) {
+        constexpr bool F = decltype(fc)::value;
+        for (auto& hb : h->blocks) {
+            const BlockDev b = make_view(h, hb);
+            const int ff = F ? S + Ord<O>::Q : 0, fd = F ? S : 0;
+            const long long nf = frame_nodes(hb.n1, hb.n2, ff), nd = frame_nodes(hb.n1, hb.n2, fd);
+            ProfScope ps(h, F ? 1 : 0, fst, 2);
+            k_wide_flux<T, O, F><<<grid_for(nf), 256, 0, fst>>>(b, a, (T*)hb.gw, ff);
+            if (mode == 0) k_wide_div<T, O, 0, F><<<grid_for(nd), 256, 0, fst>>>(b, a, (const T*)hb.gw, fd);
+            else if (mode == 2) k_wide_div<T, O, 2, F><<<grid_for(nd), 256, 0, fst>>>(b, a, (const T*)hb.gw, fd);
+            else k_wide_div<T, O, 1, F><<<grid_for(nd), 256, 0, fst>>>(b, a, (const T*)hb.gw, fd);
+        }
+    };
+    if constexpr (f32) {
+        if (march) passes(std::true_type());
+        else passes(std::false_type());
+    } else {
+        passes(std::false_type());
     }
     if (par) {
         cudaEventRecord(h->ev_join_hi, h->hi);

@@ -8,8 +8,8 @@
 //                faces), 4 planes G_10, G_11, G_20, G_21;
 //   k_wide_div:  r_j = D_1 G_1j + D_2 G_2j + the SAT terms of k_face_sat + J f, and the step epilogue
 //                (leapfrog update, operator output or RK4 stage).
-// In FP32 the two passes take only the frame of nodes near the faces (closure rows of D, SATs), and
-// k_wide_march forms both in one pass over the interior.
+// On all but small FP32 grids (wide_by_march) the two passes take only the frame of nodes near the faces (closure rows of
+// D, SATs), and k_wide_march forms both in one pass over the interior.
 #pragma once
 #include "sbp_interior_march.cuh"
 #include "sbp_kernels.cuh"
@@ -39,12 +39,24 @@ __device__ __forceinline__ void frame_node(int n1, int n2, int F, long long t, i
     i1 = k < F ? k : n1 - 2 * F + k;
 }
 
-template <typename T, int O>
-__global__ void k_wide_flux(BlockDev B, StepArgs a, T* __restrict__ G, int frame) {
+// node t of the pass (FRAME: of the frame of width `frame`); false past the last
+template <bool FRAME> __device__ __forceinline__ bool wide_node(const BlockDev& B, int frame, int& i1, int& i2) {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= frame_nodes(B.n1, B.n2, frame)) return;
+    if constexpr (FRAME) {
+        if (t >= frame_nodes(B.n1, B.n2, frame)) return false;
+        frame_node(B.n1, B.n2, frame, t, i1, i2);
+    } else {
+        if (t >= (long long)B.n1 * B.n2) return false;
+        i2 = (int)(t / B.n1);
+        i1 = (int)(t - (long long)i2 * B.n1);
+    }
+    return true;
+}
+
+template <typename T, int O, bool FRAME>
+__global__ void k_wide_flux(BlockDev B, StepArgs a, T* __restrict__ G, int frame) {
     int i1, i2;
-    frame_node(B.n1, B.n2, frame, t, i1, i2);
+    if (!wide_node<FRAME>(B, frame, i1, i2)) return;
     const int P = B.pitch;
     const size_t plane = (size_t)B.n2 * P, gi = (size_t)i2 * P + i1;
     const T* __restrict__ U0 = reinterpret_cast<const T*>(B.u[a.cur]);
@@ -66,13 +78,11 @@ __global__ void k_wide_flux(BlockDev B, StepArgs a, T* __restrict__ G, int frame
     G[3 * plane + gi] = c[7] * d10 + c[9] * d11 + c[4] * d20 + c[5] * d21;      // G_21
 }
 
-template <typename T, int O, int MODE>
+template <typename T, int O, int MODE, bool FRAME>
 __global__ void k_wide_div(BlockDev B, StepArgs a, const T* __restrict__ G, int frame) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int n1 = B.n1, n2 = B.n2;
-    if (t >= frame_nodes(n1, n2, frame)) return;
     int i1, i2;
-    frame_node(n1, n2, frame, t, i1, i2);
+    if (!wide_node<FRAME>(B, frame, i1, i2)) return;
     const int P = B.pitch;
     const size_t plane = (size_t)n2 * P, gi = (size_t)i2 * P + i1;
     const T ih1 = ih1T<T>(B), ih2 = ih2T<T>(B);
