@@ -221,12 +221,13 @@ int sbp_grid_footprint(const sbp_grid_desc* desc, long long* bytes_out);
  * for one copy of the state is allocated for the call): the FP32 interior kernel's rows per CTA (written to
  * *rows_out, 0 = the built-in heuristic; FP64 handles: 0), and whether the boundary-strip kernel
  * runs on a second stream concurrently with the interior kernel (*overlap_out, 0 or 1; the
- * default is 0).  The choice is kept by the handle.  Either pointer may be NULL. */
+ * default is 0).  Grids whose step is one launch (small and middling ones) have nothing to run side by side: 0.
+ * The choice is kept by the handle and changes no result.  Either pointer may be NULL. */
 int sbp_autotune(sbp_handle* h, int* rows_out, int* overlap_out);
 
 /* Set the tuning directly (e.g. a choice sbp_autotune made for another handle with the same
  * grid): rows per CTA of the FP32 interior kernel (0 = heuristic) and the strip/interior overlap
- * (0 off, 1 on, -1 unchanged). */
+ * (0 off, 1 on, -1 unchanged; without effect where a step is one launch).  Changes no result. */
 int sbp_set_tuning(sbp_handle* h, int rows_per_cta, int overlap);
 
 /* Apply the spatial operator to the current level of every block (synchronous):
@@ -256,7 +257,8 @@ int sbp_suggest_dt(sbp_handle* h, double cfl, double* dt_out);
 
 /* Kernel timing for benchmarks.  sbp_profile(h, 1) resets the counters and, until
  * sbp_profile(h, 0), makes every kernel launch record CUDA events (on the launch stream)
- * around its family: [0] interior stencil, [1] boundary strips (closures, and the SAT terms,
+ * around its family: [0] interior stencil, and the whole step where it is one launch (small and
+ * middling grids), [1] boundary strips (closures, and the SAT terms,
  * which the strip kernel forms itself), [2] interface traces (k_face_trace: each interface
  * side's displacement, traction and penalty share, read by the other side's SAT terms), [3] point sources,
  * [4] gradient interior, [5] gradient strips,

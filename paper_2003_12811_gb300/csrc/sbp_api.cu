@@ -1584,8 +1584,8 @@ int sbp_autotune(sbp_handle* h, int* rows_out, int* overlap_out) {
     h->rows_per_cta = best;
     // strips beside the interior or after it: the two timed alternately at the chosen height (the
     // height's own time is the minimum over the candidates, so it is not compared directly)
-    float sum_seq = 0.f, sum_ov = 0.f;
-    for (int k = 0; k < 3; ++k) {
+    float sum_seq = 0.f, sum_ov = one_launch(h, 0) ? 1.f : 0.f;   // (a step in one launch: nothing to choose)
+    for (int k = 0; k < 3 && !one_launch(h, 0); ++k) {
         float t;
         h->overlap = false;
         int rc = time_it(t);

@@ -408,15 +408,16 @@ inline int item_rows(int slots, const std::vector<int2>& grids, long long strips
     return best;
 }
 
-// Whether a step runs as one launch (sbp_step.cuh): the blocks fit the launch's tables and the kernels are not being
-// timed one by one.  FP32: leapfrog steps of the state or the adjoint fields, up to as many strip tiles as SMs
+// Whether a step runs as one launch (sbp_step.cuh): the blocks fit the launch's tables.  A property of the handle, whatever
+// its tuning and whether its kernels are being timed, so that neither changes the rounding of a result (the one-launch
+// kernels sum a face node's SAT terms by parts) and sbp_profile times the launches that steps make.  FP32: leapfrog steps of the state or the adjoint fields, up to as many strip tiles as SMs
 // (1200^2; larger grids fill the chip with either kernel, see the figures there) and without interfaces, whose
 // traces now form beside the interior (2 x 402 x 201: 38 us a step, 41 with the traces first).  FP64: leapfrog steps and RK4 stages
 // with strip tiles of 8 nodes, or 16 without interfaces (4 blocks of 401^2: 264 us in one launch, 258 in two), not on
-// the largest grids, where FP64 arithmetic alone counts.  A user's choice of streams (sbp_set_tuning) keeps the strips
-// in a launch of their own.
+// the largest grids, where FP64 arithmetic alone counts.  (Where it is one launch there is nothing for the overlap of
+// sbp_set_tuning to run side by side.)
 inline bool one_launch(const sbp_handle* h, int mode) {
-    if (h->prof || h->overlap || h->nblocks > MARCH_MAX_BLOCKS || h->stencil != SBP_STENCIL_NARROW) return false;
+    if (h->nblocks > MARCH_MAX_BLOCKS || h->stencil != SBP_STENCIL_NARROW) return false;
     if (h->precision == SBP_FP32) return mode == 0 && h->ntrefs == 0 && (h->shorts.d_tiles || h->ntiles <= h->num_sms);
     return mode != 1 && h->blocks[0].e && (h->strip_len == 8 || (h->strip_len == 16 && h->ntrefs == 0));
 }
