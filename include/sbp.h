@@ -355,8 +355,8 @@ int sbp_batch_remove(sbp_batch* b, int slot, void* stream);
  * of the admitted shots evenly over the CTAs).  Only while the batch is empty. */
 int sbp_batch_set_rows(sbp_batch* b, int rows);
 
-/* Pick the tile shape (rows of an interior work item: 32, 64, 128 or 256) by timing batch steps of
- * a representative shot h alone; h's levels, parity and time are restored afterwards (one copy of
+/* Pick the tile shape (rows of an interior work item: 0, the default of sbp_batch_set_rows, or a fixed height
+ * of 32, 64, 128 or 256 where that is clearly faster) by timing batch steps of a representative shot h alone; h's levels, parity and time are restored afterwards (one copy of
  * its state is allocated for the call).  The batch must be empty; the choice is kept by the batch
  * and written to *rows_out (may be NULL). */
 int sbp_batch_autotune(sbp_batch* b, sbp_handle* h, int* rows_out);
