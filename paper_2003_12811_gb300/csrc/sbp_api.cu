@@ -1970,8 +1970,8 @@ int batch_sync(sbp_batch* b, cudaStream_t st) {
     for (int s = 0; s < b->max_shots; ++s)
         if (b->shot[s]) {
             const int2 sz = shape[q++];
-            // bands of equal height
-            const int bands = (sz.y + rows - 1) / rows, high = (sz.y + bands - 1) / bands;
+            // bands of equal height (a caller's height may be any positive int)
+            const int r = std::min(rows, sz.y), bands = (sz.y + r - 1) / r, high = (sz.y + bands - 1) / bands;
             for (int k = 0; k < sz.x * ((sz.y + high - 1) / high); ++k) items.push_back(make_int4(s, 0, k, high));
         }
     for (int s = 0; s < b->max_shots; ++s)

@@ -166,8 +166,8 @@ int launch_step(sbp_handle* h, const StepArgs& a, int mode, cudaStream_t st, boo
             for (auto& hb : h->blocks) grids.push_back(make_int2(march_ncx(hb.n1, S), hb.n2 - 2 * S));
             const int even = h->rows_per_cta > 0 ? h->rows_per_cta : item_rows(4 * h->num_sms, grids, ss.n, false);
             for (auto& hb : h->blocks) {
-                const int ncx = march_ncx(hb.n1, S), n2i = hb.n2 - 2 * S, bands = (n2i + even - 1) / even;
-                const int rows = h->rows_per_cta > 0 ? std::min(n2i, even) : (n2i + bands - 1) / bands;
+                const int ncx = march_ncx(hb.n1, S), n2i = hb.n2 - 2 * S, most = std::min(n2i, even), bands = (n2i + most - 1) / most;
+                const int rows = h->rows_per_cta > 0 ? most : (n2i + bands - 1) / bands;
                 const int k = mm.nb++;
                 mm.maps[k] = adj ? hb.pmaps : hb.mmaps;
                 mm.b[k] = adj ? make_view_adj(h, hb) : make_view(h, hb);
