@@ -210,11 +210,18 @@ int sbp_step_graph(sbp_handle* h, int nsteps, double dt, void* stream);
 
 /* Device bytes a handle for `desc` holds after sbp_grid_create, sbp_set_material and
  * sbp_set_state (fields, coefficients, metric, closure matrices of D_xx^FC, face buffers and
- * interface traces, tensor maps), used to admit solves by HBM footprint.  No device work.  FP64
- * handles keep 18 more planes (order 6; 12 / 6 for order 4 / 2) of interior edge weights where the
- * device has eight times that much memory free at sbp_grid_create, and give them back when a later
- * allocation of the handle finds no room; they are not counted. */
+ * interface traces, tensor maps), used to admit solves by HBM footprint.  No device work.  The edge weights
+ * that an FP64 handle may hold besides (sbp_edge_weights) are not counted. */
 int sbp_grid_footprint(const sbp_grid_desc* desc, long long* bytes_out);
+
+/* FP64 handles of the narrow stencil keep 18 more planes (order 6; 12 / 6 for order 4 / 2) of interior edge weights,
+ * with which a step takes half the time, where there is room for them when the material of every block is set: within
+ * an eighth of the memory that is free then, and, over all handles of the process, within a 64th of the device's.
+ * They go back to the device, for good, when an allocation of any handle finds no room.  With and without them results
+ * differ in the last bits.  keep = 0: give them back now and take no more (callers that plan with
+ * sbp_grid_footprint to the last byte); 1: take them if there is room (the default); -1: neither.
+ * *bytes_out (may be NULL): what the handle holds of them after the call. */
+int sbp_edge_weights(sbp_handle* h, int keep, long long* bytes_out);
 
 /* Pick the launch tuning for this grid by timing candidates on leapfrog steps from the current
  * state (the overwritten level is saved and restored: the state is left unchanged; device memory

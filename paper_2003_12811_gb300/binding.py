@@ -89,6 +89,7 @@ def lib():
         L.sbp_energy.argtypes = [C.c_void_p, C.c_double, _DP]
         L.sbp_suggest_dt.argtypes = [C.c_void_p, C.c_double, _DP]
         L.sbp_get_time.argtypes = [C.c_void_p, _DP]
+        L.sbp_edge_weights.argtypes = [C.c_void_p, C.c_int, C.POINTER(C.c_longlong)]
         L.sbp_profile.argtypes = [C.c_void_p, C.c_int]
         L.sbp_step_graph.argtypes = [C.c_void_p, C.c_int, C.c_double, C.c_void_p]
         L.sbp_grid_footprint.argtypes = [C.POINTER(GridDesc), C.POINTER(C.c_longlong)]
@@ -190,7 +191,8 @@ def footprint_bytes(problem, precision="fp32"):
 class Solver:
     """A libsbp handle built from a ``workloads.Problem``."""
 
-    def __init__(self, problem, precision="fp64"):
+    def __init__(self, problem, precision="fp64", edge_weights=True):
+        """edge_weights=False: an FP64 handle holds no more than ``footprint_bytes`` (sbp_edge_weights)."""
         self.L = lib()
         self.problem = problem
         self.precision = FP64 if precision == "fp64" else FP32
@@ -201,6 +203,8 @@ class Solver:
             raise SbpError(rc, self.L.sbp_last_error(None).decode())
         self.h = h
         try:
+            if not edge_weights:
+                self.sbp_edge_weights(0)
             self._setup()
         except Exception:
             self.close()
@@ -239,6 +243,12 @@ class Solver:
                                                     s.direction[1], s.amplitude, s.alpha_p, s.t0))
 
     # ---------------------------------------------------------------- C entry points
+    def sbp_edge_weights(self, keep=-1):
+        """Give back (0), take (1) or leave (-1) the FP64 interior edge weights; returns the bytes held of them."""
+        out = C.c_longlong()
+        self._check(self.L.sbp_edge_weights(self.h, int(keep), C.byref(out)))
+        return int(out.value)
+
     def sbp_set_material(self, block, rho, Cplanes, layout=C_PAIR10):
         """rho (N2, N1); Cplanes (10, N2, N1) pair layout or (6, N2, N1) Voigt layout."""
         r, c = _f64(rho), _f64(Cplanes)

@@ -13,6 +13,10 @@
 
 using namespace sbp3;
 
+namespace sbphost {
+cudaError_t device_malloc(void** p, size_t bytes);      // sbp_api.cu
+}
+
 namespace {
 
 thread_local std::string g3_create_error;
@@ -329,7 +333,7 @@ int sbp3_create(int order, int precision, int n1, int n2, int n3, const double* 
         h->face_nodes = nodes > h->face_nodes ? nodes : h->face_nodes;
     }
     auto alloc = [&](void** p, size_t bytes) -> bool {
-        if (cudaMalloc(p, bytes) != cudaSuccess) return false;
+        if (sbphost::device_malloc(p, bytes) != cudaSuccess) return false;
         return cudaMemset(*p, 0, bytes) == cudaSuccess;
     };
     const size_t fb = (size_t)h->fs * h->es;
@@ -380,7 +384,7 @@ int sbp3_set_material(sbp3_handle* h, int i3_begin, int i3_count, const double* 
         if (!std::isfinite(C45[i])) return fail(h, SBP_E_INVALID_ARG, "C45 has a non-finite value");
     DeviceGuard dg(h->device);
     double* buf = nullptr;
-    CK3(h, cudaMalloc(&buf, 46 * np * sizeof(double)));
+    CK3(h, sbphost::device_malloc((void**)&buf, 46 * np * sizeof(double)));
     cudaError_t e = cudaMemcpy(buf, rho, np * sizeof(double), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(buf + np, C45, 45 * np * sizeof(double), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(h->d_err, 0, sizeof(int));
@@ -412,7 +416,7 @@ int sbp3_set_state(sbp3_handle* h, const double* u_prev, const double* u_cur) {
     const long long N = (long long)h->n[0] * h->n[1] * h->n[2];
     DeviceGuard dg(h->device);
     double* buf = nullptr;
-    CK3(h, cudaMalloc(&buf, 6 * N * sizeof(double)));
+    CK3(h, sbphost::device_malloc((void**)&buf, 6 * N * sizeof(double)));
     cudaError_t e = cudaMemcpy(buf, u_prev, 3 * N * sizeof(double), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(buf + 3 * N, u_cur, 3 * N * sizeof(double), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
@@ -440,7 +444,7 @@ int sbp3_get_state(sbp3_handle* h, double* u_prev, double* u_cur) {
     const long long N = (long long)h->n[0] * h->n[1] * h->n[2];
     DeviceGuard dg(h->device);
     double* buf = nullptr;
-    CK3(h, cudaMalloc(&buf, 6 * N * sizeof(double)));
+    CK3(h, sbphost::device_malloc((void**)&buf, 6 * N * sizeof(double)));
     const dim3 blk(128), grd((h->n[0] + 127) / 128, h->n[1], h->n[2]);
     if (h->precision == SBP_FP32) {
         k3_store_field<float><<<grd, blk>>>(h->g, (const float*)h->u[1 - h->cur], buf);
@@ -463,10 +467,10 @@ int sbp3_apply(sbp3_handle* h, const double* u, double* accel) {
     const long long N = (long long)h->n[0] * h->n[1] * h->n[2];
     DeviceGuard dg(h->device);
     const size_t fb = (size_t)h->fs * h->es;
-    if (!h->ain) CK3(h, cudaMalloc(&h->ain, 3 * fb));
-    if (!h->aout) CK3(h, cudaMalloc(&h->aout, 3 * fb));
+    if (!h->ain) CK3(h, sbphost::device_malloc(&h->ain, 3 * fb));
+    if (!h->aout) CK3(h, sbphost::device_malloc(&h->aout, 3 * fb));
     double* buf = nullptr;
-    CK3(h, cudaMalloc(&buf, 3 * N * sizeof(double)));
+    CK3(h, sbphost::device_malloc((void**)&buf, 3 * N * sizeof(double)));
     cudaError_t e = cudaMemcpy(buf, u, 3 * N * sizeof(double), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         cudaFree(buf);
@@ -518,8 +522,8 @@ int sbp3_autotune(sbp3_handle* h, int* variant_out, double* ms_out) {
     if (!check_range(h)) return fail(h, SBP_E_STATE, "material not set for every x3-plane");
     DeviceGuard dg(h->device);
     const size_t fb = (size_t)h->fs * h->es;
-    if (!h->ain) CK3(h, cudaMalloc(&h->ain, 3 * fb));
-    if (!h->aout) CK3(h, cudaMalloc(&h->aout, 3 * fb));
+    if (!h->ain) CK3(h, sbphost::device_malloc(&h->ain, 3 * fb));
+    if (!h->aout) CK3(h, sbphost::device_malloc(&h->aout, 3 * fb));
     // operator applications on the current level (or on zeros before any state): the state is untouched
     if (h->state) CK3(h, cudaMemcpy(h->ain, h->u[h->cur], 3 * fb, cudaMemcpyDeviceToDevice));
     else CK3(h, cudaMemset(h->ain, 0, 3 * fb));

@@ -24,23 +24,130 @@ int sync_views(sbp_handle* h) {
 
 }  // namespace
 
-// gives the edge weights of every block back to the device (an allocation of the handle found no room);
-// the interior then forms them in the kernel again.  False if there were none.
-bool sbphost::drop_edges(sbp_handle* h) {
-    bool any = false;
-    for (auto& hb : h->blocks) any = any || hb.e;
-    if (!any) return false;
-    cudaGetLastError();
+// ---------------------------------------------------------------------------------------------
+// Interior edge weights (FP64, narrow stencil): planes that a handle can do without.  They are taken once the material
+// of every block is set, within an eighth of the free memory and, over all handles of the process, a 64th of the
+// device's; and they go back to the device when an allocation of any handle finds no room, for good unless
+// sbp_edge_weights asks for them (a handle that short of memory would take and lose them again and again).
+namespace {
+struct EdgePool {
+    std::recursive_mutex m;               // taken after a handle's own `use`; other handles' `use` is only tried
+    std::vector<sbp_handle*> holders;
+    size_t bytes = 0;
+};
+EdgePool& edge_pool() {
+    static EdgePool p;
+    return p;
+}
+
+void forget_edges(sbp_handle* h) {
+    EdgePool& pool = edge_pool();
+    std::lock_guard<std::recursive_mutex> lock(pool.m);
+    auto it = std::find(pool.holders.begin(), pool.holders.end(), h);
+    if (it == pool.holders.end()) return;
+    pool.holders.erase(it);
+    pool.bytes -= h->edge_bytes;
+    h->edge_bytes = 0;
+}
+
+void drop_graph(sbp_handle* h) {
+    if (h->graph_exec) cudaGraphExecDestroy(h->graph_exec);
+    h->graph_exec = nullptr;
+}
+
+// gives the edge weights of every block back to the device (h->use is held); the interior then forms them in the
+// kernel again, as do steps that a caller has captured.  False if there were none.
+bool drop_edges(sbp_handle* h) {
+    if (h->edge_bytes == 0) return false;
+    forget_edges(h);
+    h->edges_wanted = false;
+    std::vector<void*> planes;
     cudaDeviceSynchronize();
     for (auto& hb : h->blocks) {
-        h->dfree(hb.e);
+        planes.push_back(hb.e);
         hb.e = nullptr;
     }
-    if (h->graph_exec) {
-        cudaGraphExecDestroy(h->graph_exec);
-        h->graph_exec = nullptr;
+    drop_graph(h);
+    const bool ok = sync_views(h) == SBP_OK;
+    if (ok)                               // (no kernel reads them from here on)
+        for (void* p : planes) h->dfree(p);
+    return ok;
+}
+
+// edge weights of block b
+void form_edges(sbp_handle* h, HostBlock& hb) {
+    const BlockDev b = make_view(h, hb);
+    const unsigned g = grid_for((long long)hb.n1 * hb.n2);
+    if (h->order == 2) k_edge_weights<double, 2><<<g, 256>>>(b, (double*)hb.e);
+    else if (h->order == 4) k_edge_weights<double, 4><<<g, 256>>>(b, (double*)hb.e);
+    else k_edge_weights<double, 6><<<g, 256>>>(b, (double*)hb.e);
+}
+
+// planes for the edge weights of every block, where there is room, and their values
+int take_edges(sbp_handle* h) {
+    if (h->precision != SBP_FP64 || h->stencil != SBP_STENCIL_NARROW || !h->edges_wanted || h->edge_bytes > 0) return SBP_OK;
+    auto bytes = [&](const HostBlock& hb) { return 6 * (size_t)order_q(h->order) * hb.n2 * hb.pitch * h->esize; };
+    size_t want = 0, freeb = 0, totalb = 0;
+    for (auto& hb : h->blocks) want += bytes(hb);
+    EdgePool& pool = edge_pool();
+    {
+        std::lock_guard<std::recursive_mutex> lock(pool.m);
+        if (cudaMemGetInfo(&freeb, &totalb) != cudaSuccess || want > freeb / 8 || pool.bytes + want > totalb / 64) {
+            cudaGetLastError();
+            return SBP_OK;
+        }
+        std::vector<void*> planes;
+        for (auto& hb : h->blocks) {
+            void* p = nullptr;
+            if (cudaMalloc(&p, bytes(hb)) != cudaSuccess) {
+                cudaGetLastError();
+                for (void* q : planes) cudaFree(q);
+                return SBP_OK;
+            }
+            planes.push_back(p);
+        }
+        for (size_t b = 0; b < planes.size(); ++b) {
+            h->allocs.push_back(planes[b]);
+            h->blocks[b].e = planes[b];
+        }
+        h->edge_bytes = want;
+        pool.holders.push_back(h);
+        pool.bytes += want;
     }
-    return !h->d_blocks || sync_views(h) == SBP_OK;
+    drop_graph(h);
+    for (auto& hb : h->blocks) {
+        cudaMemset(hb.e, 0, bytes(hb));
+        form_edges(h, hb);
+    }
+    const int rc = sync_views(h);
+    return rc != SBP_OK ? rc : check_cuda(h, "edge weights");
+}
+}  // namespace
+
+// an allocation found no room (h: the handle it was for, whose `use` is held, or null): the edge weights of that handle,
+// or else of another one that is not in use, go back to the device.  False if there are none.
+bool sbphost::reclaim_edges(sbp_handle* h) {
+    if (h && drop_edges(h)) return true;
+    EdgePool& pool = edge_pool();
+    std::lock_guard<std::recursive_mutex> lock(pool.m);
+    const std::vector<sbp_handle*> others = pool.holders;
+    for (sbp_handle* o : others) {
+        if (o == h || !o->use.try_lock()) continue;
+        const bool got = drop_edges(o);
+        o->use.unlock();
+        if (got) return true;
+    }
+    return false;
+}
+
+// an allocation that belongs to no 2-D handle (batches, 3-D handles)
+cudaError_t sbphost::device_malloc(void** p, size_t bytes) {
+    cudaError_t e;
+    while ((e = cudaMalloc(p, bytes)) != cudaSuccess) {
+        cudaGetLastError();
+        if (!reclaim_edges(nullptr)) break;
+    }
+    return e;
 }
 
 namespace {
@@ -634,26 +741,13 @@ int sbp_grid_create(const sbp_grid_desc* desc, sbp_handle** out) {
         cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(0) != cudaSuccess)
         return cleanup(SBP_E_CUDA, "metric setup failed");
     if (flag) return cleanup(SBP_E_JACOBIAN_NONPOSITIVE, "non-positive Jacobian determinant");
-    // FP64: planes for the interior edge weights.  They are no part of what the handle needs
-    // (sbp_grid_footprint), so they are taken only where they leave seven eighths of the free memory to
-    // others, and given back when an allocation of the handle finds no room.
-    if (h->precision == SBP_FP64 && h->stencil == SBP_STENCIL_NARROW) {
-        size_t want = 0, freeb = 0, totalb = 0;
-        for (auto& hb : h->blocks) want += 6 * (size_t)order_q(o) * hb.n2 * hb.pitch * h->esize;
-        bool room = cudaMemGetInfo(&freeb, &totalb) == cudaSuccess && want <= freeb / 8;
-        for (auto& hb : h->blocks)
-            if (room) room = (hb.e = h->dalloc(6 * (size_t)order_q(o) * hb.n2 * hb.pitch * h->esize)) != nullptr;
-        for (auto& hb : h->blocks) room = room && hb.e;    // a failing allocation takes back the ones before it
-        if (!room) drop_edges(h);
-        cudaGetLastError();
-        if (sync_views(h) != SBP_OK) return cleanup(SBP_E_CUDA, h->err);
-    }
     *out = h;
     return SBP_OK;
 }
 
 int sbp_destroy(sbp_handle* h) {
     if (!h) return SBP_OK;
+    forget_edges(h);
     for (void* p : h->allocs)
         if (p) cudaFree(p);
     for (auto& pd : h->pending) {
@@ -673,6 +767,7 @@ int sbp_destroy(sbp_handle* h) {
 
 int sbp_set_material(sbp_handle* h, int block, const double* rho, const double* C, int c_layout) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (block < 0 || block >= h->nblocks) return h->fail(SBP_E_INVALID_ARG, "bad block index");
     if (!rho || !C) return h->fail(SBP_E_INVALID_ARG, "null material arrays");
     if (c_layout != SBP_C_PAIR10 && c_layout != SBP_C_VOIGT6) return h->fail(SBP_E_INVALID_ARG, "c_layout must be SBP_C_PAIR10 or SBP_C_VOIGT6");
@@ -710,19 +805,20 @@ int sbp_set_material(sbp_handle* h, int block, const double* rho, const double* 
         else if (h->order == 4) { k_closure_mats<float, 4><<<grid_for(nx), 256>>>(b, 0, (float*)hb.mx); k_closure_mats<float, 4><<<grid_for(ny), 256>>>(b, 1, (float*)hb.my); }
         else { k_closure_mats<float, 6><<<grid_for(nx), 256>>>(b, 0, (float*)hb.mx); k_closure_mats<float, 6><<<grid_for(ny), 256>>>(b, 1, (float*)hb.my); }
     }
-    if (hb.e) {
-        if (h->order == 2) k_edge_weights<double, 2><<<grid_for((long long)n), 256>>>(b, (double*)hb.e);
-        else if (h->order == 4) k_edge_weights<double, 4><<<grid_for((long long)n), 256>>>(b, (double*)hb.e);
-        else k_edge_weights<double, 6><<<grid_for((long long)n), 256>>>(b, (double*)hb.e);
+    if (hb.e) form_edges(h, hb);
+    hb.material = true;
+    if (all_materials(h)) {
+        const int rc = take_edges(h);
+        if (rc != SBP_OK) return rc;
     }
     cudaError_t e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) return h->fail(SBP_E_CUDA, std::string("material: ") + cudaGetErrorString(e));
-    hb.material = true;
     return SBP_OK;
 }
 
 int sbp_set_robin(sbp_handle* h, int block, int face, const double* U) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (block < 0 || block >= h->nblocks || face < 0 || face > 3 || !U) return h->fail(SBP_E_INVALID_ARG, "bad arguments");
     HostFace& F = h->blocks[block].f[face];
     if (F.kind != SBP_BC_ROBIN) return h->fail(SBP_E_INVALID_ARG, "face is not a Robin face");
@@ -745,6 +841,7 @@ int sbp_set_robin(sbp_handle* h, int block, int face, const double* U) {
 
 int sbp_set_robin_damping(sbp_handle* h, int block, int face, const double* V) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (block < 0 || block >= h->nblocks || face < 0 || face > 3 || !V) return h->fail(SBP_E_INVALID_ARG, "bad arguments");
     HostFace& F = h->blocks[block].f[face];
     if (F.kind != SBP_BC_ROBIN) return h->fail(SBP_E_INVALID_ARG, "face is not a Robin face");
@@ -774,6 +871,7 @@ int sbp_set_robin_damping(sbp_handle* h, int block, int face, const double* V) {
 
 int sbp_set_layer_dissipation(sbp_handle* h, int block, const double* s) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (block < 0 || block >= h->nblocks || !s) return h->fail(SBP_E_INVALID_ARG, "bad arguments");
     HostBlock& hb = h->blocks[block];
     const size_t n = (size_t)hb.n1 * hb.n2;
@@ -828,6 +926,7 @@ int sbp_set_layer_dissipation(sbp_handle* h, int block, const double* s) {
 
 int sbp_set_time_basis(sbp_handle* h, int nbasis, const int* kinds, const double* omegas) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (nbasis < 0 || nbasis > 8 || (nbasis > 0 && (!kinds || !omegas))) return h->fail(SBP_E_INVALID_ARG, "bad time basis");
     for (int k = 0; k < nbasis; ++k)
         if (kinds[k] != 0 && kinds[k] != 1) return h->fail(SBP_E_INVALID_ARG, "basis kind must be 0 (sin) or 1 (cos)");
@@ -848,6 +947,7 @@ int sbp_set_time_basis(sbp_handle* h, int nbasis, const int* kinds, const double
 
 int sbp_set_boundary_data(sbp_handle* h, int block, int face, const double* g) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (block < 0 || block >= h->nblocks || face < 0 || face > 3 || !g) return h->fail(SBP_E_INVALID_ARG, "bad arguments");
     if (h->nbasis == 0) return h->fail(SBP_E_STATE, "set the time basis first");
     HostFace& F = h->blocks[block].f[face];
@@ -869,6 +969,7 @@ int sbp_set_boundary_data(sbp_handle* h, int block, int face, const double* g) {
 
 int sbp_set_forcing(sbp_handle* h, int block, const double* f) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (block < 0 || block >= h->nblocks || !f) return h->fail(SBP_E_INVALID_ARG, "bad arguments");
     if (h->nbasis == 0) return h->fail(SBP_E_STATE, "set the time basis first");
     HostBlock& hb = h->blocks[block];
@@ -890,6 +991,7 @@ int sbp_set_forcing(sbp_handle* h, int block, const double* f) {
 int sbp_add_point_source(sbp_handle* h, int block, double x1, double x2, double f1, double f2, double amplitude,
                          double alpha_p, double t0) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (block < 0 || block >= h->nblocks) return h->fail(SBP_E_INVALID_ARG, "bad block");
     if (!(x1 >= 0 && x1 <= 1 && x2 >= 0 && x2 <= 1)) return h->fail(SBP_E_INVALID_ARG, "source outside the block");
     if (!std::isfinite(alpha_p) || !std::isfinite(t0) || !std::isfinite(amplitude)) return h->fail(SBP_E_INVALID_ARG, "non-finite source");
@@ -931,6 +1033,7 @@ int sbp_add_point_source(sbp_handle* h, int block, double x1, double x2, double 
 
 int sbp_set_state(sbp_handle* h, int block, const double* u_prev, const double* u_cur, double t) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (block < 0 || block >= h->nblocks || !u_prev || !u_cur) return h->fail(SBP_E_INVALID_ARG, "bad arguments");
     HostBlock& hb = h->blocks[block];
     const size_t n = (size_t)hb.n1 * hb.n2;
@@ -983,6 +1086,7 @@ int check_device_buffer(sbp_handle* h, const void* p, long long pitch, const Hos
 int sbp_set_state_device(sbp_handle* h, int block, const void* u_prev, const void* u_cur, long long pitch, double t,
                          void* stream) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (block < 0 || block >= h->nblocks) return h->fail(SBP_E_INVALID_ARG, "bad block index");
     HostBlock& hb = h->blocks[block];
     int rc = check_device_buffer(h, u_prev, pitch, hb, "u_prev");
@@ -1004,6 +1108,7 @@ int sbp_set_state_device(sbp_handle* h, int block, const void* u_prev, const voi
 
 int sbp_get_field_device(sbp_handle* h, int block, int which, void* dst, long long pitch, void* stream) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (block < 0 || block >= h->nblocks || which < 0 || which > 3) return h->fail(SBP_E_INVALID_ARG, "bad arguments");
     HostBlock& hb = h->blocks[block];
     if (which == SBP_FIELD_VELOCITY && !hb.rk) return h->fail(SBP_E_STATE, "no RK4 state on this block");
@@ -1019,6 +1124,7 @@ int sbp_get_field_device(sbp_handle* h, int block, int which, void* dst, long lo
 
 int sbp_step(sbp_handle* h, int nsteps, double dt, void* stream) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (nsteps < 0 || !(dt > 0) || !std::isfinite(dt)) return h->fail(SBP_E_INVALID_ARG, "bad step arguments");
     if (!all_materials(h)) return h->fail(SBP_E_STATE, "set the material of every block first");
     cudaStream_t st = (cudaStream_t)stream;
@@ -1041,6 +1147,7 @@ int sbp_step(sbp_handle* h, int nsteps, double dt, void* stream) {
 
 int sbp_set_state_rk4(sbp_handle* h, int block, const double* u, const double* v, double t) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (block < 0 || block >= h->nblocks || !u || !v) return h->fail(SBP_E_INVALID_ARG, "bad arguments");
     HostBlock& hb = h->blocks[block];
     const size_t n = (size_t)hb.n1 * hb.n2, plane = (size_t)hb.n2 * hb.pitch;
@@ -1071,6 +1178,7 @@ int sbp_set_state_rk4(sbp_handle* h, int block, const double* u, const double* v
 
 int sbp_step_rk4(sbp_handle* h, int nsteps, double dt, void* stream) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (nsteps < 0 || !(dt > 0) || !std::isfinite(dt)) return h->fail(SBP_E_INVALID_ARG, "bad step arguments");
     if (!all_materials(h)) return h->fail(SBP_E_STATE, "set the material of every block first");
     for (auto& hb : h->blocks)
@@ -1104,6 +1212,7 @@ int sbp_step_rk4(sbp_handle* h, int nsteps, double dt, void* stream) {
 
 int sbp_apply(sbp_handle* h, int with_data, double t) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (!all_materials(h)) return h->fail(SBP_E_STATE, "set the material of every block first");
     StepArgs a{};
     a.cur = h->cur;
@@ -1118,6 +1227,7 @@ int sbp_apply(sbp_handle* h, int with_data, double t) {
 
 int sbp_get_field(sbp_handle* h, int block, int which, double* dst) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (block < 0 || block >= h->nblocks || !dst || which < 0 || which > 3) return h->fail(SBP_E_INVALID_ARG, "bad arguments");
     HostBlock& hb = h->blocks[block];
     const size_t n = (size_t)hb.n1 * hb.n2;
@@ -1135,6 +1245,7 @@ int sbp_get_field(sbp_handle* h, int block, int which, double* dst) {
 
 int sbp_energy(sbp_handle* h, double dt, double* E_out) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (!E_out || !(dt > 0)) return h->fail(SBP_E_INVALID_ARG, "bad arguments");
     if (!all_materials(h)) return h->fail(SBP_E_STATE, "set the material of every block first");
     StepArgs a{};
@@ -1168,6 +1279,7 @@ int sbp_energy(sbp_handle* h, double dt, double* E_out) {
 
 int sbp_l2_diff(sbp_handle* h, int which, const double* const* ref, double* err2_out, double* ref2_out) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (!ref || which < 0 || which > 3) return h->fail(SBP_E_INVALID_ARG, "bad arguments");
     for (int b = 0; b < h->nblocks; ++b)
         if (!ref[b]) return h->fail(SBP_E_INVALID_ARG, "null reference array");
@@ -1205,6 +1317,7 @@ int sbp_l2_diff(sbp_handle* h, int which, const double* const* ref, double* err2
 
 int sbp_suggest_dt(sbp_handle* h, double cfl, double* dt_out) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (!dt_out || !(cfl > 0)) return h->fail(SBP_E_INVALID_ARG, "bad arguments");
     if (!all_materials(h)) return h->fail(SBP_E_STATE, "set the material of every block first");
     // two passes over every block (the operator-output planes serve as scratch for the per-node
@@ -1234,8 +1347,24 @@ int sbp_suggest_dt(sbp_handle* h, double cfl, double* dt_out) {
     return SBP_OK;
 }
 
+int sbp_edge_weights(sbp_handle* h, int keep, long long* bytes_out) {
+    if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
+    if (keep < -1 || keep > 1) return h->fail(SBP_E_INVALID_ARG, "keep must be -1, 0 or 1");
+    int rc = SBP_OK;
+    if (keep >= 0) h->edges_wanted = keep != 0;
+    if (keep == 0 && h->edge_bytes > 0 && !drop_edges(h)) rc = SBP_E_CUDA;
+    if (keep == 1 && all_materials(h)) {
+        rc = take_edges(h);
+        if (rc == SBP_OK && cudaStreamSynchronize(0) != cudaSuccess) rc = h->fail(SBP_E_CUDA, "edge weights");
+    }
+    if (bytes_out) *bytes_out = (long long)h->edge_bytes;
+    return rc;
+}
+
 int sbp_profile(sbp_handle* h, int enable) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     cudaDeviceSynchronize();
     for (auto& pd : h->pending) {
         h->ev_pool.push_back(pd.a);
@@ -1252,6 +1381,7 @@ int sbp_profile(sbp_handle* h, int enable) {
 
 int sbp_profile_read(sbp_handle* h, double* ms, long long* launches) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     for (auto& pd : h->pending) {
         float t = 0;
         if (cudaEventSynchronize(pd.b) != cudaSuccess || cudaEventElapsedTime(&t, pd.a, pd.b) != cudaSuccess)
@@ -1270,6 +1400,7 @@ int sbp_profile_read(sbp_handle* h, double* ms, long long* launches) {
 
 int sbp_apply_noalloc(sbp_handle* h, const void* u_dev, void* r_dev, int with_data, double t, void* stream) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (!u_dev || !r_dev) return h->fail(SBP_E_INVALID_ARG, "null device buffer");
     if (!all_materials(h)) return h->fail(SBP_E_STATE, "set the material of every block first");
     if (h->stencil != SBP_STENCIL_NARROW) return h->fail(SBP_E_STATE, "sbp_apply_noalloc applies the narrow stencil");
@@ -1342,6 +1473,7 @@ int sbp_apply_noalloc(sbp_handle* h, const void* u_dev, void* r_dev, int with_da
 
 int sbp_step_graph(sbp_handle* h, int nsteps, double dt, void* stream) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (nsteps <= 0 || (nsteps & 1) || !(dt > 0) || !std::isfinite(dt))
         return h->fail(SBP_E_INVALID_ARG, "sbp_step_graph needs an even positive step count and dt > 0");
     if (!all_materials(h)) return h->fail(SBP_E_STATE, "set the material of every block first");
@@ -1462,6 +1594,7 @@ int sbp_grid_footprint(const sbp_grid_desc* desc, long long* bytes_out) {
 
 int sbp_set_tuning(sbp_handle* h, int rows_per_cta, int overlap) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (rows_per_cta < 0) return h->fail(SBP_E_INVALID_ARG, "rows per CTA must be >= 0");
     if (overlap < -1 || overlap > 1) return h->fail(SBP_E_INVALID_ARG, "overlap must be -1, 0 or 1");
     const bool ov = overlap < 0 ? h->overlap : overlap != 0;
@@ -1476,6 +1609,7 @@ int sbp_set_tuning(sbp_handle* h, int rows_per_cta, int overlap) {
 
 int sbp_autotune(sbp_handle* h, int* rows_out, int* overlap_out) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (!all_materials(h)) return h->fail(SBP_E_STATE, "set the material of every block first");
     // candidates for the marching kernel's rows per CTA (FP32 only); 0 = heuristic (one wave of
     // 4 CTAs/SM per block); then whether the strips run concurrently with the interior.  Beside
@@ -1615,6 +1749,7 @@ int sbp_autotune(sbp_handle* h, int* rows_out, int* overlap_out) {
 
 int sbp_debug_wait_probe(sbp_handle* h, int polls) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (polls < 1 || polls > (1 << 20)) return h->fail(SBP_E_INVALID_ARG, "polls must be in [1, 2^20]");
     k_wait_probe<<<1, 32>>>(polls, h->d_err);
     return check_cuda(h, "wait probe launch");
@@ -1622,6 +1757,7 @@ int sbp_debug_wait_probe(sbp_handle* h, int polls) {
 
 int sbp_check(sbp_handle* h) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (cudaDeviceSynchronize() != cudaSuccess) return h->fail(SBP_E_CUDA, "device error");
     return check_kernel_errors(h);
 }
@@ -1644,6 +1780,7 @@ int sbp_get_info(const sbp_handle* h, long long* nodes_out, int* precision_out, 
 
 int sbp_set_receivers(sbp_handle* h, int nrec, const int* rec) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (nrec < 0 || (nrec > 0 && !rec)) return h->fail(SBP_E_INVALID_ARG, "bad receiver arguments");
     std::vector<RecDev> v;
     std::vector<std::pair<int, long long>> seen;
@@ -1677,6 +1814,7 @@ int sbp_set_receivers(sbp_handle* h, int nrec, const int* rec) {
 
 int sbp_record(sbp_handle* h, int nsteps, double dt, double* traces) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (nsteps < 0 || !(dt > 0) || !std::isfinite(dt)) return h->fail(SBP_E_INVALID_ARG, "bad step arguments");
     if (!all_materials(h)) return h->fail(SBP_E_STATE, "set the material of every block first");
     if (h->recs.empty()) return h->fail(SBP_E_STATE, "set the receivers first");
@@ -1700,6 +1838,7 @@ int sbp_record(sbp_handle* h, int nsteps, double dt, double* traces) {
 int sbp_misfit_gradient(sbp_handle* h, int nsteps, double dt, const double* observed, int checkpoint_every,
                         double* misfit, double* const* grad_rho, double* const* grad_C, int c_layout) {
     if (!h) return SBP_E_INVALID_ARG;
+    std::lock_guard<std::recursive_mutex> use(h->use);
     if (nsteps < 1 || !(dt > 0) || !std::isfinite(dt) || !observed || !misfit || checkpoint_every < 0)
         return h->fail(SBP_E_INVALID_ARG, "bad misfit-gradient arguments");
     if (c_layout != SBP_C_PAIR10 && c_layout != SBP_C_VOIGT6) return h->fail(SBP_E_INVALID_ARG, "c_layout must be SBP_C_PAIR10 or SBP_C_VOIGT6");
@@ -1982,7 +2121,7 @@ int batch_sync(sbp_batch* b, cudaStream_t st) {
         b->d_items = nullptr;
         b->items_cap = 0;
         const int cap = (int)items.size() * 2;
-        if (cudaMalloc(&b->d_items, sizeof(int4) * cap) != cudaSuccess) return b->fail(SBP_E_OOM, "batch work list");
+        if (device_malloc((void**)&b->d_items, sizeof(int4) * cap) != cudaSuccess) return b->fail(SBP_E_OOM, "batch work list");
         b->items_cap = cap;
     }
     if (!items.empty() &&
@@ -2035,8 +2174,8 @@ int sbp_batch_create(int order, int max_shots, sbp_batch** out) {
     if (b->num_sms <= 0) b->num_sms = 1;
     const int per_sm = order == 2 ? batch_ctas_per_sm<2>() : (order == 4 ? batch_ctas_per_sm<4>() : batch_ctas_per_sm<6>());
     b->ctas = std::max(1, per_sm) * b->num_sms;      // persistent: every CTA resident at once
-    if (cudaMalloc(&b->d_head, sizeof(BatchHead)) != cudaSuccess || cudaMalloc(&b->d_shots, sizeof(BatchShot) * max_shots) != cudaSuccess ||
-        cudaMalloc(&b->d_state, sizeof(BatchState) * max_shots) != cudaSuccess || cudaMalloc(&b->d_err, 64) != cudaSuccess) {
+    if (device_malloc((void**)&b->d_head, sizeof(BatchHead)) != cudaSuccess || device_malloc((void**)&b->d_shots, sizeof(BatchShot) * max_shots) != cudaSuccess ||
+        device_malloc((void**)&b->d_state, sizeof(BatchState) * max_shots) != cudaSuccess || device_malloc((void**)&b->d_err, 64) != cudaSuccess) {
         sbp_batch_destroy(b);
         return SBP_E_OOM;
     }
@@ -2199,7 +2338,7 @@ int sbp_batch_autotune(sbp_batch* b, sbp_handle* h, int* rows_out) {
     const HostBlock& hb = h->blocks[0];
     const size_t bytes = 2 * (size_t)hb.n2 * hb.pitch * h->esize;
     void* keep[2] = {nullptr, nullptr};
-    if (cudaMalloc(&keep[0], bytes) != cudaSuccess || cudaMalloc(&keep[1], bytes) != cudaSuccess) {
+    if (device_malloc(&keep[0], bytes) != cudaSuccess || device_malloc(&keep[1], bytes) != cudaSuccess) {
         if (keep[0]) cudaFree(keep[0]);
         return b->fail(SBP_E_OOM, "autotune state copy");
     }

@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <type_traits>
 #include <vector>
@@ -70,8 +71,7 @@ struct HostBlock {
     void* lscr = nullptr;     // leapfrog: the dissipation of the listed nodes between the pre and post kernels
     void* mx = nullptr;       // closure matrices of D_xx^FC along x1 / x2 (k_closure_mats, type T)
     void* my = nullptr;
-    void* e = nullptr;        // FP64 narrow stencil: interior edge weights (6 Q planes, k_edge_weights); given back
-                              // when a later allocation of the handle finds no room (drop_edges)
+    void* e = nullptr;        // FP64 narrow stencil: interior edge weights (6 Q planes, k_edge_weights), optional (take_edges)
 };
 
 inline int order_nb(int o) { return o == 2 ? SBP2_NB : (o == 4 ? SBP4_NB : SBP6_NB); }
@@ -99,7 +99,8 @@ inline double host_hweight(int o, int N, int i) {
 
 struct sbp_handle;
 namespace sbphost {
-bool drop_edges(sbp_handle* h);
+bool reclaim_edges(sbp_handle* h);
+cudaError_t device_malloc(void** p, size_t bytes);
 }
 
 struct sbp_handle {
@@ -134,6 +135,11 @@ struct sbp_handle {
     int device = 0;             // CUDA device current at sbp_grid_create (holds every buffer)
     std::string err;
     std::vector<void*> allocs;
+    // held by every call on the handle: another handle's call that finds no memory takes the edge weights from a handle
+    // that is not in use (reclaim_edges)
+    std::recursive_mutex use;
+    bool edges_wanted = true;     // sbp_edge_weights
+    size_t edge_bytes = 0;        // bytes of HostBlock::e over the blocks
     // kernel timing (benchmarks): the families of sbp_profile in include/sbp.h
     bool prof = false;
     double prof_ms[SBP_PROF_FAMILIES] = {0};
@@ -206,9 +212,9 @@ struct sbp_handle {
     }
     void* dalloc(size_t bytes, bool clear = true) {
         void* p = nullptr;
-        if (cudaMalloc(&p, bytes) != cudaSuccess && (!sbphost::drop_edges(this) || cudaMalloc(&p, bytes) != cudaSuccess)) {
+        while (cudaMalloc(&p, bytes) != cudaSuccess) {
             cudaGetLastError();   // reported as SBP_E_OOM by the caller; the next launch check starts clean
-            return nullptr;
+            if (!sbphost::reclaim_edges(this)) return nullptr;
         }
         if (clear) cudaMemset(p, 0, bytes);
         allocs.push_back(p);

@@ -67,7 +67,8 @@ class GpuBackend:
     def create(self, problem, cfl, dt=None):
         import numpy as np
         torch = self.torch
-        S = self.Solver(problem, self.precision)
+        # admitted by footprint: no memory beyond it
+        S = self.Solver(problem, self.precision, edge_weights=False)
         if dt is None:
             dt = S.suggest_dt(cfl)
         z = [np.zeros((2, b.N2, b.N1)) for b in problem.blocks]
