@@ -217,10 +217,11 @@ int sbp_grid_footprint(const sbp_grid_desc* desc, long long* bytes_out);
 /* FP64 handles of the narrow stencil keep 18 more planes (order 6; 12 / 6 for order 4 / 2) of interior edge weights,
  * with which a step takes half the time, where there is room for them when the material of every block is set: within
  * an eighth of the memory that is free then, and, over all handles of the process, within a 64th of the device's.
- * They go back to the device, for good, when an allocation of any handle finds no room.  With and without them results
- * differ in the last bits.  keep = 0: give them back now and take no more (callers that plan with
- * sbp_grid_footprint to the last byte); 1: take them if there is room (the default); -1: neither.
- * *bytes_out (may be NULL): what the handle holds of them after the call. */
+ * They go back to the device, for good, when an allocation of any handle finds no room, but not from a handle whose steps
+ * a caller has captured into a graph of its own (sbp_step, sbp_step_rk4 or sbp_step_graph on a capturing stream).  With and
+ * without them results differ in the last bits.  keep = 0: give them back now and take no more (callers that plan with
+ * sbp_grid_footprint to the last byte; SBP_E_STATE after such a capture); 1: take them if there is room (the default);
+ * -1: neither.  *bytes_out (may be NULL): what the handle holds of them after the call. */
 int sbp_edge_weights(sbp_handle* h, int keep, long long* bytes_out);
 
 /* Pick the launch tuning for this grid by timing candidates on leapfrog steps from the current

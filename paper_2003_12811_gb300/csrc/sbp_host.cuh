@@ -140,6 +140,7 @@ struct sbp_handle {
     std::recursive_mutex use;
     bool edges_wanted = true;     // sbp_edge_weights
     size_t edge_bytes = 0;        // bytes of HostBlock::e over the blocks
+    bool captured = false;        // a caller has captured steps that read them: they stay for good
     // kernel timing (benchmarks): the families of sbp_profile in include/sbp.h
     bool prof = false;
     double prof_ms[SBP_PROF_FAMILIES] = {0};

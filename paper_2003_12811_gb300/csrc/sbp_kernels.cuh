@@ -232,26 +232,6 @@ template <typename T, int O> __global__ void k_edge_weights(BlockDev B, T* __res
     }
 }
 
-// the narrow rows of an interior node from the coefficients: a step that a caller captured may run after the edge weights
-// went back to the device (su: the node in the staged displacement, its second component US elements on, row stride SX)
-template <typename T> struct Pair {
-    T a, b;
-};
-template <typename T, int O, int SX, int US>
-__device__ __noinline__ Pair<T> narrow_rows_of_c(const BlockDev& B, size_t gi, const T* su) {
-    const size_t plane = (size_t)B.n2 * B.pitch;
-    const long long P = B.pitch;
-    const T* __restrict__ C = reinterpret_cast<const T*>(B.c) + gi;
-    T x0 = T(0), x1 = T(0), y0 = T(0), y1 = T(0);
-    dxx_interior<O, T>(0, [&](int k) { return su[k]; }, [&](int k) { return su[US + k]; }, [&](int k) { return C[k]; },
-                       [&](int k) { return C[plane + k]; }, [&](int k) { return C[2 * plane + k]; }, x0, x1);
-    dxx_interior<O, T>(0, [&](int k) { return su[k * SX]; }, [&](int k) { return su[US + k * SX]; },
-                       [&](int k) { return C[3 * plane + k * P]; }, [&](int k) { return C[4 * plane + k * P]; },
-                       [&](int k) { return C[5 * plane + k * P]; }, y0, y1);
-    const T ih1 = ih1T<T>(B), ih2 = ih2T<T>(B);
-    return {x0 * ih1 * ih1 + y0 * ih2 * ih2, x1 * ih1 * ih1 + y1 * ih2 * ih2};
-}
-
 constexpr int IE_MAX_BLOCKS = 32;
 struct InteriorTiles {
     int nb, first;                     // blocks of this launch, the first one's index
@@ -331,19 +311,13 @@ __device__ __forceinline__ void interior_edges_tile(const BlockDev& B, int tile,
         if (r >= TY || gx >= lim1 || gy >= lim2) continue;
         const size_t gi = (size_t)gy * P + gx;
         T r0 = T(0), r1 = T(0);
-        if (E) {
-            dxx_edges<O, T>(
-                0, [&](int k) { return su[0][r + Q][c + Q + k]; }, [&](int k) { return su[1][r + Q][c + Q + k]; },
-                [&](int f, int m, int k) { return __ldg(E + (size_t)edge_plane<O>(0, f, m) * plane + gi + k); }, r0, r1);
-            dxx_edges<O, T>(
-                0, [&](int k) { return su[0][r + Q + k][c + Q]; }, [&](int k) { return su[1][r + Q + k][c + Q]; },
-                [&](int f, int m, int k) { return __ldg(E + (size_t)edge_plane<O>(1, f, m) * plane + gi + (long long)k * P); },
-                r0, r1);
-        } else {
-            const Pair<T> q = narrow_rows_of_c<T, O, SX, SY * SX>(B, gi, &su[0][r + Q][c + Q]);
-            r0 = q.a;
-            r1 = q.b;
-        }
+        dxx_edges<O, T>(
+            0, [&](int k) { return su[0][r + Q][c + Q + k]; }, [&](int k) { return su[1][r + Q][c + Q + k]; },
+            [&](int f, int m, int k) { return __ldg(E + (size_t)edge_plane<O>(0, f, m) * plane + gi + k); }, r0, r1);
+        dxx_edges<O, T>(
+            0, [&](int k) { return su[0][r + Q + k][c + Q]; }, [&](int k) { return su[1][r + Q + k][c + Q]; },
+            [&](int f, int m, int k) { return __ldg(E + (size_t)edge_plane<O>(1, f, m) * plane + gi + (long long)k * P); },
+            r0, r1);
 #pragma unroll
         for (int k = 1; k <= Q; ++k) {
             r0 += a1[k - 1] * (sg1[0][r][c + Q + k] - sg1[0][r][c + Q - k]);
