@@ -19,9 +19,10 @@ What is derived (Sec. 4 and 4.1 of Almquist & Dunham; coefficients are not print
   sparse (u-column, b-column, coefficient) triples, and the interior row written through
   "edge weights": row i = sum_{m=1..q} E_m(i) (u_{i+m} - u_i) + E_m(i-m) (u_{i-m} - u_i),
   E_m(i) = sum_k e_{m,k} b_{i+k}.  For gradients with respect to b near an end: per node k the
-  (row, u-column, coefficient) list of d(row)/d b_k, and per column k the non-zeros of D.
-  Every FP64 table has an FP32 twin (suffix _F) holding exactly the values a cast of the FP64
-  entry gives, so FP32 kernels read single-precision constants without converting them.
+  (row, u-column, coefficient) list of d(row)/d b_k.
+  Every FP64 table but that one, which kernels use as compile-time constants, has an FP32 twin (suffix _F) holding
+  exactly the values a cast of the FP64 entry gives, so FP32 kernels read single-precision constants without converting
+  them.
 """
 import os
 from math import comb
@@ -182,16 +183,11 @@ def analyse(order):
             tot[k - m] = tot.get(k - m, 0) - v
     assert {k: v for k, v in tot.items() if v != 0} == diag
     clos = [sorted(W[i].items()) for i in range(nclos)]
-    # transposed views for the gradient with respect to b near the left end (node k < GS = nclos + q):
-    # every (row, u-column, coefficient) with d(row of h^2 D_xx(b) u)/d b_k = sum coefficient * u_j,
-    # and every (row, D[row][k] h) of the column k of D
+    # transposed view for the gradient with respect to b near the left end (node k < GS = nclos + q):
+    # every (row, u-column, coefficient) with d(row of h^2 D_xx(b) u)/d b_k = sum coefficient * u_j
     gs = nclos + q
-    D, _, _, _, _ = full_D(order, N)
-    gn, dt = [], []
-    for k in range(gs):
-        gn.append(sorted((i, j, v) for i in range(N) for (j, kk), v in W[i].items() if kk == k))
-        dt.append([(r, D[r, k]) for r in range(N) if D[r, k] != 0])
-    return dict(hw=hw, Dq=Dq, a=a, nclos=nclos, clos=clos, edges=edges, gs=gs, gn=gn, dt=dt)
+    gn = [sorted((i, j, v) for i in range(N) for (j, kk), v in W[i].items() if kk == k) for k in range(gs)]
+    return dict(hw=hw, Dq=Dq, a=a, nclos=nclos, clos=clos, edges=edges, gs=gs, gn=gn)
 
 
 def cnum(v):
@@ -206,7 +202,7 @@ def fnum(v):
     return "%sf" % np.format_float_scientific(f, unique=True, exp_digits=2) if f != 0 else "0.0f"
 
 
-def table(out, typ, name, vals, dims):
+def table(out, typ, name, vals, dims, twin=True):
     """Emit a double table and its FP32 twin (name_F)."""
     shape = "".join("[%d]" % d for d in dims)
     if len(dims) == 2:
@@ -217,12 +213,13 @@ def table(out, typ, name, vals, dims):
         body = ", ".join(cnum(v) for v in vals)
         fbody = ", ".join(fnum(v) for v in vals)
     out.append("SBP_TABLE double %s%s = {%s};" % (name, shape, body))
-    out.append("SBP_TABLE float %s_F%s = {%s};" % (name, shape, fbody))
+    if twin:
+        out.append("SBP_TABLE float %s_F%s = {%s};" % (name, shape, fbody))
 
 
 def emit():
     out = ["// Generated by gen_tables.py -- SBP coefficient tables (Sec. 4, 4.1). Do not edit.",
-           "// included twice by sbp.cu: with SBP_TABLE = static __constant__ (device) and static const (host)", ""]
+           "// included with SBP_TABLE = static __constant__ (device) and static const (host)", ""]
     for order in (2, 4, 6):
         t = analyse(order)
         nb, ncol = BLOCK[order]
@@ -254,23 +251,18 @@ def emit():
         for m, e in enumerate(t["edges"], start=1):
             terms = " + ".join("T(%s) * B(%d)" % (cnum(v), k) for k, v in sorted(e.items()))
             out.append("#define %s_E%d(B) (%s)" % (P, m, terms))
-        # gradient tables: node k < GS from the left end (the right end is the mirror image, with
-        # the sign of D flipped)
+        # gradient table: node k < GS from the left end (the right end is the mirror image)
         out.append("#define %s_GS %d" % (P, t["gs"]))
-        for name, tab in (("GN", t["gn"]), ("DT", t["dt"])):
-            starts, rows, js, cs = [0], [], [], []
-            for ent in tab:
-                for e in ent:
-                    rows.append(e[0])
-                    if name == "GN":
-                        js.append(e[1])
-                    cs.append(e[-1])
-                starts.append(len(rows))
-            out.append("SBP_TABLE int %s_%s_START[%d] = {%s};" % (P.lower(), name, len(starts), ", ".join(map(str, starts))))
-            out.append("SBP_TABLE int %s_%s_ROW[%d] = {%s};" % (P.lower(), name, len(rows), ", ".join(map(str, rows))))
-            if name == "GN":
-                out.append("SBP_TABLE int %s_GN_J[%d] = {%s};" % (P.lower(), len(js), ", ".join(map(str, js))))
-            table(out, "double", "%s_%s_C" % (P.lower(), name), cs, [len(cs)])
+        starts, rows, js, cs = [0], [], [], []
+        for ent in t["gn"]:
+            for row, j, c in ent:
+                rows.append(row)
+                js.append(j)
+                cs.append(c)
+            starts.append(len(rows))
+        for name, vals in (("START", starts), ("ROW", rows), ("J", js)):
+            out.append("SBP_TABLE int %s_GN_%s[%d] = {%s};" % (P.lower(), name, len(vals), ", ".join(map(str, vals))))
+        table(out, "double", "%s_GN_C" % P.lower(), cs, [len(cs)], twin=False)
         lo = min(min(e) for e in t["edges"])
         hi = max(max(e) for e in t["edges"])
         out.append("#define %s_ELO %d" % (P, lo))

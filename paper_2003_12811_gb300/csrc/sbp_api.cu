@@ -2253,8 +2253,6 @@ int sbp_batch_add(sbp_batch* b, sbp_handle* h, int nsteps, double dt, int* slot_
     sh.dt2 = dt * dt;
     sh.dt2f = (float)sh.dt2;
     sh.beta = h->beta;
-    const int S = sh.view.strip;
-    const int n2i = hb.n2 - 2 * S;
     b->nstrip[slot] = h->ntiles;
     b->pending[slot] = BatchState{nsteps, h->cur, h->t};
     b->pending_set[slot] = 1;

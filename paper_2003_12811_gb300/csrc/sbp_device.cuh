@@ -36,14 +36,6 @@ template <int O> struct Ord;
         SBP_TWIN(dqT(int r, int c), sbpdev::sbp##O##_DQ[r][c], sbpdev::sbp##O##_DQ_F[r][c])             \
         SBP_TWIN(aT(int k), sbpdev::sbp##O##_A[k], sbpdev::sbp##O##_A_F[k])                             \
         SBP_TWIN(ccT(int t), sbpdev::sbp##O##_CLOS_C[t], sbpdev::sbp##O##_CLOS_C_F[t])                  \
-        /* gradient tables: node k < GS from the left end */                                            \
-        static __device__ __forceinline__ int gn_start(int k) { return sbpdev::sbp##O##_GN_START[k]; }  \
-        static __device__ __forceinline__ int gn_row(int t) { return sbpdev::sbp##O##_GN_ROW[t]; }      \
-        static __device__ __forceinline__ int gn_j(int t) { return sbpdev::sbp##O##_GN_J[t]; }          \
-        SBP_TWIN(gn_c(int t), sbpdev::sbp##O##_GN_C[t], sbpdev::sbp##O##_GN_C_F[t])                     \
-        static __device__ __forceinline__ int dt_start(int k) { return sbpdev::sbp##O##_DT_START[k]; }  \
-        static __device__ __forceinline__ int dt_row(int t) { return sbpdev::sbp##O##_DT_ROW[t]; }      \
-        SBP_TWIN(dt_c(int t), sbpdev::sbp##O##_DT_C[t], sbpdev::sbp##O##_DT_C_F[t])                     \
     };
 SBP_ORD(2)
 SBP_ORD(4)

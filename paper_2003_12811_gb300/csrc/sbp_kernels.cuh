@@ -205,8 +205,8 @@ __global__ void __launch_bounds__(ITHREADS) k_interior(BlockDev B, StepArgs a) {
 //  * One launch covers every block (no tail per block), in tiles of a shape that launch_interior_f64
 //    picks so that small grids still spread over all SMs.
 // A step of 4 order-6 blocks of 401^2 (0.6 M interior nodes): 0.19 ms for the one launch, where the kernel
-// with its own weights took 4 launches of 0.132 ms; at the FP64 units' rate the 142 instructions per node
-// take 0.13 ms.
+// with its own weights took 4 launches of 0.132 ms; at the FP64 units' rate the 157 instructions per node
+// (counted by ncu: 227 operations) take 0.15 ms.
 template <typename T, int O> __global__ void k_edge_weights(BlockDev B, T* __restrict__ E) {
     constexpr int Q = Ord<O>::Q;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -574,8 +574,8 @@ __device__ void face_sat_node(const BlockDev* __restrict__ blocks, const BlockDe
 
 // The same terms in SAT_PARTS independent parts, for as many threads; adds the part's share to Fs, As.  Part 0 has As
 // and what needs the face node alone; the others the normal and the tangential share of a Robin face's traction, or
-// the taps of the tangential transpose.  (One function for both, the parts chosen at compile time or run in turn,
-// made face_sat_node spill in the strip kernels: 2001^2 FP32 100.5 -> 104.7 us a step.)
+// the taps of the tangential transpose.  Interfaces have their traces here (the callers' steps form them first).  Apart from
+// face_sat_node, whose callers sum the terms of a node in one go and have few registers left for them.
 constexpr int SAT_PARTS = 4;
 // face_traction's part of the normal derivative (NORMAL) or of the tangential one, added to t0, t1
 template <typename T, int O, bool NORMAL, class UA, class CA>
@@ -639,18 +639,10 @@ __device__ __forceinline__ void face_sat_part(int part, const BlockDev* __restri
         return;
     }
     const bool intf = F.kind == FACE_INTF;
-    // the neighbour across an interface: its block, face, current level and coefficients
-    const BlockDev* V = intf ? &blocks[F.nbr_block] : nullptr;
-    const FaceDev* FV = intf ? &V->f[F.nbr_face] : nullptr;
-    const T* __restrict__ Uv = intf ? reinterpret_cast<const T*>(V->u[a.cur]) : nullptr;
-    const T* __restrict__ Cv = intf ? reinterpret_cast<const T*>(V->c) : nullptr;
-    const size_t pv = intf ? (size_t)V->n2 * V->pitch : 0;
-    auto uv = [&](int L, int j1, int j2) { return Uv[(size_t)L * pv + (size_t)j2 * V->pitch + j1]; };
-    auto cv = [&](int pl, int j1, int j2) { return Cv[(size_t)pl * pv + (size_t)j2 * V->pitch + j1]; };
-    // traces of both sides (k_face_trace, same level): replace the neighbour's reads and both tractions
+    // traces of both sides of an interface (k_face_trace, same level): the neighbour's displacement, both tractions and
+    // the penalty
     const T* __restrict__ trU = intf ? reinterpret_cast<const T*>(F.tr) : nullptr;
-    const T* __restrict__ trV = intf ? reinterpret_cast<const T*>(FV->tr) : nullptr;
-    const bool traced = trU != nullptr && trV != nullptr;
+    const T* __restrict__ trV = intf ? reinterpret_cast<const T*>(blocks[F.nbr_block].f[F.nbr_face].tr) : nullptr;
     // jump w_L at face node sp (displacement: u - g(t); interface: u - v)
     auto jump = [&](int sp, T& w0, T& w1) {
         int j1, j2;
@@ -659,15 +651,8 @@ __device__ __forceinline__ void face_sat_part(int part, const BlockDev* __restri
         w1 = u(1, j1, j2);
         if (intf) {
             const int svp = F.reversed ? nf - 1 - sp : sp;
-            if (traced) {
-                w0 -= trV[svp];
-                w1 -= trV[nf + svp];
-            } else {
-                int v1, v2;
-                face_at(*V, *FV, svp, 0, v1, v2);
-                w0 -= uv(0, v1, v2);
-                w1 -= uv(1, v1, v2);
-            }
+            w0 -= trV[svp];
+            w1 -= trV[nf + svp];
         } else if (has_data) {
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
@@ -687,42 +672,20 @@ __device__ __forceinline__ void face_sat_part(int part, const BlockDev* __restri
         if (!intf) {
             const T k = T(beta * dd * F.inv_h0);
             z00 = k * c00; z01 = k * c01; z11 = k * c11;
-        } else if (traced) {
+        } else {
             const int sv = F.reversed ? nf - 1 - s : s;
             z00 = trU[4 * nf + s] + trV[4 * nf + sv];
             z01 = trU[5 * nf + s] + trV[5 * nf + sv];
             z11 = trU[6 * nf + s] + trV[6 * nf + sv];
-        } else {
-            const int sv = F.reversed ? nf - 1 - s : s;
-            int v1, v2;
-            face_at(*V, *FV, sv, 0, v1, v2);
-            const int mv = FV->m;
-            const T ku = T(beta * dd / 4.0 * F.inv_h0), kv = T(beta * dd / 4.0 * FV->inv_h0);
-            const T zu00 = ku * c00, zu01 = ku * c01, zu11 = ku * c11;
-            const T zv00 = kv * cv(plane_nn(mv, 0, 0), v1, v2), zv01 = kv * cv(plane_nn(mv, 0, 1), v1, v2),
-                    zv11 = kv * cv(plane_nn(mv, 1, 1), v1, v2);
-            z00 = zu00 + zv00;
-            z01 = zu01 + zv01;
-            z11 = zu11 + zv11;
         }
         // normal-spread amplitude a_J = half nu c_mJmL w_L
         As0 += half * nu * (c00 * w0 + c01 * w1);
         As1 += half * nu * (c01 * w0 + c11 * w1);
         T f0 = -(z00 * w0 + z01 * w1), f1 = -(z01 * w0 + z11 * w1);
         if (intf) {
-            T tu0, tu1, tv0, tv1;
             const int sv = F.reversed ? nf - 1 - s : s;
-            if (traced) {
-                tu0 = trU[2 * nf + s];
-                tu1 = trU[3 * nf + s];
-                tv0 = trV[2 * nf + sv];
-                tv1 = trV[3 * nf + sv];
-            } else {
-                face_traction<T, O>(B, F, s, u, c, tu0, tu1);
-                face_traction<T, O>(*V, *FV, sv, uv, cv, tv0, tv1);
-            }
-            f0 -= T(0.5) * (tu0 + tv0);
-            f1 -= T(0.5) * (tu1 + tv1);
+            f0 -= T(0.5) * (trU[2 * nf + s] + trV[2 * nf + sv]);
+            f1 -= T(0.5) * (trU[3 * nf + s] + trV[3 * nf + sv]);
         }
         Fs0 += inv_h0 * f0;
         Fs1 += inv_h0 * f1;
