@@ -658,8 +658,8 @@ __device__ __noinline__ void int_row(const Grid3& g, const T* __restrict__ qo, c
 // The ends of the grid lines of direction D: the partial sums
 //   r_j = D_D q_Dj + D_DD^FC(c_DjDl) u_l + the SATs of the face there
 // of the first rows from the face (line_rows<O>(); along x1 up to x1lo, or from x1hi), which k3_div completes.
-// Nodes near several faces get a sum from each direction, so every direction stores where no other does (x3: in
-// the output field; x2, x1: in planes of their own, LineParts) and one launch takes all three.
+// They go to the output field.  A node near several faces gets a sum from each direction: x3's goes there, x2's and x1's
+// to planes of their own (LineParts), so that one launch takes all three.
 // A closure row reads NCLOSJ columns of the line, the same ones for every row of the end: a
 // thread reads the columns of u, q and the 6 coefficients once (order 6: 144 loads) for all its rows,
 // where a thread per node read them for each row.  The lanes of a warp lie along x1 (D = 1, 2: coalesced)
@@ -670,7 +670,7 @@ __device__ __noinline__ void int_row(const Grid3& g, const T* __restrict__ qo, c
 // of line ends per direction for 152 SMs).  With a thread for all rows of an end, in a launch per direction one after the
 // other, nothing hid the latencies of loads and instruction fetches: FP64 steps were slower than with a thread per node
 // (a step of 40^3, order 6: 321 us with a thread per node, 436 with a thread per end, now 199; order 4: 184, 258, 147; the
-// three launches of 64 x 61 x 57, order 4: 143 us, now 64).  FP32, 160 x 151 x 144, order 6: 91 us, now 76.
+// three launches of 64 x 61 x 57, order 4: 143 us, now 64).  FP32, 160 x 151 x 144, order 6: 91 us, now 78.
 constexpr int kLines = 32;                                    // line ends of a CTA
 template <int O> constexpr int kLineGroups = O == 2 ? 1 : 3;      // groups of rows
 template <int O> constexpr int kLineThreads = kLines * kLineGroups<O>;
@@ -682,10 +682,13 @@ template <typename T, int O, int D> constexpr int line_window() {      // column
 }
 template <typename T, int O> constexpr int line_smem() { return 12 * line_window<T, O, 0>() * (kLines + 1); }
 
-// partial sums of the line ends of x2 and x1 (see Box3 for x1's rows)
+// partial sums of x2 and x1 at nodes where another direction has one in the output field (planes over all the end rows;
+// see Box3 for x1's rows)
 template <typename T> struct LineParts {
     T *x2, *x1;
 };
+// whether index i of a direction is one of the rows that k3_lines takes there
+template <int O> __device__ __forceinline__ bool line_row(int i, int n) { return i < line_rows<O>() || i >= n - line_rows<O>(); }
 // element of the sum j at the node e-th row from the nearer face x2 (the rows of the high face after those of the low one)
 template <int O> __device__ __forceinline__ long long part_x2(const Grid3& g, int e, int j, int i1, int i3) {
     return ((long long)(e * 3 + j) * g.n[2] + i3) * g.s[1] + i1;
@@ -867,8 +870,8 @@ __device__ __forceinline__ void line_ends(const Grid3& g, const Box3& bx, const 
             if (G * R3 > RX && r0 + r >= RX) continue;
             if constexpr (D == 0) sm[(j * RX + r0 + r) * (NL + 1) + tx] = rr[r][j];
             else if (live) {
-                if constexpr (D == 2) un[j * fs + o + (r0 + r) * Ss] = rr[r][j];
-                else parts.x2[part_x2<O>(g, side * line_rows<O>() + r0 + r, j, ia, ib)] = rr[r][j];
+                if (D == 1 && line_row<O>(ib, g.n[2])) parts.x2[part_x2<O>(g, side * line_rows<O>() + r0 + r, j, ia, ib)] = rr[r][j];
+                else un[j * fs + o + (r0 + r) * Ss] = rr[r][j];
             }
         }
     if constexpr (D == 0) {
@@ -878,15 +881,26 @@ __device__ __forceinline__ void line_ends(const Grid3& g, const Box3& bx, const 
         for (int idx = threadIdx.x; idx < NL * nr; idx += NT) {
             const int n = idx / nr, r = idx - n * nr, line = blk * NL + n;
             if (line >= lines) continue;
+            const int l3 = line / na, l2 = line - l3 * na;
+            const bool own = line_row<O>(l2, g.n[1]) || line_row<O>(l3, g.n[2]);
+            const long long ol = face_node(line) + r * Ss;
 #pragma unroll
-            for (int j = 0; j < 3; ++j) parts.x1[part_x1(g, bx, side, j, line, r)] = sm[(j * RX + r) * (NL + 1) + n];
+            for (int j = 0; j < 3; ++j) {
+                const T v = sm[(j * RX + r) * (NL + 1) + n];
+                if (own) parts.x1[part_x1(g, bx, side, j, line, r)] = v;
+                else un[j * fs + ol] = v;
+            }
         }
         if (live && group == 0) {
+            const bool own = line_row<O>(ia, g.n[1]) || line_row<O>(ib, g.n[2]);
             for (int r = RX; r < rows1; ++r) {
                 T v[3] = {T(0), T(0), T(0)};
                 int_row<T, O, 0>(g, q + o + r * Ss, cp + r * Ss, u + o + r * Ss, v);
 #pragma unroll
-                for (int j = 0; j < 3; ++j) parts.x1[part_x1(g, bx, side, j, tl, r)] = v[j];
+                for (int j = 0; j < 3; ++j) {
+                    if (own) parts.x1[part_x1(g, bx, side, j, tl, r)] = v[j];
+                    else un[j * fs + o + r * Ss] = v[j];
+                }
             }
         }
     }
@@ -923,12 +937,12 @@ __device__ __forceinline__ void div_int_dir(const Grid3& g, const T* __restrict_
 struct DivShape {
     int by, minb;
 };
-constexpr DivShape kDivShapes[4] = {{4, 5}, {4, 6}, {8, 3}, {2, 10}};
+constexpr DivShape kDivShapes[4] = {{4, 4}, {4, 6}, {8, 3}, {2, 10}};
 
 // Every node: the interior rows of the directions whose end rows k3_lines has not taken, on top of its partial
 // sums where it has, then the store.  NV consecutive x1 nodes per thread read as one vector
 // (float2 for FP32); the last pair of an odd row covers one element of the row's padding, whose value no
-// node reads.  160 x 151 x 144, FP32, order 6: 191 us (the
+// node reads.  160 x 151 x 144, FP32, order 6: 181 us, with the cap at 96 registers 183 (the
 // kernel with closure rows and SATs behind calls: 328 us for the x1-interior columns).
 template <typename T, int O, int MODE, int NV, int BY, int MINB>
 __global__ void __launch_bounds__(32 * BY, MINB) k3_div(Grid3 g, Box3 bx, const T* __restrict__ u,
@@ -959,17 +973,21 @@ __global__ void __launch_bounds__(32 * BY, MINB) k3_div(Grid3 g, Box3 bx, const 
 #pragma unroll
             for (int n = 0; n < NV; ++n) r[n][j] += v[n];
         };
-        const int e2 = i2 < NR ? i2 : NR + g.n[1] - 1 - i2, side = i1 >= bx.x1hi;
-        const long long line = (long long)i3 * g.n[1] + i2;
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            if (!in3) add(un + j * fs + o, j);
-            if (!in2) add(parts.x2 + part_x2<O>(g, e2, j, i1, i3), j);
-            if (!in1) {
+        for (int j = 0; j < 3; ++j) add(un + j * fs + o, j);
+        if (!in2 && !in3) {
+            const int e2 = i2 < NR ? i2 : NR + g.n[1] - 1 - i2;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) add(parts.x2 + part_x2<O>(g, e2, j, i1, i3), j);
+        }
+        if (!in1 && !(in2 && in3)) {
+            const int side = i1 >= bx.x1hi;
+            const long long line = (long long)i3 * g.n[1] + i2;
+#pragma unroll
+            for (int j = 0; j < 3; ++j)
 #pragma unroll
                 for (int n = 0; n < NV; ++n)
                     if (i1 + n < g.n[0]) r[n][j] += parts.x1[part_x1(g, bx, side, j, line, side ? g.n[0] - 1 - i1 - n : i1 + n)];
-            }
         }
     }
     if (in1) div_int_x1<T, O, NV>(q + o, cd + o, up, fs, T(g.ih[0]), r);
