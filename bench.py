@@ -38,9 +38,9 @@ UNIT = "node-updates/s"
 # 1/(rho J) 1 = 19 words
 BYTES_PER_NODE = {"fp32": 76, "fp64": 136}
 # DRAM bytes per node of one FP32 interior launch (dram__bytes_read.sum + dram__bytes_write.sum of
-# k_interior_march_multi<6,3> captured at 2 x 1601x801, scaled by nodes).  Set to None whenever that
+# k_interior_march_multi<6,3> captured at 2 x 1601x801, scaled by interior nodes).  Set to None whenever that
 # kernel changes until it is measured again.
-TRAFFIC_BYTES_PER_NODE = {"fp32": None, "fp64": None}
+TRAFFIC_BYTES_PER_NODE = {"fp32": 73.0, "fp64": None}
 FALLBACK_HBM_GBS = 6800.0
 N1, N2 = 4001, 2001
 # crop of the workload the oracle is timed on: a 401-column window around the source spanning
@@ -370,10 +370,10 @@ RK4_WORDS_PER_STAGE = (4 * 13 + 2 + 6 + 6 + 10 + 3 * 4 + 6) / 4
 WIDE_WORDS_IMPLEMENTED = {"fp32": 19, "fp64": 27}
 
 
-# FP64 operations of k_interior_edges<double, 6, 0, 32, 16> per interior node, counted from its source (narrow rows
-# 120, mixed fluxes with their halos 56, their divergence 36, update 9), and the FP64 peak
+# FP64 operations of k_interior_edges<double, 6, 0, 32, 16> per interior node (ncu thread-level counts
+# 2 x DFMA + DADD + DMUL over the 599,778 interior nodes of 2 x 801 x 401), and the FP64 peak
 # of the part: 152 SMs x 2 FP64 FMA per clock x 2 flops x 2.07 GHz
-FP64_FLOPS_PER_NODE = 221.0
+FP64_FLOPS_PER_NODE = 227.3
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 
 
@@ -843,8 +843,7 @@ def main():
     fam_ms, _ = S.sbp_profile_read()
     S.sbp_profile(False)
     interior_ms = fam_ms[0] / args.steps         # the interior launches of a step (both blocks)
-    # FP32: one launch covers the interior of both blocks; FP64: one launch per block
-    units_per_launch = interior_nodes if prec == "fp32" else interior_nodes // len(P.blocks)
+    units_per_launch = interior_nodes            # one launch covers the interior of both blocks
     bpn = BYTES_PER_NODE[prec]
     achieved = bpn * interior_nodes / (interior_ms / 1e3) / 1e9
     peak, peak_src = peaks()

@@ -4,10 +4,9 @@
 // middling grid leaves most of the chip idle in either kernel and waits for each one's latency and launch in
 // turn.  An interior tile then adds the off-strip source nodes that lie in it (as k_sources does after the step kernels; the same
 // arithmetic), which saves that launch as well.
-// A step of one block, FP32, order 6, with a source inside, against separate launches: 201^2 36.6 -> 16.5 us, 601^2
-// 37.7 -> 22.7, 1001^2 46.1 -> 29.9, but 1401^2 67.8 -> 72.7 (the strips by 128 threads then cost more than the
-// launches do); FP64, order 6: 201^2 45 -> 33 us,
-// 601^2 158 -> 136; order 4: 101^2 41 -> 27.
+// A step of one block, FP32, order 6, with a source inside, against separate launches: 201^2 36.6 -> 14.7 us, 601^2
+// 37.7 -> 20.6, 1001^2 46.1 -> 28.7, but 1401^2 66.6 -> 72.7 (the strips by 128 threads then cost more than the
+// launches do); FP64, order 6: 201^2 45 -> 32 us, 601^2 158 -> 135; order 4: 101^2 41 -> 23.
 #pragma once
 #include "sbp_interior_march.cuh"
 #include "sbp_kernels.cuh"
